@@ -8,6 +8,7 @@
 #include <string>
 #include <vector>
 
+#include "hybrid.h"
 #include "rs_device.cuh"
 #include "rs_internal.h"
 #include "rsort.h"
@@ -81,10 +82,6 @@ rs_status device_state(DeviceState** out) {
       for (int i = 0; i < cnt; ++i) {
         RS_CUDA(cudaFuncSetAttribute(ks[i].func, cudaFuncAttributeMaxDynamicSharedMemorySize, int(ks[i].smem)),
                 "cudaFuncSetAttribute(onesweep)");
-        if (ks[i].func_first)
-          RS_CUDA(cudaFuncSetAttribute(ks[i].func_first, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       int(ks[i].smem)),
-                  "cudaFuncSetAttribute(onesweep first pass)");
       }
       const HistKernel* h = hist_kernel(r);
       for (const void* f : h->funcs)
@@ -92,6 +89,7 @@ rs_status device_state(DeviceState** out) {
           RS_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(h->smem)),
                   "cudaFuncSetAttribute(hist)");
     }
+    RS_CUDA(prepare_hybrid(), "cudaFuncSetAttribute(hybrid)");
     RS_CUDA(prepare_hist64(), "cudaFuncSetAttribute(hist64)");
     for (const void* f : {msd_count_func(), msd_scatter_func()})
       RS_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(msd_smem())),
@@ -129,14 +127,16 @@ rs_status device_state(DeviceState** out) {
 // ---- tracing -------------------------------------------------------------------
 enum TraceKind {
   T_CLEAR = 0, T_HIST, T_SCAN, T_PASS8, T_PASS11, T_SEGOFF, T_SEGPLAN, T_SEGHIST, T_SEGSCAN, T_SEGPASS, T_LOCAL,
-  T_H2D, T_D2H, T_SPLIT, T_JOIN, T_MERGE, T_SELECT, T_MSDCOUNT, T_MSDSCAN, T_MSDSCATTER, T_FUSED, T_KINDS
+  T_H2D, T_D2H, T_SPLIT, T_JOIN, T_MERGE, T_SELECT, T_MSDCOUNT, T_MSDSCAN, T_MSDSCATTER, T_FUSED,
+  T_SAMPLE, T_COUNT, T_SPLIT0, T_SPLIT1, T_BUCKETS, T_KINDS
 };
 const char* const kTraceNames[T_KINDS] = {"clear",       "upfront_hist", "digit_scan", "onesweep_r8",
                                           "onesweep_r11", "seg_part_offsets", "seg_plan", "seg_hist",
                                           "seg_scan",    "seg_pass",     "local_sort", "copy_h2d",
                                           "copy_d2h",    "split64",      "join64",     "merge",
                                           "select",      "msd_count",    "msd_scan",   "msd_scatter",
-                                          "fused_sort"};
+                                          "fused_sort",  "sample",       "bucket_count", "split_high",
+                                          "split_low",   "bucket_sort"};
 
 // The selection of Sec. 4.2.1 with the paper's parameters: a 1000-point
 // sample (footnote 8), 64 cells, 65 % overlap, more than two problem cells;
@@ -338,17 +338,37 @@ rs_status make_plan(uint64_t n, bool pairs, const rs_plan* user, SortPlan* p, in
 
 // ---- temp layout ------------------------------------------------------------
 struct Layout {
-  size_t ctrl = 0;     // [0,16): tile tickets per pass; [16,32): skip flags
+  size_t ctrl = 0;     // words 0-3: tile tickets per pass; 4-7: skip flags; 12: barrier counter; 15: histogram blocks done
+  size_t cursors0 = 0; // [256] u32: the first pass's bucket cursors
   size_t hist = 0;     // [nd][2^R] u32
   size_t bases = 0;    // [nd][2^R] u32
   size_t status = 0;   // [num_tiles][2^R] status words
   size_t status_bytes = 0;
   size_t alt_k = 0, alt_v = 0;
-  size_t memset_bytes = 0;  // ctrl + hist, cleared before the histogram
+  size_t memset_bytes = 0;  // ctrl + hist (+ the buckets' counts), cleared before the histogram
+  // the sort by value buckets (buckets == 0: not offered at this size)
+  uint32_t buckets = 0, low_bits = 0, groups = 0;
+  size_t hctrl = 0, counts = 0, starts = 0, cursors = 0, group_cursors = 0, group_tiles = 0;
   size_t total = 0;
 };
 
-Layout make_layout(const SortPlan& p, uint64_t n, bool pairs) {
+// The value buckets of n keys (hybrid.cu): about 2,048 keys each, at most
+// kHybMaxBuckets, in groups of 2^low_bits that halve the bucket's bits
+// between the two splits.
+void plan_buckets(uint64_t n, uint32_t* buckets, uint32_t* low_bits, uint32_t* groups) {
+#ifndef BMEAN
+#define BMEAN 2048
+#endif
+  uint64_t b = (n + BMEAN - 1) / BMEAN;
+  if (b > kHybMaxBuckets) b = kHybMaxBuckets;
+  uint32_t bits = 0;
+  while ((uint64_t(1) << bits) < b) ++bits;
+  *buckets = uint32_t(b);
+  *low_bits = bits / 2;
+  *groups = uint32_t((b + (uint64_t(1) << *low_bits) - 1) >> *low_bits);
+}
+
+Layout make_layout(const SortPlan& p, uint64_t n, bool pairs, bool hybrid = false) {
   Layout L;
   const size_t digits = size_t(1) << p.R;
   size_t off = 0;
@@ -356,12 +376,31 @@ Layout make_layout(const SortPlan& p, uint64_t n, bool pairs) {
   off += kAlign;
   L.hist = off;
   off = align_up(off + size_t(p.nd) * digits * 4);
+  if (hybrid) {
+    plan_buckets(n, &L.buckets, &L.low_bits, &L.groups);
+    L.counts = off;
+    off = align_up(off + size_t(L.buckets) * 4);
+  }
   L.memset_bytes = off;
   L.bases = off;
   off = align_up(off + size_t(p.nd) * digits * 4);
+  L.cursors0 = off;
+  off = align_up(off + 256 * 4);
   L.status = off;
   L.status_bytes = (p.status_rows > p.num_tiles ? p.status_rows : p.num_tiles) * digits * (p.k->wide_status ? 8 : 4);
   off = align_up(off + L.status_bytes);
+  if (hybrid) {
+    for (size_t* at : {&L.starts, &L.cursors}) {
+      *at = off;
+      off = align_up(off + (size_t(L.buckets) + 1) * 4);
+    }
+    L.hctrl = off;
+    off += align_up(sizeof(HybCtrl));
+    for (size_t* at : {&L.group_cursors, &L.group_tiles}) {
+      *at = off;
+      off = align_up(off + 257 * 4);
+    }
+  }
   if (p.nd > 1 && n > 0) {
     L.alt_k = off;
     off = align_up(off + size_t(n) * 4);
@@ -398,15 +437,18 @@ void part_offsets_host(uint64_t n, uint32_t parts, uint64_t* out) {
 rs_status run_lsd(const SortPlan& p, const Layout& L, const uint32_t* keys_in, const uint32_t* vals_in,
                   uint32_t* keys_out, uint32_t* vals_out, uint32_t n, unsigned char* temp, bool force_all,
                   DeviceState* ds, cudaStream_t s, const uint32_t* vals2_in = nullptr, uint32_t* vals2_out = nullptr,
-                  uint32_t* vals2_alt = nullptr, const uint2* pair_vals_in = nullptr, uint2* pair_vals_out = nullptr) {
+                  uint32_t* vals2_alt = nullptr, const uint2* pair_vals_in = nullptr, uint2* pair_vals_out = nullptr,
+                  const uint32_t* gate = nullptr) {
   uint32_t* ctrl = reinterpret_cast<uint32_t*>(temp + L.ctrl);
   uint32_t* hist = reinterpret_cast<uint32_t*>(temp + L.hist);
   uint32_t* bases = reinterpret_cast<uint32_t*>(temp + L.bases);
   const size_t digits = size_t(1) << p.R;
-  RS_CUDA(traced(T_CLEAR, 0, s, [&] { return cudaMemsetAsync(temp, 0, L.memset_bytes, s); }),
-          "cudaMemsetAsync(temp)");
+  if (!gate)  // (a sort with a gate has cleared them)
+    RS_CUDA(traced(T_CLEAR, 0, s, [&] { return cudaMemsetAsync(temp, 0, L.memset_bytes, s); }),
+            "cudaMemsetAsync(temp)");
 
   HistArgs ha{};
+  ha.gate = gate;
   ha.keys = keys_in;
   ha.n = n;
   ha.num_digits = p.nd;
@@ -416,14 +458,25 @@ rs_status run_lsd(const SortPlan& p, const Layout& L, const uint32_t* keys_in, c
   ha.zero_vec4 = L.status_bytes / 16;
   ha.xform = p.xf;
   const HistKernel* hk = hist_kernel(p.R);
+  // byte digits: the histogram launch scans them too (control word 15 counts its blocks)
+  const bool scans = p.R == 8 && p.nd == 4 && L.cursors0;
+  uint32_t* cursors = scans && p.k->free_first && !vals_in && !force_all ? reinterpret_cast<uint32_t*>(temp + L.cursors0) : nullptr;
+  if (scans) {
+    ha.done = ctrl + 15;
+    ha.bases = bases;
+    ha.skip = force_all ? nullptr : ctrl + 4;
+    ha.cursors = cursors;
+  }
   const size_t work = (size_t(n) + 4095) / 4096;  // one block per 4096 keys at least
   unsigned hgrid = unsigned(ds->num_sms) * (hk->threads >= 1024 ? 1 : 2);
   if (work < hgrid) hgrid = unsigned(work > 0 ? work : 1);
   RS_CUDA(traced(T_HIST, n, s, [&] { return hk->launch(ha, hgrid, s); }), "launch upfront_hist");
 
-  ScanArgs sa{hist, bases, force_all ? nullptr : ctrl + 4, n};
-  RS_CUDA(traced(T_SCAN, 0, s, [&] { return scan_kernel(p.R)->launch(sa, unsigned(p.nd), s); }),
-          "launch digit_scan");
+  if (!scans) {
+    ScanArgs sa{hist, bases, force_all ? nullptr : ctrl + 4, n, gate};
+    RS_CUDA(traced(T_SCAN, 0, s, [&] { return scan_kernel(p.R)->launch(sa, unsigned(p.nd), s); }),
+            "launch digit_scan");
+  }
 
   for (int j = 0; j < p.nd; ++j) {
     PassArgs pa{};
@@ -448,12 +501,15 @@ rs_status run_lsd(const SortPlan& p, const Layout& L, const uint32_t* keys_in, c
     pa.err = ds->err;
     pa.xin = p.xf;   // the first executed pass maps the input keys
     pa.xout = p.xf;  // the last one maps them back
+    pa.gate = gate;
     pa.pair_in = pair_vals_in;  // 64-bit values read and written interleaved
     pa.pair_out = pair_vals_out;
-    // pass 0, when it runs, is the first executed pass: keys-only sorts rank it
-    // without keeping the order of equal digits (there is none to keep yet)
-    auto launch = (j == 0 && p.k->launch_first && !vals_in) ? p.k->launch_first : p.k->launch;
-    RS_CUDA(traced(p.R == 8 ? T_PASS8 : T_PASS11, n, s, [&] { return launch(pa, pass_grid(p, ds), s); }),
+    pa.cursors = cursors;
+    // pass 0, when it runs, is the first executed pass: sorts of keys alone have no order to keep yet
+    RS_CUDA(traced(p.R == 8 ? T_PASS8 : T_PASS11, n, s,
+                   [&] {
+                     return j == 0 && cursors ? launch_first_pass(pa, s) : p.k->launch(pa, pass_grid(p, ds), s);
+                   }),
             "launch onesweep");
   }
   return RS_OK;
@@ -706,6 +762,45 @@ rs_status run_msd(const SortPlan& p, const MsdLayout& M, const uint32_t* keys_in
   return run_segmented(M.seg, temp, bk, bv, keys_out, vals_out, ma.seg_off, kMsdBuckets, 3, p.xf, p.xf, ds, s);
 }
 
+// ---- the sort by value buckets -----------------------------------------------------
+// The sample, the buckets' path and, gated behind the sample's and the
+// counts' choice, the radix passes; see hybrid.cu.
+constexpr uint64_t kHybridMinKeys = uint64_t(1) << 17, kHybridMaxKeys = uint64_t(3) << 25;
+
+rs_status run_hybrid32(const SortPlan& p, const Layout& L, const uint32_t* keys_in, uint32_t* keys_out, uint32_t n,
+                       unsigned char* temp, DeviceState* ds, cudaStream_t s) {
+  HybArgs a{};
+  a.keys_in = keys_in;
+  a.keys_out = keys_out;
+  a.keys_alt = temp + L.alt_k;
+  a.n = n;
+  a.x = p.xf;
+  a.buckets = L.buckets;
+  a.low_bits = L.low_bits;
+  a.groups = L.groups;
+  a.bucket_cap = hyb_bucket_cap();
+  a.split_tile = hyb_split_tile(4);
+  a.ctrl = reinterpret_cast<HybCtrl*>(temp + L.hctrl);
+  a.counts = reinterpret_cast<uint32_t*>(temp + L.counts);
+  a.starts = reinterpret_cast<uint32_t*>(temp + L.starts);
+  a.cursors = reinterpret_cast<uint32_t*>(temp + L.cursors);
+  a.group_cursors = reinterpret_cast<uint32_t*>(temp + L.group_cursors);
+  a.group_tiles = reinterpret_cast<uint32_t*>(temp + L.group_tiles);
+  a.clear = reinterpret_cast<uint4*>(temp);
+  a.clear_vec4 = L.memset_bytes / 16;
+  a.err = ds->err;
+  const unsigned sms = unsigned(ds->num_sms);
+  const struct {
+    HybStep step;
+    int kind;
+  } steps[] = {{HybStep::kSample, T_SAMPLE}, {HybStep::kCount, T_COUNT}, {HybStep::kSplit0, T_SPLIT0},
+               {HybStep::kSplit1, T_SPLIT1}, {HybStep::kBuckets, T_BUCKETS}};
+  for (const auto& st : steps)
+    RS_CUDA(traced(st.kind, n, s, [&] { return launch_hybrid(a, st.step, 4, sms, s); }), "launch sort by buckets");
+  return run_lsd(p, L, keys_in, nullptr, keys_out, nullptr, n, temp, false, ds, s, nullptr, nullptr, nullptr, nullptr,
+                 nullptr, &a.ctrl->route);
+}
+
 // ---- the single-launch sort -----------------------------------------------------
 // Up to (resident blocks) x 9,216 keys with the automatic plan: clear + one
 // cooperative launch instead of clear + histogram + scans + four passes.  It
@@ -754,7 +849,8 @@ rs_status sort_impl(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* 
   const bool fusable = automatic && p.R == 8 && p.nd == 4 && !p.msd && !p.k->wide_status;
   if (fusable && n <= kFusedStatusMaxKeys)  // status rows for the single-launch sort's smallest tiles
     p.status_rows = size_t((n + fused_tile_keys(kFusedShapes - 1) - 1) / fused_tile_keys(kFusedShapes - 1));
-  Layout L = make_layout(p, n, pairs);
+  const bool hybrid = fusable && !pairs && n >= kHybridMinKeys && n <= kHybridMaxKeys;
+  Layout L = make_layout(p, n, pairs, hybrid);
   MsdLayout M;
   if (p.msd) {
     if (rs_status st2 = make_msd_layout(p, n, pairs, &M); st2 != RS_OK) return st2;
@@ -826,6 +922,7 @@ rs_status sort_impl(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* 
       return run_fused(p, L, keys_in, pairs ? vals_in : nullptr, keys_out, pairs ? vals_out : nullptr, uint32_t(n),
                        sh, static_cast<unsigned char*>(temp), ds, s);
   }
+  if (hybrid) return run_hybrid32(p, L, keys_in, keys_out, uint32_t(n), static_cast<unsigned char*>(temp), ds, s);
   return run_lsd(p, L, keys_in, pairs ? vals_in : nullptr, keys_out, pairs ? vals_out : nullptr, uint32_t(n),
                  static_cast<unsigned char*>(temp), false, ds, s);
 }
@@ -839,7 +936,7 @@ rs_status sort_impl(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* 
 // at the end.
 struct Layout64 {
   bool fused = false;
-  size_t ctrl = 0;    // [0, 8): tile tickets of the 8 passes; [8, 16): skip flags
+  size_t ctrl = 0;    // [0, 8): tile tickets of the 8 passes; [8, 16): skip flags; 16: histogram blocks done
   size_t hist = 0;    // [8][256]
   size_t bases = 0;   // [8][256]
   size_t status = 0, status_bytes = 0;
@@ -923,6 +1020,9 @@ rs_status run_lsd64(const SortPlan& p, const Layout64& L, const uint64_t* keys_i
     ha.hist = hist;
     ha.zero_ptr = reinterpret_cast<uint4*>(temp + L.status);
     ha.zero_vec4 = L.status_bytes / 16;
+    ha.done = ctrl + 16;  // the last block scans them
+    ha.bases = bases;
+    ha.skip = ctrl + 8;
     RS_CUDA(traced(T_HIST, n, s, [&] { return launch_hist64(ha, hgrid, s); }), "launch upfront_hist64");
   }
   for (int w = 0; w < (L.fused ? 0 : 2); ++w) {
@@ -936,8 +1036,10 @@ rs_status run_lsd64(const SortPlan& p, const Layout64& L, const uint64_t* keys_i
     ha.zero_vec4 = w == 0 ? L.status_bytes / 16 : 0;
     RS_CUDA(traced(T_HIST, n, s, [&] { return hk->launch(ha, hgrid, s); }), "launch upfront_hist");
   }
-  ScanArgs sa{hist, bases, ctrl + 8, n};
-  RS_CUDA(traced(T_SCAN, 0, s, [&] { return scan_kernel(8)->launch(sa, 8u, s); }), "launch digit_scan");
+  if (!L.fused) {
+    ScanArgs sa{hist, bases, ctrl + 8, n, nullptr};
+    RS_CUDA(traced(T_SCAN, 0, s, [&] { return scan_kernel(8)->launch(sa, 8u, s); }), "launch digit_scan");
+  }
   for (int j = 0; j < 8; ++j) {
     const bool high = j >= 4;  // which word carries the digit
     PassArgs pa{};
@@ -1402,7 +1504,7 @@ rs_status rs_digit_histograms(const uint32_t* keys, uint64_t n, uint32_t digit_b
   if (d_bases || d_skip) {
     uint32_t* b = d_bases;
     if (!b) return fail(RS_ERR_INVALID, "d_skip needs d_bases");
-    ScanArgs sa{d_hist, b, d_skip, uint32_t(n)};
+    ScanArgs sa{d_hist, b, d_skip, uint32_t(n), nullptr};
     RS_CUDA(traced(T_SCAN, 0, s, [&] { return scan_kernel(int(digit_bits))->launch(sa, unsigned(ha.num_digits), s); }),
             "launch digit_scan");
   }

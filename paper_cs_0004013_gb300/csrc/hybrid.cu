@@ -1,0 +1,514 @@
+// Sort by value buckets: two distributions by the keys' leading value range,
+// then every bucket sorted by one block in shared memory.
+//
+// Paper: the bucketing + local sort pipeline of Sec. 3 (count the keys per
+// bucket, cumulative totals, distribution, local sort of each cell's range),
+// chosen from a sample of the data as in Sec. 4.2.1, with the radix pipeline
+// as the way back.  The buckets are B equal slices of the keys' value range
+// (bucket = (key - lowest) * B / range), about 2,048 keys each, reached in two
+// distributions (first the bucket's high bits, then its low ones), because a
+// distribution to B places at once writes runs too short to be worth a
+// memory transaction.  The steps, each one launch:
+//   sample   one cluster reads an evenly spread sample: the value range, and
+//            whether the keys are spread evenly enough over it (else the
+//            radix passes sort them);
+//   counts   keys per bucket in one read; its last block scans them.  A
+//            bucket that would not fit the local sort also sends the sort to
+//            the radix passes;
+//   split    twice: tiles of keys go to their buckets' ranges;
+//   buckets  one block per bucket sorts it in place (local.cuh).
+// Every kernel returns at once when the sort takes the other way.
+//
+// Against the radix passes (8 digits of 8 bits for 64-bit keys, 4 for 32-bit
+// ones), the keys cross memory three times instead of four or eight, and keys
+// without payloads need no stable ranking: a key's place in its tile is one
+// shared atomic, and a tile's place in a bucket one global atomic.
+#include <cooperative_groups.h>
+
+#include <cstdint>
+
+#include "hybrid.h"
+#include "local.cuh"
+#include "split.cuh"
+
+namespace rs {
+namespace {
+
+constexpr int kSampleThreads = 1024;
+constexpr int kCountThreads = 1024;
+constexpr uint32_t kCoarse = 64;  // slices of the range for the evenness test
+
+// The linear map of a key's value to [0, 2^32): bucket = high word of the
+// product, place inside the bucket = low word.  Values outside the sampled
+// range [lo, hi] fall in the first or last bucket.  32-bit keys take the
+// offset and the product in one wide multiply-add: back = -lo * mult.
+template <typename K>
+struct ValueMap {
+  K lo, hi;
+  uint32_t sh, mult;
+  uint64_t back;
+  __device__ __forceinline__ K clamp(K k) const {
+    const K t = k > lo ? k : lo;
+    return t < hi ? t : hi;
+  }
+  // the product for a key inside [lo, hi]
+  __device__ __forceinline__ uint64_t product(K k) const {
+    if constexpr (sizeof(K) == 8) return uint64_t(uint32_t((k - lo) >> sh)) * mult;
+    else return uint64_t(k) * mult + back;
+  }
+  __device__ __forceinline__ uint32_t bucket(K k) const { return uint32_t(product(clamp(k)) >> 32); }
+};
+template <typename K>
+__device__ __forceinline__ ValueMap<K> load_map(const HybCtrl* c) {
+  return ValueMap<K>{K(c->lo), K(c->hi), c->sh, c->mult, 0ull - uint64_t(K(c->lo)) * c->mult};
+}
+
+// Bins of a bucket: the low word of the same product.  EDGE: the first and
+// last bucket, which also hold the values outside the sampled range.
+template <typename K, int NBITS, bool EDGE>
+struct BucketBins {
+  static constexpr bool kKnown = true;
+  ValueMap<K> m;
+  __device__ __forceinline__ uint32_t operator()(K k) const {
+    return uint32_t(m.product(EDGE ? m.clamp(k) : k)) >> (32 - NBITS);
+  }
+  __device__ __forceinline__ bool unique() const { return false; }
+};
+
+template <typename K>
+struct OrdOf;
+template <>
+struct OrdOf<uint32_t> {
+  using T = Ord32;
+  __device__ static T make(const HybArgs& a) { return Ord32{a.x}; }
+  __device__ static T identity() { return Ord32{KeyXform{0u, 0u}}; }
+};
+template <>
+struct OrdOf<uint64_t> {
+  using T = Ord64;
+  __device__ static T make(const HybArgs& a) { return Ord64{a.x64}; }
+  __device__ static T identity() { return Ord64{KeyXform64{0u, 0u, 0u}}; }
+};
+
+// ------------------------------------------------------------------ sample
+// One cluster of eight blocks.  The sample: S keys, one from each of S equal
+// stretches of the input at a place inside the stretch that a hash picks (a
+// periodic input does not line up with it).  Every block reads an eighth of
+// it into the first block's shared memory (one SM alone takes its scattered
+// reads one sector at a time), and the first block decides.  The keys count as spread
+// evenly when
+//  - no 64th of the range holds more than 1.5 times its share of the sample
+//    (uniform keys: 128 or more expected, five standard deviations below);
+//  - no bucket holds more than kFineLimit sampled keys (one expected at most);
+//  - few sampled keys are equal to another one: many equal keys end up in few
+//    bins of a bucket, which then takes the digit passes.
+constexpr int kSampleBlocks = 8;
+constexpr uint32_t kFineLimit = 12;
+template <typename K>
+struct SampleLayout {
+  static constexpr int S = 8192;
+  static constexpr int PER = S / kSampleThreads;                 // of the deciding block
+  static constexpr int LOADS = S / (kSampleThreads * kSampleBlocks);  // of every block
+  static constexpr size_t OFF_KEYS = size_t(kHybMaxBuckets) * 4;  // behind the fine counts (later the hash slots)
+  static constexpr size_t OFF_RED = OFF_KEYS + size_t(S) * sizeof(K);
+  static constexpr size_t OFF_COARSE = OFF_RED + 64 * 8;
+  static constexpr size_t SMEM = OFF_COARSE + kCoarse * 4;
+};
+
+template <typename K>
+__global__ void __cluster_dims__(kSampleBlocks, 1, 1) __launch_bounds__(kSampleThreads, 1)
+    sample_kernel(const HybArgs a) {
+  using L = SampleLayout<K>;
+  namespace cg = cooperative_groups;
+  extern __shared__ __align__(16) unsigned char smem[];
+  uint32_t* s_fine = reinterpret_cast<uint32_t*>(smem);
+  K* s_keys = reinterpret_cast<K*>(smem + L::OFF_KEYS);
+  K* s_red = reinterpret_cast<K*>(smem + L::OFF_RED);
+  uint32_t* s_coarse = reinterpret_cast<uint32_t*>(smem + L::OFF_COARSE);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const auto ord = OrdOf<K>::make(a);
+  const K* in = reinterpret_cast<const K*>(a.keys_in);
+  const uint64_t n = a.n;
+  const uint32_t stretch = uint32_t(n / L::S);
+  cg::cluster_group cluster = cg::this_cluster();
+  K got[L::LOADS];
+#pragma unroll
+  for (int i = 0; i < L::LOADS; ++i) {
+    const uint32_t q = (i * kSampleBlocks + blockIdx.x) * kSampleThreads + tid;
+    uint32_t h = q * 0x9E3779B1u;
+    h ^= h >> 15;
+    const uint64_t pos = (uint64_t(q) * n) / L::S + (stretch > 1 ? __umulhi(h * 0x85EBCA77u, stretch) : 0u);
+    got[i] = ord.map(ld_elem(in + (pos < n ? pos : n - 1)));
+  }
+  if (blockIdx.x == 0) {
+    uint4* f4 = reinterpret_cast<uint4*>(smem);
+    for (uint32_t i = tid; i < (a.buckets + 3) / 4; i += kSampleThreads) f4[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (tid < int(kCoarse)) s_coarse[tid] = 0u;
+  }
+  // the first block runs: its shared memory may be written
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+  K* to = cluster.map_shared_rank(s_keys, 0);
+#pragma unroll
+  for (int i = 0; i < L::LOADS; ++i) to[(i * kSampleBlocks + blockIdx.x) * kSampleThreads + tid] = got[i];
+  cluster.sync();
+  if (blockIdx.x != 0) {  // the others clear what the launches that follow start from
+    for (size_t i = size_t(blockIdx.x - 1) * kSampleThreads + tid; i < a.clear_vec4;
+         i += (kSampleBlocks - 1) * kSampleThreads)
+      a.clear[i] = make_uint4(0u, 0u, 0u, 0u);
+    return;
+  }
+
+  K key[L::PER];
+  K lo = ~K(0), hi = 0;
+#pragma unroll
+  for (int i = 0; i < L::PER; ++i) {
+    key[i] = s_keys[i * kSampleThreads + tid];
+    lo = key[i] < lo ? key[i] : lo;
+    hi = key[i] > hi ? key[i] : hi;
+  }
+  warp_min_max(lo, hi);
+  if (lane == 0) {
+    s_red[warp] = lo;
+    s_red[32 + warp] = hi;
+  }
+  __syncthreads();
+  lo = s_red[lane];
+  hi = s_red[32 + lane];
+  warp_min_max(lo, hi);
+  // a little wider than the sample, so that the values outside it (about
+  // 1 / S of the keys on either side) have buckets of their own
+  const K ext = (hi - lo) / (L::S / 8);
+  ValueMap<K> m;
+  m.lo = lo > ext ? lo - ext : K(0);
+  m.hi = hi < ~K(0) - ext ? hi + ext : ~K(0);
+  const K span = m.hi - m.lo;
+  const int bits = span == 0 ? 1 : 64 - __clzll((long long)(uint64_t)span);
+  m.sh = bits > 32 ? uint32_t(bits - 32) : 0u;
+  const uint64_t range = uint64_t(span >> m.sh) + 1;  // <= 2^32
+  m.mult = uint32_t((uint64_t(a.buckets) << 32) / (range > a.buckets ? range : uint64_t(a.buckets) + 1));
+  m.back = 0ull - uint64_t(m.lo) * m.mult;
+  bool bad = range <= a.buckets;
+#pragma unroll
+  for (int i = 0; i < L::PER; ++i) {
+    const uint32_t b = m.bucket(key[i]);
+    if (atomicAdd(&s_fine[b], 1u) >= kFineLimit) bad = true;
+    atomicAdd(&s_coarse[(b * kCoarse) / a.buckets], 1u);
+  }
+  __syncthreads();
+  if (a.buckets >= 4 * kCoarse && tid < int(kCoarse) && s_coarse[tid] * kCoarse * 2 > uint32_t(L::S) * 3) bad = true;
+  // equal keys: each writes its number to a hash slot, and reads back whose
+  // number stayed; an equal key's means a duplicate
+  uint16_t* s_slot = reinterpret_cast<uint16_t*>(smem);
+  auto slot_of = [](K k) { return (uint32_t(k ^ (uint64_t(k) >> 32)) * 0x9E3779B1u) >> 17; };
+#pragma unroll
+  for (int i = 0; i < L::PER; ++i) s_slot[slot_of(key[i])] = uint16_t(i * kSampleThreads + tid);
+  __syncthreads();
+  uint32_t dups = 0;
+#pragma unroll
+  for (int i = 0; i < L::PER; ++i) {
+    const uint32_t o = s_slot[slot_of(key[i])];
+    dups += o != uint32_t(i * kSampleThreads + tid) && s_keys[o] == key[i];
+  }
+  dups = __reduce_add_sync(0xffffffffu, dups);
+  uint32_t* s_sum = reinterpret_cast<uint32_t*>(s_red);
+  if (lane == 0) s_sum[warp] = dups;
+  bad = __syncthreads_or(bad);
+  dups = __reduce_add_sync(0xffffffffu, s_sum[lane]);
+  // equal keys per value of about c among n keys give S^2 c / (2 n) such
+  // pairs in the sample; c = 16 is what the bins still take well
+  if (uint64_t(dups) * n > uint64_t(L::S) * L::S * 8 + 16 * n) bad = true;
+  if (tid == 0) {
+    HybCtrl* c = a.ctrl;
+    c->lo = m.lo;
+    c->hi = m.hi;
+    c->sh = m.sh;
+    c->mult = m.mult;
+    c->done = 0;
+    c->tiles_b = 0;
+    c->route = bad ? kHybRadix : kHybBuckets;
+  }
+}
+
+// ------------------------------------------------------------------ counts
+// Keys per bucket.  32-bit shared counters for every bucket (up to 128 KiB),
+// one shared reduction per key; the blocks add them into the global counts.
+// The last block to finish scans the counts: the buckets' starts and cursors,
+// the tiles of the second split, and whether every bucket fits the local sort.
+template <typename K>
+__global__ void __launch_bounds__(kCountThreads, 1) bucket_count_kernel(const HybArgs a) {
+  extern __shared__ __align__(16) uint32_t sh[];  // [buckets]
+  __shared__ uint32_t s_warp[32];
+  __shared__ uint32_t s_last;
+  const int tid = threadIdx.x;
+  wait_for_chain();
+  if (a.ctrl->route != kHybBuckets) return;
+  const uint32_t B = a.buckets;
+  for (uint32_t i = tid; i < B; i += kCountThreads) sh[i] = 0u;
+  const ValueMap<K> m = load_map<K>(a.ctrl);
+  const auto ord = OrdOf<K>::make(a);
+  const uint32_t base = smem_addr(sh);
+  __syncthreads();
+  const uint32_t n = a.n;
+  const size_t stride = size_t(gridDim.x) * kCountThreads;
+  auto count = [&](K k) { sh_red_add(base + 4u * m.bucket(ord.map(k)), 1u); };
+  // 16-byte vectors between the first and last 16-byte boundary
+  constexpr uint32_t PV = 16 / sizeof(K);
+  const K* in = reinterpret_cast<const K*>(a.keys_in);
+  uint32_t head = uint32_t((PV - (reinterpret_cast<uintptr_t>(in) / sizeof(K)) % PV) % PV);
+  if (head > n) head = n;
+  const size_t nvec = size_t(n - head) / PV;
+  const uint32_t tail = head + uint32_t(nvec * PV);
+  if (blockIdx.x == gridDim.x - 1) {
+    for (uint32_t i = tid; i < head; i += kCountThreads) count(in[i]);
+    for (uint32_t i = tail + tid; i < n; i += kCountThreads) count(in[i]);
+  }
+  const uint4* v4 = reinterpret_cast<const uint4*>(in + head);
+  auto count4 = [&](const uint4& x) {
+    if constexpr (sizeof(K) == 4) {
+      count(x.x); count(x.y); count(x.z); count(x.w);
+    } else {
+      count((uint64_t(x.y) << 32) | x.x);
+      count((uint64_t(x.w) << 32) | x.z);
+    }
+  };
+  size_t i = size_t(blockIdx.x) * kCountThreads + tid;
+  for (; i + 7 * stride < nvec; i += 8 * stride) {
+    uint4 x[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) x[q] = ld_stream4(v4 + i + q * stride);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) count4(x[q]);
+  }
+  for (; i < nvec; i += stride) count4(ld_stream4(v4 + i));
+  // status words of the splits' chained scans
+  for (size_t z = size_t(blockIdx.x) * kCountThreads + tid; z < a.zero_vec4; z += stride)
+    a.zero_ptr[z] = make_uint4(0u, 0u, 0u, 0u);
+  __syncthreads();
+  for (uint32_t b = tid; b < B; b += kCountThreads)
+    if (sh[b]) atomicAdd(&a.counts[b], sh[b]);
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) s_last = atomicAdd(&a.ctrl->done, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  // the last block: exclusive scan of the counts, a contiguous run of buckets per
+  // warp (32 consecutive ones per step: no bank conflicts), the warps' totals scanned between
+  const int lane = tid & 31, warp = tid >> 5;
+  constexpr uint32_t WARPS = kCountThreads / 32;
+  const uint32_t per = (B + WARPS * 32 - 1) / (WARPS * 32);  // steps of a warp
+  const uint32_t b0 = uint32_t(warp) * per * 32 + lane;
+  uint32_t sum = 0, most = 0;
+  for (uint32_t i = 0; i < per; ++i) {
+    const uint32_t b = b0 + i * 32;
+    const uint32_t c = b < B ? __ldcg(&a.counts[b]) : 0u;
+    if (b < B) sh[b] = c;
+    sum += c;
+    most = c > most ? c : most;
+  }
+  sum = __reduce_add_sync(0xffffffffu, sum);
+  __syncwarp();
+  uint32_t run = block_exclusive_sum<kCountThreads>(lane == 0 ? sum : 0u, s_warp);
+  run = __shfl_sync(0xffffffffu, run, 0);
+  for (uint32_t i = 0; i < per; ++i) {
+    const uint32_t b = b0 + i * 32;
+    const uint32_t c = b < B ? sh[b] : 0u;
+    uint32_t inc = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += y;
+    }
+    if (b < B) sh[b] = run + inc - c;
+    run += __shfl_sync(0xffffffffu, inc, 31);
+  }
+  const bool over = __syncthreads_or(most > a.bucket_cap);
+  if (over) {
+    if (tid == 0) a.ctrl->route = kHybRadix;
+    return;
+  }
+  for (uint32_t b = tid; b < B; b += kCountThreads) {
+    a.starts[b] = sh[b];
+    a.cursors[b] = sh[b];
+  }
+  if (tid == 0) a.starts[B] = n;
+  // groups of the first split: starts and cursors, and the second split's tiles
+  const uint32_t groups = a.groups;
+  uint32_t g0 = 0, g1 = 0;
+  if (tid < int(groups)) {
+    g0 = sh[tid << a.low_bits];
+    g1 = ((uint32_t(tid) + 1) << a.low_bits) < B ? sh[(tid + 1) << a.low_bits] : n;
+    a.group_cursors[tid] = g0;
+  }
+  const uint32_t tiles = (g1 - g0 + a.split_tile - 1) / a.split_tile;
+  const uint32_t first = block_exclusive_sum<kCountThreads>(tid < int(groups) ? tiles : 0u, s_warp);
+  if (tid < int(groups)) a.group_tiles[tid] = first;
+  if (tid == int(groups) - 1) {
+    a.group_tiles[groups] = first + tiles;
+    a.ctrl->tiles_b = first + tiles;
+  }
+}
+
+// ------------------------------------------------------------------- split
+// One distribution of keys without payloads (split.cuh).  LEVEL 0: the
+// input's tiles to the groups (the bucket's high bits); LEVEL 1: each group's
+// tiles to its buckets (the low bits).
+template <typename K, int THREADS, int ITEMS, int MINB, int LEVEL>
+__global__ void __launch_bounds__(THREADS, MINB) split_kernel(const HybArgs a) {
+  using L = SplitLayout<K, THREADS, ITEMS>;
+  constexpr uint32_t TILE = L::TILE;
+  extern __shared__ __align__(16) unsigned char smem[];
+  wait_for_chain();
+  if (a.ctrl->route != kHybBuckets) return;
+  const int tid = threadIdx.x;
+  const ValueMap<K> m = load_map<K>(a.ctrl);
+  const uint32_t dshift = LEVEL == 0 ? a.low_bits : 0u;
+  const uint32_t dmask = LEVEL == 0 ? 0xffu : (1u << a.low_bits) - 1u;
+  auto digit = [&](K k) { return (m.bucket(k) >> dshift) & dmask; };
+  uint32_t base, valid;
+  uint32_t* cursors;
+  if constexpr (LEVEL == 0) {
+    base = blockIdx.x * TILE;
+    valid = a.n - base < TILE ? a.n - base : TILE;
+    cursors = a.group_cursors;
+  } else {
+    // the tile's group, found by every thread looking at one
+    uint32_t* s_job = reinterpret_cast<uint32_t*>(smem + L::OFF_JOB);
+    if (blockIdx.x >= a.ctrl->tiles_b) return;
+    if (tid < int(a.groups)) {
+      const uint32_t f = a.group_tiles[tid], e = a.group_tiles[tid + 1];
+      if (f <= blockIdx.x && blockIdx.x < e) {
+        const uint32_t g0 = a.starts[tid << a.low_bits];
+        const uint32_t last = (uint32_t(tid) + 1) << a.low_bits;
+        const uint32_t g1 = a.starts[last < a.buckets ? last : a.buckets];
+        const uint32_t b = g0 + (blockIdx.x - f) * TILE;
+        s_job[0] = b;
+        s_job[1] = g1 - b < TILE ? g1 - b : TILE;
+        s_job[2] = uint32_t(tid);
+      }
+    }
+    __syncthreads();
+    base = s_job[0];
+    valid = s_job[1];
+    cursors = a.cursors + (s_job[2] << a.low_bits);
+  }
+  const K* in = reinterpret_cast<const K*>(LEVEL == 0 ? a.keys_in : a.keys_alt) + base;
+  K* out = reinterpret_cast<K*>(LEVEL == 0 ? a.keys_alt : a.keys_out);
+  const auto ident = OrdOf<K>::identity();
+  const auto ordi = LEVEL == 0 ? OrdOf<K>::make(a) : ident;
+  if (valid == TILE) split_tile<K, THREADS, ITEMS, true>(in, valid, out, cursors, a.n, digit, ordi, ident, a.err, smem);
+  else split_tile<K, THREADS, ITEMS, false>(in, valid, out, cursors, a.n, digit, ordi, ident, a.err, smem);
+}
+
+// ----------------------------------------------------------------- buckets
+constexpr int kBucketThreads = 128, kBucketItems = 24, kBucketBits = 12;
+
+template <typename K, int VB, int MINB>
+__global__ void __launch_bounds__(kBucketThreads, MINB) bucket_sort_kernel(const HybArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  wait_for_chain();
+  if (a.ctrl->route != kHybBuckets) return;
+  const ValueMap<K> m = load_map<K>(a.ctrl);
+  using V = typename ValueOf<VB>::T;
+  const uint32_t b = blockIdx.x, s = a.starts[b], e = a.starts[b + 1];
+  if (s == e) return;
+  K* io = reinterpret_cast<K*>(a.keys_out) + s;
+  V* vio = VB ? reinterpret_cast<V*>(a.vals_out) + s : nullptr;
+  if (b == 0 || b == a.buckets - 1)
+    local_sort_array<kBucketThreads, kBucketItems, kBucketBits, VB, true>(
+        io, io, vio, vio, e - s, OrdOf<K>::identity(), OrdOf<K>::make(a), BucketBins<K, kBucketBits, true>{m}, smem);
+  else
+    local_sort_array<kBucketThreads, kBucketItems, kBucketBits, VB, true>(
+        io, io, vio, vio, e - s, OrdOf<K>::identity(), OrdOf<K>::make(a), BucketBins<K, kBucketBits, false>{m}, smem);
+}
+
+// ------------------------------------------------- first radix pass of keys
+// The first executed pass of a radix sort of keys without payloads: there is
+// no earlier order to keep, so it is a split by the lowest byte.
+__global__ void __launch_bounds__(kSplitThreads, kSplitBlocks) first_pass_kernel(const PassArgs a) {
+  using L = SplitLayout<uint32_t, kSplitThreads, kSplitItems>;
+  constexpr uint32_t TILE = L::TILE;
+  extern __shared__ __align__(16) unsigned char smem[];
+  if (gated_off(a.gate)) return;
+  const Route route = route_of(a.skip, 0, a.num_passes);
+  if (!route.active) return;
+  const uint32_t base = blockIdx.x * TILE, valid = a.n - base < TILE ? a.n - base : TILE;
+  uint32_t* out = route.dst == BUF_OUT ? a.keys_out : a.keys_alt;
+  const Ord32 ordi{a.xin}, ordo{route.last ? a.xout : KeyXform{0u, 0u}};
+  auto digit = [](uint32_t k) { return k & 0xffu; };
+  if (valid == TILE)
+    split_tile<uint32_t, kSplitThreads, kSplitItems, true>(a.keys_in + base, valid, out, a.cursors, a.n, digit, ordi,
+                                                           ordo, a.err, smem);
+  else
+    split_tile<uint32_t, kSplitThreads, kSplitItems, false>(a.keys_in + base, valid, out, a.cursors, a.n, digit, ordi,
+                                                            ordo, a.err, smem);
+}
+
+template <typename K>
+struct Kernels {
+  static constexpr int ST = kSplitThreads, SI = sizeof(K) == 4 ? kSplitItems : kSplitItems / 2, SB = kSplitBlocks;
+  using Split = SplitLayout<K, ST, SI>;
+  using Local = LocalLayout<kBucketThreads, kBucketItems, kBucketBits, K, 0, false>;
+  static constexpr int LB = sizeof(K) == 4 ? 8 : 4;
+  static cudaError_t prepare() {
+    cudaError_t e = cudaSuccess;
+    auto set = [&](const void* f, size_t bytes) {
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
+    };
+    set(reinterpret_cast<const void*>(&sample_kernel<K>), SampleLayout<K>::SMEM);
+    set(reinterpret_cast<const void*>(&bucket_count_kernel<K>), size_t(kHybMaxBuckets) * 4);
+    set(reinterpret_cast<const void*>(&split_kernel<K, ST, SI, SB, 0>), Split::SMEM);
+    set(reinterpret_cast<const void*>(&split_kernel<K, ST, SI, SB, 1>), Split::SMEM);
+    set(reinterpret_cast<const void*>(&bucket_sort_kernel<K, 0, LB>), Local::SMEM);
+    return e;
+  }
+};
+
+}  // namespace
+
+uint32_t hyb_split_tile(int key_bytes) {
+  return key_bytes == 4 ? uint32_t(Kernels<uint32_t>::Split::TILE) : uint32_t(Kernels<uint64_t>::Split::TILE);
+}
+uint32_t hyb_bucket_cap() { return uint32_t(kBucketThreads * kBucketItems); }
+
+cudaError_t launch_first_pass(const PassArgs& a, cudaStream_t s) {
+  using L = SplitLayout<uint32_t, kSplitThreads, kSplitItems>;
+  const unsigned tiles = unsigned((uint64_t(a.n) + L::TILE - 1) / L::TILE);
+  return launch_chained(&first_pass_kernel, tiles, kSplitThreads, L::SMEM, s, a.gate != nullptr, a);
+}
+
+cudaError_t prepare_hybrid() {
+  cudaError_t e = Kernels<uint32_t>::prepare();
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(reinterpret_cast<const void*>(&first_pass_kernel),
+                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             int(SplitLayout<uint32_t, kSplitThreads, kSplitItems>::SMEM));
+  return e == cudaSuccess ? Kernels<uint64_t>::prepare() : e;
+}
+
+template <typename K>
+static cudaError_t launch(const HybArgs& a, HybStep step, unsigned sms, cudaStream_t s) {
+  using T = Kernels<K>;
+  const unsigned tiles = (a.n + a.split_tile - 1) / a.split_tile;
+  switch (step) {
+    case HybStep::kSample:
+      sample_kernel<K><<<kSampleBlocks, kSampleThreads, SampleLayout<K>::SMEM, s>>>(a);
+      return cudaGetLastError();
+    case HybStep::kCount:
+      return launch_chained(&bucket_count_kernel<K>, sms, kCountThreads, size_t(a.buckets) * 4, s, true, a);
+    case HybStep::kSplit0:
+      return launch_chained(&split_kernel<K, T::ST, T::SI, T::SB, 0>, tiles, T::ST, T::Split::SMEM, s, true, a);
+    case HybStep::kSplit1:
+      return launch_chained(&split_kernel<K, T::ST, T::SI, T::SB, 1>, tiles + a.groups, T::ST, T::Split::SMEM, s, true,
+                            a);
+    case HybStep::kBuckets:
+      return launch_chained(&bucket_sort_kernel<K, 0, T::LB>, a.buckets, kBucketThreads, T::Local::SMEM, s, true, a);
+  }
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_hybrid(const HybArgs& a, HybStep step, int key_bytes, unsigned sms, cudaStream_t s) {
+  return key_bytes == 4 ? launch<uint32_t>(a, step, sms, s) : launch<uint64_t>(a, step, sms, s);
+}
+
+}  // namespace rs

@@ -1,0 +1,57 @@
+// The sort by value buckets (hybrid.cu): its launches' arguments.
+#pragma once
+
+#include "rs_internal.h"
+
+namespace rs {
+
+constexpr uint32_t kHybMaxBuckets = 32768;  // 32-bit shared counters of all of them: 128 KiB
+
+// Which way the sort goes, decided on the device (HybCtrl::route).
+enum : uint32_t { kHybRadix = 1, kHybBuckets = 2 };
+
+struct HybCtrl {
+  uint64_t lo, hi;     // the value map (hybrid.cu, ValueMap)
+  uint32_t sh, mult;
+  uint32_t route;
+  uint32_t done;       // count blocks that have finished
+  uint32_t tiles_b;    // tiles of the second split
+  uint32_t reserved[7];
+};
+static_assert(sizeof(HybCtrl) == 64, "one cache line or less");
+
+struct HybArgs {
+  const void* keys_in;
+  void* keys_out;
+  void* keys_alt;
+  const void* vals_in;
+  void* vals_out;
+  void* vals_alt;
+  uint32_t n;
+  KeyXform x;       // order map of 32-bit keys
+  KeyXform64 x64;   // of 64-bit keys
+  uint32_t buckets;     // B
+  uint32_t low_bits;    // the second split's digit: the bucket's low bits
+  uint32_t groups;      // digits of the first split
+  uint32_t bucket_cap;  // keys the local sort takes
+  uint32_t split_tile;  // keys of a split tile
+  HybCtrl* ctrl;
+  uint32_t* counts;         // [B], zero before the counts
+  uint32_t* starts;         // [B + 1]
+  uint32_t* cursors;        // [B]
+  uint32_t* group_cursors;  // [256]
+  uint32_t* group_tiles;    // [257]
+  uint4* clear;             // cleared by the sample
+  size_t clear_vec4;
+  uint4* zero_ptr;          // cleared by the counts
+  size_t zero_vec4;
+  uint32_t* err;
+};
+
+enum class HybStep { kSample, kCount, kSplit0, kSplit1, kBuckets };
+uint32_t hyb_split_tile(int key_bytes);
+uint32_t hyb_bucket_cap();
+cudaError_t prepare_hybrid();
+cudaError_t launch_hybrid(const HybArgs& a, HybStep step, int key_bytes, unsigned sms, cudaStream_t s);
+
+}  // namespace rs

@@ -660,6 +660,7 @@ template <int R, int THREADS, int ITEMS, int NV, typename S, int MINB, bool EARL
 __global__ void __launch_bounds__(THREADS, MINB) onesweep_kernel(const PassArgs a) {
   using L = OnesweepLayout<R, THREADS, ITEMS, NV>;
   extern __shared__ __align__(16) unsigned char smem[];
+  if (gated_off(a.gate)) return;
   const Route route = route_of(a.skip, a.pass, a.num_passes);
   if (!route.active) return;
   const uint32_t* kin = route.src == BUF_IN ? a.keys_in : (route.src == BUF_OUT ? a.keys_out : a.keys_alt);
@@ -705,8 +706,8 @@ __global__ void __launch_bounds__(THREADS, MINB) onesweep_kernel(const PassArgs 
 template <int R, int THREADS, int ITEMS, int NV, typename S, int MINB, bool EARLY_LB, bool PIO>
 cudaError_t launch_onesweep(const PassArgs& a, unsigned grid, cudaStream_t s) {
   using L = OnesweepLayout<R, THREADS, ITEMS, NV>;
-  onesweep_kernel<R, THREADS, ITEMS, NV, S, MINB, EARLY_LB, PIO><<<grid, THREADS, L::SMEM, s>>>(a);
-  return cudaGetLastError();
+  return launch_chained(&onesweep_kernel<R, THREADS, ITEMS, NV, S, MINB, EARLY_LB, PIO>, grid, THREADS, L::SMEM, s,
+                        a.gate != nullptr, a);
 }
 
 template <int R, int THREADS, int ITEMS, int NV, typename S, int MINB, bool EARLY_LB, bool PIO = false>

@@ -364,11 +364,12 @@ __device__ __forceinline__ void onesweep2_tile(const Tile2Job& job, unsigned cha
 }
 
 
-template <int THREADS, int ITEMS, int NV, typename S, int MINB, bool EARLY_LB, int LB, bool UNSTABLE>
+template <int THREADS, int ITEMS, int NV, typename S, int MINB, bool EARLY_LB, int LB>
 __global__ void __launch_bounds__(THREADS, MINB) onesweep2_kernel(const PassArgs a) {
   using L = Onesweep2Layout<THREADS, ITEMS, NV>;
   extern __shared__ __align__(16) unsigned char smem[];
-  const Route route = route_of(a.skip, a.pass, a.num_passes);
+  if (gated_off(a.gate)) return;
+  const Route route = route_of(a.skip, a.pass, a.num_passes, a.cursors != nullptr);
   if (!route.active) return;
   Tile2Job job;
   job.kin = route.src == BUF_IN ? a.keys_in : (route.src == BUF_OUT ? a.keys_out : a.keys_alt);
@@ -397,21 +398,14 @@ __global__ void __launch_bounds__(THREADS, MINB) onesweep2_kernel(const PassArgs
   }
   __syncthreads();
   job.tile = *s_tile;
-  if constexpr (UNSTABLE) {
-    // the first executed pass of this sort, on a full tile
-    if (route.src == BUF_IN && (size_t(job.tile) + 1) * L::TILE <= size_t(a.n)) {
-      onesweep2_tile<THREADS, ITEMS, NV, S, EARLY_LB, LB, false, true>(job, smem);
-      return;
-    }
-  }
   onesweep2_tile<THREADS, ITEMS, NV, S, EARLY_LB, LB, false, false>(job, smem);
 }
 
-template <int THREADS, int ITEMS, int NV, typename S, int MINB, bool EARLY_LB, int LB, bool UNSTABLE>
+template <int THREADS, int ITEMS, int NV, typename S, int MINB, bool EARLY_LB, int LB>
 cudaError_t launch_onesweep2(const PassArgs& a, unsigned grid, cudaStream_t s) {
   using L = Onesweep2Layout<THREADS, ITEMS, NV>;
-  onesweep2_kernel<THREADS, ITEMS, NV, S, MINB, EARLY_LB, LB, UNSTABLE><<<grid, THREADS, L::SMEM, s>>>(a);
-  return cudaGetLastError();
+  return launch_chained(&onesweep2_kernel<THREADS, ITEMS, NV, S, MINB, EARLY_LB, LB>, grid, THREADS, L::SMEM, s,
+                        a.gate != nullptr, a);
 }
 
 // EARLY_LB: the digit threads run the lookback before ranking their keys;
@@ -419,12 +413,6 @@ cudaError_t launch_onesweep2(const PassArgs& a, unsigned grid, cudaStream_t s) {
 template <int THREADS, int ITEMS, int NV, typename S, int MINB, bool EARLY_LB = false, int LB = 8>
 OnesweepKernel make_onesweep2(int shape_id) {
   using L = Onesweep2Layout<THREADS, ITEMS, NV>;
-  cudaError_t (*first)(const PassArgs&, unsigned, cudaStream_t) = nullptr;
-  const void* first_func = nullptr;
-  if constexpr (NV == 0) {
-    first = &launch_onesweep2<THREADS, ITEMS, NV, S, MINB, EARLY_LB, LB, true>;
-    first_func = reinterpret_cast<const void*>(&onesweep2_kernel<THREADS, ITEMS, NV, S, MINB, EARLY_LB, LB, true>);
-  }
   return OnesweepKernel{8,
                         shape_id,
                         THREADS,
@@ -433,13 +421,12 @@ OnesweepKernel make_onesweep2(int shape_id) {
                         NV >= 1,
                         sizeof(S) == 8,
                         L::SMEM,
-                        &launch_onesweep2<THREADS, ITEMS, NV, S, MINB, EARLY_LB, LB, false>,
-                        reinterpret_cast<const void*>(&onesweep2_kernel<THREADS, ITEMS, NV, S, MINB, EARLY_LB, LB, false>),
+                        &launch_onesweep2<THREADS, ITEMS, NV, S, MINB, EARLY_LB, LB>,
+                        reinterpret_cast<const void*>(&onesweep2_kernel<THREADS, ITEMS, NV, S, MINB, EARLY_LB, LB>),
                         0,
                         NV,
                         false,
-                        first,
-                        first_func};
+                        NV == 0};
 }
 
 }  // namespace rs

@@ -57,6 +57,17 @@ __device__ __forceinline__ uint32_t digit_of(uint32_t key, uint32_t shift, uint3
   return (key >> shift) & ((1u << width) - 1u);
 }
 
+// Kernels of a chain may be launched before the one in front of them has
+// finished (launch_chained): they wait for its end and its writes here, which
+// costs nothing in a kernel launched the usual way.
+__device__ __forceinline__ void wait_for_chain() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Whether a kernel launched beside another way to sort is to return at once.
+__device__ __forceinline__ bool gated_off(const uint32_t* gate) {
+  wait_for_chain();
+  return gate && *gate != kGateRadix;
+}
+
 // ---- relaxed, gpu-scope accesses for the cross-tile status words ----------
 __device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p) {
   uint32_t v;
@@ -196,7 +207,7 @@ struct Route {
 // that the last one lands in keys_out; the first reads the input.  If every
 // digit is skippable the last pass still runs (it is then a stable identity
 // copy into keys_out).  `skip` may be null (no pass skipped).
-__device__ __forceinline__ Route route_of(const uint32_t* skip, int pass, int num_passes) {
+__device__ __forceinline__ Route route_of(const uint32_t* skip, int pass, int num_passes, bool free_first = false) {
   int m = 0, idx = -1;
   for (int p = 0; p < num_passes; ++p) {
     const bool s = skip ? skip[p] != 0 : false;
@@ -220,7 +231,9 @@ __device__ __forceinline__ Route route_of(const uint32_t* skip, int pass, int nu
   r.last = idx == m - 1;
   r.dst = ((m - 1 - idx) % 2 == 0) ? BUF_OUT : BUF_ALT;
   r.src = idx == 0 ? BUF_IN : (((m - idx) % 2 == 0) ? BUF_OUT : BUF_ALT);
-  r.parity = uint32_t(idx & 1) ^ 1u;
+  // a first pass without a chained scan leaves the status words as they were cleared
+  const bool uncounted = free_first && !(skip && skip[0]);
+  r.parity = uint32_t((idx - (uncounted ? 1 : 0)) & 1) ^ 1u;
   return r;
 }
 

@@ -45,6 +45,31 @@ struct WideArgs {
   KeyXform64 x;
 };
 
+// Kernels of the radix passes launched beside another way to sort (hybrid.cu)
+// run only where the device chose them: `gate` points to that choice, null
+// where there is none.
+constexpr uint32_t kGateRadix = 1;
+
+// Launches a kernel that starts with wait_for_chain() (rs_device.cuh).
+// chained: its launch may overlap the end of the kernel in front of it on the
+// stream, which hides the launch's latency (it matters for the kernels that
+// return at once, of which a sort by value buckets has several).
+template <class Kernel, class Args>
+cudaError_t launch_chained(Kernel* kernel, unsigned grid, unsigned threads, size_t smem, cudaStream_t s, bool chained,
+                           const Args& args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = chained ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args);
+}
+
 // Upfront histogram (one read of the keys, every digit at once) and zeroing
 // of the chained-scan status array.
 struct HistArgs {
@@ -59,6 +84,13 @@ struct HistArgs {
   // launch_hist64 only: interleaved 64-bit keys and their order map
   const uint2* keys64;
   KeyXform64 x64;
+  const uint32_t* gate;  // null or the device's choice (kGateRadix: run)
+  // Byte digits: with `done` (a zeroed word) the last block also scans the
+  // histograms (ScanArgs' outputs; cursors: a copy of the first digit's bases).
+  uint32_t* done;
+  uint32_t* bases;
+  uint32_t* skip;
+  uint32_t* cursors;
 };
 
 // Exclusive scan of each digit's histogram + skip flags.
@@ -67,6 +99,7 @@ struct ScanArgs {
   uint32_t* bases;       // [num_digits][2^R]
   uint32_t* skip;        // [num_digits] (may be null)
   uint32_t n;
+  const uint32_t* gate;
 };
 
 // One onesweep LSD pass.
@@ -108,6 +141,11 @@ struct PassArgs {
   int iota;
   const uint2* gather;
   uint2* gather_out;
+  const uint32_t* gate;  // null or the device's choice (kGateRadix: run)
+  // Keys only: pass 0, when it runs, is the first executed pass and takes the
+  // tiles' places from these cursors (the digit's bases, advanced by atomics)
+  // instead of the chained scan; it then leaves the status words alone.
+  uint32_t* cursors;     // [256] or null
 };
 
 struct OnesweepKernel {
@@ -124,12 +162,12 @@ struct OnesweepKernel {
   int persistent_per_sm = 0;  // > 0: persistent kernel, grid = SMs x this (capped by tiles)
   int value_words = -1;       // payload words per key (-1: 1 if pairs else 0)
   bool pair_io = false;       // reads and writes interleaved 64-bit words (PassArgs pair_* and gather fields)
-  // Keys only: the kernel for pass 0, which ranks without keeping the order of
-  // equal digits when it is the sort's first executed pass (null: `launch`).
-  cudaError_t (*launch_first)(const PassArgs&, unsigned grid, cudaStream_t) = nullptr;
-  const void* func_first = nullptr;
+  bool free_first = false;    // keys only: pass 0 may be launch_first_pass
   int vwords() const { return value_words >= 0 ? value_words : (pairs ? 1 : 0); }
 };
+
+// Pass 0 of a sort of keys by byte digits (hybrid.cu; PassArgs::cursors).
+cudaError_t launch_first_pass(const PassArgs& a, cudaStream_t s);
 
 struct HistKernel {
   int radix_bits;
