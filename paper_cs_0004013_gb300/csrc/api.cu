@@ -108,14 +108,13 @@ rs_status device_state(DeviceState** out) {
         st.fused_tiles[pr][sh] = coop ? uint32_t(per_sm) * uint32_t(st.num_sms) : 0u;
       }
     const SegKernels* sk = seg_kernels();
-    const void* fn[12] = {sk->pass_keys[0], sk->pass_pairs[0], sk->pass_keys[1], sk->pass_pairs[1],
-                          sk->pass_keys[2], sk->pass_pairs[2], sk->tiny_keys,    sk->tiny_pairs,
-                          sk->small_keys,   sk->small_pairs,   sk->hist,         sk->hist_xf};
-    const size_t sm[12] = {sk->pass_smem_keys[0], sk->pass_smem_pairs[0], sk->pass_smem_keys[1],
-                           sk->pass_smem_pairs[1], sk->pass_smem_keys[2],  sk->pass_smem_pairs[2],
-                           sk->tiny_smem_keys,     sk->tiny_smem_pairs,    sk->small_smem_keys,
-                           sk->small_smem_pairs,   sk->hist_smem,          sk->hist_smem};
-    for (int i = 0; i < 12; ++i)
+    const void* fn[8] = {sk->pass_keys[0], sk->pass_pairs[0], sk->pass_keys[1], sk->pass_pairs[1],
+                         sk->pass_keys[2], sk->pass_pairs[2], sk->hist,         sk->hist_xf};
+    const size_t sm[8] = {sk->pass_smem_keys[0],  sk->pass_smem_pairs[0], sk->pass_smem_keys[1],
+                          sk->pass_smem_pairs[1], sk->pass_smem_keys[2],  sk->pass_smem_pairs[2],
+                          sk->hist_smem,          sk->hist_smem};
+    RS_CUDA(prepare_local(), "cudaFuncSetAttribute(local sort)");
+    for (int i = 0; i < 8; ++i)
       RS_CUDA(cudaFuncSetAttribute(fn[i], cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm[i])),
               "cudaFuncSetAttribute(segmented)");
     st.ready = true;
@@ -337,6 +336,41 @@ rs_status make_plan(uint64_t n, bool pairs, const rs_plan* user, SortPlan* p, in
 }
 
 // ---- temp layout ------------------------------------------------------------
+// The sort by value buckets (hybrid.cu): about 2,048 keys per bucket, at most
+// kHybMaxBuckets, in groups of 2^low_bits that halve the bucket's bits between
+// the two splits; up to 256 buckets take one split.
+struct HybLayout {
+  uint32_t buckets = 0, low_bits = 0, groups = 0;  // buckets == 0: not offered
+  size_t ctrl = 0, counts = 0, starts = 0, cursors = 0, group_cursors = 0, group_tiles = 0;
+  // the counts belong to what a sort clears first; returns the next offset
+  size_t place_counts(size_t off, uint64_t n, bool on) {
+    if (!on) return off;
+    uint64_t b = (n + 2047) / 2048;
+    if (b > kHybMaxBuckets) b = kHybMaxBuckets;
+    uint32_t bits = 0;
+    while ((uint64_t(1) << bits) < b) ++bits;
+    buckets = uint32_t(b);
+    low_bits = bits <= 8 ? 0u : bits / 2;
+    groups = uint32_t((b + (uint64_t(1) << low_bits) - 1) >> low_bits);
+    counts = off;
+    return align_up(off + size_t(buckets) * 4);
+  }
+  size_t place_rest(size_t off) {
+    if (!buckets) return off;
+    for (size_t* at : {&starts, &cursors}) {
+      *at = off;
+      off = align_up(off + (size_t(buckets) + 1) * 4);
+    }
+    ctrl = off;
+    off += align_up(sizeof(HybCtrl));
+    for (size_t* at : {&group_cursors, &group_tiles}) {
+      *at = off;
+      off = align_up(off + 257 * 4);
+    }
+    return off;
+  }
+};
+
 struct Layout {
   size_t ctrl = 0;     // words 0-3: tile tickets per pass; 4-7: skip flags; 12: barrier counter; 15: histogram blocks done
   size_t cursors0 = 0; // [256] u32: the first pass's bucket cursors
@@ -346,27 +380,9 @@ struct Layout {
   size_t status_bytes = 0;
   size_t alt_k = 0, alt_v = 0;
   size_t memset_bytes = 0;  // ctrl + hist (+ the buckets' counts), cleared before the histogram
-  // the sort by value buckets (buckets == 0: not offered at this size)
-  uint32_t buckets = 0, low_bits = 0, groups = 0;
-  size_t hctrl = 0, counts = 0, starts = 0, cursors = 0, group_cursors = 0, group_tiles = 0;
+  HybLayout hyb;
   size_t total = 0;
 };
-
-// The value buckets of n keys (hybrid.cu): about 2,048 keys each, at most
-// kHybMaxBuckets, in groups of 2^low_bits that halve the bucket's bits
-// between the two splits.
-void plan_buckets(uint64_t n, uint32_t* buckets, uint32_t* low_bits, uint32_t* groups) {
-#ifndef BMEAN
-#define BMEAN 2048
-#endif
-  uint64_t b = (n + BMEAN - 1) / BMEAN;
-  if (b > kHybMaxBuckets) b = kHybMaxBuckets;
-  uint32_t bits = 0;
-  while ((uint64_t(1) << bits) < b) ++bits;
-  *buckets = uint32_t(b);
-  *low_bits = bits / 2;
-  *groups = uint32_t((b + (uint64_t(1) << *low_bits) - 1) >> *low_bits);
-}
 
 Layout make_layout(const SortPlan& p, uint64_t n, bool pairs, bool hybrid = false) {
   Layout L;
@@ -376,11 +392,7 @@ Layout make_layout(const SortPlan& p, uint64_t n, bool pairs, bool hybrid = fals
   off += kAlign;
   L.hist = off;
   off = align_up(off + size_t(p.nd) * digits * 4);
-  if (hybrid) {
-    plan_buckets(n, &L.buckets, &L.low_bits, &L.groups);
-    L.counts = off;
-    off = align_up(off + size_t(L.buckets) * 4);
-  }
+  off = L.hyb.place_counts(off, n, hybrid);
   L.memset_bytes = off;
   L.bases = off;
   off = align_up(off + size_t(p.nd) * digits * 4);
@@ -389,18 +401,7 @@ Layout make_layout(const SortPlan& p, uint64_t n, bool pairs, bool hybrid = fals
   L.status = off;
   L.status_bytes = (p.status_rows > p.num_tiles ? p.status_rows : p.num_tiles) * digits * (p.k->wide_status ? 8 : 4);
   off = align_up(off + L.status_bytes);
-  if (hybrid) {
-    for (size_t* at : {&L.starts, &L.cursors}) {
-      *at = off;
-      off = align_up(off + (size_t(L.buckets) + 1) * 4);
-    }
-    L.hctrl = off;
-    off += align_up(sizeof(HybCtrl));
-    for (size_t* at : {&L.group_cursors, &L.group_tiles}) {
-      *at = off;
-      off = align_up(off + 257 * 4);
-    }
-  }
+  off = L.hyb.place_rest(off);
   if (p.nd > 1 && n > 0) {
     L.alt_k = off;
     off = align_up(off + size_t(n) * 4);
@@ -653,17 +654,15 @@ rs_status run_segmented(const SegLayout& L, unsigned char* temp, const uint32_t*
   la.vin = vin;
   la.vout = vout;
   la.seg_off = seg_off;
-  la.num_digits = nd;
-  for (int j = 0; j < nd; ++j) la.dig[j] = dig[j];
   la.xin = xin;
   la.xout = xout;
   la.list = pa.tiny_seg;
   la.count = counts + SEG_NUM_TINY;
-  RS_CUDA(traced(T_LOCAL, 0, s, [&] { return launch_local_sort(la, false, pairs, cap(num_segs, size_t(sms) * 8), s); }),
+  RS_CUDA(traced(T_LOCAL, 0, s, [&] { return launch_local_sort(la, false, pairs, num_segs, s); }),
           "launch local_sort (tiny)");
   la.list = pa.small_seg;
   la.count = counts + SEG_NUM_SMALL;
-  RS_CUDA(traced(T_LOCAL, 0, s, [&] { return launch_local_sort(la, true, pairs, cap(num_segs, size_t(sms) * 2), s); }),
+  RS_CUDA(traced(T_LOCAL, 0, s, [&] { return launch_local_sort(la, true, pairs, num_segs, s); }),
           "launch local_sort (small)");
   return RS_OK;
 }
@@ -765,7 +764,41 @@ rs_status run_msd(const SortPlan& p, const MsdLayout& M, const uint32_t* keys_in
 // ---- the sort by value buckets -----------------------------------------------------
 // The sample, the buckets' path and, gated behind the sample's and the
 // counts' choice, the radix passes; see hybrid.cu.
-constexpr uint64_t kHybridMinKeys = uint64_t(1) << 17, kHybridMaxKeys = uint64_t(3) << 25;
+constexpr uint64_t kHybridMinKeys = 8192, kHybridMaxKeys = uint64_t(3) << 25;
+
+// Launches the sample, the counts, the splits and the bucket sorts; `a` holds
+// the keys' buffers and order map.  Afterwards *gate points to the choice that
+// the radix passes' launches wait behind.
+rs_status run_buckets(HybArgs a, const HybLayout& H, size_t clear_bytes, unsigned char* temp, int key_bytes,
+                      DeviceState* ds, cudaStream_t s, const uint32_t** gate) {
+  a.buckets = H.buckets;
+  a.low_bits = H.low_bits;
+  a.groups = H.groups;
+  a.bucket_cap = hyb_bucket_cap();
+  a.split_tile = hyb_split_tile(key_bytes);
+  a.ctrl = reinterpret_cast<HybCtrl*>(temp + H.ctrl);
+  a.counts = reinterpret_cast<uint32_t*>(temp + H.counts);
+  a.starts = reinterpret_cast<uint32_t*>(temp + H.starts);
+  a.cursors = reinterpret_cast<uint32_t*>(temp + H.cursors);
+  a.group_cursors = reinterpret_cast<uint32_t*>(temp + H.group_cursors);
+  a.group_tiles = reinterpret_cast<uint32_t*>(temp + H.group_tiles);
+  a.clear = reinterpret_cast<uint4*>(temp);
+  a.clear_vec4 = clear_bytes / 16;
+  a.err = ds->err;
+  const unsigned sms = unsigned(ds->num_sms);
+  const struct {
+    HybStep step;
+    int kind;
+  } steps[] = {{HybStep::kSample, T_SAMPLE}, {HybStep::kCount, T_COUNT}, {HybStep::kSplit0, T_SPLIT0},
+               {HybStep::kSplit1, T_SPLIT1}, {HybStep::kBuckets, T_BUCKETS}};
+  for (const auto& st : steps) {
+    if (st.step == HybStep::kSplit1 && a.low_bits == 0) continue;
+    RS_CUDA(traced(st.kind, a.n, s, [&] { return launch_hybrid(a, st.step, key_bytes, sms, s); }),
+            "launch sort by buckets");
+  }
+  *gate = &a.ctrl->route;
+  return RS_OK;
+}
 
 rs_status run_hybrid32(const SortPlan& p, const Layout& L, const uint32_t* keys_in, uint32_t* keys_out, uint32_t n,
                        unsigned char* temp, DeviceState* ds, cudaStream_t s) {
@@ -775,30 +808,10 @@ rs_status run_hybrid32(const SortPlan& p, const Layout& L, const uint32_t* keys_
   a.keys_alt = temp + L.alt_k;
   a.n = n;
   a.x = p.xf;
-  a.buckets = L.buckets;
-  a.low_bits = L.low_bits;
-  a.groups = L.groups;
-  a.bucket_cap = hyb_bucket_cap();
-  a.split_tile = hyb_split_tile(4);
-  a.ctrl = reinterpret_cast<HybCtrl*>(temp + L.hctrl);
-  a.counts = reinterpret_cast<uint32_t*>(temp + L.counts);
-  a.starts = reinterpret_cast<uint32_t*>(temp + L.starts);
-  a.cursors = reinterpret_cast<uint32_t*>(temp + L.cursors);
-  a.group_cursors = reinterpret_cast<uint32_t*>(temp + L.group_cursors);
-  a.group_tiles = reinterpret_cast<uint32_t*>(temp + L.group_tiles);
-  a.clear = reinterpret_cast<uint4*>(temp);
-  a.clear_vec4 = L.memset_bytes / 16;
-  a.err = ds->err;
-  const unsigned sms = unsigned(ds->num_sms);
-  const struct {
-    HybStep step;
-    int kind;
-  } steps[] = {{HybStep::kSample, T_SAMPLE}, {HybStep::kCount, T_COUNT}, {HybStep::kSplit0, T_SPLIT0},
-               {HybStep::kSplit1, T_SPLIT1}, {HybStep::kBuckets, T_BUCKETS}};
-  for (const auto& st : steps)
-    RS_CUDA(traced(st.kind, n, s, [&] { return launch_hybrid(a, st.step, 4, sms, s); }), "launch sort by buckets");
+  const uint32_t* gate = nullptr;
+  if (rs_status st = run_buckets(a, L.hyb, L.memset_bytes, temp, 4, ds, s, &gate); st != RS_OK) return st;
   return run_lsd(p, L, keys_in, nullptr, keys_out, nullptr, n, temp, false, ds, s, nullptr, nullptr, nullptr, nullptr,
-                 nullptr, &a.ctrl->route);
+                 nullptr, gate);
 }
 
 // ---- the single-launch sort -----------------------------------------------------
@@ -888,9 +901,9 @@ rs_status sort_impl(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* 
   if (p.msd)
     return run_msd(p, M, keys_in, pairs ? vals_in : nullptr, keys_out, pairs ? vals_out : nullptr, uint32_t(n),
                    static_cast<unsigned char*>(temp), ds, s);
-  // A small array with the automatic plan fits one block: every digit is
-  // sorted in shared memory by one launch (no histogram, scans or tiled
-  // passes), which is several times faster for such sizes.
+  // A small array with the automatic plan fits one block: sorted in shared
+  // memory by one launch (no histogram, scans or tiled passes), which is
+  // several times faster for such sizes.
   const SegKernels* sk = seg_kernels();
   if (automatic && n <= sk->small_max) {
     LocalArgs la{};
@@ -899,11 +912,9 @@ rs_status sort_impl(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* 
     la.vin = pairs ? vals_in : nullptr;
     la.vout = pairs ? vals_out : nullptr;
     la.single_n = uint32_t(n);
-    la.num_digits = 4;
-    for (int j = 0; j < 4; ++j) la.dig[j] = DigitSpec{uint32_t(8 * j), 8u};
     la.xin = p.xf;
     la.xout = p.xf;
-    RS_CUDA(traced(T_LOCAL, double(n), s, [&] { return launch_local_sort(la, n > sk->tiny_max, pairs, 1u, s); }),
+    RS_CUDA(traced(T_LOCAL, double(n), s, [&] { return launch_local_array(la, 4, pairs ? 4 : 0, s); }),
             "launch local_sort (one array)");
     return RS_OK;
   }
@@ -943,10 +954,11 @@ struct Layout64 {
   size_t plane[6] = {};  // lo/hi words of the output, alternate and (split only) input order
   size_t val_alt = 0;    // the values' alternate plane (key+value sorts)
   size_t idx_out = 0;    // 64-bit values: the index plane of the output order
+  HybLayout hyb;
   size_t memset_bytes = 0, total = 0;
 };
 
-Layout64 make_layout64(const SortPlan& p, uint64_t n, bool pairs, bool vals64 = false) {
+Layout64 make_layout64(const SortPlan& p, uint64_t n, bool pairs, bool vals64 = false, bool hybrid = false) {
   Layout64 L;
   L.fused = pair_io_kernel(p.k) != nullptr;
   size_t off = 0;
@@ -954,9 +966,11 @@ Layout64 make_layout64(const SortPlan& p, uint64_t n, bool pairs, bool vals64 = 
   off += kAlign;
   L.hist = off;
   off = align_up(off + 8 * 256 * 4);
+  off = L.hyb.place_counts(off, n, hybrid);
   L.memset_bytes = off;
   L.bases = off;
   off = align_up(off + 8 * 256 * 4);
+  off = L.hyb.place_rest(off);
   L.status = off;
   L.status_bytes = p.num_tiles * 256 * (p.k->wide_status ? 8 : 4);
   off = align_up(off + L.status_bytes);
@@ -1000,8 +1014,19 @@ rs_status run_lsd64(const SortPlan& p, const Layout64& L, const uint64_t* keys_i
   const OnesweepKernel* pk = L.fused ? pair_io_kernel(p.k) : p.k;
   uint32_t *lo_out = pl[0], *hi_out = pl[1], *lo_alt = pl[2], *hi_alt = pl[3], *lo_in = pl[4], *hi_in = pl[5];
   const uint2* k2 = reinterpret_cast<const uint2*>(keys_in);
-  RS_CUDA(traced(T_CLEAR, 0, s, [&] { return cudaMemsetAsync(temp, 0, L.memset_bytes, s); }),
-          "cudaMemsetAsync(temp)");
+  const uint32_t* gate = nullptr;
+  if (L.hyb.buckets) {
+    HybArgs a{};
+    a.keys_in = keys_in;
+    a.keys_out = keys_out;
+    a.keys_alt = pl[0];  // planes 0 and 1 follow each other
+    a.n = n;
+    a.x64 = x;
+    if (rs_status st = run_buckets(a, L.hyb, L.memset_bytes, temp, 8, ds, s, &gate); st != RS_OK) return st;
+  } else {
+    RS_CUDA(traced(T_CLEAR, 0, s, [&] { return cudaMemsetAsync(temp, 0, L.memset_bytes, s); }),
+            "cudaMemsetAsync(temp)");
+  }
   const unsigned egrid = unsigned(std::min<size_t>((size_t(n) + 255) / 256, size_t(ds->num_sms) * 8));
   if (!L.fused) {
     WideArgs wa{k2, reinterpret_cast<uint2*>(keys_out), lo_in, hi_in, n, x};
@@ -1020,6 +1045,7 @@ rs_status run_lsd64(const SortPlan& p, const Layout64& L, const uint64_t* keys_i
     ha.hist = hist;
     ha.zero_ptr = reinterpret_cast<uint4*>(temp + L.status);
     ha.zero_vec4 = L.status_bytes / 16;
+    ha.gate = gate;
     ha.done = ctrl + 16;  // the last block scans them
     ha.bases = bases;
     ha.skip = ctrl + 8;
@@ -1060,6 +1086,7 @@ rs_status run_lsd64(const SortPlan& p, const Layout64& L, const uint64_t* keys_i
       pa.gather = reinterpret_cast<const uint2*>(vals64_in);
       pa.gather_out = reinterpret_cast<uint2*>(vals64_out);
     }
+    pa.gate = gate;
     pa.n = n;
     pa.shift = uint32_t(8 * (j % 4));
     pa.width = 8;
@@ -1157,7 +1184,9 @@ static rs_status sort64_impl(const uint64_t* keys_in, const void* vals_in, uint6
   if (q.tile == 0) q.tile = (vbytes == 0 && n > (uint64_t(1) << 22) && !needs_wide_status(n)) ? 8u : 1u;
   SortPlan p;
   if (rs_status st = make_plan(n, true, &q, &p, pairs ? 2 : 1); st != RS_OK) return st;
-  const Layout64 L = make_layout64(p, n, pairs, vbytes == 8);
+  const bool automatic = !plan || (plan->digit_bits == 0 && plan->mode == RS_MODE_AUTO && plan->tile == 0);
+  const bool hybrid = automatic && vbytes == 0 && n >= kHybridMinKeys && n <= kHybridMaxKeys;
+  const Layout64 L = make_layout64(p, n, pairs, vbytes == 8, hybrid);
   if (vbytes == 8 && !L.fused)
     return fail(RS_ERR_UNSUPPORTED, "64-bit values: tile shape %u has no interleaved pass kernel", q.tile);
   if (!temp) {
@@ -1189,6 +1218,18 @@ static rs_status sort64_impl(const uint64_t* keys_in, const void* vals_in, uint6
   if (n == 0) return RS_OK;
   DeviceState* ds = nullptr;
   if (rs_status st = device_state(&ds); st != RS_OK) return st;
+  if (automatic && n <= local_max_keys(8, vbytes)) {  // one block
+    LocalArgs la{};
+    la.kin = keys_in;
+    la.kout = keys_out;
+    la.vin = vals_in;
+    la.vout = vals_out;
+    la.single_n = uint32_t(n);
+    la.x64 = x;
+    RS_CUDA(traced(T_LOCAL, double(n), s, [&] { return launch_local_array(la, 8, vbytes, s); }),
+            "launch local_sort (one array)");
+    return RS_OK;
+  }
   if (vbytes == 8)
     return run_lsd64(p, L, keys_in, nullptr, keys_out, nullptr, uint32_t(n), x, static_cast<unsigned char*>(temp), ds,
                      s, static_cast<const uint64_t*>(vals_in), static_cast<uint64_t*>(vals_out));
@@ -1268,6 +1309,20 @@ rs_status rs_sort_u32_pairs64(const uint32_t* keys_in, const uint64_t* vals_in, 
   if (n == 0) return RS_OK;
   DeviceState* ds = nullptr;
   if ((st = device_state(&ds)) != RS_OK) return st;
+  const bool automatic = !plan || (plan->digit_bits == 0 && plan->mode == RS_MODE_AUTO && plan->tile == 0);
+  if (automatic && n <= local_max_keys(4, 8)) {  // one block
+    LocalArgs la{};
+    la.kin = keys_in;
+    la.kout = keys_out;
+    la.vin = vals_in;
+    la.vout = vals_out;
+    la.single_n = uint32_t(n);
+    la.xin = p.xf;
+    la.xout = p.xf;
+    RS_CUDA(traced(T_LOCAL, double(n), s, [&] { return launch_local_array(la, 4, 8, s); }),
+            "launch local_sort (one array)");
+    return RS_OK;
+  }
   unsigned char* t = static_cast<unsigned char*>(temp);
   uint32_t* pl[5] = {};
   for (int i = 0; i < nplanes; ++i) pl[i] = reinterpret_cast<uint32_t*>(t + plane[i]);

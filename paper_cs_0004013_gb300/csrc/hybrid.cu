@@ -99,7 +99,7 @@ struct OrdOf<uint64_t> {
 // evenly when
 //  - no 64th of the range holds more than 1.5 times its share of the sample
 //    (uniform keys: 128 or more expected, five standard deviations below);
-//  - no bucket holds more than kFineLimit sampled keys (one expected at most);
+//  - no bucket holds more than 1.5 times its share of the sample and kFineLimit keys;
 //  - few sampled keys are equal to another one: many equal keys end up in few
 //    bins of a bucket, which then takes the digit passes.
 constexpr int kSampleBlocks = 8;
@@ -188,10 +188,11 @@ __global__ void __cluster_dims__(kSampleBlocks, 1, 1) __launch_bounds__(kSampleT
   m.mult = uint32_t((uint64_t(a.buckets) << 32) / (range > a.buckets ? range : uint64_t(a.buckets) + 1));
   m.back = 0ull - uint64_t(m.lo) * m.mult;
   bool bad = range <= a.buckets;
+  const uint32_t fine_limit = kFineLimit + uint32_t(L::S) * 3 / (2 * a.buckets);
 #pragma unroll
   for (int i = 0; i < L::PER; ++i) {
     const uint32_t b = m.bucket(key[i]);
-    if (atomicAdd(&s_fine[b], 1u) >= kFineLimit) bad = true;
+    if (atomicAdd(&s_fine[b], 1u) >= fine_limit) bad = true;
     atomicAdd(&s_coarse[(b * kCoarse) / a.buckets], 1u);
   }
   __syncthreads();
@@ -393,7 +394,7 @@ __global__ void __launch_bounds__(THREADS, MINB) split_kernel(const HybArgs a) {
     cursors = a.cursors + (s_job[2] << a.low_bits);
   }
   const K* in = reinterpret_cast<const K*>(LEVEL == 0 ? a.keys_in : a.keys_alt) + base;
-  K* out = reinterpret_cast<K*>(LEVEL == 0 ? a.keys_alt : a.keys_out);
+  K* out = reinterpret_cast<K*>(LEVEL == 0 && a.low_bits != 0 ? a.keys_alt : a.keys_out);  // one split: no detour
   const auto ident = OrdOf<K>::identity();
   const auto ordi = LEVEL == 0 ? OrdOf<K>::make(a) : ident;
   if (valid == TILE) split_tile<K, THREADS, ITEMS, true>(in, valid, out, cursors, a.n, digit, ordi, ident, a.err, smem);

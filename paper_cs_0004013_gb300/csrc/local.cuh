@@ -40,7 +40,6 @@
 namespace rs {
 
 constexpr uint32_t kBinLimit = 29;  // eight rounds of windows
-constexpr int kMaxWindows = 3;      // windows a thread keeps in registers
 
 // What the block orders: the key, or with a payload (key, place in the input).
 struct alignas(16) KeyPlace64 {
@@ -423,7 +422,7 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
   uint32_t most = 0;
   for_items([&](int j) {
     const uint32_t b = bins(key[j]);
-    const uint32_t half = b >> (NBITS - 1);
+    const uint32_t half = (b >> (NBITS - 1)) & 1u;
     uint32_t r = 0;
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %3, %4;\n\t@p atom.shared.add.u32 %0, [%1], %2;\n\t}"
@@ -441,9 +440,10 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
     if (lane == 0) atomicMax(s_most, most);
   }
   __syncthreads();
-  // keys of the fullest bin (five at least); bins of one value need no order among equal keys
+  // keys of the fullest bin (five at least); bins of one value need no order
+  // among equal keys (as long as their turns fit their 8 bits)
   most = *s_most ? *s_most + 1u : 5u;
-  if (VB == 0 && bins.unique()) most = 1u;
+  if (VB == 0 && bins.unique() && most <= 256u) most = 1u;
   if (most <= kBinLimit) {
     // 3. counts -> starts, both halves of the words at once (sums of at most
     // CAP < 2^16 each): the low halves' total comes before the high halves'
@@ -482,7 +482,8 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
     // 4. keys into the bins' places; the windows past the end read the last element
     for_items([&](int j) {
       const uint32_t b = bins(key[j]);
-      const uint32_t p = s_start[2u * (b & uint32_t(NB / 2 - 1)) + (b >> (NBITS - 1))] +
+      // (the bin of a lane without a key is any number: both parts are masked)
+      const uint32_t p = s_start[2u * (b & uint32_t(NB / 2 - 1)) + ((b >> (NBITS - 1)) & 1u)] +
                          __byte_perm(turn[j / 4], 0u, 0x4440u + uint32_t(j % 4));
       // (a lane without a key stores to a spare slot)
       s_key[L::slot(has(j) ? p : uint32_t(L::SPARE + lane))] = EO::make(key[j], j * THREADS + tid);
@@ -491,13 +492,15 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
     __syncthreads();
     // 5. windows: those that start before the end
     constexpr int NWIN = (ITEMS + 7) / 8;  // windows per thread
-    if (NWIN <= kMaxWindows && most == 5u) {
+    // (what the block's register budget holds; else a round at a time)
+    constexpr bool HELD = NWIN * sizeof(E) <= (THREADS >= 1024 ? 8 : THREADS >= 256 ? 12 : 24);
+    if (HELD && most == 5u) {
       // Two rounds, each thread keeping its windows in registers: between
       // them it takes the next window's lower half, from the next lane or,
       // over the warp's end, through shared memory.
-      E v[NWIN][8];
+      E v[HELD ? NWIN : 1][8];
 #pragma unroll
-      for (int c = 0; c < NWIN; ++c) {
+      for (int c = 0; c < (HELD ? NWIN : 0); ++c) {
         const uint32_t p = uint32_t(c * THREADS + tid) * 8u;
         if (uint32_t(c * THREADS + warp * 32) * 8u < m) {  // the whole warp
           ld_window<L>(v[c], s_key, p < m ? p : 0u);
@@ -512,7 +515,7 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
       }
       __syncthreads();
 #pragma unroll
-      for (int c = 0; c < NWIN; ++c) {
+      for (int c = 0; c < (HELD ? NWIN : 0); ++c) {
         const uint32_t p = uint32_t(c * THREADS + tid) * 8u;
         if (uint32_t(c * THREADS + warp * 32) * 8u < m) {
           E u[8];

@@ -254,17 +254,16 @@ struct SegPassArgs {
 };
 
 struct LocalArgs {
-  const uint32_t* kin;
-  uint32_t* kout;
-  const uint32_t* vin;
-  uint32_t* vout;
+  const void* kin;
+  void* kout;
+  const void* vin;
+  void* vout;
   const uint64_t* seg_off;
   const uint32_t* list;   // segment ids (null: one array of single_n keys)
   const uint32_t* count;  // device count of list entries
-  uint32_t single_n;      // keys of the one array when list is null (<= the block's tile)
-  int num_digits;
-  DigitSpec dig[kMaxDigits];
-  KeyXform xin, xout;     // applied on loading kin, inverted on storing kout
+  uint32_t single_n;      // keys of the one array when list is null (1 .. local_max_keys)
+  KeyXform xin, xout;     // 32-bit keys: applied on loading kin, inverted on storing kout
+  KeyXform64 x64;         // 64-bit keys: both
 };
 
 // Tiled-pass shapes of the segmented pipeline (rs_plan.tile = shape + 1).
@@ -275,13 +274,8 @@ struct SegKernels {
   uint32_t blocks_per_sm[kSegShapes];  // the persistent pass's resident blocks
   uint32_t tile(bool pairs, int shape) const { return pairs ? tile_pairs[shape] : tile_keys[shape]; }
   size_t pass_smem_keys[kSegShapes], pass_smem_pairs[kSegShapes];
-  size_t tiny_smem_keys, tiny_smem_pairs, small_smem_keys, small_smem_pairs;
   const void* pass_keys[kSegShapes];
   const void* pass_pairs[kSegShapes];
-  const void* tiny_keys;
-  const void* tiny_pairs;
-  const void* small_keys;
-  const void* small_pairs;
   const void* hist;     // the segment histogram kernel for unsigned keys
   const void* hist_xf;  // and for keys of another kind
   size_t hist_smem;
@@ -292,7 +286,11 @@ cudaError_t launch_seg_plan(const SegPlanArgs& a, cudaStream_t s);
 cudaError_t launch_seg_hist(const SegHistArgs& a, unsigned grid, cudaStream_t s);
 cudaError_t launch_seg_scan(const SegScanArgs& a, unsigned grid, cudaStream_t s);
 cudaError_t launch_seg_pass(const SegPassArgs& a, bool pairs, int shape, unsigned grid, cudaStream_t s);
+// One-block sorts (local.cu): the listed segments, or one array.
+cudaError_t prepare_local();
+uint32_t local_max_keys(int key_bytes, int val_bytes);
 cudaError_t launch_local_sort(const LocalArgs& a, bool small, bool pairs, unsigned grid, cudaStream_t s);
+cudaError_t launch_local_array(const LocalArgs& a, int key_bytes, int val_bytes, cudaStream_t s);
 cudaError_t launch_bases_to_offsets(const uint32_t* bases, uint32_t num, uint64_t n, uint64_t* seg_off,
                                     cudaStream_t s);
 

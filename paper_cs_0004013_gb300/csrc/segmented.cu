@@ -17,8 +17,8 @@
 //   seg_scan      per large segment and digit: exclusive scan;
 //   seg_pass x P  onesweep passes over the large tiles, lookback confined to
 //                 the tile's own segment;
-//   local_sort    one block per tiny / small segment: every digit sorted
-//                 in shared memory, written once.
+//   local_sort    one block per tiny / small segment, in shared memory
+//                 (local.cu).
 #include <cuda_runtime.h>
 
 #include "onesweep.cuh"
@@ -224,97 +224,6 @@ __global__ void __launch_bounds__(THREADS, MINB) seg_pass_kernel(const SegPassAr
   }
 }
 
-// ------------------------------------------------------ one-block local sort
-template <int THREADS, int ITEMS, bool PAIRS>
-struct LocalLayout {
-  static constexpr int WARPS = THREADS / 32;
-  static constexpr int TILE = THREADS * ITEMS;
-  static constexpr size_t MASK_BYTES = size_t(WARPS) * kMaskSlots * 4;
-  static constexpr size_t CNT_BYTES = size_t(WARPS) * 256 * 2;
-  static constexpr size_t OFF_BUF = MASK_BYTES + CNT_BYTES;
-  static constexpr size_t BUF_BYTES = size_t(TILE) * 4 * (PAIRS ? 2 : 1);
-  static constexpr size_t OFF_WARP = OFF_BUF + BUF_BYTES;
-  static constexpr size_t SMEM = OFF_WARP + 32 * 4;
-  static_assert(THREADS >= 256, "one thread per 8-bit digit in the scan");
-  static_assert((MASK_BYTES + CNT_BYTES) % 16 == 0, "tables are cleared in 16-byte units");
-};
-
-// Sorts each listed segment (at most THREADS * ITEMS keys) by every digit
-// of the plan, least significant first, entirely in shared memory: per
-// digit a stable warp rank (the same lane-mask tables as the tiled pass),
-// per-digit tile offsets, and a scatter into the staging buffer, which the
-// next digit reads back.  Keys past the segment's end act as 0xFFFFFFFF and
-// stay behind every real key.  Writes src -> dst once.
-template <int THREADS, int ITEMS, bool PAIRS>
-__global__ void __launch_bounds__(THREADS, 1) local_sort_kernel(const LocalArgs a) {
-  using L = LocalLayout<THREADS, ITEMS, PAIRS>;
-  constexpr int TILE = L::TILE, WARPS = L::WARPS;
-  extern __shared__ __align__(16) unsigned char smem[];
-  uint32_t* s_mask = reinterpret_cast<uint32_t*>(smem);
-  uint16_t* s_cnt = reinterpret_cast<uint16_t*>(smem + L::MASK_BYTES);
-  uint32_t* s_buf = reinterpret_cast<uint32_t*>(smem + L::OFF_BUF);
-  uint32_t* s_warp = reinterpret_cast<uint32_t*>(smem + L::OFF_WARP);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // a listed set of segments, or (list == null) the one array [0, single_n)
-  const uint32_t count = a.list ? *a.count : 1u;
-  for (uint32_t k = blockIdx.x; k < count; k += gridDim.x) {
-    const uint32_t s = a.list ? a.list[k] : 0u;
-    const uint64_t start = a.list ? a.seg_off[s] : 0u;
-    const uint32_t m = a.list ? uint32_t(a.seg_off[s + 1] - start) : a.single_n;
-    uint32_t key[ITEMS], val[PAIRS ? ITEMS : 1];
-    const uint32_t wofs = uint32_t(warp) * 32 * ITEMS + lane;
-#pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-      const uint32_t i = wofs + j * 32;
-      key[j] = i < m ? to_ordered(a.kin[start + i], a.xin) : 0xffffffffu;
-      if constexpr (PAIRS) val[j] = i < m ? a.vin[start + i] : 0u;
-    }
-    for (int p = 0; p < a.num_digits; ++p) {
-      const uint32_t shift = a.dig[p].shift, width = a.dig[p].width;
-      uint4* c4 = reinterpret_cast<uint4*>(smem);
-      for (int i = tid; i < int(L::OFF_BUF / 16); i += THREADS) c4[i] = make_uint4(0u, 0u, 0u, 0u);
-      __syncthreads();
-      uint32_t rk[(ITEMS + 1) / 2];
-      warp_rank<8, ITEMS>(key, shift, width, s_mask + warp * kMaskSlots, s_cnt + warp * 256, rk);
-      __syncthreads();
-      // per digit (threads 0..255): total over warps, exclusive over digits,
-      // then exclusive (digit, warp) offsets
-      uint32_t tot = 0;
-      if (tid < 256)
-        for (int wi = 0; wi < WARPS; ++wi) tot += s_cnt[wi * 256 + tid];
-      const uint32_t excl = block_exclusive_sum<THREADS>(tid < 256 ? tot : 0u, s_warp);
-      if (tid < 256) {
-        uint32_t run = excl;
-        for (int wi = 0; wi < WARPS; ++wi) {
-          const uint32_t v = s_cnt[wi * 256 + tid];
-          s_cnt[wi * 256 + tid] = uint16_t(run);
-          run += v;
-        }
-      }
-      __syncthreads();
-#pragma unroll
-      for (int j = 0; j < ITEMS; ++j) {
-        const uint32_t pos = ((rk[j >> 1] >> (16 * (j & 1))) & 0xffffu) + s_cnt[warp * 256 + digit_of(key[j], shift, width)];
-        s_buf[pos] = key[j];
-        if constexpr (PAIRS) s_buf[TILE + pos] = val[j];
-      }
-      __syncthreads();
-#pragma unroll
-      for (int j = 0; j < ITEMS; ++j) {
-        key[j] = s_buf[wofs + j * 32];
-        if constexpr (PAIRS) val[j] = s_buf[TILE + wofs + j * 32];
-      }
-      __syncthreads();
-    }
-    // the staging buffer holds the sorted segment (then the padding)
-    for (uint32_t i = tid; i < m; i += THREADS) {
-      a.kout[start + i] = from_ordered(s_buf[i], a.xout);
-      if constexpr (PAIRS) a.vout[start + i] = s_buf[TILE + i];
-    }
-    __syncthreads();
-  }
-}
-
 // Bucket offsets of an MSD plan: the exclusive scan of the top digit as
 // segment offsets (uint64), the last one being n.
 __global__ void bases_to_offsets_kernel(const uint32_t* bases, uint32_t num, uint64_t n, uint64_t* seg_off) {
@@ -330,13 +239,6 @@ cudaError_t launch_seg_pass(const SegPassArgs& a, unsigned grid, cudaStream_t s)
   return cudaGetLastError();
 }
 
-template <int THREADS, int ITEMS, bool PAIRS>
-cudaError_t launch_local(const LocalArgs& a, unsigned grid, cudaStream_t s) {
-  using L = LocalLayout<THREADS, ITEMS, PAIRS>;
-  local_sort_kernel<THREADS, ITEMS, PAIRS><<<grid, THREADS, L::SMEM, s>>>(a);
-  return cudaGetLastError();
-}
-
 }  // namespace
 
 // Tiled passes over large segments, 8-bit digits.  Shape 0: 512 x 16 tiles
@@ -346,8 +248,8 @@ cudaError_t launch_local(const LocalArgs& a, unsigned grid, cudaStream_t s) {
 // spills in the persistent loop and takes 39.6).
 constexpr int kSegThreads = 512, kSegItemsKeys = 24, kSegItemsPairs = 22, kSegItemsSmall = 16;
 constexpr int kSegThreads3 = 384, kSegItems3 = 20;
-// Local sorts: tiny segments <= 256 x 16 keys, small ones <= 1024 x 16 keys.
-constexpr int kTinyThreads = 256, kSmallThreads = 1024, kLocalItems = 16;
+// Local sorts (local.cu): tiny segments and small ones.
+constexpr uint32_t kTinyMax = 4096, kSmallMax = 16384;
 // Segment histograms: one 1024-thread block per SM (lane copies of up to
 // four digits take 128 KiB).
 constexpr int kSegHistThreads = 1024;
@@ -358,27 +260,19 @@ const SegKernels* seg_kernels() {
        uint32_t(kSegThreads3 * kSegItems3)},
       {uint32_t(kSegThreads * kSegItemsSmall), uint32_t(kSegThreads * kSegItemsPairs),
        uint32_t(kSegThreads3 * kSegItems3)},
-      uint32_t(kTinyThreads * kLocalItems),
-      uint32_t(kSmallThreads * kLocalItems),
+      kTinyMax,
+      kSmallMax,
       {2u, 2u, 3u},
       {OnesweepLayout<8, kSegThreads, kSegItemsSmall, 0>::SMEM, OnesweepLayout<8, kSegThreads, kSegItemsKeys, 0>::SMEM,
        OnesweepLayout<8, kSegThreads3, kSegItems3, 0>::SMEM},
       {OnesweepLayout<8, kSegThreads, kSegItemsSmall, 1>::SMEM, OnesweepLayout<8, kSegThreads, kSegItemsPairs, 1>::SMEM,
        OnesweepLayout<8, kSegThreads3, kSegItems3, 1>::SMEM},
-      LocalLayout<kTinyThreads, kLocalItems, false>::SMEM,
-      LocalLayout<kTinyThreads, kLocalItems, true>::SMEM,
-      LocalLayout<kSmallThreads, kLocalItems, false>::SMEM,
-      LocalLayout<kSmallThreads, kLocalItems, true>::SMEM,
       {reinterpret_cast<const void*>(&seg_pass_kernel<kSegThreads, kSegItemsSmall, false, 2>),
        reinterpret_cast<const void*>(&seg_pass_kernel<kSegThreads, kSegItemsKeys, false, 2>),
        reinterpret_cast<const void*>(&seg_pass_kernel<kSegThreads3, kSegItems3, false, 3>)},
       {reinterpret_cast<const void*>(&seg_pass_kernel<kSegThreads, kSegItemsSmall, true, 2>),
        reinterpret_cast<const void*>(&seg_pass_kernel<kSegThreads, kSegItemsPairs, true, 2>),
        reinterpret_cast<const void*>(&seg_pass_kernel<kSegThreads3, kSegItems3, true, 3>)},
-      reinterpret_cast<const void*>(&local_sort_kernel<kTinyThreads, kLocalItems, false>),
-      reinterpret_cast<const void*>(&local_sort_kernel<kTinyThreads, kLocalItems, true>),
-      reinterpret_cast<const void*>(&local_sort_kernel<kSmallThreads, kLocalItems, false>),
-      reinterpret_cast<const void*>(&local_sort_kernel<kSmallThreads, kLocalItems, true>),
       reinterpret_cast<const void*>(&seg_hist_kernel<kSegHistThreads, false>),
       reinterpret_cast<const void*>(&seg_hist_kernel<kSegHistThreads, true>),
       size_t(kMaxDigits) * 256 * 32 * 4,
@@ -412,13 +306,6 @@ cudaError_t launch_seg_pass(const SegPassArgs& a, bool pairs, int shape, unsigne
                  : launch_seg_pass<kSegThreads, kSegItemsSmall, false, 2>(a, grid, s);
   return pairs ? launch_seg_pass<kSegThreads, kSegItemsPairs, true, 2>(a, grid, s)
                : launch_seg_pass<kSegThreads, kSegItemsKeys, false, 2>(a, grid, s);
-}
-cudaError_t launch_local_sort(const LocalArgs& a, bool small, bool pairs, unsigned grid, cudaStream_t s) {
-  if (small)
-    return pairs ? launch_local<kSmallThreads, kLocalItems, true>(a, grid, s)
-                 : launch_local<kSmallThreads, kLocalItems, false>(a, grid, s);
-  return pairs ? launch_local<kTinyThreads, kLocalItems, true>(a, grid, s)
-               : launch_local<kTinyThreads, kLocalItems, false>(a, grid, s);
 }
 cudaError_t launch_bases_to_offsets(const uint32_t* bases, uint32_t num, uint64_t n, uint64_t* seg_off,
                                     cudaStream_t s) {
