@@ -16,6 +16,7 @@ import ctypes
 import os
 
 import numpy as np
+import torch  # first: the CUDA runtime the library links against is the one torch loads
 
 from .build import LIB as LIBRARY_PATH
 
@@ -59,7 +60,7 @@ _P = ctypes.c_void_p
 _U32 = ctypes.c_uint32
 _U64 = ctypes.c_uint64
 _SZP = ctypes.POINTER(ctypes.c_size_t)
-_U64P = ctypes.POINTER(ctypes.c_uint64)
+_U64P = ctypes.c_void_p  # host uint64 arrays, passed by address
 _PLANP = ctypes.POINTER(RsPlan)
 
 _SIGS = {
@@ -93,8 +94,6 @@ def _load() -> ctypes.CDLL:
     if not os.path.exists(LIBRARY_PATH):
         raise ImportError(f"{LIBRARY_PATH} is missing: build it with "
                           "`python -c 'import __graft_entry__ as g; g.build()'`")
-    # the CUDA runtime the library links against is the one torch loaded
-    import torch  # noqa: F401
     dll = ctypes.CDLL(LIBRARY_PATH)
     for name, args in _SIGS.items():
         f = getattr(dll, name)
@@ -129,7 +128,10 @@ def _ptr(t) -> int | None:
 
 def _stream(stream) -> int | None:
     if stream is None:
-        import torch
+        # the current device's current stream, without building a Stream object
+        # for it (2.8 us of a call's 27)
+        if torch.cuda.is_initialized():
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
@@ -159,7 +161,7 @@ def rs_sort_u32(keys_in, keys_out, n: int, num_parts: int = 64, plan=None, temp=
     uint64[num_parts + 1]) or None."""
     tp, tb = _temp(temp)
     offs = np.zeros(num_parts + 1, dtype=np.uint64) if (want_offsets and temp is not None) else None
-    op = offs.ctypes.data_as(_U64P) if offs is not None else None
+    op = offs.ctypes.data if offs is not None else None
     _check(lib.rs_sort_u32(_ptr(keys_in), _ptr(keys_out), n, num_parts, op, _plan(plan), tp,
                            ctypes.byref(tb), _stream(stream) if temp is not None else None))
     return tb.value if temp is None else offs
@@ -170,7 +172,7 @@ def rs_sort_u32_pairs(keys_in, vals_in, keys_out, vals_out, n: int, num_parts: i
     """Calls rs_sort_u32_pairs; returns as rs_sort_u32."""
     tp, tb = _temp(temp)
     offs = np.zeros(num_parts + 1, dtype=np.uint64) if (want_offsets and temp is not None) else None
-    op = offs.ctypes.data_as(_U64P) if offs is not None else None
+    op = offs.ctypes.data if offs is not None else None
     _check(lib.rs_sort_u32_pairs(_ptr(keys_in), _ptr(vals_in), _ptr(keys_out), _ptr(vals_out), n, num_parts,
                                  op, _plan(plan), tp, ctypes.byref(tb),
                                  _stream(stream) if temp is not None else None))
@@ -183,7 +185,7 @@ def rs_sort_u64(keys_in, keys_out, n: int, num_parts: int = 64, plan=None, temp=
     returns as rs_sort_u32."""
     tp, tb = _temp(temp)
     offs = np.zeros(num_parts + 1, dtype=np.uint64) if (want_offsets and temp is not None) else None
-    op = offs.ctypes.data_as(_U64P) if offs is not None else None
+    op = offs.ctypes.data if offs is not None else None
     _check(lib.rs_sort_u64(_ptr(keys_in), _ptr(keys_out), n, num_parts, op, _plan(plan), tp, ctypes.byref(tb),
                            _stream(stream) if temp is not None else None))
     return tb.value if temp is None else offs
@@ -194,7 +196,7 @@ def rs_sort_u64_pairs(keys_in, vals_in, keys_out, vals_out, n: int, num_parts: i
     """Calls rs_sort_u64_pairs; returns as rs_sort_u32."""
     tp, tb = _temp(temp)
     offs = np.zeros(num_parts + 1, dtype=np.uint64) if (want_offsets and temp is not None) else None
-    op = offs.ctypes.data_as(_U64P) if offs is not None else None
+    op = offs.ctypes.data if offs is not None else None
     _check(lib.rs_sort_u64_pairs(_ptr(keys_in), _ptr(vals_in), _ptr(keys_out), _ptr(vals_out), n, num_parts, op,
                                  _plan(plan), tp, ctypes.byref(tb), _stream(stream) if temp is not None else None))
     return tb.value if temp is None else offs
@@ -206,7 +208,7 @@ def rs_sort_u64_pairs64(keys_in, vals_in, keys_out, vals_out, n: int, num_parts:
     rs_sort_u32."""
     tp, tb = _temp(temp)
     offs = np.zeros(num_parts + 1, dtype=np.uint64) if (want_offsets and temp is not None) else None
-    op = offs.ctypes.data_as(_U64P) if offs is not None else None
+    op = offs.ctypes.data if offs is not None else None
     _check(lib.rs_sort_u64_pairs64(_ptr(keys_in), _ptr(vals_in), _ptr(keys_out), _ptr(vals_out), n, num_parts,
                                    op, _plan(plan), tp, ctypes.byref(tb),
                                    _stream(stream) if temp is not None else None))
@@ -217,7 +219,6 @@ def sort64_pairs(keys, vals, num_parts: int = 64, plan=None, stream=None):
     """Stable sort of CUDA tensors of 64-bit keys and 32-bit or (by the
     values' element size) 64-bit values: (keys, vals, host partition
     offsets)."""
-    import torch
     n = keys.numel()
     ko, vo = torch.empty_like(keys), torch.empty_like(vals)
     call = rs_sort_u64_pairs64 if vals.element_size() == 8 else rs_sort_u64_pairs
@@ -232,7 +233,7 @@ def rs_sort_u32_pairs64(keys_in, vals_in, keys_out, vals_out, n: int, num_parts:
     rs_sort_u32."""
     tp, tb = _temp(temp)
     offs = np.zeros(num_parts + 1, dtype=np.uint64) if (want_offsets and temp is not None) else None
-    op = offs.ctypes.data_as(_U64P) if offs is not None else None
+    op = offs.ctypes.data if offs is not None else None
     _check(lib.rs_sort_u32_pairs64(_ptr(keys_in), _ptr(vals_in), _ptr(keys_out), _ptr(vals_out), n, num_parts,
                                    op, _plan(plan), tp, ctypes.byref(tb),
                                    _stream(stream) if temp is not None else None))
@@ -242,7 +243,6 @@ def rs_sort_u32_pairs64(keys_in, vals_in, keys_out, vals_out, n: int, num_parts:
 def sort_pairs64(keys, vals, num_parts: int = 64, plan=None, stream=None):
     """Stable (32-bit key, 64-bit value) sort of CUDA tensors: (keys, vals,
     host partition offsets)."""
-    import torch
     n = keys.numel()
     ko, vo = torch.empty_like(keys), torch.empty_like(vals)
     temp = _alloc_temp(rs_sort_u32_pairs64(None, None, None, None, n, plan=plan), keys.device)
@@ -254,7 +254,6 @@ def sort64(keys, num_parts: int = 64, plan=None, out=None, temp=None, stream=Non
     """Sorted copy of a CUDA tensor of 64-bit keys (int64 storage of uint64
     keys by default; plan={"key_kind": RS_KEY_I32 or RS_KEY_F32} for signed
     or binary64 keys) and the host partition offsets."""
-    import torch
     n = keys.numel()
     out = torch.empty_like(keys) if out is None else out
     if temp is None:
@@ -268,7 +267,7 @@ def rs_merge_u32(a, va, na: int, b, vb, nb: int, out, vout, num_parts: int = 64,
     """Calls rs_merge_u32; returns as rs_sort_u32."""
     tp, tb = _temp(temp)
     offs = np.zeros(num_parts + 1, dtype=np.uint64) if (want_offsets and temp is not None) else None
-    op = offs.ctypes.data_as(_U64P) if offs is not None else None
+    op = offs.ctypes.data if offs is not None else None
     _check(lib.rs_merge_u32(_ptr(a), _ptr(va), na, _ptr(b), _ptr(vb), nb, _ptr(out), _ptr(vout), num_parts, op,
                             _plan(plan), tp, ctypes.byref(tb), _stream(stream) if temp is not None else None))
     return tb.value if temp is None else offs
@@ -277,7 +276,6 @@ def rs_merge_u32(a, va, na: int, b, vb, nb: int, out, vout, num_parts: int = 64,
 def merge(a, b, va=None, vb=None, num_parts: int = 64, plan=None, stream=None):
     """Stable merge of two sorted CUDA tensors of 32-bit keys (and their
     payloads): (keys, vals or None, host partition offsets)."""
-    import torch
     na, nb = a.numel(), b.numel()
     out = torch.empty(na + nb, dtype=a.dtype, device=a.device)
     vout = None if va is None else torch.empty(na + nb, dtype=va.dtype, device=a.device)
@@ -293,7 +291,7 @@ def rs_sort_u32_host(h_keys_in, h_vals_in, h_keys_out, h_vals_out, n: int, num_p
     Returns as rs_sort_u32."""
     tp, tb = _temp(temp)
     offs = np.zeros(num_parts + 1, dtype=np.uint64) if (want_offsets and temp is not None) else None
-    op = offs.ctypes.data_as(_U64P) if offs is not None else None
+    op = offs.ctypes.data if offs is not None else None
     _check(lib.rs_sort_u32_host(_ptr(h_keys_in), _ptr(h_vals_in), _ptr(h_keys_out), _ptr(h_vals_out), n,
                                 num_parts, op, _plan(plan), tp, ctypes.byref(tb),
                                 _stream(stream) if temp is not None else None))
@@ -308,7 +306,7 @@ def rs_sort_u32_segmented(keys_in, vals_in, keys_out, vals_out, d_seg_offsets, h
     tp, tb = _temp(temp)
     h = np.ascontiguousarray(h_seg_offsets, dtype=np.uint64)
     _check(lib.rs_sort_u32_segmented(_ptr(keys_in), _ptr(vals_in), _ptr(keys_out), _ptr(vals_out),
-                                     _ptr(d_seg_offsets), h.ctypes.data_as(_U64P), num_segs, total_n,
+                                     _ptr(d_seg_offsets), h.ctypes.data, num_segs, total_n,
                                      num_parts, _ptr(d_part_offsets), _plan(plan), tp, ctypes.byref(tb),
                                      _stream(stream) if temp is not None else None))
     return tb.value if temp is None else None
@@ -333,7 +331,7 @@ def rs_sort_u32_noalloc(keys_in, keys_out, n: int, num_parts: int = 64, stream=N
     fixed scratch (no device allocation; n <= RS_NOALLOC_MAX_KEYS).  Returns
     the partition offsets (numpy uint64[num_parts + 1]) or None."""
     offs = np.zeros(num_parts + 1, dtype=np.uint64) if want_offsets else None
-    op = offs.ctypes.data_as(_U64P) if offs is not None else None
+    op = offs.ctypes.data if offs is not None else None
     _check(lib.rs_sort_u32_noalloc(_ptr(keys_in), _ptr(keys_out), n, num_parts, op, _stream(stream)))
     return offs
 
@@ -411,7 +409,6 @@ def rs_trace_read() -> dict:
 def _empty_u32(n, device, like=None):
     """An output buffer of n 32-bit words (the input's dtype when given:
     int32 storage of uint32 keys, or float32 / int32 keys of another kind)."""
-    import torch
     dtype = like.dtype if like is not None and like.element_size() == 4 else torch.int32
     return torch.empty(max(n, 0), dtype=dtype, device=device)
 
@@ -423,7 +420,6 @@ def temp_bytes(n: int, pairs: bool = False, plan=None) -> int:
 
 
 def _alloc_temp(nbytes: int, device):
-    import torch
     return torch.empty(max(nbytes, 1), dtype=torch.uint8, device=device)
 
 
@@ -453,7 +449,6 @@ def sort_pairs(keys, vals, num_parts: int = 64, plan=None, out_keys=None, out_va
 def sort_segmented(keys, vals, seg_offsets_host, num_parts: int = 64, plan=None, temp=None, stream=None,
                    want_part_offsets: bool = True):
     """Segmented sort; seg_offsets_host is a numpy uint64 array (num_segs+1)."""
-    import torch
     h = np.ascontiguousarray(seg_offsets_host, dtype=np.uint64)
     num_segs = h.size - 1
     total = int(h[-1]) if h.size else 0

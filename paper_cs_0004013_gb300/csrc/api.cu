@@ -381,10 +381,11 @@ struct Layout {
   size_t alt_k = 0, alt_v = 0;
   size_t memset_bytes = 0;  // ctrl + hist (+ the buckets' counts), cleared before the histogram
   HybLayout hyb;
+  size_t fcounts = 0, fcursors = 0, fctrl = 0;  // the single-launch sort's value buckets (0: none)
   size_t total = 0;
 };
 
-Layout make_layout(const SortPlan& p, uint64_t n, bool pairs, bool hybrid = false) {
+Layout make_layout(const SortPlan& p, uint64_t n, bool pairs, bool hybrid = false, bool fused = false) {
   Layout L;
   const size_t digits = size_t(1) << p.R;
   size_t off = 0;
@@ -398,10 +399,20 @@ Layout make_layout(const SortPlan& p, uint64_t n, bool pairs, bool hybrid = fals
   off = align_up(off + size_t(p.nd) * digits * 4);
   L.cursors0 = off;
   off = align_up(off + 256 * 4);
+  if (fused) {
+    for (size_t* at : {&L.fcounts, &L.fcursors}) {
+      *at = off;
+      off = align_up(off + kFusedMaxBuckets * 4);
+    }
+  }
   L.status = off;
   L.status_bytes = (p.status_rows > p.num_tiles ? p.status_rows : p.num_tiles) * digits * (p.k->wide_status ? 8 : 4);
   off = align_up(off + L.status_bytes);
   off = L.hyb.place_rest(off);
+  if (fused) {
+    L.fctrl = off;
+    off += align_up(sizeof(HybCtrl));
+  }
   if (p.nd > 1 && n > 0) {
     L.alt_k = off;
     off = align_up(off + size_t(n) * 4);
@@ -827,8 +838,14 @@ rs_status run_fused(const SortPlan& p, const Layout& L, const uint32_t* keys_in,
   const bool pairs = vals_in != nullptr;
   const uint32_t tiles = (n + fused_tile_keys(shape) - 1) / fused_tile_keys(shape);
   if (size_t(tiles) * 256 * 4 > L.status_bytes) return fail(RS_ERR_CUDA, "single-launch sort: status too small");
-  RS_CUDA(traced(T_CLEAR, 0, s, [&] { return cudaMemsetAsync(temp, 0, L.status + size_t(tiles) * 256 * 4, s); }),
-          "cudaMemsetAsync(temp)");
+  const size_t clear_bytes = L.status;  // (the launch clears its status rows itself)
+  // value buckets: as many as tiles, twice as many of the largest tiles (whose
+  // number may exceed the SMs'), when a block more than tiles, which takes the
+  // sample, is resident too
+  const uint32_t buckets = shape == 0 ? 2 * tiles : tiles;
+  const bool offered = L.fcounts && buckets >= 2 && buckets <= kFusedMaxBuckets && tiles < ds->fused_tiles[pairs][shape];
+  HybCtrl* hc = reinterpret_cast<HybCtrl*>(temp + L.fctrl);
+  RS_CUDA(traced(T_CLEAR, 0, s, [&] { return cudaMemsetAsync(temp, 0, clear_bytes, s); }), "cudaMemsetAsync(temp)");
   FusedArgs a{};
   a.keys_in = keys_in;
   a.keys_out = keys_out;
@@ -840,8 +857,15 @@ rs_status run_fused(const SortPlan& p, const Layout& L, const uint32_t* keys_in,
   a.xf = p.xf;
   a.hist = reinterpret_cast<uint32_t*>(temp + L.hist);
   a.status = temp + L.status;
+  a.first_cursors = reinterpret_cast<uint32_t*>(temp + L.cursors0);
   a.bar = reinterpret_cast<uint32_t*>(temp + L.ctrl) + 12;
   a.err = ds->err;
+  if (offered) {
+    a.ctrl = hc;
+    a.buckets = buckets;
+    a.counts = reinterpret_cast<uint32_t*>(temp + L.fcounts);
+    a.cursors = reinterpret_cast<uint32_t*>(temp + L.fcursors);
+  }
   RS_CUDA(traced(T_FUSED, n, s, [&] { return launch_fused(a, tiles, pairs, shape, s); }), "launch fused sort");
   return RS_OK;
 }
@@ -863,7 +887,7 @@ rs_status sort_impl(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* 
   if (fusable && n <= kFusedStatusMaxKeys)  // status rows for the single-launch sort's smallest tiles
     p.status_rows = size_t((n + fused_tile_keys(kFusedShapes - 1) - 1) / fused_tile_keys(kFusedShapes - 1));
   const bool hybrid = fusable && !pairs && n >= kHybridMinKeys && n <= kHybridMaxKeys;
-  Layout L = make_layout(p, n, pairs, hybrid);
+  Layout L = make_layout(p, n, pairs, hybrid, p.status_rows > 0);
   MsdLayout M;
   if (p.msd) {
     if (rs_status st2 = make_msd_layout(p, n, pairs, &M); st2 != RS_OK) return st2;
@@ -924,7 +948,7 @@ rs_status sort_impl(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* 
   if (fusable) {
     int sh = 0;
     for (int c = kFusedShapes - 1; c > 0; --c)
-      if ((n + fused_tile_keys(c) - 1) / fused_tile_keys(c) <= uint64_t(ds->num_sms)) {
+      if ((n + fused_tile_keys(c) - 1) / fused_tile_keys(c) < uint64_t(ds->num_sms)) {
         sh = c;
         break;
       }
@@ -1185,8 +1209,9 @@ static rs_status sort64_impl(const uint64_t* keys_in, const void* vals_in, uint6
   SortPlan p;
   if (rs_status st = make_plan(n, true, &q, &p, pairs ? 2 : 1); st != RS_OK) return st;
   const bool automatic = !plan || (plan->digit_bits == 0 && plan->mode == RS_MODE_AUTO && plan->tile == 0);
-  const bool hybrid = automatic && vbytes == 0 && n >= kHybridMinKeys && n <= kHybridMaxKeys;
-  const Layout64 L = make_layout64(p, n, pairs, vbytes == 8, hybrid);
+  // (the space for value buckets is part of every plan's layout)
+  Layout64 L = make_layout64(p, n, pairs, vbytes == 8, vbytes == 0 && n >= kHybridMinKeys && n <= kHybridMaxKeys);
+  if (!automatic) L.hyb.buckets = 0;
   if (vbytes == 8 && !L.fused)
     return fail(RS_ERR_UNSUPPORTED, "64-bit values: tile shape %u has no interleaved pass kernel", q.tile);
   if (!temp) {

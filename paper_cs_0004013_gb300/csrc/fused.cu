@@ -15,13 +15,25 @@
 //   3. for each executed digit: the block's tile goes through the pass of the
 //      half-warp-group kernel (onesweep2.cuh), the lookback ordering the
 //      tiles inside the pass;                                     barrier
+// One block more than tiles samples the keys (sample.cuh) during phase 1.
+// Keys that it found spread evenly over their value range take value buckets
+// instead of the passes, in the same launch: each block
+// counts its tile's keys per bucket (about as many buckets as blocks);
+// barrier; it scans the totals, claims its tile's places and writes the tile
+// to its buckets (with a payload, the key and its place in the input, so that
+// no order needs to be kept); barrier; the blocks sort the buckets
+// (local.cuh).  Three barriers and three trips of a key instead of four or five.
 // Loads use the L2 path (ld.global.cg): later passes read what other blocks
 // wrote earlier in the same launch.  Every barrier wait is bounded: a block
 // that waits too long raises the device error word and goes on, so the
 // launch always ends.
 #include <cstdint>
 
+#include "local.cuh"
+#include "sample.cuh"
 #include "onesweep2.cuh"
+#include "split.cuh"
+#include "value_map.cuh"
 
 namespace rs {
 namespace {
@@ -33,8 +45,9 @@ constexpr int kFusedThreads = 384;
 // has an SM of its own (GB300: 2^19 keys in 39.5 us with 384 x 12 against
 // 43.8 with 384 x 24) and slower once tiles share SMs (2^20 keys: 50.1
 // against 47.4).
-constexpr int kFusedItems[kFusedShapes] = {24, 18, 12};
-constexpr int fused_min_blocks(int items) { return items <= 12 ? 3 : 2; }
+constexpr int kFusedItems[kFusedShapes] = {24, 20, 12};
+// (The smaller shapes run one tile per SM.)
+constexpr int fused_min_blocks(int items) { return items <= 20 ? 1 : 2; }
 // Status rows a digit thread reads per lookback round (GB300, 2^20 keys in
 // 152 tiles of 384 x 18: the kernel takes 44.7 us with 8 rows per round,
 // 47.8 with 16 and 62.1 with 32).
@@ -42,12 +55,34 @@ constexpr int kFusedLookback = 8;
 // Rounds of a barrier wait (about 64 ns each) before it gives up.
 constexpr uint32_t kBarrierSpinLimit = 1u << 21;
 
+// Value buckets: a bucket is sorted by the block's threads, with 24 keys each
+// at 384 x 20 tiles, 16 otherwise (the buckets are a third smaller then).
+static_assert(int(kFusedMaxBuckets) == 2 * kFusedThreads, "two buckets per thread");
+constexpr int fused_bucket_items(int items) { return items == 20 ? 24 : 16; }
+constexpr int kFusedBucketBits = 13;
+
 template <int NV, int ITEMS>
 struct FusedLayout {
   using L = Onesweep2Layout<kFusedThreads, ITEMS, NV>;
   static constexpr size_t OFF_BASES = (L::SMEM + 15) / 16 * 16;  // [4][256]
   static constexpr size_t OFF_FLAGS = OFF_BASES + 4 * 256 * 4;   // [4] skip flags
-  static constexpr size_t SMEM = OFF_FLAGS + 16;
+  static constexpr size_t END_PASSES = OFF_FLAGS + 16;
+  static_assert(SplitLayout<uint32_t, kFusedThreads, ITEMS>::SMEM <= OFF_BASES, "the first pass leaves the bases alone");
+  // value buckets: the staged tile (keys, then places), counts of the two
+  // half-warps, write-out offsets; the bucket starts stay behind the local sort's space
+  static constexpr int BITEMS = fused_bucket_items(ITEMS);
+  static constexpr uint32_t BCAP = uint32_t(kFusedThreads * BITEMS);  // keys of a bucket
+  using Sample = SampleLayout<uint32_t, 1, kFusedThreads>;
+  using B = LocalLayout<kFusedThreads, BITEMS, kFusedBucketBits, uint32_t, NV ? 4 : 0,
+                        NV ? Vals::kPlaces : Vals::kAlone>;
+  static constexpr size_t OFF_CNT = size_t(L::TILE) * 4 * (1 + NV);
+  static constexpr size_t OFF_GOFF = OFF_CNT + 2 * (kFusedMaxBuckets + 1) * 4;
+  static constexpr size_t OFF_SUMS = OFF_GOFF + kFusedMaxBuckets * 4;
+  static constexpr size_t END_SPLIT = OFF_SUMS + 64 * 4;
+  static constexpr size_t OFF_STARTS = ((END_SPLIT > B::SMEM ? END_SPLIT : B::SMEM) + 15) / 16 * 16;
+  static constexpr size_t END_BUCKETS = OFF_STARTS + (kFusedMaxBuckets + 4) * 4;
+  static constexpr size_t SMEM = END_PASSES > END_BUCKETS ? END_PASSES : END_BUCKETS;
+  static_assert(Sample::SMEM <= SMEM, "the sample fits");
 };
 
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
@@ -75,6 +110,106 @@ __device__ __forceinline__ void grid_barrier(uint32_t* bar, uint32_t target, uin
   __syncthreads();
 }
 
+// The value buckets' way (see above); false, with nothing written but the
+// counts and `bar` advanced by one barrier, when a bucket does not fit the
+// local sort (every block comes to the same answer).
+template <int NV, int ITEMS>
+__device__ __forceinline__ bool fused_buckets(const FusedArgs& a, unsigned char* smem, uint32_t& barriers) {
+  using FL = FusedLayout<NV, ITEMS>;
+  constexpr uint32_t TILE = FL::L::TILE;
+  constexpr int T = kFusedThreads, ROW = kFusedMaxBuckets + 1;
+  uint32_t* s_key = reinterpret_cast<uint32_t*>(smem);
+  uint32_t* s_place = s_key + TILE;
+  uint32_t* s_cnt = reinterpret_cast<uint32_t*>(smem + FL::OFF_CNT);
+  uint32_t* s_goff = reinterpret_cast<uint32_t*>(smem + FL::OFF_GOFF);
+  uint32_t* s_sums = reinterpret_cast<uint32_t*>(smem + FL::OFF_SUMS);
+  uint32_t* s_starts = reinterpret_cast<uint32_t*>(smem + FL::OFF_STARTS);
+  const int tid = threadIdx.x, lane = tid & 31;
+  const uint32_t tiles = a.tiles, B = a.buckets, n = a.n;
+  const uint32_t base = blockIdx.x * TILE;
+  const uint32_t valid = n - base < TILE ? n - base : TILE;
+  auto has = [&](int j) { return uint32_t(j * T + tid) < valid; };
+  const ValueMap<uint32_t> map = load_map<uint32_t>(a.ctrl);
+  // 1. load, count
+  uint32_t key[ITEMS];
+#pragma unroll
+  for (int j = 0; j < ITEMS; ++j) key[j] = has(j) ? ld_stream(a.keys_in + base + j * T + tid) : 0u;
+  for (int i = tid; i < 2 * ROW; i += T) s_cnt[i] = 0u;
+  __syncthreads();
+  const uint32_t row = smem_addr(s_cnt + (lane >> 4) * ROW);
+#pragma unroll
+  for (int j = 0; j < ITEMS; ++j) {
+    key[j] = to_ordered(key[j], a.xf);
+    if (has(j)) sh_red_add(row + 4u * map.bucket(key[j]), 1u);
+  }
+  __syncthreads();
+  const uint32_t d0 = 2u * tid;  // this thread's buckets d0 and d0 + 1
+  const uint32_t c00 = s_cnt[d0], c01 = s_cnt[d0 + 1];
+  const uint32_t t0 = c00 + s_cnt[ROW + d0], t1 = c01 + s_cnt[ROW + d0 + 1];
+  if (t0) atomicAdd(a.counts + d0, t0);
+  if (t1) atomicAdd(a.counts + d0 + 1, t1);
+  grid_barrier(a.bar, gridDim.x + tiles * barriers++, a.err);
+  // 2. the buckets' starts and the tile's own scan; places claimed
+  const uint32_t g0 = d0 < B ? __ldcg(a.counts + d0) : 0u, g1 = d0 + 1 < B ? __ldcg(a.counts + d0 + 1) : 0u;
+  if (__syncthreads_or(g0 > FL::BCAP || g1 > FL::BCAP)) return false;
+  uint32_t k0 = 0, k1 = 0;
+  if (t0) k0 = atomicAdd(a.cursors + d0, t0);
+  if (t1) k1 = atomicAdd(a.cursors + d0 + 1, t1);
+  {
+    const uint32_t x[2] = {g0 + g1, 0u}, y[2] = {t0 + t1, 0u};
+    uint32_t start[2], excl[2], total;
+    block_exclusive_sums<T, 2>(x, start, s_sums, &total);
+    __syncthreads();
+    block_exclusive_sums<T, 2>(y, excl, s_sums, &total);
+    s_starts[d0] = start[0];
+    s_starts[d0 + 1] = start[0] + g0;
+    if (tid == T - 1) s_starts[2 * T] = n;
+    s_goff[d0] = start[0] + k0 - excl[0];
+    s_goff[d0 + 1] = start[0] + g0 + k1 - (excl[0] + t0);
+    s_cnt[d0] = excl[0];
+    s_cnt[ROW + d0] = excl[0] + c00;
+    s_cnt[d0 + 1] = excl[0] + t0;
+    s_cnt[ROW + d0 + 1] = excl[0] + t0 + c01;
+  }
+  __syncthreads();
+  // 3. the tile by buckets, then out
+#pragma unroll
+  for (int j = 0; j < ITEMS; ++j) {
+    if (has(j)) {
+      uint32_t p;
+      asm volatile("atom.shared.add.u32 %0, [%1], 1;" : "=r"(p) : "r"(row + 4u * map.bucket(key[j])) : "memory");
+      s_key[p] = key[j];
+      if constexpr (NV != 0) s_place[p] = base + j * T + tid;
+    }
+  }
+  __syncthreads();
+  bool oob = false;
+#pragma unroll
+  for (int j = 0; j < ITEMS; ++j) {
+    if (has(j)) {
+      const uint32_t i = j * T + tid, k = s_key[i], g = s_goff[map.bucket(k)] + i;
+      if (g < n) {
+        st_global(a.keys_alt + g, k);
+        if constexpr (NV != 0) st_global(a.vals_alt + g, s_place[i]);
+      } else {
+        oob = true;
+      }
+    }
+  }
+  if (oob) atomicOr(a.err, kErrBounds);
+  grid_barrier(a.bar, gridDim.x + tiles * barriers++, a.err);
+  // 4. the buckets
+  for (uint32_t b = blockIdx.x; b < B; b += tiles) {
+    const uint32_t s = s_starts[b], e = s_starts[b + 1];
+    if (s == e) continue;
+    uint32_t* vout = NV ? a.vals_out + s : nullptr;
+    local_sort_array<T, FL::BITEMS, kFusedBucketBits, NV ? 4 : 0, NV ? Vals::kPlaces : Vals::kAlone, true>(
+        a.keys_alt + s, a.keys_out + s, a.vals_alt + s, vout, a.vals_in, e - s, Ord32{KeyXform{0u, 0u}}, Ord32{a.xf},
+        RangeBins<uint32_t>{}, smem);
+  }
+  return true;
+}
+
 template <int NV, int ITEMS>
 __global__ void __launch_bounds__(kFusedThreads, fused_min_blocks(ITEMS)) fused_sort_kernel(const FusedArgs a) {
   using FL = FusedLayout<NV, ITEMS>;
@@ -84,11 +219,24 @@ __global__ void __launch_bounds__(kFusedThreads, fused_min_blocks(ITEMS)) fused_
   uint32_t* s_flags = reinterpret_cast<uint32_t*>(smem + FL::OFF_FLAGS);
   uint32_t* s_cnt = reinterpret_cast<uint32_t*>(smem + L::OFF_TBL);  // [4][256] while counting
   const int tid = threadIdx.x;
-  const uint32_t tile = blockIdx.x, tiles = gridDim.x;
+  const uint32_t tile = blockIdx.x, tiles = a.tiles;
   const uint32_t n = a.n;
+  uint32_t barriers = 0;  // barriers passed so far (the n-th of all tiles awaits gridDim.x + (n - 1) * tiles arrivals)
+  constexpr bool kFreeFirst = NV == 0;  // keys alone: the first executed pass keeps no order
 
-  // 1. counts of the tile's four digits (order-mapped keys)
+  if (tile == tiles) {  // one block more, when value buckets are offered: it takes the sample meanwhile
+    sample_body<uint32_t, 1, kFusedThreads>(a.keys_in, n, a.buckets, Ord32{a.xf}, a.ctrl, smem, [] {});
+    __syncthreads();
+    if (tid == 0) {
+      __threadfence();
+      atomicAdd(a.bar, 1u);
+    }
+    return;
+  }
+
+  // 1. counts of the tile's four digits (order-mapped keys); the tile's status row cleared
   for (int i = tid; i < 1024; i += kFusedThreads) s_cnt[i] = 0u;
+  if (tid < 256) static_cast<uint32_t*>(a.status)[size_t(tile) * 256 + tid] = 0u;
   __syncthreads();
   {
     const uint32_t cnt = smem_addr(s_cnt);
@@ -103,7 +251,9 @@ __global__ void __launch_bounds__(kFusedThreads, fused_min_blocks(ITEMS)) fused_
   __syncthreads();
   for (int i = tid; i < 1024; i += kFusedThreads)
     if (s_cnt[i]) atomicAdd(a.hist + i, s_cnt[i]);
-  grid_barrier(a.bar, tiles, a.err);
+  grid_barrier(a.bar, gridDim.x, a.err);  // (the sampling block passes the first barrier only)
+  barriers = 1;
+  if (a.ctrl && __ldcg(&a.ctrl->route) == kHybBuckets && fused_buckets<NV, ITEMS>(a, smem, barriers)) return;
 
   // 2. bases and skip flags of every digit (each block for itself)
   if (tid < 4) s_flags[tid] = 0u;
@@ -149,18 +299,32 @@ __global__ void __launch_bounds__(kFusedThreads, fused_min_blocks(ITEMS)) fused_
     }
     job.xin = e == 0 ? a.xf : KeyXform{0u, 0u};
     job.xout = e == m - 1 ? a.xf : KeyXform{0u, 0u};
-    job.parity = uint32_t(e & 1) ^ 1u;
+    // the status words are clear for the first pass with a chained scan
+    job.parity = uint32_t((e - (kFreeFirst ? 1 : 0)) & 1) ^ 1u;
     job.status = a.status;
     job.bases = s_bases + 256 * j;
     job.shift = uint32_t(8 * j);
     job.err = a.err;
-    bool unstable = false;  // the first executed pass of keys on a full tile: equal digits leave in any order
-    if constexpr (NV == 0) unstable = e == 0 && (size_t(tile) + 1) * L::TILE <= size_t(n);
-    if (unstable)
-      onesweep2_tile<kFusedThreads, ITEMS, NV, uint32_t, false, kFusedLookback, true, true>(job, smem);
-    else
-      onesweep2_tile<kFusedThreads, ITEMS, NV, uint32_t, false, kFusedLookback, true, false>(job, smem);
-    if (e + 1 < m) grid_barrier(a.bar, tiles * uint32_t(2 + e), a.err);
+    if constexpr (kFreeFirst) {
+      if (e == 0) {  // no earlier order to keep: a split by claims (split.cuh)
+        const uint32_t sel = 0x4440u | uint32_t(j);
+        auto digit = [&](uint32_t k) { return byte_digit(k, sel); };
+        const uint32_t base = tile * uint32_t(L::TILE), left = n - base;
+        const Ord32 ordi{job.xin}, ordo{job.xout};
+        if (left >= uint32_t(L::TILE))
+          split_tile<uint32_t, kFusedThreads, ITEMS, true>(job.kin + base, L::TILE, job.kout, a.first_cursors, n, digit,
+                                                           ordi, ordo, a.err, smem, job.bases);
+        else
+          split_tile<uint32_t, kFusedThreads, ITEMS, false>(job.kin + base, left, job.kout, a.first_cursors, n, digit,
+                                                            ordi, ordo, a.err, smem, job.bases);
+        __syncthreads();
+      }
+    }
+    // one block per SM (the smaller shapes): nothing else hides the payload loads, and registers are free
+    constexpr bool EARLY_VALS = NV != 0 && fused_min_blocks(ITEMS) == 1;
+    if (!kFreeFirst || e != 0)
+      onesweep2_tile<kFusedThreads, ITEMS, NV, uint32_t, false, kFusedLookback, true, EARLY_VALS>(job, smem);
+    if (e + 1 < m) grid_barrier(a.bar, gridDim.x + tiles * barriers++, a.err);
   }
 }
 
@@ -188,8 +352,9 @@ const void* fused_func(bool pairs, int shape) {
 
 cudaError_t launch_fused(const FusedArgs& a, unsigned tiles, bool pairs, int shape, cudaStream_t s) {
   FusedArgs args = a;
+  args.tiles = tiles;
   void* params[] = {&args};
-  return cudaLaunchCooperativeKernel(fused_func(pairs, shape), dim3(tiles), dim3(kFusedThreads), params,
+  return cudaLaunchCooperativeKernel(fused_func(pairs, shape), dim3(tiles + (a.ctrl ? 1u : 0u)), dim3(kFusedThreads), params,
                                      fused_smem(pairs, shape), s);
 }
 

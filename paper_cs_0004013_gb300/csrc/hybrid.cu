@@ -23,45 +23,19 @@
 // ones), the keys cross memory three times instead of four or eight, and keys
 // without payloads need no stable ranking: a key's place in its tile is one
 // shared atomic, and a tile's place in a bucket one global atomic.
-#include <cooperative_groups.h>
-
 #include <cstdint>
 
 #include "hybrid.h"
 #include "local.cuh"
+#include "sample.cuh"
 #include "split.cuh"
+#include "value_map.cuh"
 
 namespace rs {
 namespace {
 
 constexpr int kSampleThreads = 1024;
 constexpr int kCountThreads = 1024;
-constexpr uint32_t kCoarse = 64;  // slices of the range for the evenness test
-
-// The linear map of a key's value to [0, 2^32): bucket = high word of the
-// product, place inside the bucket = low word.  Values outside the sampled
-// range [lo, hi] fall in the first or last bucket.  32-bit keys take the
-// offset and the product in one wide multiply-add: back = -lo * mult.
-template <typename K>
-struct ValueMap {
-  K lo, hi;
-  uint32_t sh, mult;
-  uint64_t back;
-  __device__ __forceinline__ K clamp(K k) const {
-    const K t = k > lo ? k : lo;
-    return t < hi ? t : hi;
-  }
-  // the product for a key inside [lo, hi]
-  __device__ __forceinline__ uint64_t product(K k) const {
-    if constexpr (sizeof(K) == 8) return uint64_t(uint32_t((k - lo) >> sh)) * mult;
-    else return uint64_t(k) * mult + back;
-  }
-  __device__ __forceinline__ uint32_t bucket(K k) const { return uint32_t(product(clamp(k)) >> 32); }
-};
-template <typename K>
-__device__ __forceinline__ ValueMap<K> load_map(const HybCtrl* c) {
-  return ValueMap<K>{K(c->lo), K(c->hi), c->sh, c->mult, 0ull - uint64_t(K(c->lo)) * c->mult};
-}
 
 // Bins of a bucket: the low word of the same product.  EDGE: the first and
 // last bucket, which also hold the values outside the sampled range.
@@ -90,146 +64,20 @@ struct OrdOf<uint64_t> {
   __device__ static T identity() { return Ord64{KeyXform64{0u, 0u, 0u}}; }
 };
 
-// ------------------------------------------------------------------ sample
-// One cluster of eight blocks.  The sample: S keys, one from each of S equal
-// stretches of the input at a place inside the stretch that a hash picks (a
-// periodic input does not line up with it).  Every block reads an eighth of
-// it into the first block's shared memory (one SM alone takes its scattered
-// reads one sector at a time), and the first block decides.  The keys count as spread
-// evenly when
-//  - no 64th of the range holds more than 1.5 times its share of the sample
-//    (uniform keys: 128 or more expected, five standard deviations below);
-//  - no bucket holds more than 1.5 times its share of the sample and kFineLimit keys;
-//  - few sampled keys are equal to another one: many equal keys end up in few
-//    bins of a bucket, which then takes the digit passes.
+// ------------------------------------------------------------------ sample (sample.cuh)
 constexpr int kSampleBlocks = 8;
-constexpr uint32_t kFineLimit = 12;
-template <typename K>
-struct SampleLayout {
-  static constexpr int S = 8192;
-  static constexpr int PER = S / kSampleThreads;                 // of the deciding block
-  static constexpr int LOADS = S / (kSampleThreads * kSampleBlocks);  // of every block
-  static constexpr size_t OFF_KEYS = size_t(kHybMaxBuckets) * 4;  // behind the fine counts (later the hash slots)
-  static constexpr size_t OFF_RED = OFF_KEYS + size_t(S) * sizeof(K);
-  static constexpr size_t OFF_COARSE = OFF_RED + 64 * 8;
-  static constexpr size_t SMEM = OFF_COARSE + kCoarse * 4;
-};
-
 template <typename K>
 __global__ void __cluster_dims__(kSampleBlocks, 1, 1) __launch_bounds__(kSampleThreads, 1)
     sample_kernel(const HybArgs a) {
-  using L = SampleLayout<K>;
-  namespace cg = cooperative_groups;
   extern __shared__ __align__(16) unsigned char smem[];
-  uint32_t* s_fine = reinterpret_cast<uint32_t*>(smem);
-  K* s_keys = reinterpret_cast<K*>(smem + L::OFF_KEYS);
-  K* s_red = reinterpret_cast<K*>(smem + L::OFF_RED);
-  uint32_t* s_coarse = reinterpret_cast<uint32_t*>(smem + L::OFF_COARSE);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const auto ord = OrdOf<K>::make(a);
-  const K* in = reinterpret_cast<const K*>(a.keys_in);
-  const uint64_t n = a.n;
-  const uint32_t stretch = uint32_t(n / L::S);
-  cg::cluster_group cluster = cg::this_cluster();
-  K got[L::LOADS];
-#pragma unroll
-  for (int i = 0; i < L::LOADS; ++i) {
-    const uint32_t q = (i * kSampleBlocks + blockIdx.x) * kSampleThreads + tid;
-    uint32_t h = q * 0x9E3779B1u;
-    h ^= h >> 15;
-    const uint64_t pos = (uint64_t(q) * n) / L::S + (stretch > 1 ? __umulhi(h * 0x85EBCA77u, stretch) : 0u);
-    got[i] = ord.map(ld_elem(in + (pos < n ? pos : n - 1)));
-  }
-  if (blockIdx.x == 0) {
-    uint4* f4 = reinterpret_cast<uint4*>(smem);
-    for (uint32_t i = tid; i < (a.buckets + 3) / 4; i += kSampleThreads) f4[i] = make_uint4(0u, 0u, 0u, 0u);
-    if (tid < int(kCoarse)) s_coarse[tid] = 0u;
-  }
-  // the first block runs: its shared memory may be written
-  asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
-  K* to = cluster.map_shared_rank(s_keys, 0);
-#pragma unroll
-  for (int i = 0; i < L::LOADS; ++i) to[(i * kSampleBlocks + blockIdx.x) * kSampleThreads + tid] = got[i];
-  cluster.sync();
-  if (blockIdx.x != 0) {  // the others clear what the launches that follow start from
-    for (size_t i = size_t(blockIdx.x - 1) * kSampleThreads + tid; i < a.clear_vec4;
-         i += (kSampleBlocks - 1) * kSampleThreads)
+  // the blocks other than the first clear what the launches that follow start from
+  sample_body<K, kSampleBlocks, kSampleThreads>(static_cast<const K*>(a.keys_in), a.n, a.buckets, OrdOf<K>::make(a),
+                                                a.ctrl, smem, [&] {
+    for (size_t i = size_t(blockIdx.x - 1) * kSampleThreads + threadIdx.x; i < a.clear_vec4;
+         i += size_t(kSampleBlocks - 1) * kSampleThreads)
       a.clear[i] = make_uint4(0u, 0u, 0u, 0u);
-    return;
-  }
-
-  K key[L::PER];
-  K lo = ~K(0), hi = 0;
-#pragma unroll
-  for (int i = 0; i < L::PER; ++i) {
-    key[i] = s_keys[i * kSampleThreads + tid];
-    lo = key[i] < lo ? key[i] : lo;
-    hi = key[i] > hi ? key[i] : hi;
-  }
-  warp_min_max(lo, hi);
-  if (lane == 0) {
-    s_red[warp] = lo;
-    s_red[32 + warp] = hi;
-  }
-  __syncthreads();
-  lo = s_red[lane];
-  hi = s_red[32 + lane];
-  warp_min_max(lo, hi);
-  // a little wider than the sample, so that the values outside it (about
-  // 1 / S of the keys on either side) have buckets of their own
-  const K ext = (hi - lo) / (L::S / 8);
-  ValueMap<K> m;
-  m.lo = lo > ext ? lo - ext : K(0);
-  m.hi = hi < ~K(0) - ext ? hi + ext : ~K(0);
-  const K span = m.hi - m.lo;
-  const int bits = span == 0 ? 1 : 64 - __clzll((long long)(uint64_t)span);
-  m.sh = bits > 32 ? uint32_t(bits - 32) : 0u;
-  const uint64_t range = uint64_t(span >> m.sh) + 1;  // <= 2^32
-  m.mult = uint32_t((uint64_t(a.buckets) << 32) / (range > a.buckets ? range : uint64_t(a.buckets) + 1));
-  m.back = 0ull - uint64_t(m.lo) * m.mult;
-  bool bad = range <= a.buckets;
-  const uint32_t fine_limit = kFineLimit + uint32_t(L::S) * 3 / (2 * a.buckets);
-#pragma unroll
-  for (int i = 0; i < L::PER; ++i) {
-    const uint32_t b = m.bucket(key[i]);
-    if (atomicAdd(&s_fine[b], 1u) >= fine_limit) bad = true;
-    atomicAdd(&s_coarse[(b * kCoarse) / a.buckets], 1u);
-  }
-  __syncthreads();
-  if (a.buckets >= 4 * kCoarse && tid < int(kCoarse) && s_coarse[tid] * kCoarse * 2 > uint32_t(L::S) * 3) bad = true;
-  // equal keys: each writes its number to a hash slot, and reads back whose
-  // number stayed; an equal key's means a duplicate
-  uint16_t* s_slot = reinterpret_cast<uint16_t*>(smem);
-  auto slot_of = [](K k) { return (uint32_t(k ^ (uint64_t(k) >> 32)) * 0x9E3779B1u) >> 17; };
-#pragma unroll
-  for (int i = 0; i < L::PER; ++i) s_slot[slot_of(key[i])] = uint16_t(i * kSampleThreads + tid);
-  __syncthreads();
-  uint32_t dups = 0;
-#pragma unroll
-  for (int i = 0; i < L::PER; ++i) {
-    const uint32_t o = s_slot[slot_of(key[i])];
-    dups += o != uint32_t(i * kSampleThreads + tid) && s_keys[o] == key[i];
-  }
-  dups = __reduce_add_sync(0xffffffffu, dups);
-  uint32_t* s_sum = reinterpret_cast<uint32_t*>(s_red);
-  if (lane == 0) s_sum[warp] = dups;
-  bad = __syncthreads_or(bad);
-  dups = __reduce_add_sync(0xffffffffu, s_sum[lane]);
-  // equal keys per value of about c among n keys give S^2 c / (2 n) such
-  // pairs in the sample; c = 16 is what the bins still take well
-  if (uint64_t(dups) * n > uint64_t(L::S) * L::S * 8 + 16 * n) bad = true;
-  if (tid == 0) {
-    HybCtrl* c = a.ctrl;
-    c->lo = m.lo;
-    c->hi = m.hi;
-    c->sh = m.sh;
-    c->mult = m.mult;
-    c->done = 0;
-    c->tiles_b = 0;
-    c->route = bad ? kHybRadix : kHybBuckets;
-  }
+  });
 }
-
 // ------------------------------------------------------------------ counts
 // Keys per bucket.  32-bit shared counters for every bucket (up to 128 KiB),
 // one shared reduction per key; the blocks add them into the global counts.
@@ -411,16 +259,17 @@ __global__ void __launch_bounds__(kBucketThreads, MINB) bucket_sort_kernel(const
   if (a.ctrl->route != kHybBuckets) return;
   const ValueMap<K> m = load_map<K>(a.ctrl);
   using V = typename ValueOf<VB>::T;
+  constexpr Vals MODE = VB ? Vals::kStaged : Vals::kAlone;
   const uint32_t b = blockIdx.x, s = a.starts[b], e = a.starts[b + 1];
   if (s == e) return;
   K* io = reinterpret_cast<K*>(a.keys_out) + s;
   V* vio = VB ? reinterpret_cast<V*>(a.vals_out) + s : nullptr;
   if (b == 0 || b == a.buckets - 1)
-    local_sort_array<kBucketThreads, kBucketItems, kBucketBits, VB, true>(
-        io, io, vio, vio, e - s, OrdOf<K>::identity(), OrdOf<K>::make(a), BucketBins<K, kBucketBits, true>{m}, smem);
+    local_sort_array<kBucketThreads, kBucketItems, kBucketBits, VB, MODE, true>(
+        io, io, vio, vio, vio, e - s, OrdOf<K>::identity(), OrdOf<K>::make(a), BucketBins<K, kBucketBits, true>{m}, smem);
   else
-    local_sort_array<kBucketThreads, kBucketItems, kBucketBits, VB, true>(
-        io, io, vio, vio, e - s, OrdOf<K>::identity(), OrdOf<K>::make(a), BucketBins<K, kBucketBits, false>{m}, smem);
+    local_sort_array<kBucketThreads, kBucketItems, kBucketBits, VB, MODE, true>(
+        io, io, vio, vio, vio, e - s, OrdOf<K>::identity(), OrdOf<K>::make(a), BucketBins<K, kBucketBits, false>{m}, smem);
 }
 
 // ------------------------------------------------- first radix pass of keys
@@ -449,14 +298,14 @@ template <typename K>
 struct Kernels {
   static constexpr int ST = kSplitThreads, SI = sizeof(K) == 4 ? kSplitItems : kSplitItems / 2, SB = kSplitBlocks;
   using Split = SplitLayout<K, ST, SI>;
-  using Local = LocalLayout<kBucketThreads, kBucketItems, kBucketBits, K, 0, false>;
+  using Local = LocalLayout<kBucketThreads, kBucketItems, kBucketBits, K, 0, Vals::kAlone>;
   static constexpr int LB = sizeof(K) == 4 ? 8 : 4;
   static cudaError_t prepare() {
     cudaError_t e = cudaSuccess;
     auto set = [&](const void* f, size_t bytes) {
       if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
     };
-    set(reinterpret_cast<const void*>(&sample_kernel<K>), SampleLayout<K>::SMEM);
+    set(reinterpret_cast<const void*>(&sample_kernel<K>), SampleLayout<K, kSampleBlocks, kSampleThreads>::SMEM);
     set(reinterpret_cast<const void*>(&bucket_count_kernel<K>), size_t(kHybMaxBuckets) * 4);
     set(reinterpret_cast<const void*>(&split_kernel<K, ST, SI, SB, 0>), Split::SMEM);
     set(reinterpret_cast<const void*>(&split_kernel<K, ST, SI, SB, 1>), Split::SMEM);
@@ -493,7 +342,7 @@ static cudaError_t launch(const HybArgs& a, HybStep step, unsigned sms, cudaStre
   const unsigned tiles = (a.n + a.split_tile - 1) / a.split_tile;
   switch (step) {
     case HybStep::kSample:
-      sample_kernel<K><<<kSampleBlocks, kSampleThreads, SampleLayout<K>::SMEM, s>>>(a);
+      sample_kernel<K><<<kSampleBlocks, kSampleThreads, SampleLayout<K, kSampleBlocks, kSampleThreads>::SMEM, s>>>(a);
       return cudaGetLastError();
     case HybStep::kCount:
       return launch_chained(&bucket_count_kernel<K>, sms, kCountThreads, size_t(a.buckets) * 4, s, true, a);

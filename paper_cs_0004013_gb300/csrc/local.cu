@@ -36,10 +36,10 @@ __global__ void __launch_bounds__(THREADS, MINB) local_sort_kernel(const LocalAr
     start = a.seg_off[s];
     m = uint32_t(a.seg_off[s + 1] - start);
   }
-  local_sort_array<THREADS, ITEMS, NBITS, VB, false>(
+  local_sort_array<THREADS, ITEMS, NBITS, VB, VB ? Vals::kFollow : Vals::kAlone, false>(
       static_cast<const K*>(a.kin) + start, static_cast<K*>(a.kout) + start,
-      VB ? static_cast<const V*>(a.vin) + start : nullptr, VB ? static_cast<V*>(a.vout) + start : nullptr, m,
-      OrdFor<K>::in(a), OrdFor<K>::out(a), RangeBins<K>{}, smem);
+      VB ? static_cast<const V*>(a.vin) + start : nullptr, VB ? static_cast<V*>(a.vout) + start : nullptr,
+      static_cast<const V*>(nullptr), m, OrdFor<K>::in(a), OrdFor<K>::out(a), RangeBins<K>{}, smem);
 }
 
 struct Shape {
@@ -51,7 +51,7 @@ struct Shape {
 };
 template <int THREADS, int ITEMS, int NBITS, int MINB, typename K, int VB>
 Shape shape() {
-  using L = LocalLayout<THREADS, ITEMS, NBITS, K, VB, false>;
+  using L = LocalLayout<THREADS, ITEMS, NBITS, K, VB, VB ? Vals::kFollow : Vals::kAlone>;
   return Shape{uint32_t(L::CAP), unsigned(THREADS), L::SMEM,
                reinterpret_cast<const void*>(&local_sort_kernel<THREADS, ITEMS, NBITS, MINB, K, VB>),
                [](const LocalArgs& a, unsigned grid, cudaStream_t s) {

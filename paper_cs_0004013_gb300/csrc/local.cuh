@@ -23,10 +23,15 @@
 //     spans at most ceil((c + 3) / 4) such runs, is in order after that many
 //     rounds (two for c <= 5);
 //  6. out, coalesced.
+// Where (unless the caller's map is known to be even) a bin holds more than kBinLimit keys, the bins are laid again where
+// the keys are: each bin's share of a second set of bins is its share of the
+// keys (its start and count give them), and a key takes the part of that
+// share that its place inside the bin points to.  This flattens any density
+// that does not change much within a bin (normally distributed floats, wide
+// clusters).  Blocks that are crowded still sort by digits.
 // Sorts with payloads are stable: they order (key, place in the input), and
-// the payload follows its place.  Where a bin holds more than kBinLimit keys,
-// the block sorts by stable 8-bit digit passes (the digits in which the keys
-// differ) with the lane-mask tables of the tiled pass.
+// the payload follows its place.  The digit passes are stable 8-bit ones over
+// the digits in which the keys differ, with the lane-mask tables of the tiled pass.
 //
 // The work is about 55 instructions and 18 shared-memory wavefronts per 32
 // keys whatever the key width, against about 40 wavefronts per 8-bit digit
@@ -158,12 +163,21 @@ __device__ __forceinline__ void merge8(E (&v)[8]) {
   order2(v[1], v[2]); order2(v[3], v[4]); order2(v[5], v[6]);
 }
 
-// STAGED: payloads are held in shared memory in input order (a sort in place
-// overwrites them); otherwise they are read from the input when they leave.
-template <int THREADS, int ITEMS, int NBITS, typename K, int VB, bool STAGED>
+// How payloads follow their keys:
+//   kAlone    there are none;
+//   kFollow   each is read from the input, at its key's place there, when it leaves;
+//   kStaged   held in shared memory in input order meanwhile (sorts in place);
+//   kPlaces   the input's second array holds places instead of payloads: equal
+//             keys are ordered by them, and payloads are read from a third
+//             array at the place.
+enum class Vals { kAlone, kFollow, kStaged, kPlaces };
+
+template <int THREADS, int ITEMS, int NBITS, typename K, int VB, Vals MODE>
 struct LocalLayout {
+  static_assert((VB != 0) == (MODE != Vals::kAlone), "payloads and what happens to them");
   using V = typename ValueOf<VB>::T;
   using E = typename ElemOf<K, VB != 0>::E;
+  static constexpr bool STAGED = MODE == Vals::kStaged;
   static constexpr int WARPS = THREADS / 32;
   static constexpr int CAP = THREADS * ITEMS;
   static constexpr int NB = 1 << NBITS;
@@ -213,6 +227,13 @@ struct RangeBins {
   K lo;
   int sh;
   __device__ __forceinline__ uint32_t operator()(K k) const { return uint32_t((k - lo) >> sh); }
+  // how far into its bin, in units of 2^-32
+  __device__ __forceinline__ uint32_t frac(K k) const {
+    constexpr int W = int(sizeof(K)) * 8;
+    if (sh == 0) return 0u;
+    const K r = (k - lo) << (W - sh);
+    return uint32_t(r >> (W - 32));
+  }
   __device__ __forceinline__ bool unique() const { return sh == 0; }  // a bin holds one value
 };
 
@@ -267,7 +288,9 @@ __device__ __forceinline__ void block_exclusive_sums(const uint32_t (&x)[R], uin
 // The digit passes over [0, m) of s_key (see above): afterwards s_key is in
 // order.  Warp w ranks elements [w * 32 * ITEMS, ...), so that rank order is
 // the order they were in.
-template <class L, int THREADS, int ITEMS, typename K, bool PAIRS>
+// BY_PLACE: equal keys are ordered by their places too (they are not in that
+// order to begin with).
+template <class L, int THREADS, int ITEMS, typename K, bool PAIRS, bool BY_PLACE>
 __device__ __noinline__ void local_digit_passes(uint32_t m, unsigned char* smem) {
   using EO = ElemOf<K, PAIRS>;
   using E = typename EO::E;
@@ -283,11 +306,16 @@ __device__ __noinline__ void local_digit_passes(uint32_t m, unsigned char* smem)
   const uint32_t wofs = uint32_t(warp) * 32 * ITEMS + lane;
   E e[ITEMS];
   K diff = 0;
+  uint32_t pdiff = 0;
   const K k0 = EO::key(s_key[L::slot(0)]);
+  const uint32_t p0 = EO::place(s_key[L::slot(0)]);
 #pragma unroll
   for (int j = 0; j < ITEMS; ++j) {  // places past the end act as the largest key and stay behind
     e[j] = wofs + j * 32 < m ? s_key[L::slot(wofs + j * 32)] : EO::last();
-    if (wofs + j * 32 < m) diff |= EO::key(e[j]) ^ k0;
+    if (wofs + j * 32 < m) {
+      diff |= EO::key(e[j]) ^ k0;
+      pdiff |= EO::place(e[j]) ^ p0;
+    }
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) diff |= __shfl_xor_sync(0xffffffffu, diff, o);
@@ -296,15 +324,26 @@ __device__ __noinline__ void local_digit_passes(uint32_t m, unsigned char* smem)
   diff = s_red[lane < WARPS ? lane : 0];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) diff |= __shfl_xor_sync(0xffffffffu, diff, o);
-  for (uint32_t shift = 0; shift < sizeof(K) * 8; shift += 8) {
-    if (((diff >> shift) & 0xffu) == 0) continue;  // uniform
+  if constexpr (BY_PLACE) {
+    pdiff = __reduce_or_sync(0xffffffffu, pdiff);
+    __syncthreads();
+    if (lane == 0) s_warp[warp] = pdiff;
+    __syncthreads();
+    pdiff = __reduce_or_sync(0xffffffffu, s_warp[lane < WARPS ? lane : 0]);
+  }
+  // digits 0-3 are the places' (BY_PLACE), the others the keys'
+  auto digit = [&](const E& x, uint32_t d) {
+    return d < 4 ? (EO::place(x) >> (8 * d)) & 0xffu : uint32_t(EO::key(x) >> (8 * (d - 4))) & 0xffu;
+  };
+  for (uint32_t d = BY_PLACE ? 0 : 4; d < 4 + sizeof(K); ++d) {
+    if (((d < 4 ? pdiff >> (8 * d) : uint32_t(diff >> (8 * (d - 4)))) & 0xffu) == 0) continue;  // uniform
     __syncthreads();
     for (int i = tid; i < int(L::RANK_BYTES / 16); i += THREADS) b4[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
     uint32_t rk[(ITEMS + 1) / 2];
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) {
-      const uint32_t r = warp_rank_step(uint32_t(EO::key(e[j]) >> shift) & 0xffu, s_mask + warp * kMaskSlots,
+      const uint32_t r = warp_rank_step(digit(e[j], d), s_mask + warp * kMaskSlots,
                                         s_cnt + warp * 256, lt, gt, lane);
       if (j & 1) rk[j >> 1] |= r << 16;
       else rk[j >> 1] = r;
@@ -314,21 +353,21 @@ __device__ __noinline__ void local_digit_passes(uint32_t m, unsigned char* smem)
     constexpr int DPT = 256 / DT;                      // consecutive digits of such a thread
     uint32_t sum = 0;
     if (tid < DT)
-      for (int d = tid * DPT; d < (tid + 1) * DPT; ++d)
-        for (int wi = 0; wi < WARPS; ++wi) sum += s_cnt[wi * 256 + d];
+      for (int q = tid * DPT; q < (tid + 1) * DPT; ++q)
+        for (int wi = 0; wi < WARPS; ++wi) sum += s_cnt[wi * 256 + q];
     uint32_t run = block_exclusive_sum<THREADS>(sum, s_warp);
     if (tid < DT)
-      for (int d = tid * DPT; d < (tid + 1) * DPT; ++d)
+      for (int q = tid * DPT; q < (tid + 1) * DPT; ++q)
         for (int wi = 0; wi < WARPS; ++wi) {
-          const uint32_t v = s_cnt[wi * 256 + d];
-          s_cnt[wi * 256 + d] = uint16_t(run);
+          const uint32_t v = s_cnt[wi * 256 + q];
+          s_cnt[wi * 256 + q] = uint16_t(run);
           run += v;
         }
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j)
       s_key[L::slot(((rk[j >> 1] >> (16 * (j & 1))) & 0xffffu) +
-                    s_cnt[warp * 256 + (uint32_t(EO::key(e[j]) >> shift) & 0xffu)])] = e[j];
+                    s_cnt[warp * 256 + digit(e[j], d)])] = e[j];
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) e[j] = s_key[L::slot(wofs + j * 32)];
@@ -336,18 +375,21 @@ __device__ __noinline__ void local_digit_passes(uint32_t m, unsigned char* smem)
   __syncthreads();
 }
 
-// The sort of [0, m) of (in, vin) into (out, vout), 1 <= m <= THREADS * ITEMS
-// (INPLACE: in == out and vin == vout).  ordi maps a key on loading, ordo back
-// on storing.  bins: RangeBins (filled here) or a map known beforehand.  The
-// block is synchronised on return.
-template <int THREADS, int ITEMS, int NBITS, int VB, bool INPLACE, class OrdI, class OrdO, class Bins>
-__device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, typename OrdI::Key* out,
-                                                 const typename ValueOf<VB>::T* vin, typename ValueOf<VB>::T* vout,
-                                                 const uint32_t m, const OrdI ordi, const OrdO ordo, Bins bins,
-                                                 unsigned char* smem) {
+// The sort of [0, m) of (in, vin) into (out, vout), 1 <= m <= THREADS * ITEMS;
+// vin holds payloads or (kPlaces) places, and then `from` the payloads.
+// kStaged may sort in place.  COHERENT: the inputs were written by other
+// blocks of the same launch, or are overwritten by this one.  ordi maps a key
+// on loading, ordo back on storing.  bins: RangeBins (filled here) or a map
+// known beforehand.  The block is synchronised on return.
+template <int THREADS, int ITEMS, int NBITS, int VB, Vals MODE, bool COHERENT, class OrdI, class OrdO, class Bins,
+          class VIn>
+__device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, typename OrdI::Key* out, const VIn* vin,
+                                                 typename ValueOf<VB>::T* vout,
+                                                 const typename ValueOf<VB>::T* from, const uint32_t m,
+                                                 const OrdI ordi, const OrdO ordo, Bins bins, unsigned char* smem) {
   using K = typename OrdI::Key;
-  constexpr bool STAGED = VB != 0 && INPLACE;
-  using L = LocalLayout<THREADS, ITEMS, NBITS, K, VB, STAGED>;
+  constexpr bool STAGED = MODE == Vals::kStaged, PLACES = MODE == Vals::kPlaces;
+  using L = LocalLayout<THREADS, ITEMS, NBITS, K, VB, MODE>;
   using V = typename L::V;
   using EO = ElemOf<K, VB != 0>;
   using E = typename EO::E;
@@ -376,7 +418,10 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
 
   // 1. load; clear the bins
   K key[ITEMS];
-  for_items([&](int j) { key[j] = has(j) ? ld_elem<INPLACE>(in + j * THREADS + tid) : K(0); });
+  for_items([&](int j) { key[j] = has(j) ? ld_elem<COHERENT>(in + j * THREADS + tid) : K(0); });
+  uint32_t place[PLACES ? ITEMS : 1];
+  if constexpr (PLACES) for_items([&](int j) { place[j] = has(j) ? ld_elem<COHERENT>(vin + j * THREADS + tid) : 0u; });
+  auto elem = [&](int j) { return EO::make(key[j], PLACES ? place[PLACES ? j : 0] : uint32_t(j * THREADS + tid)); };
   uint4* b4 = reinterpret_cast<uint4*>(smem);
 #pragma unroll
   for (int i = 0; i < NB / 8; i += THREADS)
@@ -384,7 +429,7 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
   if (tid == 0) *s_most = 0u;
   if constexpr (STAGED) {
     for_items([&](int j) {
-      if (has(j)) s_val[j * THREADS + tid] = ld_elem<INPLACE>(vin + j * THREADS + tid);
+      if (has(j)) s_val[j * THREADS + tid] = ld_elem<COHERENT>(vin + j * THREADS + tid);
     });
   }
   if (!ordi.identity()) for_items([&](int j) { key[j] = ordi.map(key[j]); });
@@ -415,45 +460,45 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
 
   // 2. turns within the bins.  Word w of the counts holds bin w in its low and
   // bin w + NB / 2 in its high half; four 8-bit turns go to a register (a
-  // turn above kBinLimit sends the block to the digit passes, so its low bits
-  // may be lost).
+  // turn above kBinLimit sends the block another way, so its low bits may be
+  // lost).  Returns the fullest bin's keys, five at least.
   const uint32_t bin_base = static_cast<uint32_t>(__cvta_generic_to_shared(s_bin));
   uint32_t turn[(ITEMS + 3) / 4];
-  uint32_t most = 0;
-  for_items([&](int j) {
-    const uint32_t b = bins(key[j]);
-    const uint32_t half = (b >> (NBITS - 1)) & 1u;
-    uint32_t r = 0;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %3, %4;\n\t@p atom.shared.add.u32 %0, [%1], %2;\n\t}"
-        : "+r"(r)
-        : "r"(bin_base + 4u * (b & uint32_t(NB / 2 - 1))), "r"(half * 0xffffu + 1u), "r"(uint32_t(j * THREADS + tid)),
-          "r"(m)
-        : "memory");
-    r = (r >> (half * 16u)) & 0xffffu;
-    most = r > most ? r : most;
-    if (j % 4 == 0) turn[j / 4] = r;
-    else turn[j / 4] = __byte_perm(turn[j / 4], r, j % 4 == 1 ? 0x3240 : j % 4 == 2 ? 0x3410 : 0x4210);
-  });
-  if (__any_sync(0xffffffffu, most >= 5u)) {  // rare
-    most = __reduce_max_sync(0xffffffffu, most);
-    if (lane == 0) atomicMax(s_most, most);
-  }
-  __syncthreads();
-  // keys of the fullest bin (five at least); bins of one value need no order
-  // among equal keys (as long as their turns fit their 8 bits)
-  most = *s_most ? *s_most + 1u : 5u;
-  if (VB == 0 && bins.unique() && most <= 256u) most = 1u;
-  if (most <= kBinLimit) {
-    // 3. counts -> starts, both halves of the words at once (sums of at most
-    // CAP < 2^16 each): the low halves' total comes before the high halves'
-    // starts.  The words are scanned in ranges of 4 per scanning thread, one
-    // 16-byte vector per thread and range (no bank conflicts).
+  auto count = [&](auto&& bin_of) -> uint32_t {
+    uint32_t most = 0;
+    for_items([&](int j) {
+      const uint32_t b = bin_of(j);
+      const uint32_t half = (b >> (NBITS - 1)) & 1u;
+      uint32_t r = 0;
+      asm volatile(
+          "{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %3, %4;\n\t@p atom.shared.add.u32 %0, [%1], %2;\n\t}"
+          : "+r"(r)
+          : "r"(bin_base + 4u * (b & uint32_t(NB / 2 - 1))), "r"(half * 0xffffu + 1u), "r"(uint32_t(j * THREADS + tid)),
+            "r"(m)
+          : "memory");
+      r = (r >> (half * 16u)) & 0xffffu;
+      most = r > most ? r : most;
+      if (j % 4 == 0) turn[j / 4] = r;
+      else turn[j / 4] = __byte_perm(turn[j / 4], r, j % 4 == 1 ? 0x3240 : j % 4 == 2 ? 0x3410 : 0x4210);
+    });
+    if (__any_sync(0xffffffffu, most >= 5u)) {  // rare
+      most = __reduce_max_sync(0xffffffffu, most);
+      if (lane == 0) atomicMax(s_most, most);
+    }
+    __syncthreads();
+    return *s_most ? *s_most + 1u : 5u;
+  };
+  // 3. counts -> starts, both halves of the words at once (sums of at most CAP
+  // < 2^16 each): the low halves' total comes before the high halves' starts.
+  // The words are scanned in ranges of 4 per scanning thread, one 16-byte
+  // vector per thread and range (no bank conflicts).
+  auto scan = [&]() {
     constexpr int WORDS = NB / 2;
-    constexpr int ST = WORDS / 4 < THREADS ? WORDS / 4 : THREADS;  // scanning threads
+    constexpr int POW2 = THREADS >= 1024 ? 1024 : THREADS >= 512 ? 512 : THREADS >= 256 ? 256 : 128;
+    constexpr int ST = WORDS / 4 < POW2 ? WORDS / 4 : POW2;        // scanning threads
     constexpr int R = WORDS / (4 * ST);                            // ranges
     static_assert(R * 4 * ST == WORDS, "whole ranges");
-    static_assert(R <= 4, "a word of s_warp per warp and range");
+    static_assert(R <= 4, "a word of s_scan per warp and range");
     uint4 w[R];
     uint32_t sum[R], run[R];
 #pragma unroll
@@ -479,21 +524,58 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
       if (tid < ST) b4[r * ST + tid] = w[r];
     }
     __syncthreads();
-    // 4. keys into the bins' places; the windows past the end read the last element
+  };
+  auto start_of = [&](uint32_t b) -> uint32_t {  // (the bin of a lane without a key is any number: masked)
+    return s_start[2u * (b & uint32_t(NB / 2 - 1)) + ((b >> (NBITS - 1)) & 1u)];
+  };
+  // 4. keys into the bins' places (a lane without a key stores to a spare
+  // slot); the windows past the end read the last element
+  auto stage = [&](auto&& bin_of) {
     for_items([&](int j) {
-      const uint32_t b = bins(key[j]);
-      // (the bin of a lane without a key is any number: both parts are masked)
-      const uint32_t p = s_start[2u * (b & uint32_t(NB / 2 - 1)) + ((b >> (NBITS - 1)) & 1u)] +
-                         __byte_perm(turn[j / 4], 0u, 0x4440u + uint32_t(j % 4));
-      // (a lane without a key stores to a spare slot)
-      s_key[L::slot(has(j) ? p : uint32_t(L::SPARE + lane))] = EO::make(key[j], j * THREADS + tid);
+      const uint32_t p = start_of(bin_of(j)) + __byte_perm(turn[j / 4], 0u, 0x4440u + uint32_t(j % 4));
+      s_key[L::slot(has(j) ? p : uint32_t(L::SPARE + lane))] = elem(j);
     });
     if (tid < 16) s_key[L::slot(m + tid)] = EO::last();
     __syncthreads();
+  };
+  auto first_bin = [&](int j) { return bins(key[j]); };
+  uint32_t most = count(first_bin);
+  // bins of one value need no order among equal keys (as long as their turns fit their 8 bits)
+  if (VB == 0 && bins.unique() && most <= 256u) most = 1u;
+  bool staged = most <= kBinLimit;
+  if (staged) {
+    scan();
+    stage(first_bin);
+  } else if constexpr (!Bins::kKnown) {
+    if (!bins.unique()) {
+      // crowded: the second set of bins (see above), NB / m of them to a key;
+      // positions among the keys in 16.16 fixed point
+      scan();
+      const uint32_t per = (uint32_t(NB) << 16) / m;
+      uint32_t bin2[ITEMS];
+      for_items([&](int j) {
+        const uint32_t b = first_bin(j) & uint32_t(NB - 1);
+        const uint32_t s = start_of(b), e = b == uint32_t(NB - 1) ? m : start_of(b + 1);
+        bin2[j] = __umulhi((s << 16) + __umulhi(bins.frac(key[j]), (e - s) << 16), per);
+      });
+      __syncthreads();
+      for (int i = tid; i < NB / 8; i += THREADS) b4[i] = make_uint4(0u, 0u, 0u, 0u);
+      if (tid == 0) *s_most = 0u;
+      __syncthreads();
+      auto second_bin = [&](int j) { return bin2[j]; };
+      most = count(second_bin);
+      staged = most <= kBinLimit;
+      if (staged) {
+        scan();
+        stage(second_bin);
+      }
+    }
+  }
+  if (staged) {
     // 5. windows: those that start before the end
     constexpr int NWIN = (ITEMS + 7) / 8;  // windows per thread
     // (what the block's register budget holds; else a round at a time)
-    constexpr bool HELD = NWIN * sizeof(E) <= (THREADS >= 1024 ? 8 : THREADS >= 256 ? 12 : 24);
+    constexpr bool HELD = NWIN * sizeof(E) <= (THREADS >= 384 ? 8 : THREADS >= 256 ? 12 : 24);
     if (HELD && most == 5u) {
       // Two rounds, each thread keeping its windows in registers: between
       // them it takes the next window's lower half, from the next lane or,
@@ -555,10 +637,10 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
     }
   } else {
     for_items([&](int j) {
-      if (has(j)) s_key[L::slot(j * THREADS + tid)] = EO::make(key[j], j * THREADS + tid);
+      if (has(j)) s_key[L::slot(j * THREADS + tid)] = elem(j);
     });
     __syncthreads();
-    local_digit_passes<L, THREADS, ITEMS, K, VB != 0>(m, smem);
+    local_digit_passes<L, THREADS, ITEMS, K, VB != 0, PLACES>(m, smem);
   }
   // 6. out
   auto write_out = [&](auto invert) {
@@ -569,6 +651,7 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
         if constexpr (decltype(invert)::value) ordo.store(out + p, EO::key(e));
         else out[p] = EO::key(e);
         if constexpr (STAGED) vout[p] = s_val[EO::place(e)];
+        else if constexpr (PLACES) vout[p] = ld_elem(from + EO::place(e));
         else if constexpr (VB != 0) vout[p] = vin[EO::place(e)];
       }
     });

@@ -152,8 +152,10 @@ __device__ __forceinline__ uint32_t ld_pass(const uint32_t* p) {
 
 // Steps 1-6 for one tile.  The rank words must be zero and the block
 // synchronised on entry; the block is synchronised on return.
-// UNSTABLE (keys only): the first executed pass, see step 2u.
-template <int THREADS, int ITEMS, int NV, typename S, bool EARLY_LB, int LB, bool COHERENT, bool UNSTABLE = false>
+// EARLY_VALS: the payloads are loaded right after the keys and held in
+// registers (for one block per SM, whose registers are free and whose loads
+// nothing else hides).
+template <int THREADS, int ITEMS, int NV, typename S, bool EARLY_LB, int LB, bool COHERENT, bool EARLY_VALS = false>
 __device__ __forceinline__ void onesweep2_tile(const Tile2Job& job, unsigned char* smem) {
   using L = Onesweep2Layout<THREADS, ITEMS, NV>;
   constexpr int DIGITS = L::DIGITS, GROUPS = L::GROUPS, TILE = L::TILE;
@@ -174,17 +176,14 @@ __device__ __forceinline__ void onesweep2_tile(const Tile2Job& job, unsigned cha
   S* status = reinterpret_cast<S*>(job.status);
   const size_t tbase = size_t(tile) * TILE;
   const size_t left = size_t(job.n) - tbase;
-  // UNSTABLE runs on full tiles only: keys past the end would take places
-  // among the tile's real keys of digit 255 (the atomic ranking keeps no
-  // order), so the caller gives a partial tile to the stable body
-  const uint32_t valid = (NV == 0 && UNSTABLE) || left >= size_t(TILE) ? uint32_t(TILE) : uint32_t(left);
+  const uint32_t valid = left >= size_t(TILE) ? uint32_t(TILE) : uint32_t(left);
   const uint32_t sel = 0x4440u | (job.shift >> 3);
   (void)vin;
   (void)vout;
   (void)s_val;
 
   // 1p. the payload words of a full tile, prefetched into L2 for step 5
-  if constexpr (NV >= 1) {
+  if constexpr (NV >= 1 && !EARLY_VALS) {
     if (valid == TILE && (reinterpret_cast<uintptr_t>(vin + tbase) & 15u) == 0)
       prefetch_l2_tile(vin + tbase, uint32_t(TILE) * 4u);
   }
@@ -211,17 +210,23 @@ __device__ __forceinline__ void onesweep2_tile(const Tile2Job& job, unsigned cha
     }
   }
 
-  // Keys only, first executed pass of a full tile (UNSTABLE): the order of
-  // keys with the same lowest digit is free (there is no earlier order to
-  // keep, and keys with equal digits here are told apart by the later passes
-  // or are equal), so one shared counter per (half of a warp, digit)
-  // suffices and a key's position is one atomic add on it (steps 2u and 4u
-  // below) instead of the groups' mask words.  Two rows, one per half, keep
-  // the halves' accesses to one digit in different banks.
-  constexpr bool unstable = NV == 0 && UNSTABLE;
+  uint32_t val[NV >= 1 ? ITEMS : 1];
+  auto load_vals = [&]() {
+    if (valid == TILE) {
+#pragma unroll
+      for (int j = 0; j < ITEMS; ++j) val[j] = ld_pass<COHERENT>(vin + tbase + goff_in + j * 16);
+    } else {
+#pragma unroll
+      for (int j = 0; j < ITEMS; ++j) {
+        const uint32_t i = goff_in + j * 16;
+        val[j] = i < valid ? ld_pass<COHERENT>(vin + tbase + i) : 0u;
+      }
+    }
+  };
+  if constexpr (NV >= 1 && EARLY_VALS) load_vals();
 
-  // 2. early counts per (group, digit) [2u: per (half, digit)]
-  const uint32_t tb_grp = smem_addr(s_tbl + (unstable ? (lane >> 4) : grp) * L::ROW);
+  // 2. early counts per (group, digit)
+  const uint32_t tb_grp = smem_addr(s_tbl + grp * L::ROW);
 #pragma unroll
   for (int j = 0; j < ITEMS; ++j) sh_red_add(tb_grp + 4u * byte_digit(key[j], sel), 1u);
   __syncthreads();
@@ -229,30 +234,19 @@ __device__ __forceinline__ void onesweep2_tile(const Tile2Job& job, unsigned cha
   // 3. per digit (threads 0..255): the tile's count -> aggregate status now;
   // exclusive scan over digits -> where each digit's run starts in the
   // staged tile; then each group's counter -> the position of its first key
-  // of the digit [3u: the two halves' counters -> where each half's keys of
-  // the digit start]
+  // of the digit
   uint32_t tot = 0, excl = 0;
   if (tid < DIGITS) {
-    if constexpr (unstable) {
-      tot = s_tbl[tid] + s_tbl[L::ROW + tid];
-    } else {
 #pragma unroll 8
-      for (int g = 0; g < GROUPS; ++g) tot += s_tbl[g * L::ROW + tid];
-    }
+    for (int g = 0; g < GROUPS; ++g) tot += s_tbl[g * L::ROW + tid];
     st_relaxed(status + size_t(tile) * DIGITS + tid, status_word<S>(parity, tile == 0, tot));
     excl = scan256_exclusive(tot, s_scan);
-    if constexpr (unstable) {
-      const uint32_t c0 = s_tbl[tid];
-      s_tbl[tid] = excl;
-      s_tbl[L::ROW + tid] = excl + c0;
-    } else {
-      uint32_t run = excl;
+    uint32_t run = excl;
 #pragma unroll 8
-      for (int g = 0; g < GROUPS; ++g) {
-        const uint32_t c = s_tbl[g * L::ROW + tid];
-        s_tbl[g * L::ROW + tid] = run;
-        run += c;
-      }
+    for (int g = 0; g < GROUPS; ++g) {
+      const uint32_t c = s_tbl[g * L::ROW + tid];
+      s_tbl[g * L::ROW + tid] = run;
+      run += c;
     }
   }
   __syncthreads();
@@ -276,30 +270,20 @@ __device__ __forceinline__ void onesweep2_tile(const Tile2Job& job, unsigned cha
   const uint32_t mybit = 1u << (16 + l16);
   const uint32_t sk = smem_addr(s_key);
   uint32_t pos[NV >= 1 ? (ITEMS + 1) / 2 : 1];
-  if constexpr (unstable) {
-    // 4u. one atomic add per key on its digit's counter gives its place
 #pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-      uint32_t p;
-      asm volatile("atom.shared.add.u32 %0, [%1], 1;" : "=r"(p) : "r"(tb_grp + 4u * byte_digit(key[j], sel)) : "memory");
-      sh_st(sk + 4u * p, key[j]);
-    }
-  } else {
-#pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-      const uint32_t ad = tb_grp + 4u * byte_digit(key[j], sel);
-      sh_red_or(ad, mybit);
-      __syncwarp();
-      const uint32_t v = sh_ld(ad);
-      const uint32_t peers = v >> 16, base = v & 0xffffu;
-      const uint32_t p = base + __popc(peers & lt16);
-      if ((peers >> l16) == 1u) sh_st(ad, base + __popc(peers));  // the group's highest lane with this digit
-      __syncwarp();
-      sh_st(sk + 4u * p, key[j]);
-      if constexpr (NV >= 1) {
-        if (j & 1) pos[j >> 1] |= p << 16;
-        else pos[j >> 1] = p;
-      }
+  for (int j = 0; j < ITEMS; ++j) {
+    const uint32_t ad = tb_grp + 4u * byte_digit(key[j], sel);
+    sh_red_or(ad, mybit);
+    __syncwarp();
+    const uint32_t v = sh_ld(ad);
+    const uint32_t peers = v >> 16, base = v & 0xffffu;
+    const uint32_t p = base + __popc(peers & lt16);
+    if ((peers >> l16) == 1u) sh_st(ad, base + __popc(peers));  // the group's highest lane with this digit
+    __syncwarp();
+    sh_st(sk + 4u * p, key[j]);
+    if constexpr (NV >= 1) {
+      if (j & 1) pos[j >> 1] |= p << 16;
+      else pos[j >> 1] = p;
     }
   }
   if constexpr (!EARLY_LB) do_lookback();
@@ -307,17 +291,7 @@ __device__ __forceinline__ void onesweep2_tile(const Tile2Job& job, unsigned cha
 
   // 5. payloads: staged at their keys' positions (over the dead rank words)
   if constexpr (NV >= 1) {
-    uint32_t val[ITEMS];
-    if (valid == TILE) {
-#pragma unroll
-      for (int j = 0; j < ITEMS; ++j) val[j] = ld_pass<COHERENT>(vin + tbase + goff_in + j * 16);
-    } else {
-#pragma unroll
-      for (int j = 0; j < ITEMS; ++j) {
-        const uint32_t i = goff_in + j * 16;
-        val[j] = i < valid ? ld_pass<COHERENT>(vin + tbase + i) : 0u;
-      }
-    }
+    if constexpr (!EARLY_VALS) load_vals();
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) s_val[(pos[j >> 1] >> (16 * (j & 1))) & 0xffffu] = val[j];
     __syncthreads();
@@ -398,7 +372,7 @@ __global__ void __launch_bounds__(THREADS, MINB) onesweep2_kernel(const PassArgs
   }
   __syncthreads();
   job.tile = *s_tile;
-  onesweep2_tile<THREADS, ITEMS, NV, S, EARLY_LB, LB, false, false>(job, smem);
+  onesweep2_tile<THREADS, ITEMS, NV, S, EARLY_LB, LB, false>(job, smem);
 }
 
 template <int THREADS, int ITEMS, int NV, typename S, int MINB, bool EARLY_LB, int LB>

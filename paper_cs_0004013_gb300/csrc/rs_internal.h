@@ -26,6 +26,8 @@ struct KeyXform {
 };
 constexpr KeyXform kIdentityXform = {0u, 0u};
 
+struct HybCtrl;  // hybrid.h
+
 // The same map for 64-bit keys held as (low word, high word): the sign is
 // the high word's top bit; a set sign flips the low word by flo and the high
 // word by fhi, and shi is flipped in the high word of every key.
@@ -326,10 +328,18 @@ struct FusedArgs {
   uint32_t n;
   KeyXform xf;               // order map of the keys' kind
   uint32_t* hist;            // [4][256], zero on entry
-  void* status;              // [tiles][256] 32-bit status words, zero on entry
+  void* status;              // [tiles][256] 32-bit status words
+  uint32_t* first_cursors;   // [256], zero on entry
   uint32_t* bar;             // barrier counter, zero on entry
   uint32_t* err;             // device error word
+  uint32_t tiles;            // set by the launch
+  // value buckets, when offered (null: not): the sample's control block
+  HybCtrl* ctrl;
+  uint32_t buckets;
+  uint32_t* counts;          // [buckets], zero on entry
+  uint32_t* cursors;         // [buckets], zero on entry
 };
+constexpr uint32_t kFusedMaxBuckets = 768;  // value buckets of the launch
 constexpr int kFusedShapes = 3;  // tile shapes of the single-launch sort: 384 x 24, 384 x 18, 384 x 12
 uint32_t fused_tile_keys(int shape);
 size_t fused_smem(bool pairs, int shape);

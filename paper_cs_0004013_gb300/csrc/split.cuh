@@ -37,15 +37,16 @@ struct SplitLayout {
   static constexpr size_t OFF_SCAN = OFF_GOFF + 256 * 4;
   static constexpr size_t OFF_JOB = OFF_SCAN + 32 * 4;
   static constexpr size_t SMEM = OFF_JOB + 16;
-  static_assert(THREADS >= 256 && ITEMS % 4 == 0, "a thread per digit; digits are packed four to a word");
+  static_assert(THREADS >= 256 && true, "a thread per digit");
 };
 
 // The tile's keys in[0, valid) (FULL: valid is the tile's size), mapped by
-// ordi, to out[cursor of their digit ...) (mapped back by ordo).
+// ordi, to out[cursor of their digit ...) (mapped back by ordo).  bases: added
+// to the cursors (null: the cursors start at the digits' bases).
 template <typename K, int THREADS, int ITEMS, bool FULL, class Digit, class OrdI, class OrdO>
 __device__ __forceinline__ void split_tile(const K* in, uint32_t valid, K* out, uint32_t* cursors, uint32_t n,
                                            const Digit& digit, const OrdI& ordi, const OrdO& ordo, uint32_t* err,
-                                           unsigned char* smem) {
+                                           unsigned char* smem, const uint32_t* bases = nullptr) {
   using L = SplitLayout<K, THREADS, ITEMS>;
   constexpr int ROW = L::ROW;
   K* s_key = reinterpret_cast<K*>(smem);
@@ -58,7 +59,7 @@ __device__ __forceinline__ void split_tile(const K* in, uint32_t valid, K* out, 
   // 1. load, digits (four to a word), counts
   const uint32_t row = smem_addr(s_cnt + (lane >> 4) * ROW);
   K key[ITEMS];
-  uint32_t dg[ITEMS / 4];
+  uint32_t dg[(ITEMS + 3) / 4];  // digits, four to a word
 #pragma unroll
   for (int j = 0; j < ITEMS; ++j) key[j] = has(j) ? ld_elem(in + j * THREADS + tid) : K(0);
   for (int i = tid; i < 2 * ROW; i += THREADS) s_cnt[i] = 0u;
@@ -80,7 +81,7 @@ __device__ __forceinline__ void split_tile(const K* in, uint32_t valid, K* out, 
   uint32_t claim = 0, excl = 0;
   if (tid < 256) {
     const uint32_t c0 = s_cnt[tid], tot = c0 + s_cnt[ROW + tid];
-    if (tot) claim = atomicAdd(&cursors[tid], tot);
+    if (tot) claim = atomicAdd(&cursors[tid], tot) + (bases ? bases[tid] : 0u);
     excl = scan256_exclusive(tot, s_scan);
     s_cnt[tid] = excl;
     s_cnt[ROW + tid] = excl + c0;
@@ -109,7 +110,7 @@ __device__ __forceinline__ void split_tile(const K* in, uint32_t valid, K* out, 
   // against a corrupted offset (it raises an error bit instead of writing out
   // of bounds).
   uint32_t worst = 0;
-  constexpr int W = 4;
+  constexpr int W = ITEMS % 4 == 0 ? 4 : ITEMS % 3 == 0 ? 3 : 1;
   auto write_out = [&](auto invert) {
 #pragma unroll
     for (int k0 = 0; k0 < ITEMS; k0 += W) {
