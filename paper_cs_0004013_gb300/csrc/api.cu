@@ -336,16 +336,28 @@ rs_status make_plan(uint64_t n, bool pairs, const rs_plan* user, SortPlan* p, in
 }
 
 // ---- temp layout ------------------------------------------------------------
-// The sort by value buckets (hybrid.cu): about 2,048 keys per bucket, at most
-// kHybMaxBuckets, in groups of 2^low_bits that halve the bucket's bits between
-// the two splits; up to 256 buckets take one split.
+// The sort by value buckets (hybrid.cu): at most kHybMaxBuckets, in groups of
+// 2^low_bits that halve the bucket's bits between the two splits; up to 256
+// buckets take one split.
+constexpr uint64_t kHybridMinKeys = 8192;  // the sample's size
 struct HybLayout {
+  HybShape shape = {};
+  uint64_t n = 0;
+  bool pairs = false;
   uint32_t buckets = 0, low_bits = 0, groups = 0;  // buckets == 0: not offered
-  size_t ctrl = 0, counts = 0, starts = 0, cursors = 0, group_cursors = 0, group_tiles = 0;
-  // the counts belong to what a sort clears first; returns the next offset
-  size_t place_counts(size_t off, uint64_t n, bool on) {
-    if (!on) return off;
-    uint64_t b = (n + 2047) / 2048;
+  size_t ctrl = 0, counts = 0, starts = 0, cursors = 0, group_cursors = 0, group_tiles = 0, status = 0;
+  size_t status_bytes = 0;
+  // Whether n keys are offered the buckets: their mean may reach three quarters
+  // of what a bucket takes.
+  static bool offers(uint64_t n, int kb, int vb) {
+    return n >= kHybridMinKeys && n <= uint64_t(kHybMaxBuckets) * hyb_shape(kb, vb).bucket_cap * 3 / 4;
+  }
+  // the counts (and two tickets) belong to what a sort clears first; returns the next offset
+  size_t place_counts(size_t off, uint64_t n_, int kb, int vb) {
+    n = n_;
+    pairs = vb != 0;
+    shape = hyb_shape(kb, vb);
+    uint64_t b = (n + shape.bucket_mean - 1) / shape.bucket_mean;
     if (b > kHybMaxBuckets) b = kHybMaxBuckets;
     uint32_t bits = 0;
     while ((uint64_t(1) << bits) < b) ++bits;
@@ -353,7 +365,7 @@ struct HybLayout {
     low_bits = bits <= 8 ? 0u : bits / 2;
     groups = uint32_t((b + (uint64_t(1) << low_bits) - 1) >> low_bits);
     counts = off;
-    return align_up(off + size_t(buckets) * 4);
+    return align_up(off + (size_t(buckets) + 2) * 4);
   }
   size_t place_rest(size_t off) {
     if (!buckets) return off;
@@ -366,6 +378,11 @@ struct HybLayout {
     for (size_t* at : {&group_cursors, &group_tiles}) {
       *at = off;
       off = align_up(off + 257 * 4);
+    }
+    if (pairs) {
+      status = off;
+      status_bytes = (2 * size_t((n + shape.split_tile - 1) / shape.split_tile) + groups) * 1024;
+      off = align_up(off + status_bytes);
     }
     return off;
   }
@@ -385,7 +402,8 @@ struct Layout {
   size_t total = 0;
 };
 
-Layout make_layout(const SortPlan& p, uint64_t n, bool pairs, bool hybrid = false, bool fused = false) {
+// hybrid_vb: payload bytes of a sort offered value buckets (-1: it is not).
+Layout make_layout(const SortPlan& p, uint64_t n, bool pairs, int hybrid_vb = -1, bool fused = false) {
   Layout L;
   const size_t digits = size_t(1) << p.R;
   size_t off = 0;
@@ -393,7 +411,7 @@ Layout make_layout(const SortPlan& p, uint64_t n, bool pairs, bool hybrid = fals
   off += kAlign;
   L.hist = off;
   off = align_up(off + size_t(p.nd) * digits * 4);
-  off = L.hyb.place_counts(off, n, hybrid);
+  if (hybrid_vb >= 0) off = L.hyb.place_counts(off, n, 4, hybrid_vb);
   L.memset_bytes = off;
   L.bases = off;
   off = align_up(off + size_t(p.nd) * digits * 4);
@@ -441,6 +459,54 @@ void part_offsets_host(uint64_t n, uint32_t parts, uint64_t* out) {
   for (uint64_t p = 0; p <= parts; ++p) out[p] = p * q + (p < r ? p : r);
 }
 
+// ---- the sort by value buckets -----------------------------------------------------
+// The sample and the counts, the buckets' splits and sorts and, gated behind
+// the sample's and the counts' choice, the radix passes; see hybrid.cu.
+struct BucketChain {
+  HybArgs a;
+  int key_bytes, val_bytes;
+};
+// The chain for `a`, which holds the buffers and the order map of the keys.
+BucketChain make_chain(HybArgs a, const HybLayout& H, size_t clear_bytes, unsigned char* temp, int key_bytes,
+                       int val_bytes, DeviceState* ds) {
+  a.buckets = H.buckets;
+  a.low_bits = H.low_bits;
+  a.groups = H.groups;
+  a.bucket_cap = H.shape.bucket_cap;
+  a.split_tile = H.shape.split_tile;
+  a.ctrl = reinterpret_cast<HybCtrl*>(temp + H.ctrl);
+  a.counts = reinterpret_cast<uint32_t*>(temp + H.counts);
+  a.starts = reinterpret_cast<uint32_t*>(temp + H.starts);
+  a.cursors = reinterpret_cast<uint32_t*>(temp + H.cursors);
+  a.group_cursors = reinterpret_cast<uint32_t*>(temp + H.group_cursors);
+  a.group_tiles = reinterpret_cast<uint32_t*>(temp + H.group_tiles);
+  a.tickets = a.counts + H.buckets;
+  a.status = reinterpret_cast<uint32_t*>(temp + H.status);
+  a.zero_ptr = reinterpret_cast<uint4*>(temp + H.status);
+  a.zero_vec4 = H.status_bytes / 16;
+  a.clear = reinterpret_cast<uint4*>(temp);
+  a.clear_vec4 = clear_bytes / 16;
+  a.err = ds->err;
+  return BucketChain{a, key_bytes, val_bytes};
+}
+
+// The sample, the counts, the splits and the bucket sorts; the radix passes
+// that follow wait behind a.ctrl->route.
+rs_status launch_buckets(const BucketChain& c, DeviceState* ds, cudaStream_t s) {
+  const struct {
+    HybStep step;
+    int kind;
+  } steps[] = {{HybStep::kSample, T_SAMPLE}, {HybStep::kCount, T_COUNT}, {HybStep::kSplit0, T_SPLIT0},
+               {HybStep::kSplit1, T_SPLIT1}, {HybStep::kBuckets, T_BUCKETS}};
+  for (const auto& st : steps) {
+    if (st.step == HybStep::kSplit1 && c.a.low_bits == 0) continue;
+    RS_CUDA(traced(st.kind, c.a.n, s,
+                   [&] { return launch_hybrid(c.a, st.step, c.key_bytes, c.val_bytes, unsigned(ds->num_sms), s); }),
+            "launch sort by buckets");
+  }
+  return RS_OK;
+}
+
 // ---- the LSD pipeline ---------------------------------------------------------
 // memset(ctrl + hist) -> upfront histogram (+ clear status) -> digit scans ->
 // one onesweep pass per digit.
@@ -450,7 +516,8 @@ rs_status run_lsd(const SortPlan& p, const Layout& L, const uint32_t* keys_in, c
                   uint32_t* keys_out, uint32_t* vals_out, uint32_t n, unsigned char* temp, bool force_all,
                   DeviceState* ds, cudaStream_t s, const uint32_t* vals2_in = nullptr, uint32_t* vals2_out = nullptr,
                   uint32_t* vals2_alt = nullptr, const uint2* pair_vals_in = nullptr, uint2* pair_vals_out = nullptr,
-                  const uint32_t* gate = nullptr) {
+                  const BucketChain* chain = nullptr) {
+  const uint32_t* gate = chain ? &chain->a.ctrl->route : nullptr;
   uint32_t* ctrl = reinterpret_cast<uint32_t*>(temp + L.ctrl);
   uint32_t* hist = reinterpret_cast<uint32_t*>(temp + L.hist);
   uint32_t* bases = reinterpret_cast<uint32_t*>(temp + L.bases);
@@ -772,57 +839,22 @@ rs_status run_msd(const SortPlan& p, const MsdLayout& M, const uint32_t* keys_in
   return run_segmented(M.seg, temp, bk, bv, keys_out, vals_out, ma.seg_off, kMsdBuckets, 3, p.xf, p.xf, ds, s);
 }
 
-// ---- the sort by value buckets -----------------------------------------------------
-// The sample, the buckets' path and, gated behind the sample's and the
-// counts' choice, the radix passes; see hybrid.cu.
-constexpr uint64_t kHybridMinKeys = 8192, kHybridMaxKeys = uint64_t(3) << 25;
-
-// Launches the sample, the counts, the splits and the bucket sorts; `a` holds
-// the keys' buffers and order map.  Afterwards *gate points to the choice that
-// the radix passes' launches wait behind.
-rs_status run_buckets(HybArgs a, const HybLayout& H, size_t clear_bytes, unsigned char* temp, int key_bytes,
-                      DeviceState* ds, cudaStream_t s, const uint32_t** gate) {
-  a.buckets = H.buckets;
-  a.low_bits = H.low_bits;
-  a.groups = H.groups;
-  a.bucket_cap = hyb_bucket_cap();
-  a.split_tile = hyb_split_tile(key_bytes);
-  a.ctrl = reinterpret_cast<HybCtrl*>(temp + H.ctrl);
-  a.counts = reinterpret_cast<uint32_t*>(temp + H.counts);
-  a.starts = reinterpret_cast<uint32_t*>(temp + H.starts);
-  a.cursors = reinterpret_cast<uint32_t*>(temp + H.cursors);
-  a.group_cursors = reinterpret_cast<uint32_t*>(temp + H.group_cursors);
-  a.group_tiles = reinterpret_cast<uint32_t*>(temp + H.group_tiles);
-  a.clear = reinterpret_cast<uint4*>(temp);
-  a.clear_vec4 = clear_bytes / 16;
-  a.err = ds->err;
-  const unsigned sms = unsigned(ds->num_sms);
-  const struct {
-    HybStep step;
-    int kind;
-  } steps[] = {{HybStep::kSample, T_SAMPLE}, {HybStep::kCount, T_COUNT}, {HybStep::kSplit0, T_SPLIT0},
-               {HybStep::kSplit1, T_SPLIT1}, {HybStep::kBuckets, T_BUCKETS}};
-  for (const auto& st : steps) {
-    if (st.step == HybStep::kSplit1 && a.low_bits == 0) continue;
-    RS_CUDA(traced(st.kind, a.n, s, [&] { return launch_hybrid(a, st.step, key_bytes, sms, s); }),
-            "launch sort by buckets");
-  }
-  *gate = &a.ctrl->route;
-  return RS_OK;
-}
-
-rs_status run_hybrid32(const SortPlan& p, const Layout& L, const uint32_t* keys_in, uint32_t* keys_out, uint32_t n,
-                       unsigned char* temp, DeviceState* ds, cudaStream_t s) {
+rs_status run_hybrid32(const SortPlan& p, const Layout& L, const uint32_t* keys_in, const uint32_t* vals_in,
+                       uint32_t* keys_out, uint32_t* vals_out, uint32_t n, unsigned char* temp, DeviceState* ds,
+                       cudaStream_t s) {
   HybArgs a{};
   a.keys_in = keys_in;
   a.keys_out = keys_out;
   a.keys_alt = temp + L.alt_k;
+  a.vals_in = vals_in;
+  a.vals_out = vals_out;
+  a.vals_alt = temp + L.alt_v;
   a.n = n;
   a.x = p.xf;
-  const uint32_t* gate = nullptr;
-  if (rs_status st = run_buckets(a, L.hyb, L.memset_bytes, temp, 4, ds, s, &gate); st != RS_OK) return st;
-  return run_lsd(p, L, keys_in, nullptr, keys_out, nullptr, n, temp, false, ds, s, nullptr, nullptr, nullptr, nullptr,
-                 nullptr, gate);
+  const BucketChain c = make_chain(a, L.hyb, L.memset_bytes, temp, 4, vals_in ? 4 : 0, ds);
+  if (rs_status st = launch_buckets(c, ds, s); st != RS_OK) return st;
+  return run_lsd(p, L, keys_in, vals_in, keys_out, vals_out, n, temp, false, ds, s, nullptr, nullptr, nullptr, nullptr,
+                 nullptr, &c);
 }
 
 // ---- the single-launch sort -----------------------------------------------------
@@ -886,8 +918,8 @@ rs_status sort_impl(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* 
   const bool fusable = automatic && p.R == 8 && p.nd == 4 && !p.msd && !p.k->wide_status;
   if (fusable && n <= kFusedStatusMaxKeys)  // status rows for the single-launch sort's smallest tiles
     p.status_rows = size_t((n + fused_tile_keys(kFusedShapes - 1) - 1) / fused_tile_keys(kFusedShapes - 1));
-  const bool hybrid = fusable && !pairs && n >= kHybridMinKeys && n <= kHybridMaxKeys;
-  Layout L = make_layout(p, n, pairs, hybrid, p.status_rows > 0);
+  const bool hybrid = fusable && HybLayout::offers(n, 4, pairs ? 4 : 0);
+  Layout L = make_layout(p, n, pairs, hybrid ? (pairs ? 4 : 0) : -1, p.status_rows > 0);
   MsdLayout M;
   if (p.msd) {
     if (rs_status st2 = make_msd_layout(p, n, pairs, &M); st2 != RS_OK) return st2;
@@ -957,7 +989,9 @@ rs_status sort_impl(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* 
       return run_fused(p, L, keys_in, pairs ? vals_in : nullptr, keys_out, pairs ? vals_out : nullptr, uint32_t(n),
                        sh, static_cast<unsigned char*>(temp), ds, s);
   }
-  if (hybrid) return run_hybrid32(p, L, keys_in, keys_out, uint32_t(n), static_cast<unsigned char*>(temp), ds, s);
+  if (hybrid)
+    return run_hybrid32(p, L, keys_in, pairs ? vals_in : nullptr, keys_out, pairs ? vals_out : nullptr, uint32_t(n),
+                        static_cast<unsigned char*>(temp), ds, s);
   return run_lsd(p, L, keys_in, pairs ? vals_in : nullptr, keys_out, pairs ? vals_out : nullptr, uint32_t(n),
                  static_cast<unsigned char*>(temp), false, ds, s);
 }
@@ -982,7 +1016,7 @@ struct Layout64 {
   size_t memset_bytes = 0, total = 0;
 };
 
-Layout64 make_layout64(const SortPlan& p, uint64_t n, bool pairs, bool vals64 = false, bool hybrid = false) {
+Layout64 make_layout64(const SortPlan& p, uint64_t n, bool pairs, bool vals64, bool hybrid) {
   Layout64 L;
   L.fused = pair_io_kernel(p.k) != nullptr;
   size_t off = 0;
@@ -990,7 +1024,7 @@ Layout64 make_layout64(const SortPlan& p, uint64_t n, bool pairs, bool vals64 = 
   off += kAlign;
   L.hist = off;
   off = align_up(off + 8 * 256 * 4);
-  off = L.hyb.place_counts(off, n, hybrid);
+  if (hybrid) off = L.hyb.place_counts(off, n, 8, vals64 ? 8 : pairs ? 4 : 0);
   L.memset_bytes = off;
   L.bases = off;
   off = align_up(off + 8 * 256 * 4);
@@ -1044,9 +1078,15 @@ rs_status run_lsd64(const SortPlan& p, const Layout64& L, const uint64_t* keys_i
     a.keys_in = keys_in;
     a.keys_out = keys_out;
     a.keys_alt = pl[0];  // planes 0 and 1 follow each other
+    a.vals_in = vals_in ? static_cast<const void*>(vals_in) : vals64_in;
+    a.vals_out = vals_out ? static_cast<void*>(vals_out) : vals64_out;
+    a.vals_alt = temp + L.val_alt;  // (64-bit values: it and the index plane follow each other)
     a.n = n;
     a.x64 = x;
-    if (rs_status st = run_buckets(a, L.hyb, L.memset_bytes, temp, 8, ds, s, &gate); st != RS_OK) return st;
+    const int vb = vals_in ? 4 : vals64_in ? 8 : 0;
+    const BucketChain c = make_chain(a, L.hyb, L.memset_bytes, temp, 8, vb, ds);
+    if (rs_status st = launch_buckets(c, ds, s); st != RS_OK) return st;
+    gate = &c.a.ctrl->route;
   } else {
     RS_CUDA(traced(T_CLEAR, 0, s, [&] { return cudaMemsetAsync(temp, 0, L.memset_bytes, s); }),
             "cudaMemsetAsync(temp)");
@@ -1210,7 +1250,7 @@ static rs_status sort64_impl(const uint64_t* keys_in, const void* vals_in, uint6
   if (rs_status st = make_plan(n, true, &q, &p, pairs ? 2 : 1); st != RS_OK) return st;
   const bool automatic = !plan || (plan->digit_bits == 0 && plan->mode == RS_MODE_AUTO && plan->tile == 0);
   // (the space for value buckets is part of every plan's layout)
-  Layout64 L = make_layout64(p, n, pairs, vbytes == 8, vbytes == 0 && n >= kHybridMinKeys && n <= kHybridMaxKeys);
+  Layout64 L = make_layout64(p, n, pairs, vbytes == 8, HybLayout::offers(n, 8, vbytes));
   if (!automatic) L.hyb.buckets = 0;
   if (vbytes == 8 && !L.fused)
     return fail(RS_ERR_UNSUPPORTED, "64-bit values: tile shape %u has no interleaved pass kernel", q.tile);
@@ -1304,7 +1344,9 @@ rs_status rs_sort_u32_pairs64(const uint32_t* keys_in, const uint64_t* vals_in, 
   // the high words' alternate plane and (split only) both words of the input.
   // A tiled pass kernel reads and writes the interleaved values itself
   // (fused); a persistent one takes planes split and joined by kernels.
-  Layout L = make_layout(p, n, true);
+  const bool automatic = !plan || (plan->digit_bits == 0 && plan->mode == RS_MODE_AUTO && plan->tile == 0);
+  const bool hybrid = automatic && HybLayout::offers(n, 4, 8);
+  Layout L = make_layout(p, n, true, hybrid ? 8 : -1);
   const bool fused = pair_io_kernel(p.k) != nullptr;
   const int nplanes = fused ? 3 : 5;
   size_t plane[5] = {};
@@ -1334,7 +1376,6 @@ rs_status rs_sort_u32_pairs64(const uint32_t* keys_in, const uint64_t* vals_in, 
   if (n == 0) return RS_OK;
   DeviceState* ds = nullptr;
   if ((st = device_state(&ds)) != RS_OK) return st;
-  const bool automatic = !plan || (plan->digit_bits == 0 && plan->mode == RS_MODE_AUTO && plan->tile == 0);
   if (automatic && n <= local_max_keys(4, 8)) {  // one block
     LocalArgs la{};
     la.kin = keys_in;
@@ -1355,8 +1396,22 @@ rs_status rs_sort_u32_pairs64(const uint32_t* keys_in, const uint64_t* vals_in, 
   if (fused) {
     SortPlan q2 = p;
     q2.k = pair_io_kernel(p.k);
+    BucketChain c{};
+    if (hybrid) {
+      HybArgs a{};
+      a.keys_in = keys_in;
+      a.keys_out = keys_out;
+      a.keys_alt = t + L.alt_k;
+      a.vals_in = vals_in;
+      a.vals_out = vals_out;
+      a.vals_alt = pl[0];  // planes 0 and 1 follow each other
+      a.n = uint32_t(n);
+      a.x = p.xf;
+      c = make_chain(a, L.hyb, L.memset_bytes, t, 4, 8, ds);
+      if ((st = launch_buckets(c, ds, s)) != RS_OK) return st;
+    }
     return run_lsd(q2, L, keys_in, nullptr, keys_out, vlo_out, uint32_t(n), t, false, ds, s, nullptr, vhi_out,
-                   vhi_alt, reinterpret_cast<const uint2*>(vals_in), reinterpret_cast<uint2*>(vals_out));
+                   vhi_alt, reinterpret_cast<const uint2*>(vals_in), reinterpret_cast<uint2*>(vals_out), hybrid ? &c : nullptr);
   }
   const unsigned egrid = unsigned(std::min<size_t>((size_t(n) + 255) / 256, size_t(ds->num_sms) * 8));
   const KeyXform64 ident{0u, 0u, 0u};

@@ -19,6 +19,9 @@
 //   buckets  one block per bucket sorts it in place (local.cuh).
 // Every kernel returns at once when the sort takes the other way.
 //
+// Sorts with payloads take stable splits (stable_split.cuh), and a bucket's
+// equal keys are ordered by where they are in it.
+//
 // Against the radix passes (8 digits of 8 bits for 64-bit keys, 4 for 32-bit
 // ones), the keys cross memory three times instead of four or eight, and keys
 // without payloads need no stable ranking: a key's place in its tile is one
@@ -29,6 +32,7 @@
 #include "local.cuh"
 #include "sample.cuh"
 #include "split.cuh"
+#include "stable_split.cuh"
 #include "value_map.cuh"
 
 namespace rs {
@@ -78,6 +82,7 @@ __global__ void __cluster_dims__(kSampleBlocks, 1, 1) __launch_bounds__(kSampleT
       a.clear[i] = make_uint4(0u, 0u, 0u, 0u);
   });
 }
+
 // ------------------------------------------------------------------ counts
 // Keys per bucket.  32-bit shared counters for every bucket (up to 128 KiB),
 // one shared reduction per key; the blocks add them into the global counts.
@@ -199,17 +204,38 @@ __global__ void __launch_bounds__(kCountThreads, 1) bucket_count_kernel(const Hy
 }
 
 // ------------------------------------------------------------------- split
+// Tile t of the second split: its group (found by every thread looking at
+// one), the tiles before the group's first and the tile's keys; through s_job
+// (4 words).  Every thread of the block calls it.
+struct GroupTile {
+  uint32_t base, valid, group, first;
+};
+__device__ __forceinline__ GroupTile group_tile(const HybArgs& a, uint32_t t, uint32_t tile_keys, uint32_t* s_job) {
+  const uint32_t g = threadIdx.x;
+  if (g < a.groups) {
+    const uint32_t f = a.group_tiles[g], e = a.group_tiles[g + 1];
+    if (f <= t && t < e) {
+      const uint32_t g0 = a.starts[g << a.low_bits];
+      const uint32_t last = (g + 1) << a.low_bits;
+      const uint32_t g1 = a.starts[last < a.buckets ? last : a.buckets];
+      const uint32_t b = g0 + (t - f) * tile_keys;
+      s_job[0] = b;
+      s_job[1] = g1 - b < tile_keys ? g1 - b : tile_keys;
+      s_job[2] = g;
+      s_job[3] = f;
+    }
+  }
+  __syncthreads();
+  return GroupTile{s_job[0], s_job[1], s_job[2], s_job[3]};
+}
+
 // One distribution of keys without payloads (split.cuh).  LEVEL 0: the
 // input's tiles to the groups (the bucket's high bits); LEVEL 1: each group's
 // tiles to its buckets (the low bits).
-template <typename K, int THREADS, int ITEMS, int MINB, int LEVEL>
-__global__ void __launch_bounds__(THREADS, MINB) split_kernel(const HybArgs a) {
+template <typename K, int THREADS, int ITEMS, int LEVEL>
+__device__ __forceinline__ void split_body(const HybArgs& a, unsigned char* smem) {
   using L = SplitLayout<K, THREADS, ITEMS>;
   constexpr uint32_t TILE = L::TILE;
-  extern __shared__ __align__(16) unsigned char smem[];
-  wait_for_chain();
-  if (a.ctrl->route != kHybBuckets) return;
-  const int tid = threadIdx.x;
   const ValueMap<K> m = load_map<K>(a.ctrl);
   const uint32_t dshift = LEVEL == 0 ? a.low_bits : 0u;
   const uint32_t dmask = LEVEL == 0 ? 0xffu : (1u << a.low_bits) - 1u;
@@ -221,25 +247,11 @@ __global__ void __launch_bounds__(THREADS, MINB) split_kernel(const HybArgs a) {
     valid = a.n - base < TILE ? a.n - base : TILE;
     cursors = a.group_cursors;
   } else {
-    // the tile's group, found by every thread looking at one
-    uint32_t* s_job = reinterpret_cast<uint32_t*>(smem + L::OFF_JOB);
     if (blockIdx.x >= a.ctrl->tiles_b) return;
-    if (tid < int(a.groups)) {
-      const uint32_t f = a.group_tiles[tid], e = a.group_tiles[tid + 1];
-      if (f <= blockIdx.x && blockIdx.x < e) {
-        const uint32_t g0 = a.starts[tid << a.low_bits];
-        const uint32_t last = (uint32_t(tid) + 1) << a.low_bits;
-        const uint32_t g1 = a.starts[last < a.buckets ? last : a.buckets];
-        const uint32_t b = g0 + (blockIdx.x - f) * TILE;
-        s_job[0] = b;
-        s_job[1] = g1 - b < TILE ? g1 - b : TILE;
-        s_job[2] = uint32_t(tid);
-      }
-    }
-    __syncthreads();
-    base = s_job[0];
-    valid = s_job[1];
-    cursors = a.cursors + (s_job[2] << a.low_bits);
+    const GroupTile t = group_tile(a, blockIdx.x, TILE, reinterpret_cast<uint32_t*>(smem + L::OFF_JOB));
+    base = t.base;
+    valid = t.valid;
+    cursors = a.cursors + (t.group << a.low_bits);
   }
   const K* in = reinterpret_cast<const K*>(LEVEL == 0 ? a.keys_in : a.keys_alt) + base;
   K* out = reinterpret_cast<K*>(LEVEL == 0 && a.low_bits != 0 ? a.keys_alt : a.keys_out);  // one split: no detour
@@ -249,37 +261,115 @@ __global__ void __launch_bounds__(THREADS, MINB) split_kernel(const HybArgs a) {
   else split_tile<K, THREADS, ITEMS, false>(in, valid, out, cursors, a.n, digit, ordi, ident, a.err, smem);
 }
 
-// ----------------------------------------------------------------- buckets
-constexpr int kBucketThreads = 128, kBucketItems = 24, kBucketBits = 12;
+template <typename K, int THREADS, int ITEMS, int MINB, int LEVEL>
+__global__ void __launch_bounds__(THREADS, MINB) split_kernel(const HybArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  wait_for_chain();
+  if (a.ctrl->route == kHybBuckets) split_body<K, THREADS, ITEMS, LEVEL>(a, smem);
+}
 
-template <typename K, int VB, int MINB>
-__global__ void __launch_bounds__(kBucketThreads, MINB) bucket_sort_kernel(const HybArgs a) {
+// The same with payloads, stable (stable_split.cuh): tiles by ticket, ordered
+// by a chained scan, of the whole input (LEVEL 0) or within the group (LEVEL 1).
+template <typename K, int VB, int THREADS, int ITEMS, int LEVEL>
+__device__ __forceinline__ void stable_split_body(const HybArgs& a, unsigned char* smem) {
+  using L = StableSplitLayout<K, VB, THREADS, ITEMS>;
+  using V = typename L::V;
+  constexpr uint32_t TILE = L::TILE;
+  // as many blocks as tiles take tickets
+  if (blockIdx.x >= (LEVEL == 0 ? (a.n + TILE - 1) / TILE : a.ctrl->tiles_b)) return;
+  uint32_t* s_job = reinterpret_cast<uint32_t*>(smem + L::OFF_JOB);
+  uint4* c4 = reinterpret_cast<uint4*>(smem);
+  for (int i = threadIdx.x; i < int(L::RANK_BYTES / 16); i += THREADS) c4[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (threadIdx.x == 0) s_job[0] = atomicAdd(a.tickets + LEVEL, 1u);
+  const ValueMap<K> m = load_map<K>(a.ctrl);
+  __syncthreads();
+  const uint32_t tile = s_job[0];
+  const uint32_t dshift = LEVEL == 0 ? a.low_bits : 0u;
+  const uint32_t dmask = LEVEL == 0 ? 0xffu : (1u << a.low_bits) - 1u;
+  auto digit = [&](K k) { return (m.bucket(k) >> dshift) & dmask; };
+  GroupTile t{0u, 0u, 0u, 0u};
+  if constexpr (LEVEL == 0) {
+    t.base = tile * TILE;
+    t.valid = a.n - t.base < TILE ? a.n - t.base : TILE;
+  } else {
+    __syncthreads();  // the ticket is read
+    t = group_tile(a, tile, TILE, s_job);
+  }
+  // a digit's first place: its bucket's start (a digit that no bucket has moves nothing)
+  auto base = [&](uint32_t d) {
+    const uint32_t b = LEVEL == 0 ? d << a.low_bits : (t.group << a.low_bits) + d;
+    return a.starts[b < a.buckets ? b : a.buckets];
+  };
+  const bool to_alt = LEVEL == 0 && a.low_bits != 0;  // one split: no detour
+  const K* in = reinterpret_cast<const K*>(LEVEL == 0 ? a.keys_in : a.keys_alt) + t.base;
+  const V* vin = reinterpret_cast<const V*>(LEVEL == 0 ? a.vals_in : a.vals_alt) + t.base;
+  K* out = reinterpret_cast<K*>(to_alt ? a.keys_alt : a.keys_out);
+  V* vout = reinterpret_cast<V*>(to_alt ? a.vals_alt : a.vals_out);
+  uint32_t* status = LEVEL == 0 ? a.status : a.status + size_t((a.n + TILE - 1) / TILE) * 256;
+  const auto ordi = LEVEL == 0 ? OrdOf<K>::make(a) : OrdOf<K>::identity();
+  if (t.valid == TILE)
+    stable_split_tile<K, VB, THREADS, ITEMS, true>(in, vin, t.valid, out, vout, a.n, status, tile, t.first, digit, base,
+                                                   ordi, a.err, smem);
+  else
+    stable_split_tile<K, VB, THREADS, ITEMS, false>(in, vin, t.valid, out, vout, a.n, status, tile, t.first, digit, base,
+                                                    ordi, a.err, smem);
+}
+
+template <typename K, int VB, int THREADS, int ITEMS, int MINB, int LEVEL>
+__global__ void __launch_bounds__(THREADS, MINB) stable_split_kernel(const HybArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  wait_for_chain();
+  if (a.ctrl->route == kHybBuckets) stable_split_body<K, VB, THREADS, ITEMS, LEVEL>(a, smem);
+}
+
+// ----------------------------------------------------------------- buckets
+// One block per bucket, in place.  (A loop over a few buckets per block, which
+// a sort that goes the other way would leave sooner, spills: 203 us -> 394 for
+// 2^26 keys.)
+template <typename K, int VB, int THREADS, int ITEMS, int MINB>
+__global__ void __launch_bounds__(THREADS, MINB) bucket_sort_kernel(const HybArgs a) {
+  constexpr int BITS = 12;
   extern __shared__ __align__(16) unsigned char smem[];
   wait_for_chain();
   if (a.ctrl->route != kHybBuckets) return;
   const ValueMap<K> m = load_map<K>(a.ctrl);
   using V = typename ValueOf<VB>::T;
-  constexpr Vals MODE = VB ? Vals::kStaged : Vals::kAlone;
   const uint32_t b = blockIdx.x, s = a.starts[b], e = a.starts[b + 1];
   if (s == e) return;
   K* io = reinterpret_cast<K*>(a.keys_out) + s;
   V* vio = VB ? reinterpret_cast<V*>(a.vals_out) + s : nullptr;
-  if (b == 0 || b == a.buckets - 1)
-    local_sort_array<kBucketThreads, kBucketItems, kBucketBits, VB, MODE, true>(
-        io, io, vio, vio, vio, e - s, OrdOf<K>::identity(), OrdOf<K>::make(a), BucketBins<K, kBucketBits, true>{m}, smem);
-  else
-    local_sort_array<kBucketThreads, kBucketItems, kBucketBits, VB, MODE, true>(
-        io, io, vio, vio, vio, e - s, OrdOf<K>::identity(), OrdOf<K>::make(a), BucketBins<K, kBucketBits, false>{m}, smem);
+  auto sort = [&](auto edge, auto mode, auto eo) {
+    local_sort_array<THREADS, ITEMS, BITS, VB, decltype(mode)::value, true>(io, io, vio, vio, vio, e - s, OrdOf<K>::identity(),
+                                                           OrdOf<K>::make(a),
+                                                           BucketBins<K, BITS, decltype(edge)::value>{m}, smem, eo);
+  };
+  const bool edge = b == 0 || b == a.buckets - 1;
+  if constexpr (VB == 0) {
+    using Alone = std::integral_constant<Vals, Vals::kAlone>;
+    if (edge) sort(std::true_type{}, Alone{}, ElemOf<K, false>{});
+    else sort(std::false_type{}, Alone{}, ElemOf<K, false>{});
+  } else {
+    // A key's distance from its bucket's first possible key and its place
+    // share a word when they fit: half the work of ordering them side by side.
+    constexpr int PBITS = THREADS * ITEMS <= 2048 ? 11 : 12;
+    static_assert(THREADS * ITEMS < (1 << 12), "a place's bits");
+    const uint64_t step = 0xffffffffull / m.mult + 1;  // offsets per bucket, at most
+    const uint64_t t0 = ((uint64_t(b) << 32) + m.mult - 1) / m.mult;  // the bucket's first offset
+    const int bits = 64 - __clzll((long long)step) + int(m.sh);
+    if (!edge && bits + PBITS <= int(sizeof(K) * 8))
+      sort(std::false_type{}, std::integral_constant<Vals, Vals::kStaged>{},
+           PackedElem<K, PBITS>{K(m.lo + (K(t0) << m.sh))});
+    else
+      sort(std::true_type{}, std::integral_constant<Vals, Vals::kInPlace>{}, ElemOf<K, true>{});
+  }
 }
 
 // ------------------------------------------------- first radix pass of keys
 // The first executed pass of a radix sort of keys without payloads: there is
 // no earlier order to keep, so it is a split by the lowest byte.
-__global__ void __launch_bounds__(kSplitThreads, kSplitBlocks) first_pass_kernel(const PassArgs a) {
+__device__ __forceinline__ void first_pass_body(const PassArgs& a, unsigned char* smem) {
   using L = SplitLayout<uint32_t, kSplitThreads, kSplitItems>;
   constexpr uint32_t TILE = L::TILE;
-  extern __shared__ __align__(16) unsigned char smem[];
-  if (gated_off(a.gate)) return;
   const Route route = route_of(a.skip, 0, a.num_passes);
   if (!route.active) return;
   const uint32_t base = blockIdx.x * TILE, valid = a.n - base < TILE ? a.n - base : TILE;
@@ -293,13 +383,71 @@ __global__ void __launch_bounds__(kSplitThreads, kSplitBlocks) first_pass_kernel
     split_tile<uint32_t, kSplitThreads, kSplitItems, false>(a.keys_in + base, valid, out, a.cursors, a.n, digit, ordi,
                                                             ordo, a.err, smem);
 }
+__global__ void __launch_bounds__(kSplitThreads, kSplitBlocks) first_pass_kernel(const PassArgs p) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  if (!gated_off(p.gate)) first_pass_body(p, smem);
+}
 
-template <typename K>
+// Shapes per key and payload bytes: the splits' threads, items and blocks per
+// SM (ST, SI, SB), the bucket sort's (BT, BI, BB).  MEAN: keys per bucket that
+// the plan aims at; a bucket takes half as many again.  GB300, us per launch:
+//   32-bit keys, 2^26: bucket sort 128 x 24 at 8 blocks 203, 256 x 12 at 5 230;
+//   with a 32-bit payload: splits 384 x 16 at 3 blocks 353 and 320 (256 x 24 at
+//   4: 383, 365; 384 x 20 at 3: 361, 341; 512 x 20 at 2: 356, 340), bucket sort
+//   256 x 12 at 5 303 (at 4: 331; 128 x 24 at 5: 369; 384 x 8 at 3: 401);
+//   64-bit keys, 2^24: bucket sort 256 x 12 101 (128 x 24: 108 to 114).
+template <typename K, int VB>
+struct Shape;
+template <>
+struct Shape<uint32_t, 0> {
+  static constexpr int ST = kSplitThreads, SI = kSplitItems, SB = kSplitBlocks, BT = 128, BI = 24, BB = 8, MEAN = 2048;
+};
+template <>
+struct Shape<uint64_t, 0> {
+  static constexpr int ST = kSplitThreads, SI = kSplitItems / 2, SB = kSplitBlocks, BT = 256, BI = 12, BB = 4,
+                       MEAN = 2048;
+};
+template <>
+struct Shape<uint32_t, 4> {
+  static constexpr int ST = 384, SI = 16, SB = 3, BT = 256, BI = 12, BB = 5, MEAN = 2048;
+};
+template <>
+struct Shape<uint32_t, 8> {
+  static constexpr int ST = 384, SI = 16, SB = 3, BT = 256, BI = 8, BB = 3, MEAN = 1365;
+};
+template <>
+struct Shape<uint64_t, 4> {
+  static constexpr int ST = 384, SI = 12, SB = 3, BT = 256, BI = 8, BB = 3, MEAN = 1365;
+};
+template <>
+struct Shape<uint64_t, 8> {
+  static constexpr int ST = 384, SI = 12, SB = 3, BT = 256, BI = 8, BB = 3, MEAN = 1365;
+};
+
+template <typename K, int VB>
 struct Kernels {
-  static constexpr int ST = kSplitThreads, SI = sizeof(K) == 4 ? kSplitItems : kSplitItems / 2, SB = kSplitBlocks;
-  using Split = SplitLayout<K, ST, SI>;
-  using Local = LocalLayout<kBucketThreads, kBucketItems, kBucketBits, K, 0, Vals::kAlone>;
-  static constexpr int LB = sizeof(K) == 4 ? 8 : 4;
+  using T = Shape<K, VB>;
+  // the larger of a bucket's two ways (keys and places packed, or side by side)
+  static constexpr size_t local_smem() {
+    if constexpr (VB == 0) {
+      return LocalLayout<T::BT, T::BI, 12, K, 0, Vals::kAlone>::SMEM;
+    } else {
+      constexpr size_t packed = LocalLayout<T::BT, T::BI, 12, K, VB, Vals::kStaged, PackedElem<K, 12>>::SMEM;
+      constexpr size_t wide = LocalLayout<T::BT, T::BI, 12, K, VB, Vals::kInPlace>::SMEM;
+      return packed > wide ? packed : wide;
+    }
+  }
+  static constexpr uint32_t TILE = uint32_t(T::ST * T::SI), CAP = uint32_t(T::BT * T::BI);
+  template <int LEVEL>
+  static auto split() {
+    if constexpr (VB != 0) return &stable_split_kernel<K, VB, T::ST, T::SI, T::SB, LEVEL>;
+    else return &split_kernel<K, T::ST, T::SI, T::SB, LEVEL>;
+  }
+  static constexpr size_t split_smem() {
+    if constexpr (VB != 0) return StableSplitLayout<K, VB, T::ST, T::SI>::SMEM;
+    else return SplitLayout<K, T::ST, T::SI>::SMEM;
+  }
+  static auto buckets() { return &bucket_sort_kernel<K, VB, T::BT, T::BI, T::BB>; }
   static cudaError_t prepare() {
     cudaError_t e = cudaSuccess;
     auto set = [&](const void* f, size_t bytes) {
@@ -307,19 +455,41 @@ struct Kernels {
     };
     set(reinterpret_cast<const void*>(&sample_kernel<K>), SampleLayout<K, kSampleBlocks, kSampleThreads>::SMEM);
     set(reinterpret_cast<const void*>(&bucket_count_kernel<K>), size_t(kHybMaxBuckets) * 4);
-    set(reinterpret_cast<const void*>(&split_kernel<K, ST, SI, SB, 0>), Split::SMEM);
-    set(reinterpret_cast<const void*>(&split_kernel<K, ST, SI, SB, 1>), Split::SMEM);
-    set(reinterpret_cast<const void*>(&bucket_sort_kernel<K, 0, LB>), Local::SMEM);
+    set(reinterpret_cast<const void*>(split<0>()), split_smem());
+    set(reinterpret_cast<const void*>(split<1>()), split_smem());
+    set(reinterpret_cast<const void*>(buckets()), local_smem());
     return e;
+  }
+  static HybShape shape() { return HybShape{TILE, CAP, uint32_t(T::MEAN)}; }
+  static cudaError_t launch(const HybArgs& a, HybStep step, unsigned sms, cudaStream_t s) {
+    const unsigned tiles = (a.n + TILE - 1) / TILE;
+    switch (step) {
+      case HybStep::kSample:
+        sample_kernel<K>
+            <<<kSampleBlocks, kSampleThreads, SampleLayout<K, kSampleBlocks, kSampleThreads>::SMEM, s>>>(a);
+        return cudaGetLastError();
+      case HybStep::kCount:
+        return launch_chained(&bucket_count_kernel<K>, sms, kCountThreads, size_t(a.buckets) * 4, s, true, a);
+      case HybStep::kSplit0: return launch_chained(split<0>(), tiles, T::ST, split_smem(), s, true, a);
+      case HybStep::kSplit1: return launch_chained(split<1>(), tiles + a.groups, T::ST, split_smem(), s, true, a);
+      case HybStep::kBuckets: return launch_chained(buckets(), a.buckets, T::BT, local_smem(), s, true, a);
+    }
+    return cudaErrorInvalidValue;
   }
 };
 
+// f(Kernels) of the key and payload widths.
+template <class F>
+auto with_kernels(int kb, int vb, F&& f) {
+  if (kb == 4) return vb == 0 ? f(Kernels<uint32_t, 0>{}) : vb == 4 ? f(Kernels<uint32_t, 4>{}) : f(Kernels<uint32_t, 8>{});
+  return vb == 0 ? f(Kernels<uint64_t, 0>{}) : vb == 4 ? f(Kernels<uint64_t, 4>{}) : f(Kernels<uint64_t, 8>{});
+}
+
 }  // namespace
 
-uint32_t hyb_split_tile(int key_bytes) {
-  return key_bytes == 4 ? uint32_t(Kernels<uint32_t>::Split::TILE) : uint32_t(Kernels<uint64_t>::Split::TILE);
+HybShape hyb_shape(int key_bytes, int val_bytes) {
+  return with_kernels(key_bytes, val_bytes, [](auto k) { return decltype(k)::shape(); });
 }
-uint32_t hyb_bucket_cap() { return uint32_t(kBucketThreads * kBucketItems); }
 
 cudaError_t launch_first_pass(const PassArgs& a, cudaStream_t s) {
   using L = SplitLayout<uint32_t, kSplitThreads, kSplitItems>;
@@ -328,37 +498,17 @@ cudaError_t launch_first_pass(const PassArgs& a, cudaStream_t s) {
 }
 
 cudaError_t prepare_hybrid() {
-  cudaError_t e = Kernels<uint32_t>::prepare();
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(reinterpret_cast<const void*>(&first_pass_kernel),
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(SplitLayout<uint32_t, kSplitThreads, kSplitItems>::SMEM));
-  return e == cudaSuccess ? Kernels<uint64_t>::prepare() : e;
+  cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(&first_pass_kernel),
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       int(SplitLayout<uint32_t, kSplitThreads, kSplitItems>::SMEM));
+  for (int kb : {4, 8})
+    for (int vb : {0, 4, 8})
+      if (e == cudaSuccess) e = with_kernels(kb, vb, [](auto k) { return decltype(k)::prepare(); });
+  return e;
 }
 
-template <typename K>
-static cudaError_t launch(const HybArgs& a, HybStep step, unsigned sms, cudaStream_t s) {
-  using T = Kernels<K>;
-  const unsigned tiles = (a.n + a.split_tile - 1) / a.split_tile;
-  switch (step) {
-    case HybStep::kSample:
-      sample_kernel<K><<<kSampleBlocks, kSampleThreads, SampleLayout<K, kSampleBlocks, kSampleThreads>::SMEM, s>>>(a);
-      return cudaGetLastError();
-    case HybStep::kCount:
-      return launch_chained(&bucket_count_kernel<K>, sms, kCountThreads, size_t(a.buckets) * 4, s, true, a);
-    case HybStep::kSplit0:
-      return launch_chained(&split_kernel<K, T::ST, T::SI, T::SB, 0>, tiles, T::ST, T::Split::SMEM, s, true, a);
-    case HybStep::kSplit1:
-      return launch_chained(&split_kernel<K, T::ST, T::SI, T::SB, 1>, tiles + a.groups, T::ST, T::Split::SMEM, s, true,
-                            a);
-    case HybStep::kBuckets:
-      return launch_chained(&bucket_sort_kernel<K, 0, T::LB>, a.buckets, kBucketThreads, T::Local::SMEM, s, true, a);
-  }
-  return cudaErrorInvalidValue;
-}
-
-cudaError_t launch_hybrid(const HybArgs& a, HybStep step, int key_bytes, unsigned sms, cudaStream_t s) {
-  return key_bytes == 4 ? launch<uint32_t>(a, step, sms, s) : launch<uint64_t>(a, step, sms, s);
+cudaError_t launch_hybrid(const HybArgs& a, HybStep step, int key_bytes, int val_bytes, unsigned sms, cudaStream_t s) {
+  return with_kernels(key_bytes, val_bytes, [&](auto k) { return decltype(k)::launch(a, step, sms, s); });
 }
 
 }  // namespace rs

@@ -41,6 +41,8 @@ struct HybArgs {
   uint32_t* cursors;        // [B]
   uint32_t* group_cursors;  // [256]
   uint32_t* group_tiles;    // [257]
+  uint32_t* tickets;        // [2], zero before the splits (sorts with payloads)
+  uint32_t* status;         // [tiles + second split's tiles][256], zero before the splits (with payloads)
   uint4* clear;             // cleared by the sample
   size_t clear_vec4;
   uint4* zero_ptr;          // cleared by the counts
@@ -49,9 +51,13 @@ struct HybArgs {
 };
 
 enum class HybStep { kSample, kCount, kSplit0, kSplit1, kBuckets };
-uint32_t hyb_split_tile(int key_bytes);
-uint32_t hyb_bucket_cap();
+struct HybShape {
+  uint32_t split_tile;   // keys of a split tile
+  uint32_t bucket_cap;   // keys the local sort takes
+  uint32_t bucket_mean;  // keys per bucket that the plan aims at
+};
+HybShape hyb_shape(int key_bytes, int val_bytes);
 cudaError_t prepare_hybrid();
-cudaError_t launch_hybrid(const HybArgs& a, HybStep step, int key_bytes, unsigned sms, cudaStream_t s);
+cudaError_t launch_hybrid(const HybArgs& a, HybStep step, int key_bytes, int val_bytes, unsigned sms, cudaStream_t s);
 
 }  // namespace rs

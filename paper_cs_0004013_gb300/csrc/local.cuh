@@ -86,6 +86,19 @@ struct ElemOf<uint64_t, true> {
   static __device__ __forceinline__ E last() { return E{~0ull, ~0u}; }
 };
 
+// (key, place) of keys from one narrow range in a single word: the key's
+// distance from the range's start above the place's PBITS bits.  The caller
+// makes sure that it fits.
+template <typename K, int PBITS>
+struct PackedElem {
+  using E = K;
+  K base;
+  __device__ __forceinline__ E make(K k, uint32_t i) const { return ((k - base) << PBITS) | K(i); }
+  __device__ __forceinline__ K key(E e) const { return base + (e >> PBITS); }
+  __device__ __forceinline__ uint32_t place(E e) const { return uint32_t(e) & ((1u << PBITS) - 1u); }
+  __device__ __forceinline__ E last() const { return ~K(0); }  // (no key has the place of all ones)
+};
+
 __device__ __forceinline__ void order2(uint32_t& a, uint32_t& b) {
   const uint32_t lo = min(a, b);
   b = max(a, b);
@@ -166,17 +179,19 @@ __device__ __forceinline__ void merge8(E (&v)[8]) {
 // How payloads follow their keys:
 //   kAlone    there are none;
 //   kFollow   each is read from the input, at its key's place there, when it leaves;
-//   kStaged   held in shared memory in input order meanwhile (sorts in place);
+//   kStaged   copied to shared memory in input order meanwhile (sorts in place);
+//   kInPlace  read like kFollow, but all of them before the first is written
+//             (sorts in place, less shared memory, slower);
 //   kPlaces   the input's second array holds places instead of payloads: equal
 //             keys are ordered by them, and payloads are read from a third
 //             array at the place.
-enum class Vals { kAlone, kFollow, kStaged, kPlaces };
+enum class Vals { kAlone, kFollow, kStaged, kInPlace, kPlaces };
 
-template <int THREADS, int ITEMS, int NBITS, typename K, int VB, Vals MODE>
+template <int THREADS, int ITEMS, int NBITS, typename K, int VB, Vals MODE, class Elem = ElemOf<K, VB != 0>>
 struct LocalLayout {
   static_assert((VB != 0) == (MODE != Vals::kAlone), "payloads and what happens to them");
   using V = typename ValueOf<VB>::T;
-  using E = typename ElemOf<K, VB != 0>::E;
+  using E = typename Elem::E;
   static constexpr bool STAGED = MODE == Vals::kStaged;
   static constexpr int WARPS = THREADS / 32;
   static constexpr int CAP = THREADS * ITEMS;
@@ -290,9 +305,8 @@ __device__ __forceinline__ void block_exclusive_sums(const uint32_t (&x)[R], uin
 // the order they were in.
 // BY_PLACE: equal keys are ordered by their places too (they are not in that
 // order to begin with).
-template <class L, int THREADS, int ITEMS, typename K, bool PAIRS, bool BY_PLACE>
-__device__ __noinline__ void local_digit_passes(uint32_t m, unsigned char* smem) {
-  using EO = ElemOf<K, PAIRS>;
+template <class L, int THREADS, int ITEMS, typename K, class EO, bool BY_PLACE>
+__device__ __noinline__ void local_digit_passes(uint32_t m, const EO eo, unsigned char* smem) {
   using E = typename EO::E;
   constexpr int WARPS = L::WARPS;
   E* s_key = reinterpret_cast<E*>(smem + L::OFF_KEY);
@@ -307,14 +321,14 @@ __device__ __noinline__ void local_digit_passes(uint32_t m, unsigned char* smem)
   E e[ITEMS];
   K diff = 0;
   uint32_t pdiff = 0;
-  const K k0 = EO::key(s_key[L::slot(0)]);
-  const uint32_t p0 = EO::place(s_key[L::slot(0)]);
+  const K k0 = eo.key(s_key[L::slot(0)]);
+  const uint32_t p0 = eo.place(s_key[L::slot(0)]);
 #pragma unroll
   for (int j = 0; j < ITEMS; ++j) {  // places past the end act as the largest key and stay behind
-    e[j] = wofs + j * 32 < m ? s_key[L::slot(wofs + j * 32)] : EO::last();
+    e[j] = wofs + j * 32 < m ? s_key[L::slot(wofs + j * 32)] : eo.last();
     if (wofs + j * 32 < m) {
-      diff |= EO::key(e[j]) ^ k0;
-      pdiff |= EO::place(e[j]) ^ p0;
+      diff |= eo.key(e[j]) ^ k0;
+      pdiff |= eo.place(e[j]) ^ p0;
     }
   }
 #pragma unroll
@@ -333,7 +347,7 @@ __device__ __noinline__ void local_digit_passes(uint32_t m, unsigned char* smem)
   }
   // digits 0-3 are the places' (BY_PLACE), the others the keys'
   auto digit = [&](const E& x, uint32_t d) {
-    return d < 4 ? (EO::place(x) >> (8 * d)) & 0xffu : uint32_t(EO::key(x) >> (8 * (d - 4))) & 0xffu;
+    return d < 4 ? (eo.place(x) >> (8 * d)) & 0xffu : uint32_t(eo.key(x) >> (8 * (d - 4))) & 0xffu;
   };
   for (uint32_t d = BY_PLACE ? 0 : 4; d < 4 + sizeof(K); ++d) {
     if (((d < 4 ? pdiff >> (8 * d) : uint32_t(diff >> (8 * (d - 4)))) & 0xffu) == 0) continue;  // uniform
@@ -380,18 +394,19 @@ __device__ __noinline__ void local_digit_passes(uint32_t m, unsigned char* smem)
 // kStaged may sort in place.  COHERENT: the inputs were written by other
 // blocks of the same launch, or are overwritten by this one.  ordi maps a key
 // on loading, ordo back on storing.  bins: RangeBins (filled here) or a map
-// known beforehand.  The block is synchronised on return.
+// known beforehand.  eo: what is ordered (by default the key, or key and
+// place side by side).  The block is synchronised on return.
 template <int THREADS, int ITEMS, int NBITS, int VB, Vals MODE, bool COHERENT, class OrdI, class OrdO, class Bins,
-          class VIn>
+          class VIn, class EO = ElemOf<typename OrdI::Key, VB != 0>>
 __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, typename OrdI::Key* out, const VIn* vin,
                                                  typename ValueOf<VB>::T* vout,
                                                  const typename ValueOf<VB>::T* from, const uint32_t m,
-                                                 const OrdI ordi, const OrdO ordo, Bins bins, unsigned char* smem) {
+                                                 const OrdI ordi, const OrdO ordo, Bins bins, unsigned char* smem,
+                                                 const EO eo = EO{}) {
   using K = typename OrdI::Key;
   constexpr bool STAGED = MODE == Vals::kStaged, PLACES = MODE == Vals::kPlaces;
-  using L = LocalLayout<THREADS, ITEMS, NBITS, K, VB, MODE>;
+  using L = LocalLayout<THREADS, ITEMS, NBITS, K, VB, MODE, EO>;
   using V = typename L::V;
-  using EO = ElemOf<K, VB != 0>;
   using E = typename EO::E;
   constexpr int WARPS = L::WARPS, NB = L::NB;
   uint32_t* s_bin = reinterpret_cast<uint32_t*>(smem);  // two 16-bit counts per word
@@ -401,7 +416,8 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
   K* s_red = reinterpret_cast<K*>(smem + L::OFF_WARP);
   uint32_t* s_scan = reinterpret_cast<uint32_t*>(smem + L::OFF_SCAN);
   uint32_t* s_most = reinterpret_cast<uint32_t*>(smem + L::OFF_MOST);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x;
+  const int lane = tid & 31, warp = tid >> 5;
   // Items go by groups of G: a group past the last key is skipped by the whole
   // block (a uniform branch); inside a group a lane without a key has its
   // shared atomic and its stores predicated off.
@@ -421,16 +437,22 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
   for_items([&](int j) { key[j] = has(j) ? ld_elem<COHERENT>(in + j * THREADS + tid) : K(0); });
   uint32_t place[PLACES ? ITEMS : 1];
   if constexpr (PLACES) for_items([&](int j) { place[j] = has(j) ? ld_elem<COHERENT>(vin + j * THREADS + tid) : 0u; });
-  auto elem = [&](int j) { return EO::make(key[j], PLACES ? place[PLACES ? j : 0] : uint32_t(j * THREADS + tid)); };
+  auto elem = [&](int j) { return eo.make(key[j], PLACES ? place[PLACES ? j : 0] : uint32_t(j * THREADS + tid)); };
   uint4* b4 = reinterpret_cast<uint4*>(smem);
 #pragma unroll
   for (int i = 0; i < NB / 8; i += THREADS)
     if (i + THREADS <= NB / 8 || i + tid < NB / 8) b4[i + tid] = make_uint4(0u, 0u, 0u, 0u);
   if (tid == 0) *s_most = 0u;
   if constexpr (STAGED) {
+    // asynchronous copies: nothing waits for them before the payloads leave
     for_items([&](int j) {
-      if (has(j)) s_val[j * THREADS + tid] = ld_elem<COHERENT>(vin + j * THREADS + tid);
+      if (has(j))
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(static_cast<uint32_t>(
+                         __cvta_generic_to_shared(s_val + j * THREADS + tid))),
+                     "l"(vin + j * THREADS + tid), "n"(VB)
+                     : "memory");
     });
+    asm volatile("cp.async.commit_group;" ::: "memory");
   }
   if (!ordi.identity()) for_items([&](int j) { key[j] = ordi.map(key[j]); });
   if constexpr (!Bins::kKnown) {
@@ -535,7 +557,7 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
       const uint32_t p = start_of(bin_of(j)) + __byte_perm(turn[j / 4], 0u, 0x4440u + uint32_t(j % 4));
       s_key[L::slot(has(j) ? p : uint32_t(L::SPARE + lane))] = elem(j);
     });
-    if (tid < 16) s_key[L::slot(m + tid)] = EO::last();
+    if (tid < 16) s_key[L::slot(m + tid)] = eo.last();
     __syncthreads();
   };
   auto first_bin = [&](int j) { return bins(key[j]); };
@@ -614,7 +636,7 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
           }
           if (p + 8u >= m) {  // no next window
 #pragma unroll
-            for (int i = 4; i < 8; ++i) u[i] = EO::last();
+            for (int i = 4; i < 8; ++i) u[i] = eo.last();
           }
           merge8(u);
           __syncwarp();
@@ -640,19 +662,31 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
       if (has(j)) s_key[L::slot(j * THREADS + tid)] = elem(j);
     });
     __syncthreads();
-    local_digit_passes<L, THREADS, ITEMS, K, VB != 0, PLACES>(m, smem);
+    local_digit_passes<L, THREADS, ITEMS, K, EO, PLACES>(m, eo, smem);
   }
   // 6. out
+  if constexpr (STAGED) {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+  }
+  V held[MODE == Vals::kInPlace ? ITEMS : 1];
+  if constexpr (MODE == Vals::kInPlace) {
+    for_items([&](int j) {
+      if (has(j)) held[j] = ld_elem<COHERENT>(vin + eo.place(s_key[L::slot(j * THREADS + tid)]));
+    });
+    __syncthreads();
+  }
   auto write_out = [&](auto invert) {
     for_items([&](int j) {
       if (has(j)) {
         const uint32_t p = j * THREADS + tid;
         const E e = s_key[L::slot(p)];
-        if constexpr (decltype(invert)::value) ordo.store(out + p, EO::key(e));
-        else out[p] = EO::key(e);
-        if constexpr (STAGED) vout[p] = s_val[EO::place(e)];
-        else if constexpr (PLACES) vout[p] = ld_elem(from + EO::place(e));
-        else if constexpr (VB != 0) vout[p] = vin[EO::place(e)];
+        if constexpr (decltype(invert)::value) ordo.store(out + p, eo.key(e));
+        else out[p] = eo.key(e);
+        if constexpr (STAGED) vout[p] = s_val[eo.place(e)];
+        else if constexpr (MODE == Vals::kInPlace) vout[p] = held[j];
+        else if constexpr (PLACES) vout[p] = ld_elem(from + eo.place(e));
+        else if constexpr (VB != 0) vout[p] = vin[eo.place(e)];
       }
     });
   };

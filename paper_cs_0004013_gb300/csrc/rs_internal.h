@@ -56,9 +56,9 @@ constexpr uint32_t kGateRadix = 1;
 // chained: its launch may overlap the end of the kernel in front of it on the
 // stream, which hides the launch's latency (it matters for the kernels that
 // return at once, of which a sort by value buckets has several).
-template <class Kernel, class Args>
+template <class Kernel, class... Args>
 cudaError_t launch_chained(Kernel* kernel, unsigned grid, unsigned threads, size_t smem, cudaStream_t s, bool chained,
-                           const Args& args) {
+                           const Args&... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(threads);
@@ -69,7 +69,7 @@ cudaError_t launch_chained(Kernel* kernel, unsigned grid, unsigned threads, size
   attr.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &attr;
   cfg.numAttrs = chained ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, args);
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 // Upfront histogram (one read of the keys, every digit at once) and zeroing
