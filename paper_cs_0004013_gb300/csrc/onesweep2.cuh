@@ -74,9 +74,6 @@ struct Onesweep2Layout {
 };
 
 // 32-bit shared-memory accesses by address (the hot loop's tables).
-__device__ __forceinline__ uint32_t smem_addr(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
 __device__ __forceinline__ void sh_red_add(uint32_t a, uint32_t v) {
   asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }

@@ -89,6 +89,11 @@ __device__ __forceinline__ void st_relaxed(unsigned long long* p, unsigned long 
 }
 
 // ---- L2 prefetch of a tile's payloads ---------------------------------------
+// A shared-memory address for inline PTX.
+__device__ __forceinline__ uint32_t smem_addr(const void* p) {
+  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+
 // The pass kernels load a tile's payload words only after ranking its keys;
 // asking the TMA unit at the start of the tile to bring them into L2 turns
 // that load's DRAM latency into an L2 hit.  Threads 0.. of the block each
