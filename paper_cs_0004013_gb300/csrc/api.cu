@@ -388,6 +388,29 @@ struct HybLayout {
   }
 };
 
+// When the radix passes, which leave out a digit that all keys share, are the
+// faster way for evenly spread keys too.  Measured, us, buckets against radix
+// passes over the digits given (2^23 and 2^24 keys, c equal keys per value):
+//   pairs, 3 digits: c = 2 166 / 166 and 297 / 299, c = 8 174 / 170 and 314 /
+//     294; 4 digits 162 / 215 and 292 / 390;
+//   64-bit payloads, 3 digits: c = 2 219 / 214 and 405 / 393, but 2.5M keys 90 /
+//     103 (c = 16 99 / 107); 2 digits, 1M 65 / 56, but 277,635 41 / 52;
+//   keys, 3 digits: c = 8 115 / 132 and 191 / 213, c = 16 139 / 131 and 229 / 213;
+//   64-bit keys: 5 digits 157-181 / 324-281, a digit less about 47 less; with
+//     32-bit payloads 249-274 / 426-370, a digit 63; with 64-bit ones 281-305 / 659-611.
+SampleRule hyb_rule(uint64_t n, int kb, int vb) {
+  const bool large = n > uint64_t(1) << 22;
+  if (kb == 4) return SampleRule{vb == 0 ? 1u : vb == 4 || large ? 4u : n > uint64_t(1) << 19 ? 3u : 1u, vb == 8 && !large ? 16u : 8u};
+  return SampleRule{!large || vb == 8 ? 1u : vb == 4 ? 4u : 3u, 8u};
+}
+// The same for the sorts of one launch.  Keys alone gain or lose little with
+// two digits (277,635 keys 24.5 / 26.6, 50,000 23 / 22), pairs lose: 277,635
+// 33-47 / 29 (three digits 30.6 / 37.5), 2^20 66 / 36 (three 47-49 / 47-48, four 47 / 59).
+// The largest tiles' pairs lose with any (2.5M: 92 / 86): not offered.
+SampleRule fused_rule(bool pairs, int shape) {
+  return SampleRule{!pairs ? 1u : shape == 1 ? 4u : 3u, 16u};
+}
+
 struct Layout {
   size_t ctrl = 0;     // words 0-3: tile tickets per pass; 4-7: skip flags; 12: barrier counter; 15: histogram blocks done
   size_t cursors0 = 0; // [256] u32: the first pass's bucket cursors
@@ -474,6 +497,7 @@ BucketChain make_chain(HybArgs a, const HybLayout& H, size_t clear_bytes, unsign
   a.groups = H.groups;
   a.bucket_cap = H.shape.bucket_cap;
   a.split_tile = H.shape.split_tile;
+  a.rule = hyb_rule(H.n, key_bytes, val_bytes);
   a.ctrl = reinterpret_cast<HybCtrl*>(temp + H.ctrl);
   a.counts = reinterpret_cast<uint32_t*>(temp + H.counts);
   a.starts = reinterpret_cast<uint32_t*>(temp + H.starts);
@@ -875,7 +899,8 @@ rs_status run_fused(const SortPlan& p, const Layout& L, const uint32_t* keys_in,
   // number may exceed the SMs'), when a block more than tiles, which takes the
   // sample, is resident too
   const uint32_t buckets = shape == 0 ? 2 * tiles : tiles;
-  const bool offered = L.fcounts && buckets >= 2 && buckets <= kFusedMaxBuckets && tiles < ds->fused_tiles[pairs][shape];
+  const bool offered = L.fcounts && buckets >= 2 && buckets <= kFusedMaxBuckets &&
+                       tiles < ds->fused_tiles[pairs][shape] && !(pairs && shape == 0);
   HybCtrl* hc = reinterpret_cast<HybCtrl*>(temp + L.fctrl);
   RS_CUDA(traced(T_CLEAR, 0, s, [&] { return cudaMemsetAsync(temp, 0, clear_bytes, s); }), "cudaMemsetAsync(temp)");
   FusedArgs a{};
@@ -894,6 +919,7 @@ rs_status run_fused(const SortPlan& p, const Layout& L, const uint32_t* keys_in,
   a.err = ds->err;
   if (offered) {
     a.ctrl = hc;
+    a.rule = fused_rule(pairs, shape);
     a.buckets = buckets;
     a.counts = reinterpret_cast<uint32_t*>(temp + L.fcounts);
     a.cursors = reinterpret_cast<uint32_t*>(temp + L.fcursors);

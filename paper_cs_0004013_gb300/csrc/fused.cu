@@ -91,14 +91,18 @@ __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
   return v;
 }
 
-// Arrival number `target` of the launch's monotone barrier counter.
-__device__ __forceinline__ void grid_barrier(uint32_t* bar, uint32_t target, uint32_t* err) {
+// Arrival number `target` of the launch's monotone barrier counter.  True when
+// the sampling block has chosen the value buckets: it arrives with a bit set
+// above the count, so that its answer costs no read after the barrier.
+constexpr uint32_t kBucketsBit = 1u << 24;
+__device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t target, uint32_t* err) {
+  uint32_t seen = 0;
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
     atomicAdd(bar, 1u);
     uint32_t spins = 0;
-    while (ld_acquire(bar) < target) {
+    while (((seen = ld_acquire(bar)) & (kBucketsBit - 1u)) < target) {
       if (++spins > kBarrierSpinLimit) {
         atomicOr(err, kErrTimeout);
         break;
@@ -107,14 +111,15 @@ __device__ __forceinline__ void grid_barrier(uint32_t* bar, uint32_t target, uin
     }
     __threadfence();
   }
-  __syncthreads();
+  return __syncthreads_or(seen & kBucketsBit);
 }
 
 // The value buckets' way (see above); false, with nothing written but the
 // counts and `bar` advanced by one barrier, when a bucket does not fit the
 // local sort (every block comes to the same answer).
 template <int NV, int ITEMS>
-__device__ __forceinline__ bool fused_buckets(const FusedArgs& a, unsigned char* smem, uint32_t& barriers) {
+__device__ __forceinline__ bool fused_buckets(const FusedArgs& a, uint32_t tile, unsigned char* smem,
+                                              uint32_t& barriers) {
   using FL = FusedLayout<NV, ITEMS>;
   constexpr uint32_t TILE = FL::L::TILE;
   constexpr int T = kFusedThreads, ROW = kFusedMaxBuckets + 1;
@@ -126,7 +131,7 @@ __device__ __forceinline__ bool fused_buckets(const FusedArgs& a, unsigned char*
   uint32_t* s_starts = reinterpret_cast<uint32_t*>(smem + FL::OFF_STARTS);
   const int tid = threadIdx.x, lane = tid & 31;
   const uint32_t tiles = a.tiles, B = a.buckets, n = a.n;
-  const uint32_t base = blockIdx.x * TILE;
+  const uint32_t base = tile * TILE;
   const uint32_t valid = n - base < TILE ? n - base : TILE;
   auto has = [&](int j) { return uint32_t(j * T + tid) < valid; };
   const ValueMap<uint32_t> map = load_map<uint32_t>(a.ctrl);
@@ -199,7 +204,7 @@ __device__ __forceinline__ bool fused_buckets(const FusedArgs& a, unsigned char*
   if (oob) atomicOr(a.err, kErrBounds);
   grid_barrier(a.bar, gridDim.x + tiles * barriers++, a.err);
   // 4. the buckets
-  for (uint32_t b = blockIdx.x; b < B; b += tiles) {
+  for (uint32_t b = tile; b < B; b += tiles) {
     const uint32_t s = s_starts[b], e = s_starts[b + 1];
     if (s == e) continue;
     uint32_t* vout = NV ? a.vals_out + s : nullptr;
@@ -219,17 +224,18 @@ __global__ void __launch_bounds__(kFusedThreads, fused_min_blocks(ITEMS)) fused_
   uint32_t* s_flags = reinterpret_cast<uint32_t*>(smem + FL::OFF_FLAGS);
   uint32_t* s_cnt = reinterpret_cast<uint32_t*>(smem + L::OFF_TBL);  // [4][256] while counting
   const int tid = threadIdx.x;
-  const uint32_t tile = blockIdx.x, tiles = a.tiles;
+  const uint32_t tiles = a.tiles, tile = blockIdx.x - (gridDim.x - tiles);
   const uint32_t n = a.n;
   uint32_t barriers = 0;  // barriers passed so far (the n-th of all tiles awaits gridDim.x + (n - 1) * tiles arrivals)
   constexpr bool kFreeFirst = NV == 0;  // keys alone: the first executed pass keeps no order
 
-  if (tile == tiles) {  // one block more, when value buckets are offered: it takes the sample meanwhile
-    sample_body<uint32_t, 1, kFusedThreads>(a.keys_in, n, a.buckets, Ord32{a.xf}, a.ctrl, smem, [] {});
-    __syncthreads();
+  // one block more, when value buckets are offered: it takes the sample meanwhile (the first, it starts soonest)
+  if (tile >= tiles) {
+    sample_body<uint32_t, 1, kFusedThreads>(a.keys_in, n, a.buckets, Ord32{a.xf}, a.rule, a.ctrl, smem, [] {});
     if (tid == 0) {
+      const bool buckets = a.ctrl->route == kHybBuckets;  // (written by this thread)
       __threadfence();
-      atomicAdd(a.bar, 1u);
+      atomicAdd(a.bar, buckets ? 1u + kBucketsBit : 1u);
     }
     return;
   }
@@ -240,31 +246,43 @@ __global__ void __launch_bounds__(kFusedThreads, fused_min_blocks(ITEMS)) fused_
   __syncthreads();
   {
     const uint32_t cnt = smem_addr(s_cnt);
-    const uint64_t lo = uint64_t(tile) * L::TILE;
-    const uint64_t hi = lo + L::TILE < n ? lo + L::TILE : n;
-    for (uint64_t i = lo + tid; i < hi; i += kFusedThreads) {
-      const uint32_t k = to_ordered(a.keys_in[i], a.xf);
+    const uint32_t base = tile * uint32_t(L::TILE);
+    const uint32_t valid = n - base < uint32_t(L::TILE) ? n - base : uint32_t(L::TILE);
+    uint32_t key[ITEMS];  // (every load before the first count)
 #pragma unroll
-      for (uint32_t j = 0; j < 4; ++j) sh_red_add(cnt + 4u * (256u * j + byte_digit(k, 0x4440u | j)), 1u);
+    for (int i = 0; i < ITEMS; ++i)
+      if (uint32_t(i * kFusedThreads + tid) < valid) key[i] = a.keys_in[base + i * kFusedThreads + tid];
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+      if (uint32_t(i * kFusedThreads + tid) < valid) {
+        const uint32_t k = to_ordered(key[i], a.xf);
+#pragma unroll
+        for (uint32_t j = 0; j < 4; ++j) sh_red_add(cnt + 4u * (256u * j + byte_digit(k, 0x4440u | j)), 1u);
+      }
     }
   }
   __syncthreads();
   for (int i = tid; i < 1024; i += kFusedThreads)
     if (s_cnt[i]) atomicAdd(a.hist + i, s_cnt[i]);
-  grid_barrier(a.bar, gridDim.x, a.err);  // (the sampling block passes the first barrier only)
+  const bool buckets = grid_barrier(a.bar, gridDim.x, a.err);  // (the sampling block passes the first barrier only)
   barriers = 1;
-  if (a.ctrl && __ldcg(&a.ctrl->route) == kHybBuckets && fused_buckets<NV, ITEMS>(a, smem, barriers)) return;
+  if (buckets && fused_buckets<NV, ITEMS>(a, tile, smem, barriers)) return;
 
   // 2. bases and skip flags of every digit (each block for itself)
-  if (tid < 4) s_flags[tid] = 0u;
-  __syncthreads();
-  for (int j = 0; j < 4; ++j) {
-    if (tid < 256) {
-      const uint32_t v = ld_pass<true>(a.hist + 256 * j + tid);
-      if (v == n) s_flags[j] = 1u;  // one bucket holds every key: the digit moves nothing
-      s_bases[256 * j + tid] = scan256_exclusive(v, reinterpret_cast<uint32_t*>(smem + L::OFF_SCAN));
-    }
+  {
+    uint32_t v[4];  // (all four reads before the first scan)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = tid < 256 ? ld_pass<true>(a.hist + 256 * j + tid) : 0u;
+    if (tid < 4) s_flags[tid] = 0u;
     __syncthreads();
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (tid < 256) {
+        if (v[j] == n) s_flags[j] = 1u;  // one bucket holds every key: the digit moves nothing
+        s_bases[256 * j + tid] = scan256_exclusive(v[j], reinterpret_cast<uint32_t*>(smem + L::OFF_SCAN));
+      }
+      __syncthreads();
+    }
   }
 
   // 3. the executed passes: the skipped digits are left out; if every digit

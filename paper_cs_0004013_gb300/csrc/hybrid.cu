@@ -74,9 +74,10 @@ template <typename K>
 __global__ void __cluster_dims__(kSampleBlocks, 1, 1) __launch_bounds__(kSampleThreads, 1)
     sample_kernel(const HybArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
+  launch_next();
   // the blocks other than the first clear what the launches that follow start from
   sample_body<K, kSampleBlocks, kSampleThreads>(static_cast<const K*>(a.keys_in), a.n, a.buckets, OrdOf<K>::make(a),
-                                                a.ctrl, smem, [&] {
+                                                a.rule, a.ctrl, smem, [&] {
     for (size_t i = size_t(blockIdx.x - 1) * kSampleThreads + threadIdx.x; i < a.clear_vec4;
          i += size_t(kSampleBlocks - 1) * kSampleThreads)
       a.clear[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -94,10 +95,10 @@ __global__ void __launch_bounds__(kCountThreads, 1) bucket_count_kernel(const Hy
   __shared__ uint32_t s_warp[32];
   __shared__ uint32_t s_last;
   const int tid = threadIdx.x;
+  const uint32_t B = a.buckets;
+  for (uint32_t i = tid; i < B; i += kCountThreads) sh[i] = 0u;  // while the sample is taken
   wait_for_chain();
   if (a.ctrl->route != kHybBuckets) return;
-  const uint32_t B = a.buckets;
-  for (uint32_t i = tid; i < B; i += kCountThreads) sh[i] = 0u;
   const ValueMap<K> m = load_map<K>(a.ctrl);
   const auto ord = OrdOf<K>::make(a);
   const uint32_t base = smem_addr(sh);

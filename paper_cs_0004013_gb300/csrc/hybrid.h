@@ -35,6 +35,7 @@ struct HybArgs {
   uint32_t groups;      // digits of the first split
   uint32_t bucket_cap;  // keys the local sort takes
   uint32_t split_tile;  // keys of a split tile
+  SampleRule rule;
   HybCtrl* ctrl;
   uint32_t* counts;         // [B], zero before the counts
   uint32_t* starts;         // [B + 1]

@@ -269,6 +269,31 @@ __device__ __forceinline__ uint32_t warp_rank_step(uint32_t d, uint32_t* wm, uin
   return before + __popc(peers & lt);
 }
 
+// The same of the lanes that have a key (lane 0 does); a row of one digit, as
+// few distinct keys make many, needs no table: its lanes would all meet in one word.
+__device__ __forceinline__ uint32_t warp_rank_row(uint32_t d, bool has, uint32_t* wm, uint16_t* wc, uint32_t lt,
+                                                  uint32_t gt, int lane) {
+  const uint32_t live = __ballot_sync(0xffffffffu, has), d0 = __shfl_sync(0xffffffffu, d, 0);
+  if (__all_sync(0xffffffffu, !has || d == d0)) {
+    const uint32_t before = wc[d0];
+    __syncwarp();
+    if (lane == 0) wc[d0] = uint16_t(before + __popc(live));
+    __syncwarp();
+    return before + __popc(live & lt);
+  }
+  if (has) atomicOr(&wm[d], 1u << lane);
+  __syncwarp();
+  const uint32_t peers = wm[d];
+  const uint32_t before = wc[d];
+  __syncwarp();
+  if (has && (peers & gt) == 0) {
+    wc[d] = uint16_t(before + __popc(peers));
+    wm[d] = 0u;
+  }
+  __syncwarp();
+  return before + __popc(peers & lt);
+}
+
 // Block-wide exclusive prefix sums of R ranges of words that follow each other
 // (range r's sums come after the whole of range r - 1), and the total, with
 // one barrier: every warp scans the warps' sums for itself.  s (R * 32 words)
@@ -302,7 +327,7 @@ __device__ __forceinline__ void block_exclusive_sums(const uint32_t (&x)[R], uin
 
 // The digit passes over [0, m) of s_key (see above): afterwards s_key is in
 // order.  Warp w ranks elements [w * 32 * ITEMS, ...), so that rank order is
-// the order they were in.
+// the order they were in; places past the end take no part.
 // BY_PLACE: equal keys are ordered by their places too (they are not in that
 // order to begin with).
 template <class L, int THREADS, int ITEMS, typename K, class EO, bool BY_PLACE>
@@ -318,15 +343,17 @@ __device__ __noinline__ void local_digit_passes(uint32_t m, const EO eo, unsigne
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t lt = lanemask_lt(), gt = lanemask_gt();
   const uint32_t wofs = uint32_t(warp) * 32 * ITEMS + lane;
+  auto row = [&](int j) { return uint32_t(warp * 32 * ITEMS + j * 32) < m; };  // the warp's row has keys
+  auto has = [&](int j) { return wofs + j * 32 < m; };
   E e[ITEMS];
   K diff = 0;
   uint32_t pdiff = 0;
   const K k0 = eo.key(s_key[L::slot(0)]);
   const uint32_t p0 = eo.place(s_key[L::slot(0)]);
 #pragma unroll
-  for (int j = 0; j < ITEMS; ++j) {  // places past the end act as the largest key and stay behind
-    e[j] = wofs + j * 32 < m ? s_key[L::slot(wofs + j * 32)] : eo.last();
-    if (wofs + j * 32 < m) {
+  for (int j = 0; j < ITEMS; ++j) {
+    if (has(j)) {
+      e[j] = s_key[L::slot(wofs + j * 32)];
       diff |= eo.key(e[j]) ^ k0;
       pdiff |= eo.place(e[j]) ^ p0;
     }
@@ -346,7 +373,8 @@ __device__ __noinline__ void local_digit_passes(uint32_t m, const EO eo, unsigne
     pdiff = __reduce_or_sync(0xffffffffu, s_warp[lane < WARPS ? lane : 0]);
   }
   // digits 0-3 are the places' (BY_PLACE), the others the keys'
-  auto digit = [&](const E& x, uint32_t d) {
+  auto digit = [&](int j, uint32_t d) {
+    const E& x = e[j];
     return d < 4 ? (eo.place(x) >> (8 * d)) & 0xffu : uint32_t(eo.key(x) >> (8 * (d - 4))) & 0xffu;
   };
   for (uint32_t d = BY_PLACE ? 0 : 4; d < 4 + sizeof(K); ++d) {
@@ -357,8 +385,8 @@ __device__ __noinline__ void local_digit_passes(uint32_t m, const EO eo, unsigne
     uint32_t rk[(ITEMS + 1) / 2];
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) {
-      const uint32_t r = warp_rank_step(digit(e[j], d), s_mask + warp * kMaskSlots,
-                                        s_cnt + warp * 256, lt, gt, lane);
+      const uint32_t r =
+          row(j) ? warp_rank_row(digit(j, d), has(j), s_mask + warp * kMaskSlots, s_cnt + warp * 256, lt, gt, lane) : 0u;
       if (j & 1) rk[j >> 1] |= r << 16;
       else rk[j >> 1] = r;
     }
@@ -380,11 +408,12 @@ __device__ __noinline__ void local_digit_passes(uint32_t m, const EO eo, unsigne
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j)
-      s_key[L::slot(((rk[j >> 1] >> (16 * (j & 1))) & 0xffffu) +
-                    s_cnt[warp * 256 + digit(e[j], d)])] = e[j];
+      if (has(j))
+        s_key[L::slot(((rk[j >> 1] >> (16 * (j & 1))) & 0xffffu) + s_cnt[warp * 256 + digit(j, d)])] = e[j];
     __syncthreads();
 #pragma unroll
-    for (int j = 0; j < ITEMS; ++j) e[j] = s_key[L::slot(wofs + j * 32)];
+    for (int j = 0; j < ITEMS; ++j)
+      if (has(j)) e[j] = s_key[L::slot(wofs + j * 32)];
   }
   __syncthreads();
 }
@@ -435,9 +464,12 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
   // 1. load; clear the bins
   K key[ITEMS];
   for_items([&](int j) { key[j] = has(j) ? ld_elem<COHERENT>(in + j * THREADS + tid) : K(0); });
-  uint32_t place[PLACES ? ITEMS : 1];
+  [[maybe_unused]] uint32_t place[PLACES ? ITEMS : 1];
   if constexpr (PLACES) for_items([&](int j) { place[j] = has(j) ? ld_elem<COHERENT>(vin + j * THREADS + tid) : 0u; });
-  auto elem = [&](int j) { return eo.make(key[j], PLACES ? place[PLACES ? j : 0] : uint32_t(j * THREADS + tid)); };
+  auto elem = [&](int j) {
+    if constexpr (PLACES) return eo.make(key[j], place[j]);
+    else return eo.make(key[j], uint32_t(j * THREADS + tid));
+  };
   uint4* b4 = reinterpret_cast<uint4*>(smem);
 #pragma unroll
   for (int i = 0; i < NB / 8; i += THREADS)
@@ -569,7 +601,19 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
     scan();
     stage(first_bin);
   } else if constexpr (!Bins::kKnown) {
-    if (!bins.unique()) {
+    // Few distinct keys: D of them leave a lane without its like in the warp with
+    // a chance of (1 - 1 / D)^31, and with m / D above kBinLimit other bins are
+    // as crowded, so the digit passes sort them at once (16,000 keys of 8 values
+    // 40 us with the second bins tried first, 35 without).
+    const uint32_t live = __ballot_sync(0xffffffffu, has(0));
+    const uint32_t same = __match_any_sync(0xffffffffu, key[0]) & live;  // (every lane takes part)
+    const uint32_t likes = __popc(__ballot_sync(0xffffffffu, has(0) && (same & (same - 1u)) != 0u));
+    if (lane == 0) s_scan[warp] = likes;
+    __syncthreads();
+    const uint32_t sum = __reduce_add_sync(0xffffffffu, lane < WARPS ? s_scan[lane] : 0u);
+    __syncthreads();
+    const bool repeats = sum * m > 31u * kBinLimit * (m < uint32_t(THREADS) ? m : uint32_t(THREADS));
+    if (!repeats && !bins.unique()) {
       // crowded: the second set of bins (see above), NB / m of them to a key;
       // positions among the keys in 16.16 fixed point
       scan();

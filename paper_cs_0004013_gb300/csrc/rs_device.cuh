@@ -63,6 +63,9 @@ __device__ __forceinline__ uint32_t digit_of(uint32_t key, uint32_t shift, uint3
 // be launched at this one's start instead of its end was slower: 2^26 keys 581
 // us against 561, its blocks take room from the tail of this kernel's.)
 __device__ __forceinline__ void wait_for_chain() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The next kernel of the chain may be launched from here on: for kernels that
+// leave room beside them.
+__device__ __forceinline__ void launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Whether a kernel launched beside another way to sort is to return at once.
 __device__ __forceinline__ bool gated_off(const uint32_t* gate) {

@@ -316,6 +316,12 @@ cudaError_t launch_merge(const MergeArgs& m, cudaStream_t s);
 cudaError_t launch_split64(const WideArgs& a, unsigned grid, cudaStream_t s);
 cudaError_t launch_join64(const WideArgs& a, unsigned grid, cudaStream_t s);
 
+// What the sample of a sort asks of its keys beyond an even spread (sample.cuh).
+struct SampleRule {
+  uint32_t min_digits;   // bytes in which the keys differ, at least: fewer radix passes are faster
+  uint32_t narrow_dups;  // equal keys per value, at most, of keys that differ in three bytes or less (otherwise 16)
+};
+
 // A whole sort of up to a few million keys in one cooperative launch
 // (fused.cu): 8-bit digits, one 384 x 24, 384 x 18 or 384 x 12 tile per block, every block resident.
 struct FusedArgs {
@@ -335,12 +341,13 @@ struct FusedArgs {
   uint32_t tiles;            // set by the launch
   // value buckets, when offered (null: not): the sample's control block
   HybCtrl* ctrl;
+  SampleRule rule;
   uint32_t buckets;
   uint32_t* counts;          // [buckets], zero on entry
   uint32_t* cursors;         // [buckets], zero on entry
 };
 constexpr uint32_t kFusedMaxBuckets = 768;  // value buckets of the launch
-constexpr int kFusedShapes = 3;  // tile shapes of the single-launch sort: 384 x 24, 384 x 18, 384 x 12
+constexpr int kFusedShapes = 3;  // tile shapes of the single-launch sort: 384 x 24, 384 x 20, 384 x 12
 uint32_t fused_tile_keys(int shape);
 size_t fused_smem(bool pairs, int shape);
 const void* fused_func(bool pairs, int shape);

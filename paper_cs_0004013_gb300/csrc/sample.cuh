@@ -24,7 +24,9 @@ namespace rs {
 //    the sample (uniform keys: 128 expected, five standard deviations below);
 //  - no bucket holds more than 1.5 times its share of the sample and kFineLimit keys;
 //  - few sampled keys are equal to another one: many equal keys end up in few
-//    bins of a bucket, which then takes the digit passes.
+//    bins of a bucket, which then takes the digit passes;
+//  - the keys differ in enough bytes: the radix passes leave out the others
+//    (hyb_rule in api.cu).
 // In the sorts of one launch (fused.cu) a block of its own takes a quarter of
 // the sample; their buckets are few and large.
 constexpr uint32_t kFineLimit = 12;
@@ -41,21 +43,20 @@ struct SampleLayout {
   static constexpr size_t FINE_BYTES = size_t(MAXB) * 4 > SLOT_BYTES ? size_t(MAXB) * 4 : SLOT_BYTES;
   static constexpr size_t OFF_KEYS = FINE_BYTES;
   static constexpr size_t OFF_RED = OFF_KEYS + size_t(S) * sizeof(K);
-  static constexpr size_t OFF_COARSE = OFF_RED + 64 * 8;
-  static constexpr size_t SMEM = OFF_COARSE + COARSE * 4;
+  static constexpr size_t SMEM = OFF_RED + 64 * 8;
 };
 
 // The sample of in[0, n) for `buckets` value buckets, to *ctrl.  The blocks
 // other than the first call others() and leave after their reads.
 template <typename K, int BLOCKS, int THREADS, class Ord, class Others>
-__device__ __forceinline__ void sample_body(const K* in, uint64_t n, uint32_t buckets, const Ord& ord, HybCtrl* ctrl,
-                                            unsigned char* smem, Others&& others) {
+__device__ __forceinline__ void sample_body(const K* in, uint64_t n, uint32_t buckets, const Ord& ord,
+                                            const SampleRule& rule, HybCtrl* ctrl, unsigned char* smem,
+                                            Others&& others) {
   using L = SampleLayout<K, BLOCKS, THREADS>;
   namespace cg = cooperative_groups;
   uint32_t* s_fine = reinterpret_cast<uint32_t*>(smem);
   K* s_keys = reinterpret_cast<K*>(smem + L::OFF_KEYS);
   K* s_red = reinterpret_cast<K*>(smem + L::OFF_RED);
-  uint32_t* s_coarse = reinterpret_cast<uint32_t*>(smem + L::OFF_COARSE);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t block = BLOCKS > 1 ? blockIdx.x : 0u;
   const uint32_t stretch = uint32_t(n / L::S);
@@ -71,7 +72,6 @@ __device__ __forceinline__ void sample_body(const K* in, uint64_t n, uint32_t bu
   if (block == 0) {
     uint4* f4 = reinterpret_cast<uint4*>(smem);
     for (uint32_t i = tid; i < (buckets + 3) / 4; i += THREADS) f4[i] = make_uint4(0u, 0u, 0u, 0u);
-    if (tid < int(L::COARSE)) s_coarse[tid] = 0u;
   }
   K key[L::PER];
   if constexpr (BLOCKS > 1) {
@@ -121,16 +121,24 @@ __device__ __forceinline__ void sample_body(const K* in, uint64_t n, uint32_t bu
   m.mult = uint32_t((uint64_t(buckets) << 32) / (range > buckets ? range : uint64_t(buckets) + 1));
   m.back = 0ull - uint64_t(m.lo) * m.mult;
   bool bad = range <= buckets;
+  K diff = 0;
   const uint32_t fine_limit = kFineLimit + uint32_t(L::S) * 3 / (2 * buckets);
 #pragma unroll
   for (int i = 0; i < L::PER; ++i) {
+    diff |= key[i] ^ lo;
     const uint32_t b = m.bucket(key[i]);
     if (atomicAdd(&s_fine[b], 1u) >= fine_limit) bad = true;
-    atomicAdd(&s_coarse[(b * L::COARSE) / buckets], 1u);
   }
   __syncthreads();
-  if (buckets >= 4 * L::COARSE && tid < int(L::COARSE) && s_coarse[tid] * L::COARSE * 2 > uint32_t(L::S) * 3)
-    bad = true;
+  if (buckets >= 4 * L::COARSE) {  // a warp per slice
+    for (uint32_t c = warp; c < L::COARSE; c += L::WARPS) {
+      const uint32_t from = (c * buckets + L::COARSE - 1) / L::COARSE, to = ((c + 1) * buckets + L::COARSE - 1) / L::COARSE;
+      uint32_t sum = 0;
+      for (uint32_t b = from + lane; b < to; b += 32) sum += s_fine[b];
+      if (__reduce_add_sync(0xffffffffu, sum) * L::COARSE * 2 > uint32_t(L::S) * 3) bad = true;
+    }
+  }
+  __syncthreads();  // (the hash slots take the counts' place)
   // equal keys: each writes its number to a hash slot, and reads back whose
   // number stayed; an equal key's means a duplicate
   uint16_t* s_slot = reinterpret_cast<uint16_t*>(smem);
@@ -146,12 +154,25 @@ __device__ __forceinline__ void sample_body(const K* in, uint64_t n, uint32_t bu
   }
   dups = __reduce_add_sync(0xffffffffu, dups);
   uint32_t* s_sum = reinterpret_cast<uint32_t*>(s_red);
-  if (lane == 0) s_sum[warp] = dups;
+  const uint32_t diff_lo = __reduce_or_sync(0xffffffffu, uint32_t(diff));
+  const uint32_t diff_hi = sizeof(K) == 8 ? __reduce_or_sync(0xffffffffu, uint32_t(uint64_t(diff) >> 32)) : 0u;
+  if (lane == 0) {
+    s_sum[warp] = dups;
+    s_sum[32 + warp] = diff_lo;
+    s_sum[64 + warp] = diff_hi;
+  }
   bad = __syncthreads_or(bad);
-  dups = __reduce_add_sync(0xffffffffu, lane < L::WARPS ? s_sum[lane] : 0u);
+  const int w = lane < L::WARPS ? lane : 0;
+  dups = __reduce_add_sync(0xffffffffu, lane < L::WARPS ? s_sum[w] : 0u);
+  const uint32_t words[2] = {__reduce_or_sync(0xffffffffu, s_sum[32 + w]), __reduce_or_sync(0xffffffffu, s_sum[64 + w])};
+  uint32_t digits = 0;
+#pragma unroll
+  for (int i = 0; i < int(sizeof(K)); ++i) digits += ((words[i / 4] >> (8 * (i % 4))) & 0xffu) != 0u;
+  if (digits < rule.min_digits) bad = true;
   // equal keys per value of about c among n keys give S^2 c / (2 n) such
   // pairs in the sample; c = 16 is what the bins still take well
-  if (uint64_t(dups) * n > uint64_t(L::S) * L::S * 8 + 16 * n) bad = true;
+  const uint32_t c = digits <= 3 ? rule.narrow_dups : 16u;
+  if (uint64_t(dups) * n > uint64_t(L::S) * L::S * c / 2 + 8 * n) bad = true;
   if (tid == 0) {
     HybCtrl* c = ctrl;
     c->lo = m.lo;
