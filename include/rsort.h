@@ -95,7 +95,11 @@ typedef struct rs_plan {
 
 /* Sort n keys ascending into keys_out and write the num_parts + 1 partition
  * offsets (Sec. 1.1, footnote 7) to the HOST array h_part_offsets (may be
- * NULL if not wanted).  num_parts >= 1.  plan may be NULL (automatic).      */
+ * NULL if not wanted).  num_parts >= 1.  plan may be NULL (automatic): up to
+ * 16,384 keys are sorted by one block, up to 2.8 M in one launch, more by
+ * value buckets where a sample taken on the device finds the keys spread
+ * evenly over their value range, else by the radix passes.  Either way the
+ * result is the same.                                                       */
 rs_status rs_sort_u32(const uint32_t* keys_in, uint32_t* keys_out, uint64_t n,
                       uint32_t num_parts, uint64_t* h_part_offsets,
                       const rs_plan* plan, void* temp, size_t* temp_bytes,
@@ -183,7 +187,9 @@ rs_status rs_sort_u32_pairs64(const uint32_t* keys_in, const uint64_t* vals_in,
  * key for digits 0-3 and the high word for digits 4-7.  plan: digit_bits must be 0
  * or 8, mode LSD (or 0), tile selects the key+payload tile shape, and
  * key_kind orders the 64-bit words as unsigned (RS_KEY_U32), two's-complement
- * signed (RS_KEY_I32) or IEEE-754 binary64 totalOrder (RS_KEY_F32).  Temp:
+ * signed (RS_KEY_I32) or IEEE-754 binary64 totalOrder (RS_KEY_F32).  With the
+ * automatic plan up to 8,192 keys are sorted by one block, and more by value
+ * buckets where a sample finds them spread evenly (as rs_sort_u32).  Temp:
  * four n-word planes (six with the tile shapes other than 1 and 3, which
  * split the keys into planes first) plus histograms and status.  The
  * default tile is 3 above 2^22 keys (below 2^30 - 2^16), else 1.           */

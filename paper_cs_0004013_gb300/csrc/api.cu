@@ -1002,7 +1002,8 @@ rs_status sort_impl(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* 
   }
   // Up to a few million keys: every tile resident at once, the whole sort in
   // one launch (8-bit digits, the same passes).  The tile shape: the smallest
-  // whose tiles still number at most one per SM, else the largest.
+  // whose tiles number fewer than the SMs (one is left to the sampling block),
+  // else the largest.
   if (fusable) {
     int sh = 0;
     for (int c = kFusedShapes - 1; c > 0; --c)

@@ -24,6 +24,13 @@ struct OrdFor<uint64_t> {
 
 // A block per listed segment (list != null; the grid holds a block for every
 // segment that may be listed), or the one array [0, single_n).
+// One array is one block's chain of steps, bound by its latency: bins and sorting
+// networks instead of four digit passes, traced (about 4 us of it the events),
+// us: 1,000 keys 15.7 -> 7.5, 4,000 16.4 -> 8.0, 8,000 27.2 -> 11.1, 16,000 35.5 ->
+// 14.7, with payloads 44.8 -> 24.8; 8,000 64-bit keys, which eight launches of
+// passes sorted, 123 -> 15, with 64-bit payloads 141 -> 23.  Few distinct values
+// still end in the digit passes: 8,000 keys of 8 values 23.8 -> 29.2 (the pass
+// over the bins that found them crowded comes on top).
 template <int THREADS, int ITEMS, int NBITS, int MINB, typename K, int VB>
 __global__ void __launch_bounds__(THREADS, MINB) local_sort_kernel(const LocalArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];

@@ -23,8 +23,8 @@
 //     spans at most ceil((c + 3) / 4) such runs, is in order after that many
 //     rounds (two for c <= 5);
 //  6. out, coalesced.
-// Where (unless the caller's map is known to be even) a bin holds more than kBinLimit keys, the bins are laid again where
-// the keys are: each bin's share of a second set of bins is its share of the
+// Where (unless the caller's map is known to be even) a bin holds more than
+// kBinLimit keys, the bins are laid again where the keys are: each bin's share of a second set of bins is its share of the
 // keys (its start and count give them), and a key takes the part of that
 // share that its place inside the bin points to.  This flattens any density
 // that does not change much within a bin (normally distributed floats, wide
@@ -36,7 +36,7 @@
 // The work is about 55 instructions and 18 shared-memory wavefronts per 32
 // keys whatever the key width, against about 40 wavefronts per 8-bit digit
 // of the digit passes; what it measured stands at the kernels that use it
-// (local_sort_kernel in segmented.cu, bucket_sort_kernel in hybrid.cu).
+// (local_sort_kernel in local.cu, bucket_sort_kernel in hybrid.cu).
 #pragma once
 
 #include "elem.cuh"

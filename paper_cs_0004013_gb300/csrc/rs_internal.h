@@ -293,8 +293,6 @@ cudaError_t prepare_local();
 uint32_t local_max_keys(int key_bytes, int val_bytes);
 cudaError_t launch_local_sort(const LocalArgs& a, bool small, bool pairs, unsigned grid, cudaStream_t s);
 cudaError_t launch_local_array(const LocalArgs& a, int key_bytes, int val_bytes, cudaStream_t s);
-cudaError_t launch_bases_to_offsets(const uint32_t* bases, uint32_t num, uint64_t n, uint64_t* seg_off,
-                                    cudaStream_t s);
 
 // Stable merge of two sorted runs (merge.cu).
 struct MergeArgs {
@@ -323,7 +321,7 @@ struct SampleRule {
 };
 
 // A whole sort of up to a few million keys in one cooperative launch
-// (fused.cu): 8-bit digits, one 384 x 24, 384 x 18 or 384 x 12 tile per block, every block resident.
+// (fused.cu): 8-bit digits, one 384 x 24, 384 x 20 or 384 x 12 tile per block, every block resident.
 struct FusedArgs {
   const uint32_t* keys_in;
   uint32_t* keys_out;

@@ -224,14 +224,6 @@ __global__ void __launch_bounds__(THREADS, MINB) seg_pass_kernel(const SegPassAr
   }
 }
 
-// Bucket offsets of an MSD plan: the exclusive scan of the top digit as
-// segment offsets (uint64), the last one being n.
-__global__ void bases_to_offsets_kernel(const uint32_t* bases, uint32_t num, uint64_t n, uint64_t* seg_off) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < num) seg_off[i] = bases[i];
-  if (i == num) seg_off[i] = n;
-}
-
 template <int THREADS, int ITEMS, bool PAIRS, int MINB>
 cudaError_t launch_seg_pass(const SegPassArgs& a, unsigned grid, cudaStream_t s) {
   using L = OnesweepLayout<8, THREADS, ITEMS, PAIRS>;
@@ -306,11 +298,6 @@ cudaError_t launch_seg_pass(const SegPassArgs& a, bool pairs, int shape, unsigne
                  : launch_seg_pass<kSegThreads, kSegItemsSmall, false, 2>(a, grid, s);
   return pairs ? launch_seg_pass<kSegThreads, kSegItemsPairs, true, 2>(a, grid, s)
                : launch_seg_pass<kSegThreads, kSegItemsKeys, false, 2>(a, grid, s);
-}
-cudaError_t launch_bases_to_offsets(const uint32_t* bases, uint32_t num, uint64_t n, uint64_t* seg_off,
-                                    cudaStream_t s) {
-  bases_to_offsets_kernel<<<(num + 256) / 256, 256, 0, s>>>(bases, num, n, seg_off);
-  return cudaGetLastError();
 }
 
 }  // namespace rs
