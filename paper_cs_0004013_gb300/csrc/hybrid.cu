@@ -85,7 +85,7 @@ __global__ void __cluster_dims__(kSampleBlocks, 1, 1) __launch_bounds__(kSampleT
 }
 
 // ------------------------------------------------------------------ counts
-// Keys per bucket.  32-bit shared counters for every bucket (up to 128 KiB),
+// Keys per bucket.  32-bit shared counters for every bucket (up to 192 KiB),
 // one shared reduction per key; the blocks add them into the global counts.
 // The last block to finish scans the counts: the buckets' starts and cursors,
 // the tiles of the second split, and whether every bucket fits the local sort.

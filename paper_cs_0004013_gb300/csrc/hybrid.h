@@ -5,7 +5,8 @@
 
 namespace rs {
 
-constexpr uint32_t kHybMaxBuckets = 32768;  // 32-bit shared counters of all of them: 128 KiB
+// 32-bit shared counters of all of them are 192 KiB; the two digits of a split allow 65,536.
+constexpr uint32_t kHybMaxBuckets = 49152;
 
 // Which way the sort goes, decided on the device (HybCtrl::route).
 enum : uint32_t { kHybRadix = 1, kHybBuckets = 2 };

@@ -40,7 +40,8 @@ struct SampleLayout {
   static constexpr int SLOT_BITS = BLOCKS > 1 ? 15 : 13;               // hash slots, in the fine counts' place
   static constexpr size_t SLOT_BYTES = (size_t(1) << SLOT_BITS) * 2;
   static constexpr int WARPS = THREADS / 32;
-  static constexpr size_t FINE_BYTES = size_t(MAXB) * 4 > SLOT_BYTES ? size_t(MAXB) * 4 : SLOT_BYTES;
+  static constexpr size_t FINE_BYTES = size_t(MAXB) * 2 > SLOT_BYTES ? size_t(MAXB) * 2 : SLOT_BYTES;  // 16-bit counts
+  static_assert(S < 65536 && FINE_BYTES % 16 == 0, "16-bit counts, cleared in 16-byte units");
   static constexpr size_t OFF_KEYS = FINE_BYTES;
   static constexpr size_t OFF_RED = OFF_KEYS + size_t(S) * sizeof(K);
   static constexpr size_t SMEM = OFF_RED + 64 * 8;
@@ -71,7 +72,7 @@ __device__ __forceinline__ void sample_body(const K* in, uint64_t n, uint32_t bu
   }
   if (block == 0) {
     uint4* f4 = reinterpret_cast<uint4*>(smem);
-    for (uint32_t i = tid; i < (buckets + 3) / 4; i += THREADS) f4[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (uint32_t i = tid; i < (buckets + 7) / 8; i += THREADS) f4[i] = make_uint4(0u, 0u, 0u, 0u);
   }
   K key[L::PER];
   if constexpr (BLOCKS > 1) {
@@ -127,14 +128,15 @@ __device__ __forceinline__ void sample_body(const K* in, uint64_t n, uint32_t bu
   for (int i = 0; i < L::PER; ++i) {
     diff |= key[i] ^ lo;
     const uint32_t b = m.bucket(key[i]);
-    if (atomicAdd(&s_fine[b], 1u) >= fine_limit) bad = true;
+    const uint32_t at = 16u * (b & 1u);  // two counts to a word
+    if (((atomicAdd(&s_fine[b >> 1], 1u << at) >> at) & 0xffffu) >= fine_limit) bad = true;
   }
   __syncthreads();
   if (buckets >= 4 * L::COARSE) {  // a warp per slice
     for (uint32_t c = warp; c < L::COARSE; c += L::WARPS) {
       const uint32_t from = (c * buckets + L::COARSE - 1) / L::COARSE, to = ((c + 1) * buckets + L::COARSE - 1) / L::COARSE;
       uint32_t sum = 0;
-      for (uint32_t b = from + lane; b < to; b += 32) sum += s_fine[b];
+      for (uint32_t b = from + lane; b < to; b += 32) sum += reinterpret_cast<const uint16_t*>(s_fine)[b];
       if (__reduce_add_sync(0xffffffffu, sum) * L::COARSE * 2 > uint32_t(L::S) * 3) bad = true;
     }
   }
