@@ -235,7 +235,8 @@ struct SortPlan {
   DigitSpec dig[kMaxDigits] = {};
   const OnesweepKernel* k = nullptr;
   size_t num_tiles = 0;
-  size_t status_rows = 0;  // status rows to hold when more than num_tiles (the single-launch sort's small tiles)
+  size_t status_rows = 0;  // status rows to clear when more than num_tiles (the single-launch sort's small tiles)
+  size_t held_rows = 0;    // status rows to have space for when more than those (smaller sorts' small tiles)
 };
 
 // Defaults from measurement on GB300 (uniform 31-bit keys, 2^16 .. 2^26):
@@ -347,10 +348,14 @@ struct HybLayout {
   uint32_t buckets = 0, low_bits = 0, groups = 0;  // buckets == 0: not offered
   size_t ctrl = 0, counts = 0, starts = 0, cursors = 0, group_cursors = 0, group_tiles = 0, status = 0;
   size_t status_bytes = 0;
-  // Whether n keys are offered the buckets: their mean may reach three quarters
-  // of what a bucket takes.
-  static bool offers(uint64_t n, int kb, int vb) {
-    return n >= kHybridMinKeys && n <= uint64_t(kHybMaxBuckets) * hyb_shape(kb, vb).bucket_cap * 3 / 4;
+  // The most keys that are offered the buckets: their mean may reach three
+  // quarters of what a bucket takes.
+  static uint64_t most(int kb, int vb) { return uint64_t(kHybMaxBuckets) * hyb_shape(kb, vb).bucket_cap * 3 / 4; }
+  static bool offers(uint64_t n, int kb, int vb) { return n >= kHybridMinKeys && n <= most(kb, vb); }
+  // The space of that many, which larger sorts hold too: a workspace for more keys takes fewer.
+  static size_t most_bytes(int kb, int vb) {
+    HybLayout h;
+    return h.place_rest(h.place_counts(0, most(kb, vb), kb, vb));
   }
   // the counts (and two tickets) belong to what a sort clears first; returns the next offset
   size_t place_counts(size_t off, uint64_t n_, int kb, int vb) {
@@ -381,8 +386,10 @@ struct HybLayout {
     }
     if (pairs) {
       status = off;
-      status_bytes = (2 * size_t((n + shape.split_tile - 1) / shape.split_tile) + groups) * 1024;
-      off = align_up(off + status_bytes);
+      const size_t rows = 2 * size_t((n + shape.split_tile - 1) / shape.split_tile);
+      status_bytes = (rows + groups) * 1024;
+      // (the groups fall where the second split takes a bit more: as many rows as fewer buckets may have groups)
+      off = align_up(off + (rows + (buckets < 256 ? buckets : 256)) * 1024);
     }
     return off;
   }
@@ -425,7 +432,9 @@ struct Layout {
   size_t total = 0;
 };
 
-// hybrid_vb: payload bytes of a sort offered value buckets (-1: it is not).
+// hybrid_vb: payload bytes of a sort whose sizes offers() are offered value
+// buckets (-1: it is not).  fused: with the space of the single-launch sort.
+// No part gets smaller as n grows, so that a workspace for more keys takes fewer.
 Layout make_layout(const SortPlan& p, uint64_t n, bool pairs, int hybrid_vb = -1, bool fused = false) {
   Layout L;
   const size_t digits = size_t(1) << p.R;
@@ -434,7 +443,8 @@ Layout make_layout(const SortPlan& p, uint64_t n, bool pairs, int hybrid_vb = -1
   off += kAlign;
   L.hist = off;
   off = align_up(off + size_t(p.nd) * digits * 4);
-  if (hybrid_vb >= 0) off = L.hyb.place_counts(off, n, 4, hybrid_vb);
+  const bool hybrid = hybrid_vb >= 0 && HybLayout::offers(n, 4, hybrid_vb);
+  if (hybrid) off = L.hyb.place_counts(off, n, 4, hybrid_vb);
   L.memset_bytes = off;
   L.bases = off;
   off = align_up(off + size_t(p.nd) * digits * 4);
@@ -447,9 +457,11 @@ Layout make_layout(const SortPlan& p, uint64_t n, bool pairs, int hybrid_vb = -1
     }
   }
   L.status = off;
-  L.status_bytes = (p.status_rows > p.num_tiles ? p.status_rows : p.num_tiles) * digits * (p.k->wide_status ? 8 : 4);
-  off = align_up(off + L.status_bytes);
-  off = L.hyb.place_rest(off);
+  const size_t row_bytes = digits * (p.k->wide_status ? 8 : 4);
+  L.status_bytes = std::max(p.status_rows, p.num_tiles) * row_bytes;
+  off = align_up(off + std::max(L.status_bytes, p.held_rows * row_bytes));
+  if (hybrid) off = L.hyb.place_rest(off);
+  else if (hybrid_vb >= 0 && n >= kHybridMinKeys) off += HybLayout::most_bytes(4, hybrid_vb);
   if (fused) {
     L.fctrl = off;
     off += align_up(sizeof(HybCtrl));
@@ -942,10 +954,14 @@ rs_status sort_impl(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* 
   if (st != RS_OK) return st;
   const bool automatic = plan->digit_bits == 0 && plan->mode == RS_MODE_AUTO && plan->tile == 0;
   const bool fusable = automatic && p.R == 8 && p.nd == 4 && !p.msd && !p.k->wide_status;
-  if (fusable && n <= kFusedStatusMaxKeys)  // status rows for the single-launch sort's smallest tiles
-    p.status_rows = size_t((n + fused_tile_keys(kFusedShapes - 1) - 1) / fused_tile_keys(kFusedShapes - 1));
-  const bool hybrid = fusable && HybLayout::offers(n, 4, pairs ? 4 : 0);
-  Layout L = make_layout(p, n, pairs, hybrid ? (pairs ? 4 : 0) : -1, p.status_rows > 0);
+  const bool spaced = automatic && p.R == 8 && !p.msd;  // with the other routes' space, whatever n
+  if (spaced) {  // status rows for the single-launch sort's smallest tiles
+    const uint32_t tile = fused_tile_keys(kFusedShapes - 1);
+    p.held_rows = size_t((std::min(n, kFusedStatusMaxKeys) + tile - 1) / tile);
+    if (n <= kFusedStatusMaxKeys) p.status_rows = p.held_rows;
+  }
+  Layout L = make_layout(p, n, pairs, spaced ? (pairs ? 4 : 0) : -1, spaced);
+  const bool hybrid = fusable && L.hyb.buckets;
   MsdLayout M;
   if (p.msd) {
     if (rs_status st2 = make_msd_layout(p, n, pairs, &M); st2 != RS_OK) return st2;
@@ -1043,7 +1059,9 @@ struct Layout64 {
   size_t memset_bytes = 0, total = 0;
 };
 
-Layout64 make_layout64(const SortPlan& p, uint64_t n, bool pairs, bool vals64, bool hybrid) {
+// As make_layout, no part gets smaller as n grows.
+Layout64 make_layout64(const SortPlan& p, uint64_t n, int vbytes) {
+  const bool pairs = vbytes != 0, vals64 = vbytes == 8, hybrid = HybLayout::offers(n, 8, vbytes);
   Layout64 L;
   L.fused = pair_io_kernel(p.k) != nullptr;
   size_t off = 0;
@@ -1051,14 +1069,15 @@ Layout64 make_layout64(const SortPlan& p, uint64_t n, bool pairs, bool vals64, b
   off += kAlign;
   L.hist = off;
   off = align_up(off + 8 * 256 * 4);
-  if (hybrid) off = L.hyb.place_counts(off, n, 8, vals64 ? 8 : pairs ? 4 : 0);
+  if (hybrid) off = L.hyb.place_counts(off, n, 8, vbytes);
   L.memset_bytes = off;
   L.bases = off;
   off = align_up(off + 8 * 256 * 4);
-  off = L.hyb.place_rest(off);
+  if (hybrid) off = L.hyb.place_rest(off);
+  else if (n >= kHybridMinKeys) off += HybLayout::most_bytes(8, vbytes);
   L.status = off;
   L.status_bytes = p.num_tiles * 256 * (p.k->wide_status ? 8 : 4);
-  off = align_up(off + L.status_bytes);
+  off = align_up(off + std::max(L.status_bytes, p.held_rows * 1024));
   for (int i = 0; i < (L.fused ? 4 : 6); ++i) {
     L.plane[i] = off;
     off = align_up(off + size_t(n) * 4);
@@ -1272,12 +1291,15 @@ static rs_status sort64_impl(const uint64_t* keys_in, const void* vals_in, uint6
   // SM) for keys alone above 2^22 keys (GB300, 2^26 keys: 335 us per pass
   // against 349 at 512 x 24; 2^23: 20.0 against 18.7 Gkeys/s), else 512 x 16
   // (the one with 64-bit status words and two payload words)
-  if (q.tile == 0) q.tile = (vbytes == 0 && n > (uint64_t(1) << 22) && !needs_wide_status(n)) ? 8u : 1u;
+  constexpr uint64_t kSmallTileMax = uint64_t(1) << 22;
+  const bool own_tile = q.tile != 0;
+  if (!own_tile) q.tile = (vbytes == 0 && n > kSmallTileMax && !needs_wide_status(n)) ? 8u : 1u;
   SortPlan p;
   if (rs_status st = make_plan(n, true, &q, &p, pairs ? 2 : 1); st != RS_OK) return st;
   const bool automatic = !plan || (plan->digit_bits == 0 && plan->mode == RS_MODE_AUTO && plan->tile == 0);
+  if (!own_tile && n > kSmallTileMax) p.held_rows = size_t(kSmallTileMax / (512 * 16));  // tile 1 takes more rows than 8
   // (the space for value buckets is part of every plan's layout)
-  Layout64 L = make_layout64(p, n, pairs, vbytes == 8, HybLayout::offers(n, 8, vbytes));
+  Layout64 L = make_layout64(p, n, vbytes);
   if (!automatic) L.hyb.buckets = 0;
   if (vbytes == 8 && !L.fused)
     return fail(RS_ERR_UNSUPPORTED, "64-bit values: tile shape %u has no interleaved pass kernel", q.tile);
@@ -1372,8 +1394,8 @@ rs_status rs_sort_u32_pairs64(const uint32_t* keys_in, const uint64_t* vals_in, 
   // A tiled pass kernel reads and writes the interleaved values itself
   // (fused); a persistent one takes planes split and joined by kernels.
   const bool automatic = !plan || (plan->digit_bits == 0 && plan->mode == RS_MODE_AUTO && plan->tile == 0);
-  const bool hybrid = automatic && HybLayout::offers(n, 4, 8);
-  Layout L = make_layout(p, n, true, hybrid ? 8 : -1);
+  Layout L = make_layout(p, n, true, automatic ? 8 : -1);
+  const bool hybrid = L.hyb.buckets != 0;
   const bool fused = pair_io_kernel(p.k) != nullptr;
   const int nplanes = fused ? 3 : 5;
   size_t plane[5] = {};
