@@ -685,9 +685,12 @@ SegLayout make_seg_layout(size_t off, uint32_t num_segs, uint64_t total_n, int n
 
 // small_max: segments up to this many keys are sorted by one block in shared
 // memory (at most the local sort's capacity); larger ones by tiled passes.
+// few_tiny: fewer than half of the segments are expected in the smallest
+// class.  (Any offsets on the device are sorted, whatever the host expects.)
 rs_status run_segmented(const SegLayout& L, unsigned char* temp, const uint32_t* kin, const uint32_t* vin,
-                        uint32_t* kout, uint32_t* vout, const uint64_t* seg_off, uint32_t num_segs, int nd,
-                        KeyXform xin, KeyXform xout, DeviceState* ds, cudaStream_t s, uint32_t small_max = 0) {
+                        uint32_t* kout, uint32_t* vout, const uint64_t* seg_off, uint32_t num_segs, uint64_t total_n,
+                        int nd, KeyXform xin, KeyXform xout, DeviceState* ds, cudaStream_t s, bool few_tiny,
+                        uint32_t small_max = 0) {
   const SegKernels* sk = seg_kernels();
   if (small_max == 0 || small_max > sk->small_max) small_max = sk->small_max;
   const uint32_t tiny_max = small_max < sk->tiny_max ? small_max : sk->tiny_max;
@@ -772,12 +775,17 @@ rs_status run_segmented(const SegLayout& L, unsigned char* temp, const uint32_t*
   la.xout = xout;
   la.list = pa.tiny_seg;
   la.count = counts + SEG_NUM_TINY;
-  RS_CUDA(traced(T_LOCAL, 0, s, [&] { return launch_local_sort(la, false, pairs, num_segs, s); }),
+  RS_CUDA(traced(T_LOCAL, 0, s, [&] { return launch_tiny_segments(la, pairs, num_segs, few_tiny ? sms : 0u, s); }),
           "launch local_sort (tiny)");
   la.list = pa.small_seg;
   la.count = counts + SEG_NUM_SMALL;
-  RS_CUDA(traced(T_LOCAL, 0, s, [&] { return launch_local_sort(la, true, pairs, num_segs, s); }),
-          "launch local_sort (small)");
+  // (a block per SM, whose empty ones take their time: no more of them than
+  // segments of that size fit.  100,000 empty segments beside one of 50,000 keys
+  // 545 us with one for every segment, 360 without, 312 with few_tiny too)
+  const unsigned small_ub = unsigned(std::min<uint64_t>(num_segs, total_n / (tiny_max + 1)));
+  if (small_ub)
+    RS_CUDA(traced(T_LOCAL, 0, s, [&] { return launch_small_segments(la, pairs, small_ub, s); }),
+            "launch local_sort (small)");
   return RS_OK;
 }
 
@@ -868,11 +876,11 @@ rs_status run_msd(const SortPlan& p, const MsdLayout& M, const uint32_t* keys_in
   if (!pairs) {
     RS_CUDA(traced(T_MSDSCATTER, n, s, [&] { return launch_msd_scatter(ma, s); }), "launch msd_scatter");
     // the bucket buffer holds order-mapped keys; the local phase maps them back
-    return run_segmented(M.seg, temp, bk, nullptr, keys_out, nullptr, ma.seg_off, kMsdBuckets, 3, kIdentityXform,
-                         p.xf, ds, s);
+    return run_segmented(M.seg, temp, bk, nullptr, keys_out, nullptr, ma.seg_off, kMsdBuckets, n, 3, kIdentityXform,
+                         p.xf, ds, s, true);
   }
   if (rs_status st = run_lsd(M.q, M.lsd, keys_in, vals_in, bk, bv, n, temp, true, ds, s); st != RS_OK) return st;
-  return run_segmented(M.seg, temp, bk, bv, keys_out, vals_out, ma.seg_off, kMsdBuckets, 3, p.xf, p.xf, ds, s);
+  return run_segmented(M.seg, temp, bk, bv, keys_out, vals_out, ma.seg_off, kMsdBuckets, n, 3, p.xf, p.xf, ds, s, true);
 }
 
 rs_status run_hybrid32(const SortPlan& p, const Layout& L, const uint32_t* keys_in, const uint32_t* vals_in,
@@ -1595,14 +1603,14 @@ rs_status rs_sort_u32_segmented(const uint32_t* keys_in, const uint32_t* vals_in
   if (num_parts < 1) return fail(RS_ERR_INVALID, "num_parts must be >= 1");
   if (num_segs > 0 && !h_seg_offsets) return fail(RS_ERR_INVALID, "h_seg_offsets is NULL");
   if (total_n >= (uint64_t(1) << 32)) return fail(RS_ERR_INVALID, "total_n must be below 2^32");
-  uint64_t max_seg = 0;
+  uint32_t tiny = 0;  // segments of the smallest class
   if (num_segs > 0) {
     if (h_seg_offsets[0] != 0 || h_seg_offsets[num_segs] != total_n)
       return fail(RS_ERR_INVALID, "segment offsets must start at 0 and end at total_n");
     for (uint32_t i = 0; i < num_segs; ++i) {
       if (h_seg_offsets[i + 1] < h_seg_offsets[i]) return fail(RS_ERR_INVALID, "segment offsets decrease at %u", i);
       const uint64_t m = h_seg_offsets[i + 1] - h_seg_offsets[i];
-      if (m > max_seg) max_seg = m;
+      tiny += m > 0 && m <= seg_kernels()->tiny_max;
     }
   }
   const rs_plan eff = resolve_plan(pairs ? RS_ENTRY_SEGMENTED_PAIRS : RS_ENTRY_SEGMENTED,
@@ -1619,7 +1627,6 @@ rs_status rs_sort_u32_segmented(const uint32_t* keys_in, const uint32_t* vals_in
   KeyXform xf;
   if (rs_status st = key_xform(&eff, &xf); st != RS_OK) return st;
   if (needs_wide_status(total_n)) return fail(RS_ERR_UNSUPPORTED, "the segmented sort needs total_n < 2^30 - 2^16");
-  (void)max_seg;
   const SegLayout L = make_seg_layout(0, num_segs, total_n, 4, pairs, shape);
   if (!temp) {
     *temp_bytes = L.end;
@@ -1651,7 +1658,8 @@ rs_status rs_sort_u32_segmented(const uint32_t* keys_in, const uint32_t* vals_in
   }
   if (total_n == 0) return RS_OK;
   return run_segmented(L, static_cast<unsigned char*>(temp), keys_in, pairs ? vals_in : nullptr, keys_out,
-                       pairs ? vals_out : nullptr, d_seg_offsets, num_segs, 4, xf, xf, ds, s, small_max);
+                       pairs ? vals_out : nullptr, d_seg_offsets, num_segs, total_n, 4, xf, xf, ds, s,
+                       tiny < num_segs / 2, small_max);
 }
 
 rs_status rs_digit_histograms(const uint32_t* keys, uint64_t n, uint32_t digit_bits, uint32_t* d_hist,

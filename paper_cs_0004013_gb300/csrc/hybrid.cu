@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(THREADS, MINB) bucket_sort_kernel(const HybArg
   K* io = reinterpret_cast<K*>(a.keys_out) + s;
   V* vio = VB ? reinterpret_cast<V*>(a.vals_out) + s : nullptr;
   auto sort = [&](auto edge, auto mode, auto eo) {
-    local_sort_array<THREADS, ITEMS, BITS, VB, decltype(mode)::value, true>(io, io, vio, vio, vio, e - s, OrdOf<K>::identity(),
+    local_sort_array<THREADS, ITEMS, BITS, VB, decltype(mode)::value, true, false>(io, io, vio, vio, vio, e - s, OrdOf<K>::identity(),
                                                            OrdOf<K>::make(a),
                                                            BucketBins<K, BITS, decltype(edge)::value>{m}, smem, eo);
   };

@@ -1,6 +1,8 @@
 // Arrays and segments that fit one block, sorted in shared memory (local.cuh).
 //
 // Paper: the local sort of each cell's keys (Sec. 3.3).
+#include <algorithm>
+
 #include "local.cuh"
 #include "rs_internal.h"
 
@@ -23,7 +25,11 @@ struct OrdFor<uint64_t> {
 };
 
 // A block per listed segment (list != null; the grid holds a block for every
-// segment that may be listed), or the one array [0, single_n).
+// segment that may be listed), or the one array [0, single_n).  LOOP: a grid of
+// any size, whose blocks take segments in turn; for lists that are short beside
+// what may be listed, as an empty block takes about 0.3 us of its place on the SM
+// (MSD plan's 16,384 buckets of clustered keys: 140 us -> 130), while full lists
+// lose by it (16,384 segments of 4,096 keys: 291 us against 310).
 // One array is one block's chain of steps, bound by its latency: bins and sorting
 // networks instead of four digit passes, traced (about 4 us of it the events),
 // us: 1,000 keys 15.7 -> 7.5, 4,000 16.4 -> 8.0, 8,000 27.2 -> 11.1, 16,000 35.5 ->
@@ -31,22 +37,34 @@ struct OrdFor<uint64_t> {
 // passes sorted, 123 -> 15, with 64-bit payloads 141 -> 23.  Few distinct values
 // still end in the digit passes: 8,000 keys of 8 values 23.8 -> 29.2 (the pass
 // over the bins that found them crowded comes on top).
-template <int THREADS, int ITEMS, int NBITS, int MINB, typename K, int VB>
+template <int THREADS, int ITEMS, int NBITS, int MINB, typename K, int VB, bool LOOP>
 __global__ void __launch_bounds__(THREADS, MINB) local_sort_kernel(const LocalArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   using V = typename ValueOf<VB>::T;
-  uint64_t start = 0;
-  uint32_t m = a.single_n;
-  if (a.list) {
-    if (blockIdx.x >= *a.count) return;
-    const uint32_t s = a.list[blockIdx.x];
-    start = a.seg_off[s];
-    m = uint32_t(a.seg_off[s + 1] - start);
+  auto sort = [&](uint64_t start, uint32_t m) {
+    local_sort_array<THREADS, ITEMS, NBITS, VB, VB ? Vals::kFollow : Vals::kAlone, false, LOOP>(
+        static_cast<const K*>(a.kin) + start, static_cast<K*>(a.kout) + start,
+        VB ? static_cast<const V*>(a.vin) + start : nullptr, VB ? static_cast<V*>(a.vout) + start : nullptr,
+        static_cast<const V*>(nullptr), m, OrdFor<K>::in(a), OrdFor<K>::out(a), RangeBins<K>{}, smem);
+  };
+  if constexpr (LOOP) {
+    const uint32_t count = *a.count;
+    for (uint32_t k = blockIdx.x; k < count; k += gridDim.x) {
+      const uint32_t s = a.list[k];
+      const uint64_t start = a.seg_off[s];
+      sort(start, uint32_t(a.seg_off[s + 1] - start));
+    }
+  } else {
+    uint64_t start = 0;
+    uint32_t m = a.single_n;
+    if (a.list) {
+      if (blockIdx.x >= *a.count) return;
+      const uint32_t s = a.list[blockIdx.x];
+      start = a.seg_off[s];
+      m = uint32_t(a.seg_off[s + 1] - start);
+    }
+    sort(start, m);
   }
-  local_sort_array<THREADS, ITEMS, NBITS, VB, VB ? Vals::kFollow : Vals::kAlone, false>(
-      static_cast<const K*>(a.kin) + start, static_cast<K*>(a.kout) + start,
-      VB ? static_cast<const V*>(a.vin) + start : nullptr, VB ? static_cast<V*>(a.vout) + start : nullptr,
-      static_cast<const V*>(nullptr), m, OrdFor<K>::in(a), OrdFor<K>::out(a), RangeBins<K>{}, smem);
 }
 
 struct Shape {
@@ -56,13 +74,13 @@ struct Shape {
   const void* func;
   cudaError_t (*launch)(const LocalArgs&, unsigned, cudaStream_t);
 };
-template <int THREADS, int ITEMS, int NBITS, int MINB, typename K, int VB>
+template <int THREADS, int ITEMS, int NBITS, int MINB, typename K, int VB, bool LOOP = false>
 Shape shape() {
   using L = LocalLayout<THREADS, ITEMS, NBITS, K, VB, VB ? Vals::kFollow : Vals::kAlone>;
   return Shape{uint32_t(L::CAP), unsigned(THREADS), L::SMEM,
-               reinterpret_cast<const void*>(&local_sort_kernel<THREADS, ITEMS, NBITS, MINB, K, VB>),
+               reinterpret_cast<const void*>(&local_sort_kernel<THREADS, ITEMS, NBITS, MINB, K, VB, LOOP>),
                [](const LocalArgs& a, unsigned grid, cudaStream_t s) {
-                 local_sort_kernel<THREADS, ITEMS, NBITS, MINB, K, VB><<<grid, THREADS, L::SMEM, s>>>(a);
+                 local_sort_kernel<THREADS, ITEMS, NBITS, MINB, K, VB, LOOP><<<grid, THREADS, L::SMEM, s>>>(a);
                  return cudaGetLastError();
                }};
 }
@@ -70,7 +88,7 @@ Shape shape() {
 // Segments: tiny ones (up to 4,096 keys) by 256 threads, small ones (up to
 // 16,384) by 1,024.  One array: the smallest of its shapes that holds it.
 struct Shapes {
-  Shape tiny[2], small[2];                                  // [payload]
+  Shape tiny[2], few_tiny[2], small[2];                     // [payload]
   Shape one32[2], mid32[2], one32v8, big32v8, one64[3], big64[3];  // one array; [0, 4 or 8 payload bytes]
 };
 const Shapes& shapes() {
@@ -78,6 +96,7 @@ const Shapes& shapes() {
   using u64 = uint64_t;
   static const Shapes s = {
       {shape<256, 16, 12, 4, u32, 0>(), shape<256, 16, 12, 3, u32, 4>()},
+      {shape<256, 16, 12, 4, u32, 0, true>(), shape<256, 16, 12, 3, u32, 4, true>()},
       {shape<1024, 16, 14, 1, u32, 0>(), shape<1024, 16, 14, 1, u32, 4>()},
       {shape<256, 4, 11, 1, u32, 0>(), shape<256, 4, 11, 1, u32, 4>()},
       {shape<1024, 4, 13, 1, u32, 0>(), shape<1024, 4, 13, 1, u32, 4>()},
@@ -93,7 +112,7 @@ const Shapes& shapes() {
 
 cudaError_t prepare_local() {
   const Shapes& s = shapes();
-  const Shape* all[] = {&s.tiny[0],  &s.tiny[1],  &s.small[0], &s.small[1], &s.one32[0], &s.one32[1],
+  const Shape* all[] = {&s.tiny[0],  &s.tiny[1],  &s.few_tiny[0], &s.few_tiny[1], &s.small[0], &s.small[1], &s.one32[0], &s.one32[1],
                         &s.mid32[0], &s.mid32[1], &s.one32v8,  &s.big32v8,  &s.one64[0], &s.one64[1],
                         &s.one64[2], &s.big64[0], &s.big64[1], &s.big64[2]};
   for (const Shape* p : all)
@@ -105,9 +124,13 @@ cudaError_t prepare_local() {
 
 uint32_t local_max_keys(int key_bytes, int val_bytes) { return key_bytes == 4 && val_bytes < 8 ? 16384u : 8192u; }
 
-cudaError_t launch_local_sort(const LocalArgs& a, bool small, bool pairs, unsigned grid, cudaStream_t s) {
+cudaError_t launch_tiny_segments(const LocalArgs& a, bool pairs, uint32_t num_segs, unsigned few_sms, cudaStream_t s) {
   const Shapes& sh = shapes();
-  return (small ? sh.small[pairs] : sh.tiny[pairs]).launch(a, grid, s);
+  return few_sms ? sh.few_tiny[pairs].launch(a, std::min(num_segs, few_sms * 16u), s)  // four times what is resident
+                 : sh.tiny[pairs].launch(a, num_segs, s);
+}
+cudaError_t launch_small_segments(const LocalArgs& a, bool pairs, uint32_t max_listed, cudaStream_t s) {
+  return shapes().small[pairs].launch(a, max_listed, s);
 }
 
 cudaError_t launch_local_array(const LocalArgs& a, int key_bytes, int val_bytes, cudaStream_t s) {

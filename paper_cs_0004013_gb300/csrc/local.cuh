@@ -425,7 +425,12 @@ __device__ __noinline__ void local_digit_passes(uint32_t m, const EO eo, unsigne
 // on loading, ordo back on storing.  bins: RangeBins (filled here) or a map
 // known beforehand.  eo: what is ordered (by default the key, or key and
 // place side by side).  The block is synchronised on return.
-template <int THREADS, int ITEMS, int NBITS, int VB, Vals MODE, bool COHERENT, class OrdI, class OrdO, class Bins,
+// LOOPED: for a call inside a loop.  There the registers of items that a short
+// array leaves out would be carried round the loop, and what depends on the
+// thread's index alone would be kept over it (288 bytes of spills for 4,096 keys):
+// they start defined, and the index is read anew (20 bytes).  Other calls are up
+// to 7 % slower with that.
+template <int THREADS, int ITEMS, int NBITS, int VB, Vals MODE, bool COHERENT, bool LOOPED, class OrdI, class OrdO, class Bins,
           class VIn, class EO = ElemOf<typename OrdI::Key, VB != 0>>
 __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, typename OrdI::Key* out, const VIn* vin,
                                                  typename ValueOf<VB>::T* vout,
@@ -445,7 +450,14 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
   K* s_red = reinterpret_cast<K*>(smem + L::OFF_WARP);
   uint32_t* s_scan = reinterpret_cast<uint32_t*>(smem + L::OFF_SCAN);
   uint32_t* s_most = reinterpret_cast<uint32_t*>(smem + L::OFF_MOST);
-  const int tid = threadIdx.x;
+  int tid = threadIdx.x;
+  if constexpr (LOOPED) asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
+  auto define = [](auto* a, int count) {
+    if constexpr (LOOPED) {
+#pragma unroll
+      for (int i = 0; i < count; ++i) a[i] = {};
+    }
+  };
   const int lane = tid & 31, warp = tid >> 5;
   // Items go by groups of G: a group past the last key is skipped by the whole
   // block (a uniform branch); inside a group a lane without a key has its
@@ -463,8 +475,10 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
 
   // 1. load; clear the bins
   K key[ITEMS];
+  define(key, ITEMS);
   for_items([&](int j) { key[j] = has(j) ? ld_elem<COHERENT>(in + j * THREADS + tid) : K(0); });
   [[maybe_unused]] uint32_t place[PLACES ? ITEMS : 1];
+  define(place, PLACES ? ITEMS : 1);
   if constexpr (PLACES) for_items([&](int j) { place[j] = has(j) ? ld_elem<COHERENT>(vin + j * THREADS + tid) : 0u; });
   auto elem = [&](int j) {
     if constexpr (PLACES) return eo.make(key[j], place[j]);
@@ -518,6 +532,7 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
   // lost).  Returns the fullest bin's keys, five at least.
   const uint32_t bin_base = static_cast<uint32_t>(__cvta_generic_to_shared(s_bin));
   uint32_t turn[(ITEMS + 3) / 4];
+  define(turn, (ITEMS + 3) / 4);
   auto count = [&](auto&& bin_of) -> uint32_t {
     uint32_t most = 0;
     for_items([&](int j) {
@@ -619,6 +634,7 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
       scan();
       const uint32_t per = (uint32_t(NB) << 16) / m;
       uint32_t bin2[ITEMS];
+      define(bin2, ITEMS);
       for_items([&](int j) {
         const uint32_t b = first_bin(j) & uint32_t(NB - 1);
         const uint32_t s = start_of(b), e = b == uint32_t(NB - 1) ? m : start_of(b + 1);
@@ -647,6 +663,7 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
       // them it takes the next window's lower half, from the next lane or,
       // over the warp's end, through shared memory.
       E v[HELD ? NWIN : 1][8];
+      define(v[0], (HELD ? NWIN : 1) * 8);
 #pragma unroll
       for (int c = 0; c < (HELD ? NWIN : 0); ++c) {
         const uint32_t p = uint32_t(c * THREADS + tid) * 8u;
@@ -714,6 +731,7 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
     __syncthreads();
   }
   V held[MODE == Vals::kInPlace ? ITEMS : 1];
+  define(held, MODE == Vals::kInPlace ? ITEMS : 1);
   if constexpr (MODE == Vals::kInPlace) {
     for_items([&](int j) {
       if (has(j)) held[j] = ld_elem<COHERENT>(vin + eo.place(s_key[L::slot(j * THREADS + tid)]));

@@ -291,7 +291,10 @@ cudaError_t launch_seg_pass(const SegPassArgs& a, bool pairs, int shape, unsigne
 // One-block sorts (local.cu): the listed segments, or one array.
 cudaError_t prepare_local();
 uint32_t local_max_keys(int key_bytes, int val_bytes);
-cudaError_t launch_local_sort(const LocalArgs& a, bool small, bool pairs, unsigned grid, cudaStream_t s);
+// few_sms: 0, or the number of SMs when few of the segments are listed.
+cudaError_t launch_tiny_segments(const LocalArgs& a, bool pairs, uint32_t num_segs, unsigned few_sms, cudaStream_t s);
+// max_listed: at least as many as are listed.
+cudaError_t launch_small_segments(const LocalArgs& a, bool pairs, uint32_t max_listed, cudaStream_t s);
 cudaError_t launch_local_array(const LocalArgs& a, int key_bytes, int val_bytes, cudaStream_t s);
 
 // Stable merge of two sorted runs (merge.cu).
