@@ -215,7 +215,7 @@ __device__ __forceinline__ bool fused_buckets(const FusedArgs& a, uint32_t tile,
     uint32_t* vout = NV ? a.vals_out + s : nullptr;
     local_sort_array<T, FL::BITEMS, kFusedBucketBits, NV ? 4 : 0, NV ? Vals::kPlaces : Vals::kAlone, true, false>(
         a.keys_alt + s, a.keys_out + s, a.vals_alt + s, vout, a.vals_in, e - s, Ord32{KeyXform{0u, 0u}}, Ord32{a.xf},
-        RangeBins<uint32_t>{}, smem);
+        RangeBins<uint32_t, false>{}, smem);
   }
   return true;
 }

@@ -45,7 +45,7 @@ constexpr int kCountThreads = 1024;
 // last bucket, which also hold the values outside the sampled range.
 template <typename K, int NBITS, bool EDGE>
 struct BucketBins {
-  static constexpr bool kKnown = true;
+  static constexpr bool kKnown = true, kLook = false;
   ValueMap<K> m;
   __device__ __forceinline__ uint32_t operator()(K k) const {
     return uint32_t(m.product(EDGE ? m.clamp(k) : k)) >> (32 - NBITS);

@@ -34,9 +34,11 @@ struct OrdFor<uint64_t> {
 // networks instead of four digit passes, traced (about 4 us of it the events),
 // us: 1,000 keys 15.7 -> 7.5, 4,000 16.4 -> 8.0, 8,000 27.2 -> 11.1, 16,000 35.5 ->
 // 14.7, with payloads 44.8 -> 24.8; 8,000 64-bit keys, which eight launches of
-// passes sorted, 123 -> 15, with 64-bit payloads 141 -> 23.  Few distinct values
-// still end in the digit passes: 8,000 keys of 8 values 23.8 -> 29.2 (the pass
-// over the bins that found them crowded comes on top).
+// passes sorted, 123 -> 15, with 64-bit payloads 141 -> 23.  Values that
+// crowd end in the digit passes after a look at a sample (in graphs, us, before any
+// bins / bins tried first / now): 8,000 keys of 8 values 18.1 / 25.7 / 20.1, 16,000
+// 20.8 / 32.2 / 25, log-uniform ones 32.3 / 48 / 35, clusters 25.5 / 40 / 35; 4,000
+// keys, which are not looked at, of 8 values 10.3 / 12.8 / 12.8.
 template <int THREADS, int ITEMS, int NBITS, int MINB, typename K, int VB, bool LOOP>
 __global__ void __launch_bounds__(THREADS, MINB) local_sort_kernel(const LocalArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];

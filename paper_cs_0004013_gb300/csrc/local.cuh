@@ -28,7 +28,8 @@
 // keys (its start and count give them), and a key takes the part of that
 // share that its place inside the bin points to.  This flattens any density
 // that does not change much within a bin (normally distributed floats, wide
-// clusters).  Blocks that are crowded still sort by digits.
+// clusters).  Blocks that are crowded still, or that a sample shows to be, sort
+// by digits.
 // Sorts with payloads are stable: they order (key, place in the input), and
 // the payload follows its place.  The digit passes are stable 8-bit ones over
 // the digits in which the keys differ, with the lane-mask tables of the tiled pass.
@@ -45,6 +46,10 @@
 namespace rs {
 
 constexpr uint32_t kBinLimit = 29;  // eight rounds of windows
+constexpr uint32_t kCrowded = 24;   // mean keys per bin that a small sample shows well enough
+// Arrays of more keys are looked at before their bins are laid (up to 0.3 us;
+// 16,000 keys of 8 values 32 us -> 25, 4,000 even ones 4.0 -> 4.4).
+constexpr uint32_t kLookKeys = 4096;
 
 // What the block orders: the key, or with a payload (key, place in the input).
 struct alignas(16) KeyPlace64 {
@@ -236,9 +241,10 @@ __device__ __forceinline__ void warp_min_max(K& lo, K& hi) {
 }
 
 // Bins from the array's own range: bin = (key - lo) >> sh.
-template <typename K>
+// LOOK: whether its values may crowd (not where a sample has found them spread evenly).
+template <typename K, bool LOOK = true>
 struct RangeBins {
-  static constexpr bool kKnown = false;
+  static constexpr bool kKnown = false, kLook = LOOK;
   K lo;
   int sh;
   __device__ __forceinline__ uint32_t operator()(K k) const { return uint32_t((k - lo) >> sh); }
@@ -262,31 +268,6 @@ __device__ __forceinline__ uint32_t warp_rank_step(uint32_t d, uint32_t* wm, uin
   const uint32_t before = wc[d];
   __syncwarp();
   if ((peers & gt) == 0) {
-    wc[d] = uint16_t(before + __popc(peers));
-    wm[d] = 0u;
-  }
-  __syncwarp();
-  return before + __popc(peers & lt);
-}
-
-// The same of the lanes that have a key (lane 0 does); a row of one digit, as
-// few distinct keys make many, needs no table: its lanes would all meet in one word.
-__device__ __forceinline__ uint32_t warp_rank_row(uint32_t d, bool has, uint32_t* wm, uint16_t* wc, uint32_t lt,
-                                                  uint32_t gt, int lane) {
-  const uint32_t live = __ballot_sync(0xffffffffu, has), d0 = __shfl_sync(0xffffffffu, d, 0);
-  if (__all_sync(0xffffffffu, !has || d == d0)) {
-    const uint32_t before = wc[d0];
-    __syncwarp();
-    if (lane == 0) wc[d0] = uint16_t(before + __popc(live));
-    __syncwarp();
-    return before + __popc(live & lt);
-  }
-  if (has) atomicOr(&wm[d], 1u << lane);
-  __syncwarp();
-  const uint32_t peers = wm[d];
-  const uint32_t before = wc[d];
-  __syncwarp();
-  if (has && (peers & gt) == 0) {
     wc[d] = uint16_t(before + __popc(peers));
     wm[d] = 0u;
   }
@@ -382,13 +363,29 @@ __device__ __noinline__ void local_digit_passes(uint32_t m, const EO eo, unsigne
     __syncthreads();
     for (int i = tid; i < int(L::RANK_BYTES / 16); i += THREADS) b4[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
+    // Rows of 32 two at a time: one vote tells whether both hold one digit only
+    // (as few distinct keys make many), whose lanes would all meet in one word.
+    // Places past the end act as the largest digit: they come after every key.
     uint32_t rk[(ITEMS + 1) / 2];
+    uint32_t* wm = s_mask + warp * kMaskSlots;
+    uint16_t* wc = s_cnt + warp * 256;
+    auto rank = [&](uint32_t x, bool uniform) -> uint32_t {
+      if (!uniform) return warp_rank_step(x, wm, wc, lt, gt, lane);
+      const uint32_t before = wc[x];
+      __syncwarp();
+      if (lane == 0) wc[x] = uint16_t(before + 32u);
+      __syncwarp();
+      return before + uint32_t(lane);
+    };
 #pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-      const uint32_t r =
-          row(j) ? warp_rank_row(digit(j, d), has(j), s_mask + warp * kMaskSlots, s_cnt + warp * 256, lt, gt, lane) : 0u;
-      if (j & 1) rk[j >> 1] |= r << 16;
-      else rk[j >> 1] = r;
+    for (int j = 0; j < ITEMS; j += 2) {
+      if (!row(j)) break;
+      const uint32_t x0 = has(j) ? digit(j, d) : 255u;
+      const uint32_t x1 = j + 1 < ITEMS && has(j + 1) ? digit(j + 1, d) : 255u;
+      const uint32_t both = x0 | (x1 << 8);
+      const bool uniform = __all_sync(0xffffffffu, both == __shfl_sync(0xffffffffu, both, 0));
+      rk[j >> 1] = rank(x0, uniform);
+      if (j + 1 < ITEMS) rk[j >> 1] |= rank(x1, uniform) << 16;
     }
     __syncthreads();
     constexpr int DT = THREADS < 256 ? THREADS : 256;  // threads with digits
@@ -473,10 +470,47 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
       }
   };
 
+  // How crowded the bins are is told by a sample, each lane's key from a stretch
+  // of its own: D bins in use give a key its like among its warp's others with a
+  // chance of about 31 / D, and m / D keys to a bin.  Counted are likes in the
+  // second set of bins, with a bin's share taken from the warp's keys in it:
+  // those that neither set tells apart.  Four warps look (a match takes 0.1 us of
+  // them, 1 us of 32): before the bins are laid where there are keys enough,
+  // otherwise when they are found crowded.
+  constexpr int FEW = WARPS < 4 ? WARPS : 4;
+  constexpr uint32_t LANES = uint32_t(FEW) * 32;
+  const bool looked = Bins::kLook && m > kLookKeys;
+  auto sampled = [&]() {  // (fewer keys than lanes: the lane's own)
+    const uint32_t q = uint32_t(tid);
+    return m < LANES ? q : q * m / LANES + __umulhi(q * 0x9E3779B1u, m / LANES);
+  };
+  auto count_likes = [&](K k, bool live) {
+    if constexpr (!Bins::kKnown) {
+      if (warp < FEW) {
+        const uint32_t lives = __ballot_sync(0xffffffffu, live);
+        const uint32_t b = bins(k);
+        const uint32_t same = __match_any_sync(0xffffffffu, b) & lives;
+        uint32_t likes = __ballot_sync(0xffffffffu, live && (same & (same - 1u)) != 0u);
+        if (likes) {
+          const uint32_t part = __umulhi(bins.frac(k), uint32_t(__popc(same)) * uint32_t(NB / 32));
+          const uint32_t same2 = __match_any_sync(0xffffffffu, (b << NBITS) + part) & same;
+          likes = __ballot_sync(0xffffffffu, live && (same2 & (same2 - 1u)) != 0u);
+        }
+        if (lane == 0) s_scan[warp] = uint32_t(__popc(likes));
+      }
+    }
+  };
+  uint32_t likes = 0;
+  auto read_likes = [&]() { return __reduce_add_sync(0xffffffffu, lane < FEW ? s_scan[lane] : 0u); };
+  // whether the likes mean more than `limit` keys to a bin
+  auto more_than = [&](uint32_t limit) { return likes * m > 31u * limit * (m < LANES ? m : LANES); };
+
   // 1. load; clear the bins
   K key[ITEMS];
   define(key, ITEMS);
   for_items([&](int j) { key[j] = has(j) ? ld_elem<COHERENT>(in + j * THREADS + tid) : K(0); });
+  K probe = 0;
+  if (looked && warp < FEW) probe = ld_elem<COHERENT>(in + sampled());
   [[maybe_unused]] uint32_t place[PLACES ? ITEMS : 1];
   define(place, PLACES ? ITEMS : 1);
   if constexpr (PLACES) for_items([&](int j) { place[j] = has(j) ? ld_elem<COHERENT>(vin + j * THREADS + tid) : 0u; });
@@ -524,7 +558,13 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
     bins.lo = lo;
     bins.sh = bits > NBITS ? bits - NBITS : 0;
   }
+  // Far too crowded for either set of bins: the digit passes sort them at once
+  // (the bins' atomics would meet in few words).  Bins of one value, whose keys
+  // need no order, hold 256.
+  if (looked) count_likes(ordi.map(probe), true);
   __syncthreads();
+  if (looked) likes = read_likes();
+  const bool crowded = looked && more_than(VB == 0 && bins.unique() ? 256u : kCrowded);
 
   // 2. turns within the bins.  Word w of the counts holds bin w in its low and
   // bin w + NB / 2 in its high half; four 8-bit turns go to a register (a
@@ -608,48 +648,50 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
     __syncthreads();
   };
   auto first_bin = [&](int j) { return bins(key[j]); };
-  uint32_t most = count(first_bin);
-  // bins of one value need no order among equal keys (as long as their turns fit their 8 bits)
-  if (VB == 0 && bins.unique() && most <= 256u) most = 1u;
-  bool staged = most <= kBinLimit;
-  if (staged) {
-    scan();
-    stage(first_bin);
-  } else if constexpr (!Bins::kKnown) {
-    // Few distinct keys: D of them leave a lane without its like in the warp with
-    // a chance of (1 - 1 / D)^31, and with m / D above kBinLimit other bins are
-    // as crowded, so the digit passes sort them at once (16,000 keys of 8 values
-    // 40 us with the second bins tried first, 35 without).
-    const uint32_t live = __ballot_sync(0xffffffffu, has(0));
-    const uint32_t same = __match_any_sync(0xffffffffu, key[0]) & live;  // (every lane takes part)
-    const uint32_t likes = __popc(__ballot_sync(0xffffffffu, has(0) && (same & (same - 1u)) != 0u));
-    if (lane == 0) s_scan[warp] = likes;
-    __syncthreads();
-    const uint32_t sum = __reduce_add_sync(0xffffffffu, lane < WARPS ? s_scan[lane] : 0u);
-    __syncthreads();
-    const bool repeats = sum * m > 31u * kBinLimit * (m < uint32_t(THREADS) ? m : uint32_t(THREADS));
-    if (!repeats && !bins.unique()) {
-      // crowded: the second set of bins (see above), NB / m of them to a key;
-      // positions among the keys in 16.16 fixed point
+  uint32_t most = 0;
+  bool staged = false;
+  if (!crowded) {
+    most = count(first_bin);
+    // bins of one value need no order among equal keys (as long as their turns fit their 8 bits)
+    if (VB == 0 && bins.unique() && most <= 256u) most = 1u;
+    staged = most <= kBinLimit;
+    if (staged) {
       scan();
-      const uint32_t per = (uint32_t(NB) << 16) / m;
-      uint32_t bin2[ITEMS];
-      define(bin2, ITEMS);
-      for_items([&](int j) {
-        const uint32_t b = first_bin(j) & uint32_t(NB - 1);
-        const uint32_t s = start_of(b), e = b == uint32_t(NB - 1) ? m : start_of(b + 1);
-        bin2[j] = __umulhi((s << 16) + __umulhi(bins.frac(key[j]), (e - s) << 16), per);
-      });
-      __syncthreads();
-      for (int i = tid; i < NB / 8; i += THREADS) b4[i] = make_uint4(0u, 0u, 0u, 0u);
-      if (tid == 0) *s_most = 0u;
-      __syncthreads();
-      auto second_bin = [&](int j) { return bin2[j]; };
-      most = count(second_bin);
-      staged = most <= kBinLimit;
-      if (staged) {
-        scan();
-        stage(second_bin);
+      stage(first_bin);
+    } else if (!Bins::kKnown && !bins.unique()) {
+      if constexpr (!Bins::kKnown) {
+        // (a mean of 18 keys leaves some bin of the second set above the limit)
+        if (!looked) {
+          const uint32_t at = sampled();
+          count_likes(warp < FEW && at < m ? ordi.map(ld_elem<COHERENT>(in + at)) : K(0), at < m);
+          __syncthreads();
+          likes = read_likes();
+          __syncthreads();
+        }
+        if (!more_than(18u)) {
+          // the second set of bins (see above), NB / m of them to a key;
+          // positions among the keys in 16.16 fixed point
+          scan();
+          const uint32_t per = (uint32_t(NB) << 16) / m;
+          uint32_t bin2[ITEMS];
+          define(bin2, ITEMS);
+          for_items([&](int j) {
+            const uint32_t b = first_bin(j) & uint32_t(NB - 1);
+            const uint32_t s = start_of(b), e = b == uint32_t(NB - 1) ? m : start_of(b + 1);
+            bin2[j] = __umulhi((s << 16) + __umulhi(bins.frac(key[j]), (e - s) << 16), per);
+          });
+          __syncthreads();
+          for (int i = tid; i < NB / 8; i += THREADS) b4[i] = make_uint4(0u, 0u, 0u, 0u);
+          if (tid == 0) *s_most = 0u;
+          __syncthreads();
+          auto second_bin = [&](int j) { return bin2[j]; };
+          most = count(second_bin);
+          staged = most <= kBinLimit;
+          if (staged) {
+            scan();
+            stage(second_bin);
+          }
+        }
       }
     }
   }
