@@ -341,6 +341,11 @@ rs_status make_plan(uint64_t n, bool pairs, const rs_plan* user, SortPlan* p, in
 // 2^low_bits that halve the bucket's bits between the two splits; up to 256
 // buckets take one split.
 constexpr uint64_t kHybridMinKeys = 8192;  // the sample's size
+// 32-bit pairs: smaller sorts gain nothing (full-range keys take the wide elements
+// up to 2^23, 31-bit ones up to 2^22) and pay the sample: 2.9M even pairs 98 us by
+// passes, 94 by buckets, 3.5M 104 / 109, normally distributed ones 107 / 121; 4.3M
+// even 31-bit ones 124 / 98.
+constexpr uint64_t kHybridMinPairs = uint64_t(1) << 22;
 struct HybLayout {
   HybShape shape = {};
   uint64_t n = 0;
@@ -351,7 +356,8 @@ struct HybLayout {
   // The most keys that are offered the buckets: their mean may reach three
   // quarters of what a bucket takes.
   static uint64_t most(int kb, int vb) { return uint64_t(kHybMaxBuckets) * hyb_shape(kb, vb).bucket_cap * 3 / 4; }
-  static bool offers(uint64_t n, int kb, int vb) { return n >= kHybridMinKeys && n <= most(kb, vb); }
+  static uint64_t fewest(int kb, int vb) { return kb == 4 && vb == 4 ? kHybridMinPairs : kHybridMinKeys; }
+  static bool offers(uint64_t n, int kb, int vb) { return n >= fewest(kb, vb) && n <= most(kb, vb); }
   // The space of that many, which larger sorts hold too: a workspace for more keys takes fewer.
   static size_t most_bytes(int kb, int vb) {
     HybLayout h;
@@ -405,17 +411,29 @@ struct HybLayout {
 //   keys, 3 digits: c = 8 115 / 132 and 191 / 213, c = 16 139 / 131 and 229 / 213;
 //   64-bit keys: 5 digits 157-181 / 324-281, a digit less about 47 less; with
 //     32-bit payloads 249-274 / 426-370, a digit 63; with 64-bit ones 281-305 / 659-611.
+// c equal keys per value in all four digits (eight), where more of them crowd
+// some bin, buckets / radix passes behind the sample: 14.7M keys c = 12 228 /
+// 240, 14 254 / 240; pairs 12 325 / 362, 14 355 / 362; 64-bit payloads 14 419 /
+// 457, 16 475 / 460; 64-bit keys 20 665 / 740, 2.5M 147 / 215.
 SampleRule hyb_rule(uint64_t n, int kb, int vb) {
   const bool large = n > uint64_t(1) << 22;
-  if (kb == 4) return SampleRule{vb == 0 ? 1u : vb == 4 || large ? 4u : n > uint64_t(1) << 19 ? 3u : 1u, vb == 8 && !large ? 16u : 8u};
-  return SampleRule{!large || vb == 8 ? 1u : vb == 4 ? 4u : 3u, 8u};
+  // up to 2^16 keys of 64 bits, or with 64-bit payloads, any number: eight passes
+  // of launches are slower than crowded blocks (50,000 keys of 1,000 values 55 / 102)
+  const uint32_t wide_dups = n <= uint64_t(1) << 16 ? 1u << 16 : kb == 8 ? 20u : 16u;
+  if (kb == 4)
+    return SampleRule{vb == 0 ? 1u : vb == 4 || large ? 4u : n > uint64_t(1) << 19 ? 3u : 1u,
+                      vb == 8 && !large ? 16u : 8u, vb == 8 ? wide_dups : 12u};
+  return SampleRule{!large || vb == 8 ? 1u : vb == 4 ? 4u : 3u, 8u, wide_dups};
 }
 // The same for the sorts of one launch.  Keys alone gain or lose little with
 // two digits (277,635 keys 24.5 / 26.6, 50,000 23 / 22), pairs lose: 277,635
 // 33-47 / 29 (three digits 30.6 / 37.5), 2^20 66 / 36 (three 47-49 / 47-48, four 47 / 59).
 // The largest tiles' pairs lose with any (2.5M: 92 / 86): not offered.
+// c equal keys per value: 2^20 keys c = 10 45 / 43, 12 46 / 43, 50,000 keys 10 19
+// / 26, 12 31 / 26; 277,635 pairs 8 31 / 37, 10 46 / 37, 2^20 pairs 6 47 / 51, 8 67 / 51.
 SampleRule fused_rule(bool pairs, int shape) {
-  return SampleRule{!pairs ? 1u : shape == 1 ? 4u : 3u, 16u};
+  const uint32_t dups = !pairs ? 10u : shape == 1 ? 5u : 7u;
+  return SampleRule{!pairs ? 1u : shape == 1 ? 4u : 3u, dups, dups};
 }
 
 struct Layout {
@@ -461,7 +479,7 @@ Layout make_layout(const SortPlan& p, uint64_t n, bool pairs, int hybrid_vb = -1
   L.status_bytes = std::max(p.status_rows, p.num_tiles) * row_bytes;
   off = align_up(off + std::max(L.status_bytes, p.held_rows * row_bytes));
   if (hybrid) off = L.hyb.place_rest(off);
-  else if (hybrid_vb >= 0 && n >= kHybridMinKeys) off += HybLayout::most_bytes(4, hybrid_vb);
+  else if (hybrid_vb >= 0 && n >= HybLayout::fewest(4, hybrid_vb)) off += HybLayout::most_bytes(4, hybrid_vb);
   if (fused) {
     L.fctrl = off;
     off += align_up(sizeof(HybCtrl));
@@ -1082,7 +1100,7 @@ Layout64 make_layout64(const SortPlan& p, uint64_t n, int vbytes) {
   L.bases = off;
   off = align_up(off + 8 * 256 * 4);
   if (hybrid) off = L.hyb.place_rest(off);
-  else if (n >= kHybridMinKeys) off += HybLayout::most_bytes(8, vbytes);
+  else if (n >= HybLayout::fewest(8, vbytes)) off += HybLayout::most_bytes(8, vbytes);
   L.status = off;
   L.status_bytes = p.num_tiles * 256 * (p.k->wide_status ? 8 : 4);
   off = align_up(off + std::max(L.status_bytes, p.held_rows * 1024));

@@ -320,7 +320,8 @@ cudaError_t launch_join64(const WideArgs& a, unsigned grid, cudaStream_t s);
 // What the sample of a sort asks of its keys beyond an even spread (sample.cuh).
 struct SampleRule {
   uint32_t min_digits;   // bytes in which the keys differ, at least: fewer radix passes are faster
-  uint32_t narrow_dups;  // equal keys per value, at most, of keys that differ in three bytes or less (otherwise 16)
+  uint32_t narrow_dups;  // equal keys per value, at most, of keys that differ in three bytes or less
+  uint32_t dups;         // and of others
 };
 
 // A whole sort of up to a few million keys in one cooperative launch

@@ -171,10 +171,10 @@ __device__ __forceinline__ void sample_body(const K* in, uint64_t n, uint32_t bu
 #pragma unroll
   for (int i = 0; i < int(sizeof(K)); ++i) digits += ((words[i / 4] >> (8 * (i % 4))) & 0xffu) != 0u;
   if (digits < rule.min_digits) bad = true;
-  // equal keys per value of about c among n keys give S^2 c / (2 n) such
-  // pairs in the sample; c = 16 is what the bins still take well
-  const uint32_t c = digits <= 3 ? rule.narrow_dups : 16u;
-  if (uint64_t(dups) * n > uint64_t(L::S) * L::S * c / 2 + 8 * n) bad = true;
+  // n keys of n / c values give the sample S / (n / c) of each on average, and
+  // as many duplicates as it has keys beyond the values that it meets
+  const float values = float(n) / float(digits <= 3 ? rule.narrow_dups : rule.dups);
+  if (float(dups) > float(L::S) + values * expm1f(-float(L::S) / values) + 4.0f) bad = true;
   if (tid == 0) {
     HybCtrl* c = ctrl;
     c->lo = m.lo;
