@@ -412,6 +412,19 @@ rs_status rs_trace_read(rs_trace_entry* out, uint32_t capacity, uint32_t* count)
  * reports RS_ERR_TIMEOUT and the context stays usable.                     */
 rs_status rs_selftest_wait_timeout(void* temp, size_t temp_bytes, rs_stream_t stream);
 
+/* Self-test of the routes: which way the last sort with the automatic plan
+ * that used temp (DEVICE) went, for n keys of key_bytes (4, 8) and payloads of
+ * val_bytes (0: none, 4, 8), as the sort was called.  The route is chosen on
+ * the device, and every route gives the same result, so only this tells.
+ * *h_route: RS_ROUTE_FIXED (sizes without a choice: one block, or the radix
+ * passes), RS_ROUTE_RADIX (the sample chose the radix passes),
+ * RS_ROUTE_BUCKETS (value buckets), RS_ROUTE_OVERFULL (the sample chose the
+ * buckets, one of them held too many keys, and the radix passes took over).
+ * Waits for `stream`.                                                       */
+enum { RS_ROUTE_FIXED = 0, RS_ROUTE_RADIX = 1, RS_ROUTE_BUCKETS = 2, RS_ROUTE_OVERFULL = 3 };
+rs_status rs_selftest_route(uint32_t key_bytes, uint32_t val_bytes, uint64_t n, const void* temp,
+                            uint32_t* h_route, rs_stream_t stream);
+
 /* Library version as MAJOR * 10000 + MINOR * 100 + PATCH. */
 uint32_t rs_version(void);
 

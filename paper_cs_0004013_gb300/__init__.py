@@ -25,6 +25,7 @@ __all__ = [
     "rs_sort_u32", "rs_sort_u32_pairs", "rs_sort_u32_segmented", "rs_digit_histograms",
     "rs_radix_pass", "rs_last_error", "rs_check_device_error", "rs_peek_device_error_async", "rs_version", "rs_trace_enable",
     "rs_trace_read", "rs_sort_u32_noalloc", "RS_NOALLOC_MAX_KEYS", "rs_selftest_wait_timeout",
+    "rs_selftest_route", "RS_ROUTE_FIXED", "RS_ROUTE_RADIX", "RS_ROUTE_BUCKETS", "RS_ROUTE_OVERFULL",
     "rs_sort_u32_host", "rs_sort_u64", "sort64", "rs_sort_u64_pairs", "rs_sort_u64_pairs64", "sort64_pairs", "rs_sort_u32_pairs64", "sort_pairs64", "rs_merge_u32", "merge",
     "sort", "sort_pairs", "sort_segmented", "temp_bytes",
     "STATUS_NAMES", "RS_MODE_AUTO", "RS_MODE_LSD", "RS_MODE_MSD", "RS_KEY_U32", "RS_KEY_I32", "RS_KEY_F32",
@@ -38,6 +39,8 @@ RS_MODE_AUTO, RS_MODE_LSD, RS_MODE_MSD = 0, 1, 2
 # key kinds (rs_plan.key_kind): how 32-bit key words are ordered
 RS_KEY_U32, RS_KEY_I32, RS_KEY_F32 = 0, 1, 2
 RS_NOALLOC_MAX_KEYS = 1 << 20
+# rs_selftest_route
+RS_ROUTE_FIXED, RS_ROUTE_RADIX, RS_ROUTE_BUCKETS, RS_ROUTE_OVERFULL = 0, 1, 2, 3
 
 
 class RsError(RuntimeError):
@@ -82,6 +85,7 @@ _SIGS = {
     "rs_merge_u32": [_P, _P, _U64, _P, _P, _U64, _P, _P, _U32, _U64P, _PLANP, _P, _SZP, _P],
     "rs_sort_u32_noalloc": [_P, _P, _U64, _U32, _U64P, _P],
     "rs_selftest_wait_timeout": [_P, ctypes.c_size_t, _P],
+    "rs_selftest_route": [_U32, _U32, _U64, _P, _P, _P],
     "rs_trace_read": [ctypes.POINTER(RsTraceEntry), _U32, ctypes.POINTER(ctypes.c_uint32)],
     "rs_set_default_plan": [_U32, _U32, _PLANP],
     "rs_sample_overlap": [_P, _U64, _U32, _U32, _U32, _U32, _U32, _P, ctypes.POINTER(ctypes.c_uint32), _P],
@@ -390,6 +394,14 @@ def rs_peek_device_error_async(h_word, stream=None) -> None:
 def rs_selftest_wait_timeout(temp, stream=None) -> None:
     """Runs the bounded-wait self-test (see include/rsort.h)."""
     _check(lib.rs_selftest_wait_timeout(_ptr(temp), temp.numel() * temp.element_size(), _stream(stream)))
+
+
+def rs_selftest_route(key_bytes: int, val_bytes: int, n: int, temp, stream=None) -> int:
+    """Calls rs_selftest_route; returns the route (RS_ROUTE_...) of the last
+    automatic sort of n such keys that used temp."""
+    route = ctypes.c_uint32(0)
+    _check(lib.rs_selftest_route(key_bytes, val_bytes, n, _ptr(temp), ctypes.byref(route), _stream(stream)))
+    return route.value
 
 
 def rs_trace_enable(on: bool = True) -> None:

@@ -926,6 +926,17 @@ rs_status run_hybrid32(const SortPlan& p, const Layout& L, const uint32_t* keys_
 // histograms, status rows (the layout holds a row per tile of the smallest
 // shape up to kFusedStatusMaxKeys keys) and alternate buffers.
 constexpr uint64_t kFusedStatusMaxKeys = uint64_t(1) << 22;
+// Value buckets that the launch offers (0: none): as many as tiles, twice as many
+// of the largest tiles (whose number may exceed the SMs'), when a block more than
+// tiles, which takes the sample, is resident too.
+uint32_t fused_buckets(const Layout& L, uint32_t tiles, bool pairs, int shape, const DeviceState* ds) {
+  const uint32_t buckets = shape == 0 ? 2 * tiles : tiles;
+  return L.fcounts && buckets >= 2 && buckets <= kFusedMaxBuckets && tiles < ds->fused_tiles[pairs][shape] &&
+                 !(pairs && shape == 0)
+             ? buckets
+             : 0u;
+}
+
 rs_status run_fused(const SortPlan& p, const Layout& L, const uint32_t* keys_in, const uint32_t* vals_in,
                     uint32_t* keys_out, uint32_t* vals_out, uint32_t n, int shape, unsigned char* temp,
                     DeviceState* ds, cudaStream_t s) {
@@ -933,12 +944,7 @@ rs_status run_fused(const SortPlan& p, const Layout& L, const uint32_t* keys_in,
   const uint32_t tiles = (n + fused_tile_keys(shape) - 1) / fused_tile_keys(shape);
   if (size_t(tiles) * 256 * 4 > L.status_bytes) return fail(RS_ERR_CUDA, "single-launch sort: status too small");
   const size_t clear_bytes = L.status;  // (the launch clears its status rows itself)
-  // value buckets: as many as tiles, twice as many of the largest tiles (whose
-  // number may exceed the SMs'), when a block more than tiles, which takes the
-  // sample, is resident too
-  const uint32_t buckets = shape == 0 ? 2 * tiles : tiles;
-  const bool offered = L.fcounts && buckets >= 2 && buckets <= kFusedMaxBuckets &&
-                       tiles < ds->fused_tiles[pairs][shape] && !(pairs && shape == 0);
+  const uint32_t buckets = fused_buckets(L, tiles, pairs, shape, ds);
   HybCtrl* hc = reinterpret_cast<HybCtrl*>(temp + L.fctrl);
   RS_CUDA(traced(T_CLEAR, 0, s, [&] { return cudaMemsetAsync(temp, 0, clear_bytes, s); }), "cudaMemsetAsync(temp)");
   FusedArgs a{};
@@ -955,7 +961,7 @@ rs_status run_fused(const SortPlan& p, const Layout& L, const uint32_t* keys_in,
   a.first_cursors = reinterpret_cast<uint32_t*>(temp + L.cursors0);
   a.bar = reinterpret_cast<uint32_t*>(temp + L.ctrl) + 12;
   a.err = ds->err;
-  if (offered) {
+  if (buckets) {
     a.ctrl = hc;
     a.rule = fused_rule(pairs, shape);
     a.buckets = buckets;
@@ -964,6 +970,44 @@ rs_status run_fused(const SortPlan& p, const Layout& L, const uint32_t* keys_in,
   }
   RS_CUDA(traced(T_FUSED, n, s, [&] { return launch_fused(a, tiles, pairs, shape, s); }), "launch fused sort");
   return RS_OK;
+}
+
+// The plan and the layout of a 32-bit sort (keys, or key + uint32 payload).
+struct Sort32 {
+  SortPlan p;
+  Layout L;
+  bool automatic = false, fusable = false, hybrid = false;
+};
+rs_status plan_sort32(uint64_t n, bool pairs, const rs_plan* plan, Sort32* out) {
+  Sort32& o = *out;
+  SortPlan& p = o.p;
+  if (rs_status st = make_plan(n, pairs, plan, &p); st != RS_OK) return st;
+  o.automatic = plan->digit_bits == 0 && plan->mode == RS_MODE_AUTO && plan->tile == 0;
+  o.fusable = o.automatic && p.R == 8 && p.nd == 4 && !p.msd && !p.k->wide_status;
+  const bool spaced = o.automatic && p.R == 8 && !p.msd;  // with the other routes' space, whatever n
+  if (spaced) {  // status rows for the single-launch sort's smallest tiles
+    const uint32_t tile = fused_tile_keys(kFusedShapes - 1);
+    p.held_rows = size_t((std::min(n, kFusedStatusMaxKeys) + tile - 1) / tile);
+    if (n <= kFusedStatusMaxKeys) p.status_rows = p.held_rows;
+  }
+  o.L = make_layout(p, n, pairs, spaced ? (pairs ? 4 : 0) : -1, spaced);
+  o.hybrid = o.fusable && o.L.hyb.buckets;
+  return RS_OK;
+}
+
+// The single launch's tile shape for n keys (-1: it does not take them).  The
+// smallest whose tiles number fewer than the SMs (one is left to the sampling
+// block), else the largest.
+int fused_shape(const Sort32& o, uint64_t n, bool pairs, const DeviceState* ds) {
+  if (!o.fusable) return -1;
+  int sh = 0;
+  for (int c = kFusedShapes - 1; c > 0; --c)
+    if ((n + fused_tile_keys(c) - 1) / fused_tile_keys(c) < uint64_t(ds->num_sms)) {
+      sh = c;
+      break;
+    }
+  const size_t tiles = (n + fused_tile_keys(sh) - 1) / fused_tile_keys(sh);
+  return tiles <= ds->fused_tiles[pairs ? 1 : 0][sh] && tiles * 1024 <= o.L.status_bytes ? sh : -1;
 }
 
 rs_status sort_impl(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* keys_out, uint32_t* vals_out,
@@ -975,19 +1019,10 @@ rs_status sort_impl(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* 
   rs_status st = check_common(keys_in, keys_out, n, temp, temp_bytes);
   if (st != RS_OK) return st;
   if (num_parts < 1) return fail(RS_ERR_INVALID, "num_parts must be >= 1");
-  SortPlan p;
-  st = make_plan(n, pairs, plan, &p);
-  if (st != RS_OK) return st;
-  const bool automatic = plan->digit_bits == 0 && plan->mode == RS_MODE_AUTO && plan->tile == 0;
-  const bool fusable = automatic && p.R == 8 && p.nd == 4 && !p.msd && !p.k->wide_status;
-  const bool spaced = automatic && p.R == 8 && !p.msd;  // with the other routes' space, whatever n
-  if (spaced) {  // status rows for the single-launch sort's smallest tiles
-    const uint32_t tile = fused_tile_keys(kFusedShapes - 1);
-    p.held_rows = size_t((std::min(n, kFusedStatusMaxKeys) + tile - 1) / tile);
-    if (n <= kFusedStatusMaxKeys) p.status_rows = p.held_rows;
-  }
-  Layout L = make_layout(p, n, pairs, spaced ? (pairs ? 4 : 0) : -1, spaced);
-  const bool hybrid = fusable && L.hyb.buckets;
+  Sort32 o;
+  if ((st = plan_sort32(n, pairs, plan, &o)) != RS_OK) return st;
+  SortPlan& p = o.p;
+  Layout& L = o.L;
   MsdLayout M;
   if (p.msd) {
     if (rs_status st2 = make_msd_layout(p, n, pairs, &M); st2 != RS_OK) return st2;
@@ -1029,7 +1064,7 @@ rs_status sort_impl(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* 
   // memory by one launch (no histogram, scans or tiled passes), which is
   // several times faster for such sizes.
   const SegKernels* sk = seg_kernels();
-  if (automatic && n <= sk->small_max) {
+  if (o.automatic && n <= sk->small_max) {
     LocalArgs la{};
     la.kin = keys_in;
     la.kout = keys_out;
@@ -1043,22 +1078,11 @@ rs_status sort_impl(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* 
     return RS_OK;
   }
   // Up to a few million keys: every tile resident at once, the whole sort in
-  // one launch (8-bit digits, the same passes).  The tile shape: the smallest
-  // whose tiles number fewer than the SMs (one is left to the sampling block),
-  // else the largest.
-  if (fusable) {
-    int sh = 0;
-    for (int c = kFusedShapes - 1; c > 0; --c)
-      if ((n + fused_tile_keys(c) - 1) / fused_tile_keys(c) < uint64_t(ds->num_sms)) {
-        sh = c;
-        break;
-      }
-    const size_t tiles = (n + fused_tile_keys(sh) - 1) / fused_tile_keys(sh);
-    if (tiles <= ds->fused_tiles[pairs ? 1 : 0][sh] && tiles * 1024 <= L.status_bytes)
-      return run_fused(p, L, keys_in, pairs ? vals_in : nullptr, keys_out, pairs ? vals_out : nullptr, uint32_t(n),
-                       sh, static_cast<unsigned char*>(temp), ds, s);
-  }
-  if (hybrid)
+  // one launch (8-bit digits, the same passes).
+  if (const int sh = fused_shape(o, n, pairs, ds); sh >= 0)
+    return run_fused(p, L, keys_in, pairs ? vals_in : nullptr, keys_out, pairs ? vals_out : nullptr, uint32_t(n), sh,
+                     static_cast<unsigned char*>(temp), ds, s);
+  if (o.hybrid)
     return run_hybrid32(p, L, keys_in, pairs ? vals_in : nullptr, keys_out, pairs ? vals_out : nullptr, uint32_t(n),
                         static_cast<unsigned char*>(temp), ds, s);
   return run_lsd(p, L, keys_in, pairs ? vals_in : nullptr, keys_out, pairs ? vals_out : nullptr, uint32_t(n),
@@ -1294,6 +1318,36 @@ rs_status rs_sort_u32_pairs(const uint32_t* keys_in, const uint32_t* vals_in, ui
                    reinterpret_cast<cudaStream_t>(stream), true);
 }
 
+// The plan and the layout of a sort of 64-bit keys; vbytes as below.
+struct Sort64 {
+  SortPlan p;
+  Layout64 L;
+  bool automatic = false;
+};
+static rs_status plan_sort64(uint64_t n, int vbytes, const rs_plan* plan, Sort64* out) {
+  rs_plan q = plan ? *plan : rs_plan{0, 0, 0, 0};
+  q.digit_bits = 8;
+  q.mode = RS_MODE_LSD;
+  q.key_kind = RS_KEY_U32;
+  // the shapes with interleaved-word pass kernels: 384 x 24 (three blocks per
+  // SM) for keys alone above 2^22 keys (GB300, 2^26 keys: 335 us per pass
+  // against 349 at 512 x 24; 2^23: 20.0 against 18.7 Gkeys/s), else 512 x 16
+  // (the one with 64-bit status words and two payload words)
+  constexpr uint64_t kSmallTileMax = uint64_t(1) << 22;
+  const bool own_tile = q.tile != 0;
+  if (!own_tile) q.tile = (vbytes == 0 && n > kSmallTileMax && !needs_wide_status(n)) ? 8u : 1u;
+  SortPlan& p = out->p;
+  if (rs_status st = make_plan(n, true, &q, &p, vbytes != 0 ? 2 : 1); st != RS_OK) return st;
+  out->automatic = !plan || (plan->digit_bits == 0 && plan->mode == RS_MODE_AUTO && plan->tile == 0);
+  if (!own_tile && n > kSmallTileMax) p.held_rows = size_t(kSmallTileMax / (512 * 16));  // tile 1 takes more rows than 8
+  // (the space for value buckets is part of every plan's layout)
+  out->L = make_layout64(p, n, vbytes);
+  if (!out->automatic) out->L.hyb.buckets = 0;
+  if (vbytes == 8 && !out->L.fused)
+    return fail(RS_ERR_UNSUPPORTED, "64-bit values: tile shape %u has no interleaved pass kernel", q.tile);
+  return RS_OK;
+}
+
 // vbytes: 0 (keys only), 4 (uint32 values) or 8 (uint64 values).
 static rs_status sort64_impl(const uint64_t* keys_in, const void* vals_in, uint64_t* keys_out, void* vals_out,
                              uint64_t n, uint32_t num_parts, uint64_t* h_part_offsets, const rs_plan* plan,
@@ -1309,26 +1363,10 @@ static rs_status sort64_impl(const uint64_t* keys_in, const void* vals_in, uint6
   if (plan && plan->mode == RS_MODE_MSD) return fail(RS_ERR_UNSUPPORTED, "64-bit keys use the LSD plan");
   KeyXform64 x;
   if (rs_status st = key_xform64(plan, &x); st != RS_OK) return st;
-  rs_plan q = plan ? *plan : rs_plan{0, 0, 0, 0};
-  q.digit_bits = 8;
-  q.mode = RS_MODE_LSD;
-  q.key_kind = RS_KEY_U32;
-  // the shapes with interleaved-word pass kernels: 384 x 24 (three blocks per
-  // SM) for keys alone above 2^22 keys (GB300, 2^26 keys: 335 us per pass
-  // against 349 at 512 x 24; 2^23: 20.0 against 18.7 Gkeys/s), else 512 x 16
-  // (the one with 64-bit status words and two payload words)
-  constexpr uint64_t kSmallTileMax = uint64_t(1) << 22;
-  const bool own_tile = q.tile != 0;
-  if (!own_tile) q.tile = (vbytes == 0 && n > kSmallTileMax && !needs_wide_status(n)) ? 8u : 1u;
-  SortPlan p;
-  if (rs_status st = make_plan(n, true, &q, &p, pairs ? 2 : 1); st != RS_OK) return st;
-  const bool automatic = !plan || (plan->digit_bits == 0 && plan->mode == RS_MODE_AUTO && plan->tile == 0);
-  if (!own_tile && n > kSmallTileMax) p.held_rows = size_t(kSmallTileMax / (512 * 16));  // tile 1 takes more rows than 8
-  // (the space for value buckets is part of every plan's layout)
-  Layout64 L = make_layout64(p, n, vbytes);
-  if (!automatic) L.hyb.buckets = 0;
-  if (vbytes == 8 && !L.fused)
-    return fail(RS_ERR_UNSUPPORTED, "64-bit values: tile shape %u has no interleaved pass kernel", q.tile);
+  Sort64 o;
+  if (rs_status st = plan_sort64(n, vbytes, plan, &o); st != RS_OK) return st;
+  const SortPlan& p = o.p;
+  const Layout64& L = o.L;
   if (!temp) {
     *temp_bytes = L.total;
     return RS_OK;
@@ -1358,7 +1396,7 @@ static rs_status sort64_impl(const uint64_t* keys_in, const void* vals_in, uint6
   if (n == 0) return RS_OK;
   DeviceState* ds = nullptr;
   if (rs_status st = device_state(&ds); st != RS_OK) return st;
-  if (automatic && n <= local_max_keys(8, vbytes)) {  // one block
+  if (o.automatic && n <= local_max_keys(8, vbytes)) {  // one block
     LocalArgs la{};
     la.kin = keys_in;
     la.kout = keys_out;
@@ -1398,6 +1436,17 @@ rs_status rs_sort_u64_pairs64(const uint64_t* keys_in, const uint64_t* vals_in, 
                      stream, 8);
 }
 
+// The plan and the key + payload part of the layout of 32-bit keys with 64-bit values.
+static rs_status plan_pairs64(uint64_t n, const rs_plan* plan, bool automatic, SortPlan* p, Layout* L) {
+  rs_plan q = plan ? *plan : rs_plan{0, 0, 0, 0};
+  q.digit_bits = 8;
+  q.mode = RS_MODE_LSD;
+  if (q.tile == 0) q.tile = 1;  // the shape with two-payload-word pass kernels
+  if (rs_status st = make_plan(n, true, &q, p, 2); st != RS_OK) return st;
+  *L = make_layout(*p, n, true, automatic ? 8 : -1);
+  return RS_OK;
+}
+
 rs_status rs_sort_u32_pairs64(const uint32_t* keys_in, const uint64_t* vals_in, uint32_t* keys_out,
                               uint64_t* vals_out, uint64_t n, uint32_t num_parts, uint64_t* h_part_offsets,
                               const rs_plan* plan, void* temp, size_t* temp_bytes, rs_stream_t stream) {
@@ -1408,19 +1457,15 @@ rs_status rs_sort_u32_pairs64(const uint32_t* keys_in, const uint64_t* vals_in, 
   if (num_parts < 1) return fail(RS_ERR_INVALID, "num_parts must be >= 1");
   if (plan && plan->mode == RS_MODE_MSD) return fail(RS_ERR_UNSUPPORTED, "64-bit values use the LSD plan");
   if (plan && plan->digit_bits && plan->digit_bits != 8) return fail(RS_ERR_UNSUPPORTED, "64-bit values use 8-bit digits");
-  rs_plan q = plan ? *plan : rs_plan{0, 0, 0, 0};
-  q.digit_bits = 8;
-  q.mode = RS_MODE_LSD;
-  if (q.tile == 0) q.tile = 1;  // the shape with two-payload-word pass kernels
   SortPlan p;
-  if ((st = make_plan(n, true, &q, &p, 2)) != RS_OK) return st;
+  Layout L;
+  const bool automatic = !plan || (plan->digit_bits == 0 && plan->mode == RS_MODE_AUTO && plan->tile == 0);
+  if ((st = plan_pairs64(n, plan, automatic, &p, &L)) != RS_OK) return st;
   // the sort's own layout (keys, the low value words as the first payload
   // plane) followed by the value planes: low and high words of the output,
   // the high words' alternate plane and (split only) both words of the input.
   // A tiled pass kernel reads and writes the interleaved values itself
   // (fused); a persistent one takes planes split and joined by kernels.
-  const bool automatic = !plan || (plan->digit_bits == 0 && plan->mode == RS_MODE_AUTO && plan->tile == 0);
-  Layout L = make_layout(p, n, true, automatic ? 8 : -1);
   const bool hybrid = L.hyb.buckets != 0;
   const bool fused = pair_io_kernel(p.k) != nullptr;
   const int nplanes = fused ? 3 : 5;
@@ -1923,6 +1968,51 @@ rs_status rs_selftest_wait_timeout(void* temp, size_t temp_bytes, rs_stream_t st
   const cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   RS_CUDA(cudaMemsetAsync(temp, 0, 4096, s), "cudaMemsetAsync(self-test)");
   RS_CUDA(launch_lookback_timeout(static_cast<const uint32_t*>(temp), ds->err, s), "launch self-test");
+  return RS_OK;
+}
+
+rs_status rs_selftest_route(uint32_t key_bytes, uint32_t val_bytes, uint64_t n, const void* temp, uint32_t* h_route,
+                            rs_stream_t stream) {
+  g_last_error.clear();
+  if (!temp || !h_route) return fail(RS_ERR_INVALID, "NULL temp or output");
+  if ((key_bytes != 4 && key_bytes != 8) || (val_bytes != 0 && val_bytes != 4 && val_bytes != 8))
+    return fail(RS_ERR_INVALID, "keys of 4 or 8 bytes, values of 0, 4 or 8 (got %u, %u)", key_bytes, val_bytes);
+  if (n >= (uint64_t(1) << 32)) return fail(RS_ERR_INVALID, "n must be below 2^32");
+  DeviceState* ds = nullptr;
+  rs_status st = device_state(&ds);
+  if (st != RS_OK) return st;
+  *h_route = RS_ROUTE_FIXED;
+  size_t ctrl = 0;  // (no layout starts with it)
+  if (key_bytes == 8) {
+    Sort64 o;
+    if ((st = plan_sort64(n, int(val_bytes), nullptr, &o)) != RS_OK) return st;
+    if (o.L.hyb.buckets && n > local_max_keys(8, int(val_bytes))) ctrl = o.L.hyb.ctrl;
+  } else if (val_bytes == 8) {
+    SortPlan p;
+    Layout L;
+    if ((st = plan_pairs64(n, nullptr, true, &p, &L)) != RS_OK) return st;
+    if (L.hyb.buckets && n > local_max_keys(4, 8)) ctrl = L.hyb.ctrl;
+  } else {
+    const bool pairs = val_bytes != 0;
+    const rs_plan eff = resolve_plan(pairs ? RS_ENTRY_SORT_U32_PAIRS : RS_ENTRY_SORT_U32, n, nullptr);
+    Sort32 o;
+    if ((st = plan_sort32(n, pairs, &eff, &o)) != RS_OK) return st;
+    if (n > seg_kernels()->small_max) {
+      if (const int sh = fused_shape(o, n, pairs, ds); sh >= 0) {
+        const uint32_t tiles = uint32_t((n + fused_tile_keys(sh) - 1) / fused_tile_keys(sh));
+        if (fused_buckets(o.L, tiles, pairs, sh, ds)) ctrl = o.L.fctrl;
+      } else if (o.hybrid) {
+        ctrl = o.L.hyb.ctrl;
+      }
+    }
+  }
+  if (!ctrl) return RS_OK;
+  const cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  HybCtrl c;
+  RS_CUDA(cudaMemcpyAsync(&c, static_cast<const unsigned char*>(temp) + ctrl, sizeof(c), cudaMemcpyDeviceToHost, s),
+          "read the sample's choice");
+  RS_CUDA(cudaStreamSynchronize(s), "cudaStreamSynchronize");
+  *h_route = c.over ? RS_ROUTE_OVERFULL : c.route == kHybBuckets ? RS_ROUTE_BUCKETS : RS_ROUTE_RADIX;
   return RS_OK;
 }
 

@@ -17,7 +17,8 @@ struct HybCtrl {
   uint32_t route;
   uint32_t done;       // count blocks that have finished
   uint32_t tiles_b;    // tiles of the second split
-  uint32_t reserved[7];
+  uint32_t over;       // a bucket did not fit the local sort: the radix passes took over
+  uint32_t reserved[6];
 };
 static_assert(sizeof(HybCtrl) == 64, "one cache line or less");
 
