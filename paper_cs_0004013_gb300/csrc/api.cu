@@ -606,7 +606,7 @@ rs_status run_lsd(const SortPlan& p, const Layout& L, const uint32_t* keys_in, c
   RS_CUDA(traced(T_HIST, n, s, [&] { return hk->launch(ha, hgrid, s); }), "launch upfront_hist");
 
   if (!scans) {
-    ScanArgs sa{hist, bases, force_all ? nullptr : ctrl + 4, n, gate};
+    ScanArgs sa{hist, bases, force_all ? nullptr : ctrl + 4, n};  // (a sort with a gate has byte digits)
     RS_CUDA(traced(T_SCAN, 0, s, [&] { return scan_kernel(p.R)->launch(sa, unsigned(p.nd), s); }),
             "launch digit_scan");
   }
@@ -1223,7 +1223,7 @@ rs_status run_lsd64(const SortPlan& p, const Layout64& L, const uint64_t* keys_i
     RS_CUDA(traced(T_HIST, n, s, [&] { return hk->launch(ha, hgrid, s); }), "launch upfront_hist");
   }
   if (!L.fused) {
-    ScanArgs sa{hist, bases, ctrl + 8, n, nullptr};
+    ScanArgs sa{hist, bases, ctrl + 8, n};
     RS_CUDA(traced(T_SCAN, 0, s, [&] { return scan_kernel(8)->launch(sa, 8u, s); }), "launch digit_scan");
   }
   for (int j = 0; j < 8; ++j) {
@@ -1759,7 +1759,7 @@ rs_status rs_digit_histograms(const uint32_t* keys, uint64_t n, uint32_t digit_b
   if (d_bases || d_skip) {
     uint32_t* b = d_bases;
     if (!b) return fail(RS_ERR_INVALID, "d_skip needs d_bases");
-    ScanArgs sa{d_hist, b, d_skip, uint32_t(n), nullptr};
+    ScanArgs sa{d_hist, b, d_skip, uint32_t(n)};
     RS_CUDA(traced(T_SCAN, 0, s, [&] { return scan_kernel(int(digit_bits))->launch(sa, unsigned(ha.num_digits), s); }),
             "launch digit_scan");
   }

@@ -53,9 +53,9 @@ constexpr int kFusedThreads = 384;
 constexpr int kFusedItems[kFusedShapes] = {24, 20, 12};
 // (The smaller shapes run one tile per SM.)
 constexpr int fused_min_blocks(int items) { return items <= 20 ? 1 : 2; }
-// Status rows a digit thread reads per lookback round (GB300, 2^20 keys in
-// 152 tiles of 384 x 18: the kernel takes 44.7 us with 8 rows per round,
-// 47.8 with 16 and 62.1 with 32).
+// Status rows a digit thread reads per lookback round (GB300, clustered data: 2^20
+// keys 42.7 us with 8 rows per round, 44.3 with 16 and 44.3 with 32, 2.5M pairs
+// in 272 tiles of 384 x 24 78, 82 and 95).
 constexpr int kFusedLookback = 8;
 // Rounds of a barrier wait (about 64 ns each) before it gives up.
 constexpr uint32_t kBarrierSpinLimit = 1u << 21;

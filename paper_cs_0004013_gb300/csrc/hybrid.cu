@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(THREADS, MINB) bucket_sort_kernel(const HybArg
     // A key's distance from its bucket's first possible key and its place
     // share a word when they fit: half the work of ordering them side by side.
     constexpr int PBITS = THREADS * ITEMS <= 2048 ? 11 : 12;
-    static_assert(THREADS * ITEMS < (1 << 12), "a place's bits");
+    static_assert(THREADS * ITEMS <= (1 << PBITS), "a place's bits");
     const uint64_t step = 0xffffffffull / m.mult + 1;  // offsets per bucket, at most
     const uint64_t t0 = ((uint64_t(b) << 32) + m.mult - 1) / m.mult;  // the bucket's first offset
     const int bits = 64 - __clzll((long long)step) + int(m.sh);

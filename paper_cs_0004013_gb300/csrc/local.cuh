@@ -93,7 +93,8 @@ struct ElemOf<uint64_t, true> {
 
 // (key, place) of keys from one narrow range in a single word: the key's
 // distance from the range's start above the place's PBITS bits.  The caller
-// makes sure that it fits.
+// makes sure that it fits.  (Where a block takes 2^PBITS keys, the last place of
+// the largest distance is the padding's word: either may be written for the other.)
 template <typename K, int PBITS>
 struct PackedElem {
   using E = K;
@@ -101,7 +102,7 @@ struct PackedElem {
   __device__ __forceinline__ E make(K k, uint32_t i) const { return ((k - base) << PBITS) | K(i); }
   __device__ __forceinline__ K key(E e) const { return base + (e >> PBITS); }
   __device__ __forceinline__ uint32_t place(E e) const { return uint32_t(e) & ((1u << PBITS) - 1u); }
-  __device__ __forceinline__ E last() const { return ~K(0); }  // (no key has the place of all ones)
+  __device__ __forceinline__ E last() const { return ~K(0); }
 };
 
 __device__ __forceinline__ void order2(uint32_t& a, uint32_t& b) {

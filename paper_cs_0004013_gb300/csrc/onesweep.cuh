@@ -656,9 +656,11 @@ __device__ __forceinline__ uint32_t begin_tile(uint32_t* counter, unsigned char*
 }
 
 // The plain pass: tile i covers keys [i * TILE, (i + 1) * TILE) of one array.
-template <int R, int THREADS, int ITEMS, int NV, typename S, bool EARLY_LB, bool PIO>
-__device__ __forceinline__ void onesweep_pass(const PassArgs& a, unsigned char* smem) {
+template <int R, int THREADS, int ITEMS, int NV, typename S, int MINB, bool EARLY_LB, bool PIO>
+__global__ void __launch_bounds__(THREADS, MINB) onesweep_kernel(const PassArgs a) {
   using L = OnesweepLayout<R, THREADS, ITEMS, NV>;
+  extern __shared__ __align__(16) unsigned char smem[];
+  if (gated_off(a.gate)) return;
   const Route route = route_of(a.skip, a.pass, a.num_passes);
   if (!route.active) return;
   const uint32_t* kin = route.src == BUF_IN ? a.keys_in : (route.src == BUF_OUT ? a.keys_out : a.keys_alt);
@@ -699,13 +701,6 @@ __device__ __forceinline__ void onesweep_pass(const PassArgs& a, unsigned char* 
                                                         reinterpret_cast<S*>(a.status), route.parity, a.err,
                                                         route.src == BUF_IN ? a.xin : KeyXform{0u, 0u},
                                                         route.last ? a.xout : KeyXform{0u, 0u}, smem);
-}
-
-template <int R, int THREADS, int ITEMS, int NV, typename S, int MINB, bool EARLY_LB, bool PIO>
-__global__ void __launch_bounds__(THREADS, MINB) onesweep_kernel(const PassArgs a) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  if (gated_off(a.gate)) return;
-  onesweep_pass<R, THREADS, ITEMS, NV, S, EARLY_LB, PIO>(a, smem);
 }
 
 template <int R, int THREADS, int ITEMS, int NV, typename S, int MINB, bool EARLY_LB, bool PIO>

@@ -86,7 +86,7 @@ struct HistArgs {
   // launch_hist64 only: interleaved 64-bit keys and their order map
   const uint2* keys64;
   KeyXform64 x64;
-  const uint32_t* gate;  // null or the device's choice (kGateRadix: run)
+  const uint32_t* gate;  // byte digits: null or the device's choice (kGateRadix: run)
   // Byte digits: with `done` (a zeroed word) the last block also scans the
   // histograms (ScanArgs' outputs; cursors: a copy of the first digit's bases).
   uint32_t* done;
@@ -101,7 +101,6 @@ struct ScanArgs {
   uint32_t* bases;       // [num_digits][2^R]
   uint32_t* skip;        // [num_digits] (may be null)
   uint32_t n;
-  const uint32_t* gate;
 };
 
 // One onesweep LSD pass.

@@ -37,7 +37,7 @@ struct SplitLayout {
   static constexpr size_t OFF_SCAN = OFF_GOFF + 256 * 4;
   static constexpr size_t OFF_JOB = OFF_SCAN + 32 * 4;
   static constexpr size_t SMEM = OFF_JOB + 16;
-  static_assert(THREADS >= 256 && true, "a thread per digit");
+  static_assert(THREADS >= 256, "a thread per digit");
 };
 
 // The tile's keys in[0, valid) (FULL: valid is the tile's size), mapped by

@@ -173,3 +173,46 @@ def test_two_streams_at_once():
             s.run(streams[i % 2])
     for s, data in zip(sorts, ("even", "clusters", "even", "even")):
         s.check(s.rs.RS_ROUTE_RADIX if data == "clusters" else s.rs.RS_ROUTE_BUCKETS)
+
+
+def _fill_one_bucket(w, bits, mean, count):
+    """w with keys from elsewhere moved into a middle bucket until it holds `count`, as the sort will
+    see it: the value map of a sample at fixed places, which stay as they are."""
+    n, S = w.size, 8192
+    q = np.arange(S, dtype=np.uint64)
+    m32 = np.uint64(0xFFFFFFFF)
+    h = (q * np.uint64(0x9E3779B1)) & m32
+    h ^= h >> np.uint64(15)
+    pos = q * np.uint64(n) // np.uint64(S)
+    if n // S > 1:
+        pos = pos + ((((h * np.uint64(0x85EBCA77)) & m32) * np.uint64(n // S)) >> np.uint64(32))
+    pos = pos.astype(np.int64)
+    buckets = -(-n // mean)
+    lo, hi = int(w[pos].min()), int(w[pos].max())
+    ext = (hi - lo) // (S // 8)
+    lo, hi = max(lo - ext, 0), min(hi + ext, (1 << bits) - 1)
+    sh = max((hi - lo).bit_length() - 32, 0)
+    mult = (buckets << 32) // (((hi - lo) >> sh) + 1)
+    x = np.clip(w.astype(np.uint64), np.uint64(lo), np.uint64(hi)) - np.uint64(lo)
+    bucket = ((x >> np.uint64(sh)) * np.uint64(mult)) >> np.uint64(32)
+    b = buckets // 2
+    first, last = -(-(b << 32) // mult), -(-((b + 1) << 32) // mult)  # its offsets: [first, last)
+    need = count - int((bucket == b).sum())
+    free = np.ones(n, bool)
+    free[pos] = False
+    move = np.flatnonzero(free & (bucket != b))[:: 97][:need]
+    assert 0 < need == move.size
+    step = (synth.splitmix64(17, need) % np.uint64((last - first) << sh)) + np.uint64((first << sh) + lo)
+    out = w.copy()
+    out[move] = step.astype(w.dtype)
+    return out
+
+
+@pytest.mark.parametrize("over", [0, 1])
+@pytest.mark.parametrize("bits,vb,n,mean,most", [(32, 0, 3_000_001, 2048, 3072), (32, 8, 1_000_001, 1365, 2048), (64, 0, 1_000_001, 2048, 3072),
+                                                 (64, 4, 1_000_001, 1365, 2048), (64, 8, 3_000_001, 1365, 2048),
+                                                 (32, 4, (1 << 23) + 500_001, 2048, 3072)])
+def test_a_bucket_at_its_most_keys(bits, vb, n, mean, most, over):
+    w = _fill_one_bucket(_words(bits, n, "even"), bits, mean, most + over)
+    s = Sort(bits, vb, n).put(w).run()
+    s.check(s.rs.RS_ROUTE_OVERFULL if over else s.rs.RS_ROUTE_BUCKETS)
