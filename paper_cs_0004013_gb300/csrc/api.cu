@@ -1560,10 +1560,10 @@ rs_status rs_merge_u32(const uint32_t* a, const uint32_t* va, uint64_t na, const
     return fail(RS_ERR_INVALID, "va, vb and vout go together");
   KeyXform x;
   if (rs_status st = key_xform(plan, &x); st != RS_OK) return st;
-  const uint32_t tile = merge_tile_keys(plan ? plan->tile : 0u, pairs);
-  if (tile == 0) return fail(RS_ERR_UNSUPPORTED, "no merge tile shape %u", plan->tile);
-  const size_t tiles = (size_t(n) + tile - 1) / tile;
-  const size_t need = align_up((tiles + 1) * 4);
+  const uint32_t shape = plan ? plan->tile : 0u;
+  const uint32_t tile = merge_tile_keys(shape, n, pairs);
+  if (tile == 0) return fail(RS_ERR_UNSUPPORTED, "no merge tile shape %u", shape);
+  const size_t need = align_up((merge_max_tiles(shape, n, pairs) + 1) * 4);
   if (!temp) {
     *temp_bytes = need;
     return RS_OK;

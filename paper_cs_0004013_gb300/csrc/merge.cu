@@ -17,6 +17,7 @@
 // KeyXform.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "rs_device.cuh"
@@ -314,12 +315,30 @@ cudaError_t launch_tiles(const MergeArgs& m, unsigned tiles, cudaStream_t s) {
 }  // namespace
 
 // Outputs per tile of merge tile shape `shape` (1-based), or 0 if there is
-// no such shape.  Shape 0 picks the measured default, 23 items per thread (two
-// runs of 2^26: 261 us against 281 for 19; with payloads 443 against 466).
-uint32_t merge_tile_keys(uint32_t shape, bool pairs) {
-  const uint32_t idx = shape == 0 ? 2u : shape - 1;
+// no such shape.  Shape 0 picks by the number of outputs: while tiles are few a
+// merge lasts as long as one of them, and short networks are faster; many tiles
+// pay for their boundaries.  Items per thread 11 / 15 / 23, us: keys 1,007 3.1 / 3.5
+// / 3.7, 305,000 5.1 / 5.3 / 5.9, 2.1M 7.5 / 7.5 / 8.0, 5M 12.0 / 11.4 / 11.2, 21.8M 43.1
+// / 41.8 / 38.7; with payloads 20 3.7 / 4.6 / 5.1, 305,000 6.0 / 6.7 / 8.0, 1M 8.0 / 8.0 /
+// 9.8, 5M 21.6 / 19.7 / 20.5, 21.8M 83 / 71.5 / 72.3 (two runs of 2^26: 261 with 23
+// against 281 with 19; with payloads 443 against 466).
+constexpr uint64_t kMergeSmall = uint64_t(1) << 20;
+constexpr uint64_t merge_mid(bool pairs) { return uint64_t(1) << (pairs ? 24 : 22); }
+uint32_t merge_tile_keys(uint32_t shape, uint64_t n, bool pairs) {
+  const uint32_t idx = shape != 0 ? shape - 1 : n <= kMergeSmall ? 1u : n <= merge_mid(pairs) ? 0u : 2u;
   if (idx >= sizeof(kMergeItemsChoice) / sizeof(kMergeItemsChoice[0])) return 0;
   return uint32_t(kMergeThreads * kMergeItemsChoice[idx]);
+}
+
+// Tile boundaries to have space for: those of any merge of at most n outputs
+// with that shape (a workspace for more outputs takes fewer).
+size_t merge_max_tiles(uint32_t shape, uint64_t n, bool pairs) {
+  size_t most = 0;
+  for (uint64_t m : {std::min(n, kMergeSmall), std::min(n, merge_mid(pairs)), n}) {
+    const uint32_t tile = merge_tile_keys(shape, m, pairs);
+    most = std::max(most, size_t((m + tile - 1) / tile));
+  }
+  return most;
 }
 
 cudaError_t launch_merge(const MergeArgs& m, cudaStream_t s) {

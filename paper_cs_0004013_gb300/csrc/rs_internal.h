@@ -310,7 +310,8 @@ struct MergeArgs {
   uint32_t* err;       // device error word
   uint32_t tile;       // outputs per tile (merge_tile_keys of the chosen shape)
 };
-uint32_t merge_tile_keys(uint32_t shape, bool pairs);
+uint32_t merge_tile_keys(uint32_t shape, uint64_t n, bool pairs);
+size_t merge_max_tiles(uint32_t shape, uint64_t n, bool pairs);
 cudaError_t launch_merge(const MergeArgs& m, cudaStream_t s);
 
 cudaError_t launch_split64(const WideArgs& a, unsigned grid, cudaStream_t s);

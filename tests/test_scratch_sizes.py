@@ -30,11 +30,12 @@ def _queries():
         "host": lambda n: rs.rs_sort_u32_host(None, None, None, None, n),
         "host_pairs": lambda n: rs.rs_sort_u32_host(None, 1, None, 2, n),
         "merge": lambda n: rs.rs_merge_u32(None, None, n // 3, None, None, n - n // 3, None, None),
+        "merge_pairs": lambda n: rs.rs_merge_u32(None, 1, n // 3, None, 1, n - n // 3, None, 1),
     }
 
 
 @pytest.mark.parametrize("entry", ["sort", "sort_pairs", "sort_pairs64", "sort64", "sort64_pairs", "sort64_pairs64",
-                                   "host", "host_pairs", "merge"])
+                                   "host", "host_pairs", "merge", "merge_pairs"])
 def test_scratch_never_falls(entry):
     query = _queries()[entry]
     at = _sizes()
