@@ -481,12 +481,12 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
   constexpr int FEW = WARPS < 4 ? WARPS : 4;
   constexpr uint32_t LANES = uint32_t(FEW) * 32;
   const bool looked = Bins::kLook && m > kLookKeys;
-  auto sampled = [&]() {  // (fewer keys than lanes: the lane's own)
+  auto sampled = [&]() {
     const uint32_t q = uint32_t(tid);
-    return m < LANES ? q : q * m / LANES + __umulhi(q * 0x9E3779B1u, m / LANES);
+    return q * m / LANES + __umulhi(q * 0x9E3779B1u, m / LANES);
   };
   auto count_likes = [&](K k, bool live) {
-    if constexpr (!Bins::kKnown) {
+    if constexpr (Bins::kLook) {
       if (warp < FEW) {
         const uint32_t lives = __ballot_sync(0xffffffffu, live);
         const uint32_t b = bins(k);
@@ -661,15 +661,14 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
       stage(first_bin);
     } else if (!Bins::kKnown && !bins.unique()) {
       if constexpr (!Bins::kKnown) {
-        // (a mean of 18 keys leaves some bin of the second set above the limit)
-        if (!looked) {
-          const uint32_t at = sampled();
-          count_likes(warp < FEW && at < m ? ordi.map(ld_elem<COHERENT>(in + at)) : K(0), at < m);
+        constexpr uint32_t LIMIT = 18;  // a mean that leaves some bin of the second set above kBinLimit
+        if (Bins::kLook && !looked && m > 31u * LIMIT) {  // (fewer keys cannot tell)
+          count_likes(key[0], has(0));  // the first lanes' own keys
           __syncthreads();
           likes = read_likes();
           __syncthreads();
         }
-        if (!more_than(18u)) {
+        if (!more_than(LIMIT)) {
           // the second set of bins (see above), NB / m of them to a key;
           // positions among the keys in 16.16 fixed point
           scan();
