@@ -1,6 +1,7 @@
 // C ABI of librsort (declared in include/rsort.h): argument checks, the
 // radix plan, the layout of the caller's temp buffer and the launches.
 #include <algorithm>
+#include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -401,6 +402,14 @@ struct HybLayout {
   }
 };
 
+// Duplicates that a sample of s keys may have when at most c equal keys per
+// value are taken: those of n keys of n / c values (keys beyond the values that
+// the sample meets), and a few.
+uint32_t sample_dups(uint64_t n, uint32_t c, uint32_t s) {
+  const double values = double(n) / c;
+  return uint32_t(double(s) + values * std::expm1(-double(s) / values) + 4.0);
+}
+
 // When the radix passes, which leave out a digit that all keys share, are the
 // faster way for evenly spread keys too.  Measured, us, buckets against radix
 // passes over the digits given (2^23 and 2^24 keys, c equal keys per value):
@@ -416,14 +425,15 @@ struct HybLayout {
 // 240, 14 254 / 240; pairs 12 325 / 362, 14 355 / 362; 64-bit payloads 14 419 /
 // 457, 16 475 / 460; 64-bit keys 20 665 / 740, 2.5M 147 / 215.
 SampleRule hyb_rule(uint64_t n, int kb, int vb) {
+  auto dups = [n](uint32_t c) { return sample_dups(n, c, kSampleKeys); };
   const bool large = n > uint64_t(1) << 22;
   // up to 2^16 keys of 64 bits, or with 64-bit payloads, any number: eight passes
   // of launches are slower than crowded blocks (50,000 keys of 1,000 values 55 / 102)
   const uint32_t wide_dups = n <= uint64_t(1) << 16 ? 1u << 16 : kb == 8 ? 20u : 16u;
   if (kb == 4)
     return SampleRule{vb == 0 ? 1u : vb == 4 || large ? 4u : n > uint64_t(1) << 19 ? 3u : 1u,
-                      vb == 8 && !large ? 16u : 8u, vb == 8 ? wide_dups : 12u};
-  return SampleRule{!large || vb == 8 ? 1u : vb == 4 ? 4u : 3u, 8u, wide_dups};
+                      dups(vb == 8 && !large ? 16u : 8u), dups(vb == 8 ? wide_dups : 12u)};
+  return SampleRule{!large || vb == 8 ? 1u : vb == 4 ? 4u : 3u, dups(8u), dups(wide_dups)};
 }
 // The same for the sorts of one launch.  Keys alone gain or lose little with
 // two digits (277,635 keys 24.5 / 26.6, 50,000 23 / 22), pairs lose: 277,635
@@ -431,8 +441,8 @@ SampleRule hyb_rule(uint64_t n, int kb, int vb) {
 // The largest tiles' pairs lose with any (2.5M: 92 / 86): not offered.
 // c equal keys per value: 2^20 keys c = 10 45 / 43, 12 46 / 43, 50,000 keys 10 19
 // / 26, 12 31 / 26; 277,635 pairs 8 31 / 37, 10 46 / 37, 2^20 pairs 6 47 / 51, 8 67 / 51.
-SampleRule fused_rule(bool pairs, int shape) {
-  const uint32_t dups = !pairs ? 10u : shape == 1 ? 5u : 7u;
+SampleRule fused_rule(uint64_t n, bool pairs, int shape) {
+  const uint32_t dups = sample_dups(n, !pairs ? 10u : shape == 1 ? 5u : 7u, kFusedSampleKeys);
   return SampleRule{!pairs ? 1u : shape == 1 ? 4u : 3u, dups, dups};
 }
 
@@ -963,7 +973,7 @@ rs_status run_fused(const SortPlan& p, const Layout& L, const uint32_t* keys_in,
   a.err = ds->err;
   if (buckets) {
     a.ctrl = hc;
-    a.rule = fused_rule(pairs, shape);
+    a.rule = fused_rule(n, pairs, shape);
     a.buckets = buckets;
     a.counts = reinterpret_cast<uint32_t*>(temp + L.fcounts);
     a.cursors = reinterpret_cast<uint32_t*>(temp + L.fcursors);

@@ -320,9 +320,10 @@ cudaError_t launch_join64(const WideArgs& a, unsigned grid, cudaStream_t s);
 // What the sample of a sort asks of its keys beyond an even spread (sample.cuh).
 struct SampleRule {
   uint32_t min_digits;   // bytes in which the keys differ, at least: fewer radix passes are faster
-  uint32_t narrow_dups;  // equal keys per value, at most, of keys that differ in three bytes or less
+  uint32_t narrow_dups;  // duplicates in the sample, at most, of keys that differ in three bytes or less
   uint32_t dups;         // and of others
 };
+constexpr uint32_t kSampleKeys = 8192, kFusedSampleKeys = 2304;  // the sample's size; in the sorts of one launch
 
 // A whole sort of up to a few million keys in one cooperative launch
 // (fused.cu): 8-bit digits, one 384 x 24, 384 x 20 or 384 x 12 tile per block, every block resident.

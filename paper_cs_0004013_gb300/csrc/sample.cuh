@@ -32,7 +32,8 @@ namespace rs {
 constexpr uint32_t kFineLimit = 12;
 template <typename K, int BLOCKS, int THREADS>
 struct SampleLayout {
-  static constexpr int S = BLOCKS > 1 ? 8192 : 6 * THREADS;
+  static constexpr int S = int(BLOCKS > 1 ? kSampleKeys : kFusedSampleKeys);
+  static_assert(S % (THREADS * BLOCKS) == 0, "whole rows of the sample");
   static constexpr uint32_t COARSE = BLOCKS > 1 ? 64 : 16;            // slices of the range for the evenness test
   static constexpr uint32_t MAXB = BLOCKS > 1 ? kHybMaxBuckets : kFusedMaxBuckets;
   static constexpr int PER = S / THREADS;                       // of the deciding block
@@ -171,10 +172,7 @@ __device__ __forceinline__ void sample_body(const K* in, uint64_t n, uint32_t bu
 #pragma unroll
   for (int i = 0; i < int(sizeof(K)); ++i) digits += ((words[i / 4] >> (8 * (i % 4))) & 0xffu) != 0u;
   if (digits < rule.min_digits) bad = true;
-  // n keys of n / c values give the sample S / (n / c) of each on average, and
-  // as many duplicates as it has keys beyond the values that it meets
-  const float values = float(n) / float(digits <= 3 ? rule.narrow_dups : rule.dups);
-  if (float(dups) > float(L::S) + values * expm1f(-float(L::S) / values) + 4.0f) bad = true;
+  if (dups > (digits <= 3 ? rule.narrow_dups : rule.dups)) bad = true;
   if (tid == 0) {
     HybCtrl* c = ctrl;
     c->lo = m.lo;
