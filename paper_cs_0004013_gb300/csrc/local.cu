@@ -128,8 +128,8 @@ uint32_t local_max_keys(int key_bytes, int val_bytes) { return key_bytes == 4 &&
 
 cudaError_t launch_tiny_segments(const LocalArgs& a, bool pairs, uint32_t num_segs, unsigned few_sms, cudaStream_t s) {
   const Shapes& sh = shapes();
-  return few_sms ? sh.few_tiny[pairs].launch(a, std::min(num_segs, few_sms * 16u), s)  // four times what is resident
-                 : sh.tiny[pairs].launch(a, num_segs, s);
+  const uint32_t few = few_sms * 16u;  // four times what is resident
+  return few_sms && num_segs > few ? sh.few_tiny[pairs].launch(a, few, s) : sh.tiny[pairs].launch(a, num_segs, s);
 }
 cudaError_t launch_small_segments(const LocalArgs& a, bool pairs, uint32_t max_listed, cudaStream_t s) {
   return shapes().small[pairs].launch(a, max_listed, s);
