@@ -424,8 +424,8 @@ uint32_t sample_dups(uint64_t n, uint32_t c, uint32_t s) {
 // some bin, buckets / radix passes behind the sample: 14.7M keys c = 12 228 /
 // 240, 14 254 / 240; pairs 12 325 / 362, 14 355 / 362; 64-bit payloads 14 419 /
 // 457, 16 475 / 460; 64-bit keys 20 665 / 740, 2.5M 147 / 215.
-SampleRule hyb_rule(uint64_t n, int kb, int vb) {
-  auto dups = [n](uint32_t c) { return sample_dups(n, c, kSampleKeys); };
+SampleRule hyb_rule(uint64_t n, uint32_t buckets, int kb, int vb) {
+  auto dups = [=](uint32_t c) { return sample_dups(n, c, hyb_sample_keys(buckets)); };
   const bool large = n > uint64_t(1) << 22;
   // up to 2^16 keys of 64 bits, or with 64-bit payloads, any number: eight passes
   // of launches are slower than crowded blocks (50,000 keys of 1,000 values 55 / 102)
@@ -537,7 +537,7 @@ BucketChain make_chain(HybArgs a, const HybLayout& H, size_t clear_bytes, unsign
   a.groups = H.groups;
   a.bucket_cap = H.shape.bucket_cap;
   a.split_tile = H.shape.split_tile;
-  a.rule = hyb_rule(H.n, key_bytes, val_bytes);
+  a.rule = hyb_rule(H.n, H.buckets, key_bytes, val_bytes);
   a.ctrl = reinterpret_cast<HybCtrl*>(temp + H.ctrl);
   a.counts = reinterpret_cast<uint32_t*>(temp + H.counts);
   a.starts = reinterpret_cast<uint32_t*>(temp + H.starts);

@@ -53,6 +53,8 @@ struct HybArgs {
   uint32_t* err;
 };
 
+// Keys of the sample for so many buckets.
+constexpr uint32_t hyb_sample_keys(uint32_t buckets) { return buckets <= kFusedMaxBuckets ? kFusedSampleKeys : kSampleKeys; }
 enum class HybStep { kSample, kCount, kSplit0, kSplit1, kBuckets };
 struct HybShape {
   uint32_t split_tile;   // keys of a split tile

@@ -22,20 +22,21 @@ namespace rs {
 // evenly when
 //  - no slice of the range (of COARSE) holds more than 1.5 times its share of
 //    the sample (uniform keys: 128 expected, five standard deviations below);
-//  - no bucket holds more than 1.5 times its share of the sample and kFineLimit keys;
+//  - no bucket holds more than 1.5 times its share of the sample and 12 keys (of
+//    the small sample 16: even keys passed it but for one time in 1,000 with 12);
 //  - few sampled keys are equal to another one: many equal keys end up in few
 //    bins of a bucket, which then takes the digit passes;
 //  - the keys differ in enough bytes: the radix passes leave out the others
 //    (hyb_rule in api.cu).
-// In the sorts of one launch (fused.cu) a block of its own takes a quarter of
-// the sample; their buckets are few and large.
-constexpr uint32_t kFineLimit = 12;
+// Where buckets are few, one block takes a sample of about a quarter the size: in
+// the sorts of one launch (fused.cu) and for few buckets of the others.
 template <typename K, int BLOCKS, int THREADS>
 struct SampleLayout {
   static constexpr int S = int(BLOCKS > 1 ? kSampleKeys : kFusedSampleKeys);
   static_assert(S % (THREADS * BLOCKS) == 0, "whole rows of the sample");
   static constexpr uint32_t COARSE = BLOCKS > 1 ? 64 : 16;            // slices of the range for the evenness test
   static constexpr uint32_t MAXB = BLOCKS > 1 ? kHybMaxBuckets : kFusedMaxBuckets;
+  static constexpr uint32_t FINE = BLOCKS > 1 ? 12 : 16;
   static constexpr int PER = S / THREADS;                       // of the deciding block
   static constexpr int LOADS = S / (THREADS * BLOCKS);          // of every block
   static constexpr int SLOT_BITS = BLOCKS > 1 ? 15 : 13;               // hash slots, in the fine counts' place
@@ -124,7 +125,7 @@ __device__ __forceinline__ void sample_body(const K* in, uint64_t n, uint32_t bu
   m.back = 0ull - uint64_t(m.lo) * m.mult;
   bool bad = range <= buckets;
   K diff = 0;
-  const uint32_t fine_limit = kFineLimit + uint32_t(L::S) * 3 / (2 * buckets);
+  const uint32_t fine_limit = L::FINE + uint32_t(L::S) * 3 / (2 * buckets);
 #pragma unroll
   for (int i = 0; i < L::PER; ++i) {
     diff |= key[i] ^ lo;

@@ -178,7 +178,8 @@ def test_two_streams_at_once():
 def _fill_one_bucket(w, bits, mean, count):
     """w with keys from elsewhere moved into a middle bucket until it holds `count`, as the sort will
     see it: the value map of a sample at fixed places, which stay as they are."""
-    n, S = w.size, 8192
+    n = w.size
+    S = 2304 if -(-n // mean) <= 768 else 8192
     q = np.arange(S, dtype=np.uint64)
     m32 = np.uint64(0xFFFFFFFF)
     h = (q * np.uint64(0x9E3779B1)) & m32
