@@ -1993,6 +1993,9 @@ rs_status rs_selftest_route(uint32_t key_bytes, uint32_t val_bytes, uint64_t n, 
   if (st != RS_OK) return st;
   *h_route = RS_ROUTE_FIXED;
   size_t ctrl = 0;  // (no layout starts with it)
+  size_t counts_at = 0;
+  std::vector<uint32_t> counts;  // of the single launch's buckets
+  uint32_t most = 0;
   if (key_bytes == 8) {
     Sort64 o;
     if ((st = plan_sort64(n, int(val_bytes), nullptr, &o)) != RS_OK) return st;
@@ -2010,7 +2013,12 @@ rs_status rs_selftest_route(uint32_t key_bytes, uint32_t val_bytes, uint64_t n, 
     if (n > seg_kernels()->small_max) {
       if (const int sh = fused_shape(o, n, pairs, ds); sh >= 0) {
         const uint32_t tiles = uint32_t((n + fused_tile_keys(sh) - 1) / fused_tile_keys(sh));
-        if (fused_buckets(o.L, tiles, pairs, sh, ds)) ctrl = o.L.fctrl;
+        if (const uint32_t buckets = fused_buckets(o.L, tiles, pairs, sh, ds); buckets) {
+          ctrl = o.L.fctrl;
+          counts_at = o.L.fcounts;
+          counts.resize(buckets);
+          most = fused_bucket_keys(sh);
+        }
       } else if (o.hybrid) {
         ctrl = o.L.hyb.ctrl;
       }
@@ -2021,8 +2029,16 @@ rs_status rs_selftest_route(uint32_t key_bytes, uint32_t val_bytes, uint64_t n, 
   HybCtrl c;
   RS_CUDA(cudaMemcpyAsync(&c, static_cast<const unsigned char*>(temp) + ctrl, sizeof(c), cudaMemcpyDeviceToHost, s),
           "read the sample's choice");
+  if (!counts.empty())
+    RS_CUDA(cudaMemcpyAsync(counts.data(), static_cast<const unsigned char*>(temp) + counts_at, counts.size() * 4,
+                            cudaMemcpyDeviceToHost, s),
+            "read the buckets' counts");
   RS_CUDA(cudaStreamSynchronize(s), "cudaStreamSynchronize");
-  *h_route = c.over ? RS_ROUTE_OVERFULL : c.route == kHybBuckets ? RS_ROUTE_BUCKETS : RS_ROUTE_RADIX;
+  // The counts' last block turns the route of the larger sorts; the single
+  // launch's blocks see for themselves that a bucket holds too many.
+  const bool over = counts.empty() ? c.route == kHybRadix && c.done != 0
+                                   : c.route == kHybBuckets && *std::max_element(counts.begin(), counts.end()) > most;
+  *h_route = over ? RS_ROUTE_OVERFULL : c.route == kHybBuckets ? RS_ROUTE_BUCKETS : RS_ROUTE_RADIX;
   return RS_OK;
 }
 

@@ -161,10 +161,7 @@ __device__ __forceinline__ bool fused_buckets(const FusedArgs& a, uint32_t tile,
   grid_barrier(a.bar, gridDim.x + tiles * barriers++, a.err);
   // 2. the buckets' starts and the tile's own scan; places claimed
   const uint32_t g0 = d0 < B ? __ldcg(a.counts + d0) : 0u, g1 = d0 + 1 < B ? __ldcg(a.counts + d0 + 1) : 0u;
-  if (__syncthreads_or(g0 > FL::BCAP || g1 > FL::BCAP)) {
-    if (tile == 0 && tid == 0) a.ctrl->over = 1u;
-    return false;
-  }
+  if (__syncthreads_or(g0 > FL::BCAP || g1 > FL::BCAP)) return false;
   uint32_t k0 = 0, k1 = 0;
   if (t0) k0 = atomicAdd(a.cursors + d0, t0);
   if (t1) k1 = atomicAdd(a.cursors + d0 + 1, t1);
@@ -357,6 +354,7 @@ __global__ void __launch_bounds__(kFusedThreads, fused_min_blocks(ITEMS)) fused_
 }  // namespace
 
 uint32_t fused_tile_keys(int shape) { return uint32_t(kFusedThreads * kFusedItems[shape]); }
+uint32_t fused_bucket_keys(int shape) { return uint32_t(kFusedThreads * fused_bucket_items(kFusedItems[shape])); }
 
 template <int SH>
 struct FusedShape {

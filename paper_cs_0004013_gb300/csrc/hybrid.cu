@@ -191,10 +191,7 @@ __global__ void __launch_bounds__(kCountThreads, 1) bucket_count_kernel(const Hy
   }
   const bool over = __syncthreads_or(most > a.bucket_cap);
   if (over) {
-    if (tid == 0) {
-      a.ctrl->over = 1u;
-      a.ctrl->route = kHybRadix;
-    }
+    if (tid == 0) a.ctrl->route = kHybRadix;
     return;
   }
   for (uint32_t b = tid; b < B; b += kCountThreads) {

@@ -15,10 +15,9 @@ struct HybCtrl {
   uint64_t lo, hi;     // the value map (hybrid.cu, ValueMap)
   uint32_t sh, mult;
   uint32_t route;
-  uint32_t done;       // count blocks that have finished
+  uint32_t done;       // count blocks that have finished (none when the sample chose the radix passes)
   uint32_t tiles_b;    // tiles of the second split
-  uint32_t over;       // a bucket did not fit the local sort: the radix passes took over
-  uint32_t reserved[6];
+  uint32_t reserved[7];
 };
 static_assert(sizeof(HybCtrl) == 64, "one cache line or less");
 

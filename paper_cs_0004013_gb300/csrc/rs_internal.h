@@ -352,6 +352,7 @@ struct FusedArgs {
 constexpr uint32_t kFusedMaxBuckets = 768;  // value buckets of the launch
 constexpr int kFusedShapes = 3;  // tile shapes of the single-launch sort: 384 x 24, 384 x 20, 384 x 12
 uint32_t fused_tile_keys(int shape);
+uint32_t fused_bucket_keys(int shape);  // keys a bucket takes
 size_t fused_smem(bool pairs, int shape);
 const void* fused_func(bool pairs, int shape);
 cudaError_t launch_fused(const FusedArgs& a, unsigned tiles, bool pairs, int shape, cudaStream_t s);

@@ -182,7 +182,6 @@ __device__ __forceinline__ void sample_body(const K* in, uint64_t n, uint32_t bu
     c->mult = m.mult;
     c->done = 0;
     c->tiles_b = 0;
-    c->over = 0;
     c->route = bad ? kHybRadix : kHybBuckets;
   }
 }
