@@ -98,8 +98,9 @@ typedef struct rs_plan {
  * NULL if not wanted).  num_parts >= 1.  plan may be NULL (automatic): up to
  * 16,384 keys are sorted by one block, up to 2.8 M in one launch, more by
  * value buckets where a sample taken on the device finds the keys spread
- * evenly over their value range, else by the radix passes.  Either way the
- * result is the same.                                                       */
+ * evenly over their value range, else by the radix passes (pairs from 2^22 on).
+ * Either way the result is the same.  With the automatic plan no size query
+ * falls as n grows: a temp for more keys takes fewer.                       */
 rs_status rs_sort_u32(const uint32_t* keys_in, uint32_t* keys_out, uint64_t n,
                       uint32_t num_parts, uint64_t* h_part_offsets,
                       const rs_plan* plan, void* temp, size_t* temp_bytes,
