@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kMergeThreads, PAIRS ? 4 : 6) merge_tile_kerne
     slice_ends(cvb, lb, 128, [&](uint32_t e) { svb[cvb.off + e] = gvb[e]; });
   }
   __syncthreads();  // the ends, and the barrier's start
-  {
+  auto arrived = [&]() {
     uint32_t done = 0;
     for (int i = 0; i < kMergeWaits && !done; ++i)
       asm volatile(
@@ -225,10 +225,14 @@ __global__ void __launch_bounds__(kMergeThreads, PAIRS ? 4 : 6) merge_tile_kerne
           : "=r"(done)
           : "r"(bar)
           : "memory");
-    if (__syncthreads_or(!done)) {
-      if (tid == 0) atomicOr(m.err, kErrTimeout);
-      return;
+    return done;
+  };
+  if (__syncthreads_or(!arrived())) {
+    if (tid == 0) {
+      atomicOr(m.err, kErrTimeout);
+      arrived();  // the copies in flight write this block's shared memory: it is held as long again
     }
+    return;
   }
   // this thread's ITEMS outputs start on the path at diagonal tid * ITEMS
   auto mapped = [&](uint32_t k) { return XF ? to_ordered(k, m.x) : k; };
