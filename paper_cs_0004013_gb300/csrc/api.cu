@@ -421,28 +421,30 @@ uint32_t sample_dups(uint64_t n, uint32_t c, uint32_t s) {
 //   64-bit keys: 5 digits 157-181 / 324-281, a digit less about 47 less; with
 //     32-bit payloads 249-274 / 426-370, a digit 63; with 64-bit ones 281-305 / 659-611.
 // c equal keys per value in all four digits (eight), where more of them crowd
-// some bin, buckets / radix passes behind the sample: 14.7M keys c = 12 228 /
-// 240, 14 254 / 240; pairs 12 325 / 362, 14 355 / 362; 64-bit payloads 14 419 /
-// 457, 16 475 / 460; 64-bit keys 20 665 / 740, 2.5M 147 / 215.
+// some bin, buckets / radix passes behind the sample: 14.7M keys c = 20 187 /
+// 241, 30 225 / 242, 40 258 / 242; pairs 20 292 / 363, 30 322 / 367, 40 383 / 366;
+// 64-bit payloads 2.5M 20 106 / 125, 25 112 / 127, 30 132 / 125; 64-bit keys 20 358 /
+// 750, 30 443 / 755 (with more their number per bucket varies too much).
 SampleRule hyb_rule(uint64_t n, uint32_t buckets, int kb, int vb) {
   auto dups = [=](uint32_t c) { return sample_dups(n, c, hyb_sample_keys(buckets)); };
   const bool large = n > uint64_t(1) << 22;
   // up to 2^16 keys of 64 bits, or with 64-bit payloads, any number: eight passes
   // of launches are slower than crowded blocks (50,000 keys of 1,000 values 55 / 102)
-  const uint32_t wide_dups = n <= uint64_t(1) << 16 ? 1u << 16 : kb == 8 ? 20u : 16u;
+  const uint32_t wide_dups = n <= uint64_t(1) << 16 ? 1u << 16 : kb == 8 ? 28u : 20u;
   if (kb == 4)
     return SampleRule{vb == 0 ? 1u : vb == 4 || large ? 4u : n > uint64_t(1) << 19 ? 3u : 1u,
-                      dups(vb == 8 && !large ? 16u : 8u), dups(vb == 8 ? wide_dups : 12u)};
+                      dups(vb == 8 && !large ? 16u : 8u), dups(vb == 8 ? wide_dups : 28u)};
   return SampleRule{!large || vb == 8 ? 1u : vb == 4 ? 4u : 3u, dups(8u), dups(wide_dups)};
 }
 // The same for the sorts of one launch.  Keys alone gain or lose little with
 // two digits (277,635 keys 24.5 / 26.6, 50,000 23 / 22), pairs lose: 277,635
 // 33-47 / 29 (three digits 30.6 / 37.5), 2^20 66 / 36 (three 47-49 / 47-48, four 47 / 59).
 // The largest tiles' pairs lose with any (2.5M: 92 / 86): not offered.
-// c equal keys per value: 2^20 keys c = 10 45 / 43, 12 46 / 43, 50,000 keys 10 19
-// / 26, 12 31 / 26; 277,635 pairs 8 31 / 37, 10 46 / 37, 2^20 pairs 6 47 / 51, 8 67 / 51.
+// c equal keys per value: 2^20 keys c = 20 31 / 43, 25 44 / 43, 50,000 keys 30 23
+// / 27, 50 34 / 27; 277,635 pairs 20 33 / 37, 30 36 / 37, 40 49 / 37, 2^20 pairs 16 49 /
+// 51, 20 50 / 51, 25 72 / 51.
 SampleRule fused_rule(uint64_t n, bool pairs, int shape) {
-  const uint32_t dups = sample_dups(n, !pairs ? 10u : shape == 1 ? 5u : 7u, kFusedSampleKeys);
+  const uint32_t dups = sample_dups(n, !pairs || shape != 1 ? 20u : 14u, kFusedSampleKeys);
   return SampleRule{!pairs ? 1u : shape == 1 ? 4u : 3u, dups, dups};
 }
 

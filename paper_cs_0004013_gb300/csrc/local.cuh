@@ -24,8 +24,8 @@
 //     rounds (two for c <= 5);
 //  6. out, coalesced.
 // Where (unless the caller's map is known to be even) a bin holds more than
-// kBinLimit keys, the bins are laid again where the keys are: each bin's share of a second set of bins is its share of the
-// keys (its start and count give them), and a key takes the part of that
+// kBinLimit keys, the bins are laid again where the keys are: each bin's share of
+// a second set of bins is its share of the keys (its start and count give them), and a key takes the part of that
 // share that its place inside the bin points to.  This flattens any density
 // that does not change much within a bin (normally distributed floats, wide
 // clusters).  Blocks that are crowded still, or that a sample shows to be, sort
@@ -45,8 +45,12 @@
 
 namespace rs {
 
-constexpr uint32_t kBinLimit = 29;  // eight rounds of windows
-constexpr uint32_t kCrowded = 24;   // mean keys per bin that a small sample shows well enough
+// Keys in the fullest bin: above kBinLimit (eight rounds of windows) the second
+// set of bins is laid where there is one; above kLastLimit (sixteen rounds) the
+// digit passes take over.  16,000 keys of 1,000 values: digit passes above 29 keys
+// 43 us, above 61 18; 14.7M keys of as many values as give 14 to each 254 and 172.
+constexpr uint32_t kBinLimit = 29, kLastLimit = 61;
+constexpr uint32_t kCrowded = 40;  // mean keys per bin that leave some bin above kLastLimit
 // Arrays of more keys are looked at before their bins are laid (up to 0.3 us;
 // 16,000 keys of 8 values 32 us -> 25, 4,000 even ones 4.0 -> 4.4).
 constexpr uint32_t kLookKeys = 4096;
@@ -569,7 +573,7 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
 
   // 2. turns within the bins.  Word w of the counts holds bin w in its low and
   // bin w + NB / 2 in its high half; four 8-bit turns go to a register (a
-  // turn above kBinLimit sends the block another way, so its low bits may be
+  // turn above kLastLimit sends the block another way, so its high bits may be
   // lost).  Returns the fullest bin's keys, five at least.
   const uint32_t bin_base = static_cast<uint32_t>(__cvta_generic_to_shared(s_bin));
   uint32_t turn[(ITEMS + 3) / 4];
@@ -655,20 +659,19 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
     most = count(first_bin);
     // bins of one value need no order among equal keys (as long as their turns fit their 8 bits)
     if (VB == 0 && bins.unique() && most <= 256u) most = 1u;
-    staged = most <= kBinLimit;
+    staged = most <= (Bins::kKnown ? kLastLimit : kBinLimit);
     if (staged) {
       scan();
       stage(first_bin);
     } else if (!Bins::kKnown && !bins.unique()) {
       if constexpr (!Bins::kKnown) {
-        constexpr uint32_t LIMIT = 18;  // a mean that leaves some bin of the second set above kBinLimit
-        if (Bins::kLook && !looked && m > 31u * LIMIT) {  // (fewer keys cannot tell)
+        if (Bins::kLook && !looked && m > 31u * kCrowded) {  // (fewer keys cannot tell)
           count_likes(key[0], has(0));  // the first lanes' own keys
           __syncthreads();
           likes = read_likes();
           __syncthreads();
         }
-        if (!more_than(LIMIT)) {
+        if (!more_than(kCrowded)) {
           // the second set of bins (see above), NB / m of them to a key;
           // positions among the keys in 16.16 fixed point
           scan();
@@ -686,7 +689,7 @@ __device__ __forceinline__ void local_sort_array(const typename OrdI::Key* in, t
           __syncthreads();
           auto second_bin = [&](int j) { return bin2[j]; };
           most = count(second_bin);
-          staged = most <= kBinLimit;
+          staged = most <= kLastLimit;
           if (staged) {
             scan();
             stage(second_bin);
