@@ -1678,14 +1678,11 @@ rs_status rs_sort_u32_segmented(const uint32_t* keys_in, const uint32_t* vals_in
   if (num_parts < 1) return fail(RS_ERR_INVALID, "num_parts must be >= 1");
   if (num_segs > 0 && !h_seg_offsets) return fail(RS_ERR_INVALID, "h_seg_offsets is NULL");
   if (total_n >= (uint64_t(1) << 32)) return fail(RS_ERR_INVALID, "total_n must be below 2^32");
-  uint32_t tiny = 0;  // segments of the smallest class
   if (num_segs > 0) {
     if (h_seg_offsets[0] != 0 || h_seg_offsets[num_segs] != total_n)
       return fail(RS_ERR_INVALID, "segment offsets must start at 0 and end at total_n");
     for (uint32_t i = 0; i < num_segs; ++i) {
       if (h_seg_offsets[i + 1] < h_seg_offsets[i]) return fail(RS_ERR_INVALID, "segment offsets decrease at %u", i);
-      const uint64_t m = h_seg_offsets[i + 1] - h_seg_offsets[i];
-      tiny += m > 0 && m <= seg_kernels()->tiny_max;
     }
   }
   const rs_plan eff = resolve_plan(pairs ? RS_ENTRY_SEGMENTED_PAIRS : RS_ENTRY_SEGMENTED,
@@ -1732,9 +1729,15 @@ rs_status rs_sort_u32_segmented(const uint32_t* keys_in, const uint32_t* vals_in
             "launch seg_part_offsets");
   }
   if (total_n == 0) return RS_OK;
+  // whether fewer than half are of the smallest class, from 256 of them (it only picks a grid)
+  uint32_t seen = 0, tiny = 0;
+  for (uint32_t i = 0, step = num_segs / 256 + 1; i < num_segs; i += step, ++seen) {
+    const uint64_t m = h_seg_offsets[i + 1] - h_seg_offsets[i];
+    tiny += m > 0 && m <= seg_kernels()->tiny_max;
+  }
   return run_segmented(L, static_cast<unsigned char*>(temp), keys_in, pairs ? vals_in : nullptr, keys_out,
                        pairs ? vals_out : nullptr, d_seg_offsets, num_segs, total_n, 4, xf, xf, ds, s,
-                       tiny < num_segs / 2, small_max);
+                       2 * tiny < seen, small_max);
 }
 
 rs_status rs_digit_histograms(const uint32_t* keys, uint64_t n, uint32_t digit_bits, uint32_t* d_hist,
